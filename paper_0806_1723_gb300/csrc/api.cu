@@ -230,8 +230,7 @@ struct lasto_poisson {
     int device = 0;
     char* pool = nullptr;
     size_t pool_bytes = 0;
-    double* quad = nullptr;
-    int nq = 0;
+    SphereRule rule;                     // the sphere quadrature of the projection
     cudaStream_t cs = nullptr, cs2 = nullptr, cs3 = nullptr;
     cudaEvent_t ev_origin = nullptr;
     // per batch slot: the cluster's branch stream, its setup stream and fork/join/done events
@@ -864,7 +863,7 @@ int enqueue_finish(lasto_poisson* h, ClusterPlan& P, const lasto_cluster& cl, do
     const LevelT<double> V = F.view64();
     const bool dc = is_defect_correction(h);
     if (!dc) TRY(launch_resid_norm(V, F.u, F.b, nullptr, nullptr, 0u, P.red(FIN_TRUE), s));
-    TRY(launch_project(cl.n, cl.x, cl.y, cl.z, F.u, cl.n_atoms, cl.pos, cl.R, h->quad, h->nq, vlm, P.status, s));
+    TRY(launch_project(cl.n, cl.x, cl.y, cl.z, F.u, cl.n_atoms, cl.pos, cl.R, h->rule, vlm, P.status, s));
     if (potential) TRY(cudaMemcpyAsync(potential, F.u, sizeof(double) * F.N(), cudaMemcpyDeviceToDevice, s));
     k_write_stats<<<1, 1, 0, s>>>(P.ctl, P.status, P.gl >= 0 ? 1 : 0, dc ? 1 : 0, P.stats_dev);
     TRY(cudaGetLastError());
@@ -1458,12 +1457,8 @@ int lasto_poisson_create(const lasto_config* cfg, lasto_poisson** out)
         delete h;
         return e == cudaErrorMemoryAllocation ? LASTO_ERR_NO_MEMORY : LASTO_ERR_CUDA;
     }
-    h->nq = cfg->n_theta * cfg->n_phi;
-    std::vector<double> tab((size_t)h->nq * 28);
-    host_quadrature(cfg->n_theta, cfg->n_phi, tab.data());
-    e = cudaMalloc(&h->quad, sizeof(double) * tab.size());
-    if (e == cudaSuccess) e = cudaMemcpy(h->quad, tab.data(), sizeof(double) * tab.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->cs, cudaStreamNonBlocking);
+    h->rule = sphere_rule(cfg->n_theta, cfg->n_phi);
+    e = cudaStreamCreateWithFlags(&h->cs, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->cs2, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->cs3, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_origin, cudaEventDisableTiming);
@@ -1504,7 +1499,6 @@ void lasto_poisson_destroy(lasto_poisson* h)
     if (h->exec) cudaGraphExecDestroy(h->exec);
     if (h->graph) cudaGraphDestroy(h->graph);
     if (h->pool) cudaFree(h->pool);
-    if (h->quad) cudaFree(h->quad);
     if (h->stats_pinned) cudaFreeHost(h->stats_pinned);
     if (h->cs) cudaStreamDestroy(h->cs);
     if (h->cs2) cudaStreamDestroy(h->cs2);
@@ -2026,16 +2020,8 @@ int lasto_op_project(const int n[3], const double* x, const double* y, const dou
     if (!op_grid_ok(n, x, y, z) || !u || n_atoms < 0 || (n_atoms > 0 && (!pos || !R || !vlm)) || n_theta < 1 ||
         n_theta > 32 || n_phi < 1 || n_phi > 64)
         return LASTO_ERR_INVALID_ARG;
-    cudaStream_t s = (cudaStream_t)stream;
-    const int nq = n_theta * n_phi;
-    std::vector<double> tab((size_t)nq * 28);
-    host_quadrature(n_theta, n_phi, tab.data());
-    Scratch q(sizeof(double) * tab.size(), s);
-    if (!q.p) return LASTO_ERR_NO_MEMORY;
-    cudaError_t e = cudaMemcpyAsync(q.p, tab.data(), sizeof(double) * tab.size(), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e == cudaSuccess) e = launch_project(n, x, y, z, u, n_atoms, pos, R, q.as<double>(), nq, vlm, status, s);
-    return op_status(e);
+    return op_status(launch_project(n, x, y, z, u, n_atoms, pos, R, sphere_rule(n_theta, n_phi), vlm, status,
+                                    (cudaStream_t)stream));
 }
 
 int lasto_op_sphere_density(const lasto_cluster* cl, int n_rad, double r_min, int n_theta, int n_phi, double* rho_lm,
@@ -2049,19 +2035,13 @@ int lasto_op_sphere_density(const lasto_cluster* cl, int n_rad, double r_min, in
         if (cl->n[d] < 5) return LASTO_ERR_INVALID_ARG;
     init_device_constants();
     cudaStream_t s = (cudaStream_t)stream;
-    const int nq = n_theta * n_phi;
-    std::vector<double> tab((size_t)nq * 28);
-    host_quadrature(n_theta, n_phi, tab.data());
-    Scratch q(sizeof(double) * tab.size(), s);
+    const SphereRule& q = sphere_rule(n_theta, n_phi);
     Scratch rec(sizeof(double) * SPHERE_REC_DOUBLES * (size_t)cl->n_atoms, s);
-    if (!q.p || !rec.p) return LASTO_ERR_NO_MEMORY;
-    cudaError_t e = cudaMemcpyAsync(q.p, tab.data(), sizeof(double) * tab.size(), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (!rec.p) return LASTO_ERR_NO_MEMORY;
+    cudaError_t e = launch_sphere_params(*cl, cl->x, cl->y, cl->z, rec.as<double>(), nullptr, nullptr, nullptr,
+                                         nullptr, status, s);
     if (e == cudaSuccess)
-        e = launch_sphere_params(*cl, cl->x, cl->y, cl->z, rec.as<double>(), nullptr, nullptr, nullptr, nullptr,
-                                 status, s);
-    if (e == cudaSuccess)
-        e = launch_sphere_density(cl->n_atoms, rec.as<double>(), cl->c_lm, q.as<double>(), nq, n_rad, r_min, rho_lm, s);
+        e = launch_sphere_density(cl->n_atoms, rec.as<double>(), cl->c_lm, q, n_rad, r_min, rho_lm, s);
     return op_status(e);
 }
 

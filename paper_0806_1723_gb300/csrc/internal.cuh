@@ -15,7 +15,6 @@ namespace lasto {
 constexpr int NLM = 25;
 constexpr int MAX_LEVELS = 10;
 constexpr int MAX_COARSE = 9;        // nodes per axis on the coarsest level
-constexpr int MAX_QUAD = 2048;       // n_theta * n_phi
 constexpr int RED_THREADS = 256;     // block size of reducing kernels
 constexpr double PI = 3.141592653589793238462643383279502884;
 
@@ -56,6 +55,19 @@ void host_monomials(Mono* out);      // the 56 terms, coefficients in FP64
 void host_solid_harmonics(double x, double y, double z, double* S);
 
 __host__ __device__ __forceinline__ int l_of_lm(int lm) { return lm >= 16 ? 4 : lm >= 9 ? 3 : lm >= 4 ? 2 : lm >= 1 ? 1 : 0; }
+
+// ---------------------------------------------------------------- sphere quadrature
+// Gauss-Legendre in cos(theta) x uniform phi: point (a, b) is (st_a cos phi_b, st_a sin phi_b,
+// ct_a); wf[a][slot(l, m)] = w_a f_lm(theta_a), f_lm = y_lm at phi = 0, m >= 0; trig[2b] = cos
+// phi_b, trig[2b + 1] = sin phi_b.  Passed to the kernels by value.
+constexpr int RULE_NT = 32, RULE_NP = 64;   // largest n_theta, n_phi
+struct SphereRule {
+    int nt, np;
+    double ct[RULE_NT], st[RULE_NT];
+    double wf[RULE_NT][15];
+    double trig[2 * RULE_NP];
+};
+__host__ __device__ constexpr int rule_slot(int l, int m) { return l * (l + 1) / 2 + m; }
 
 // ---------------------------------------------------------------- FP32 point update
 // u = acc / (-dsum) of a red-black FP32 update as acc times the hardware's approximate
@@ -366,8 +378,8 @@ cudaError_t launch_raw_sphere_params(const RawArgs& a, double* rec, int* status,
 cudaError_t launch_raw_deposit(const RawArgs& a, const double* rec, double* b, int* owner, int* status, cudaStream_t s);
 
 // inner.cu: inside the spheres (Eq. 3.4-3.7)
-cudaError_t launch_sphere_density(int na, const double* rec, const double* clm, const double* quad, int nq,
-                                  int n_rad, double r_min, double* out, cudaStream_t s);
+cudaError_t launch_sphere_density(int na, const double* rec, const double* clm, const SphereRule& q, int n_rad,
+                                  double r_min, double* out, cudaStream_t s);
 cudaError_t launch_inner_solve(int na, const double* R, const double* Z, int n_rad, double r_min,
                                const double* rho_lm, const double* vR, double* v, cudaStream_t s);
 
@@ -409,10 +421,10 @@ cudaError_t launch_resample(const int na[3], const double* ax, const double* ay,
                             int interior_only, cudaStream_t s);
 
 // project.cu
-void host_quadrature(int n_theta, int n_phi, double* table /* [nq][28]: unit xyz, w*S_lm */);
+const SphereRule& sphere_rule(int n_theta, int n_phi);   // valid until this thread asks for another
 cudaError_t launch_project(const int n[3], const double* x, const double* y, const double* z, const double* u,
-                           int n_atoms, const double* pos, const double* R, const double* quad, int nq,
-                           double* vlm, int* status, cudaStream_t s);
+                           int n_atoms, const double* pos, const double* R, const SphereRule& q, double* vlm,
+                           int* status, cudaStream_t s);
 
 // ---------------------------------------------------------------- lockstep batches (mg.cu)
 // Clusters whose grids have the same shape advance together: each kernel of the FP32 cycle and
