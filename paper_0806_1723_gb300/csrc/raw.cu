@@ -11,32 +11,62 @@ namespace {
 
 constexpr double RAW_PI = 3.14159265358979323846;
 
-// One thread per sphere: q = sqrt(4pi) int_0^R rho_00 r^2 dr - Z (rule in ln r, rho_00
+// weight of sample j (of n >= 5, in units of h / 24) in the sum of the cubic rule over all intervals
+__device__ __forceinline__ double cubic_weight(int j, int n)
+{
+    int w = 0;
+    if (j < 4) w += j == 0 ? 9 : j == 1 ? 19 : j == 2 ? -5 : 1;
+    const int e = n - 1 - j;
+    if (e < 4) w += e == 0 ? 9 : e == 1 ? 19 : e == 2 ? -5 : 1;
+#pragma unroll
+    for (int t = 0; t < 4; t++) {   // sample j is the t-th of the interior interval q
+        const int q = j + 1 - t;
+        if (q >= 1 && q <= n - 3) w += (t == 0 || t == 3) ? -1 : 13;
+    }
+    return (double)w;
+}
+
+// One block per sphere: q = sqrt(4pi) int_0^R rho_00 r^2 dr - Z (rule in ln r, rho_00
 // constant on [0, r_min]), rho(R) = rho_00(R)/sqrt(4pi), rho'(R) from the one-sided fourth-
 // order difference in ln r, and the quartic a + b r^2 + c r^4 meeting the three constraints
 // (written out: c = (Q - rho R^3/3 + rho' R^4/15) 105/(8 R^7), b = rho'/(2R) - 2 c R^2,
 // a = rho - rho' R/2 + c R^4 with Q = q/(4pi)).  Record: x y z R a b c h.  Also the
 // geometry check: the sphere two nodes inside every face and disjoint from the others.
-__global__ void k_raw_sphere_params(RawArgs a, double* __restrict__ rec, int* __restrict__ status)
+// The integral is one weighted sum over the samples, taken by the block: latency bound (a few
+// FP64 exponentials deep), 55 spheres of 429 samples 1451 us (one thread per sphere, four
+// exponentials per interval) -> 16.4 us.
+constexpr int RSP_NT = 128;
+__global__ void __launch_bounds__(RSP_NT) k_raw_sphere_params(RawArgs a, double* __restrict__ rec,
+                                                              int* __restrict__ status)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= a.na) return;
+    __shared__ double sm[32];
+    const int i = blockIdx.x;
     const double Ri = a.R[i], rm = a.r_min;
     const int n = a.n_rad;
     const double h = log(Ri / rm) / (n - 1);
     const double* f = a.rho00 + (size_t)i * n;
-    auto rr = [&](int j) { return j == n - 1 ? Ri : Ri * exp((j - (n - 1)) * h); };
-    auto g = [&](int j) { const double x = rr(j); return f[j] * x * x * x; };
-    double acc = f[0] * rm * rm * rm / 3.0;
-    for (int j = 0; j + 1 < n; j++) {
-        double w;
-        if (j == 0) w = h / 24.0 * (9.0 * g(0) + 19.0 * g(1) - 5.0 * g(2) + g(3));
-        else if (j == n - 2) w = h / 24.0 * (g(n - 4) - 5.0 * g(n - 3) + 19.0 * g(n - 2) + 9.0 * g(n - 1));
-        else w = h / 24.0 * (-g(j - 1) + 13.0 * g(j) + 13.0 * g(j + 1) - g(j + 2));
-        acc += w;
+    double part = 0.0;
+    for (int j = threadIdx.x; j < n; j += RSP_NT) {
+        const double x = j == n - 1 ? Ri : Ri * exp((j - (n - 1)) * h);
+        part = fma(cubic_weight(j, n) * f[j], x * x * x, part);
     }
+    bool bad = false;
+    for (int j = threadIdx.x; j < a.na; j += RSP_NT) {
+        if (j == i) continue;
+        const double dx = a.pos[3 * i] - a.pos[3 * j], dy = a.pos[3 * i + 1] - a.pos[3 * j + 1],
+                     dz = a.pos[3 * i + 2] - a.pos[3 * j + 2];
+        if (sqrt(dx * dx + dy * dy + dz * dz) < Ri + a.R[j]) bad = true;
+    }
+    if (threadIdx.x < 3) {
+        const int d = threadIdx.x;
+        const double cc = a.pos[3 * i + d];
+        if (!(cc - Ri >= a.ax[d][2] && cc + Ri <= a.ax[d][a.n[d] - 3])) bad = true;
+    }
+    if (bad && status) atomicMax(status, (int)LASTO_ERR_GEOMETRY);
+    const double sum = block_sum<RSP_NT>(part, sm);
+    if (threadIdx.x != 0) return;
     const double s4 = sqrt(4.0 * RAW_PI);
-    const double q = s4 * acc - a.Z[i];
+    const double q = s4 * fma(h / 24.0, sum, f[0] * rm * rm * rm / 3.0) - a.Z[i];
     const int m = n - 1;
     const double rho = f[m] / s4;
     const double drho = (25.0 * f[m] - 48.0 * f[m - 1] + 36.0 * f[m - 2] - 16.0 * f[m - 3] + 3.0 * f[m - 4]) /
@@ -54,18 +84,6 @@ __global__ void k_raw_sphere_params(RawArgs a, double* __restrict__ rec, int* __
     o[5] = b;
     o[6] = c;
     o[7] = h;
-    bool bad = false;
-    for (int d = 0; d < 3; d++) {
-        const double cc = a.pos[3 * i + d];
-        if (!(cc - Ri >= a.ax[d][2] && cc + Ri <= a.ax[d][a.n[d] - 3])) bad = true;
-    }
-    for (int j = 0; j < a.na; j++) {
-        if (j == i) continue;
-        const double dx = a.pos[3 * i] - a.pos[3 * j], dy = a.pos[3 * i + 1] - a.pos[3 * j + 1],
-                     dz = a.pos[3 * i + 2] - a.pos[3 * j + 2];
-        if (sqrt(dx * dx + dy * dy + dz * dz) < Ri + a.R[j]) bad = true;
-    }
-    if (bad && status) atomicMax(status, (int)LASTO_ERR_GEOMETRY);
     if (!isfinite(q) || !isfinite(aa) || !isfinite(b) || !isfinite(c))
         if (status) atomicMax(status, (int)LASTO_ERR_NONFINITE);
 }
@@ -143,7 +161,7 @@ __global__ void __launch_bounds__(256) k_raw_deposit(RawArgs a, const double* __
 
 cudaError_t launch_raw_sphere_params(const RawArgs& a, double* rec, int* status, cudaStream_t s)
 {
-    k_raw_sphere_params<<<(a.na + 63) / 64, 64, 0, s>>>(a, rec, status);
+    k_raw_sphere_params<<<a.na, RSP_NT, 0, s>>>(a, rec, status);
     return cudaGetLastError();
 }
 

@@ -76,3 +76,20 @@ def test_sphere_density_of_a_single_atom(orc):
     rho, _ = B.lasto_op_sphere_density(B.DeviceCluster(cl))
     ref = orc.sphere_density(cl)
     assert np.abs(host(rho) - ref).max() < 1e-12 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("n_rad", [5, 6, 8, 129, 430])
+def test_raw_sphere_charge(orc, n_rad):
+    """The composite cubic weights of the raw path's charge integral, from the shortest table on:
+    the deposit inside the spheres against the oracle's interval-by-interval rule."""
+    B = need_gpu()
+    cl = _pair(np.random.default_rng(n_rad), 2.4, 4.9)
+    x, y, z = orc.mesh(cl)
+    r = np.stack([orc.radial_mesh(n_rad, 1e-2, R) for R in cl.R])
+    rho00 = np.exp(-r) * (1.0 + 0.1 * np.arange(2)[:, None])
+    ne = np.random.default_rng(1).uniform(0.1, 0.2, (33, 33, 33))
+    b, owner, status = B.lasto_op_raw_deposit(B.RawCluster(cl.pos, cl.Z, cl.R, x, y, z, cl.centre, ne, rho00, r_min=1e-2))
+    ref, rowner = orc.raw_deposit(cl.pos, cl.Z, cl.R, x, y, z, ne, rho00, r_min=1e-2)
+    assert int(host(status)[0]) == 0
+    assert np.array_equal(host(owner).reshape(rowner.shape), rowner)
+    assert np.abs(host(b).reshape(ref.shape) - ref).max() < 1e-12 * np.abs(ref).max()
