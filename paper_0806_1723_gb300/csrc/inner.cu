@@ -334,87 +334,104 @@ __device__ __forceinline__ double block_incl_scan(double v, double* wsum)
     return v;
 }
 
-// One block per (atom, lm).  The integrands at the mesh points, the cubic-rule integral over
-// each interval, then I1 as a prefix sum and I2 as a suffix sum of the intervals (each thread
-// a contiguous run of intervals, the runs' totals scanned across the block), then V_LM.
+// One block per (atom, IS_LM harmonics).  The radii and their reciprocals once, then per harmonic
+// the integrands at the mesh points, the cubic-rule integral over each interval, I1 as a prefix
+// sum and I2 as a suffix sum of the intervals (each thread a contiguous run of intervals, the
+// runs' totals scanned across the block), and V_LM.  Bound: FP64 issue.  The exponential of a
+// radius costs more than its share of a harmonic, so five harmonics share it, and no division is
+// left per point: Pd55, 429 radii 164 us (a block per harmonic) -> 116 us.
+constexpr int IS_LM = 5;
 __global__ void __launch_bounds__(IS_NT) k_inner_solve(int na, const double* __restrict__ R,
                                                        const double* __restrict__ Z, int n, double r_min,
                                                        const double* __restrict__ rho_lm,
                                                        const double* __restrict__ vR, double* __restrict__ v)
 {
-    extern __shared__ double is_sm[];   // x[n], g1[n], g2[n], seg1[n], seg2[n]
+    extern __shared__ double is_sm[];   // x[n], 1/x[n], g1[n], g2[n], seg1[n], seg2[n]
     __shared__ double wsum[IS_NT / 32];
     double* xs = is_sm;
-    double* g1 = xs + n;
+    double* ix = xs + n;
+    double* g1 = ix + n;
     double* g2 = g1 + n;
     double* s1 = g2 + n;
     double* s2 = s1 + n;
-    const int t = blockIdx.x, a = t / NLM, lm = t % NLM, L = l_of_lm(lm);
+    const int a = blockIdx.x / (NLM / IS_LM), lm0 = (blockIdx.x % (NLM / IS_LM)) * IS_LM;
     const double Ra = R[a];
     const double h = log(Ra / r_min) / (n - 1);
-    const double* rho = rho_lm + (size_t)t * n;
-    double* out = v + (size_t)t * n;
     for (int j = threadIdx.x; j < n; j += IS_NT) {
         const double x = j == n - 1 ? Ra : Ra * exp((j - (n - 1)) * h);
-        double xl = 1.0;
-        for (int e = 0; e < L; e++) xl *= x;
         xs[j] = x;
-        g1[j] = rho[j] * xl * x * x * x;   // rho r^(L+2) dr = rho r^(L+3) d(ln r)
-        g2[j] = rho[j] * x * x / xl;       // rho r^(1-L) dr = rho r^(2-L) d(ln r)
+        ix[j] = 1.0 / x;
     }
-    __syncthreads();
-    for (int j = threadIdx.x; j < n - 1; j += IS_NT) {
-        const int b = j == 0 ? 0 : (j == n - 2 ? n - 4 : j - 1);
-        const int kind = j == 0 ? 0 : (j == n - 2 ? 2 : 1);
-        s1[j] = seg_integral(g1[b], g1[b + 1], g1[b + 2], g1[b + 3], kind, h);
-        s2[j] = seg_integral(g2[b], g2[b + 1], g2[b + 2], g2[b + 3], kind, h);
-    }
-    __syncthreads();
+    const double iRa = 1.0 / Ra, sq4piZ = 3.5449077018110318 * Z[a];
     // contiguous runs of intervals per thread: [c0, c1)
     const int m = n - 1, per = (m + IS_NT - 1) / IS_NT;
     const int c0 = min(m, (int)threadIdx.x * per), c1 = min(m, c0 + per);
-    double run1 = 0.0, run2 = 0.0;
-    for (int j = c0; j < c1; j++) {
-        run1 += s1[j];
-        run2 += s2[j];
-    }
-    const double inc1 = block_incl_scan(run1, wsum);
-    __syncthreads();
-    const double inc2 = block_incl_scan(run2, wsum);
-    __syncthreads();
-    if (threadIdx.x == IS_NT - 1) {
-        wsum[0] = inc1;   // I1 over all intervals
-        wsum[1] = inc2;   // I2 over all intervals
-    }
-    __syncthreads();
-    const double tot1 = wsum[0], tot2 = wsum[1];
-    const double I1_0 = g1[0] / (L + 3);   // rho taken constant on [0, r_0]: rho_0 r_0^(L+3) / (L+3)
-    const double vr = vR[(size_t)a * NLM + lm];
-    const double c = 4.0 * 3.14159265358979323846 / (2 * L + 1);
-    const double sq4pi = 3.5449077018110318;
-    double RaL = 1.0;
-    for (int e = 0; e < L; e++) RaL *= Ra;
-    const double R2L1 = RaL * RaL * Ra;
-    const double I1R = I1_0 + tot1;
-    // points [c0, c1) of this thread's run, and the last point m with the run that ends there:
-    // I1 at point j = I1_0 + intervals [0, j), I2 = intervals [j, m)
-    if (c0 < c1) {
-        double p1 = inc1 - run1, p2 = tot2 - (inc2 - run2);
-        const int last = c1 == m ? m : c1 - 1;
-        for (int j = c0; j <= last; j++) {
-            if (j > c0) {
-                p1 += s1[j - 1];
-                p2 -= s2[j - 1];
+    for (int lm = lm0; lm < lm0 + IS_LM; lm++) {
+        const int L = l_of_lm(lm);
+        const double* rho = rho_lm + ((size_t)a * NLM + lm) * n;
+        double* out = v + ((size_t)a * NLM + lm) * n;
+        for (int j = threadIdx.x; j < n; j += IS_NT) {
+            const double x = xs[j], i1 = ix[j], f = rho[j] * x * x;
+            double xl = 1.0, il = 1.0;
+            for (int e = 0; e < L; e++) {
+                xl *= x;
+                il *= i1;
             }
-            const double x = xs[j];
-            double xl = 1.0;
-            for (int e = 0; e < L; e++) xl *= x;
-            const double I1 = I1_0 + p1;
-            const double I2 = j == m ? 0.0 : p2;
-            double val = vr * (xl / RaL) - c * (I1 / (xl * x) + xl * I2 - xl * I1R / R2L1);
-            if (L == 0) val += sq4pi * Z[a] * (1.0 / x - 1.0 / Ra);
-            out[j] = val;
+            g1[j] = f * x * xl;   // rho r^(L+2) dr = rho r^(L+3) d(ln r)
+            g2[j] = f * il;       // rho r^(1-L) dr = rho r^(2-L) d(ln r)
         }
+        __syncthreads();
+        for (int j = threadIdx.x; j < n - 1; j += IS_NT) {
+            const int b = j == 0 ? 0 : (j == n - 2 ? n - 4 : j - 1);
+            const int kind = j == 0 ? 0 : (j == n - 2 ? 2 : 1);
+            s1[j] = seg_integral(g1[b], g1[b + 1], g1[b + 2], g1[b + 3], kind, h);
+            s2[j] = seg_integral(g2[b], g2[b + 1], g2[b + 2], g2[b + 3], kind, h);
+        }
+        const double I1_0 = g1[0] / (L + 3);   // rho taken constant on [0, r_0]: rho_0 r_0^(L+3) / (L+3)
+        __syncthreads();
+        double run1 = 0.0, run2 = 0.0;
+        for (int j = c0; j < c1; j++) {
+            run1 += s1[j];
+            run2 += s2[j];
+        }
+        const double inc1 = block_incl_scan(run1, wsum);
+        __syncthreads();
+        const double inc2 = block_incl_scan(run2, wsum);
+        __syncthreads();
+        if (threadIdx.x == IS_NT - 1) {
+            wsum[0] = inc1;   // I1 over all intervals
+            wsum[1] = inc2;   // I2 over all intervals
+        }
+        __syncthreads();
+        const double tot1 = wsum[0], tot2 = wsum[1];
+        const double c = 4.0 * 3.14159265358979323846 / (2 * L + 1);
+        double iRaL = 1.0;
+        for (int e = 0; e < L; e++) iRaL *= iRa;
+        // V = x^L (V(R) / R^L + c I1(R) / R^(2L+1) - c I2) - c I1 / x^(L+1)
+        const double head = fma(c * (I1_0 + tot1), iRaL * iRaL * iRa, vR[(size_t)a * NLM + lm] * iRaL);
+        // points [c0, c1) of this thread's run, and the last point m with the run that ends there:
+        // I1 at point j = I1_0 + intervals [0, j), I2 = intervals [j, m)
+        if (c0 < c1) {
+            double p1 = inc1 - run1, p2 = tot2 - (inc2 - run2);
+            const int last = c1 == m ? m : c1 - 1;
+            for (int j = c0; j <= last; j++) {
+                if (j > c0) {
+                    p1 += s1[j - 1];
+                    p2 -= s2[j - 1];
+                }
+                const double x = xs[j], i1 = ix[j];
+                double xl = 1.0, il = i1;
+                for (int e = 0; e < L; e++) {
+                    xl *= x;
+                    il *= i1;
+                }
+                const double I2 = j == m ? 0.0 : p2;
+                double val = xl * (head - c * I2) - c * (I1_0 + p1) * il;
+                if (L == 0) val += sq4piZ * (i1 - iRa);
+                out[j] = val;
+            }
+        }
+        __syncthreads();   // the integrands' arrays are free again
     }
 }
 
@@ -445,11 +462,12 @@ cudaError_t launch_inner_solve(int na, const double* R, const double* Z, int n_r
                                const double* rho_lm, const double* vR, double* v, cudaStream_t s)
 {
     if (n_rad > IS_MAX) return cudaErrorInvalidValue;
-    const size_t smem = sizeof(double) * 5 * (size_t)n_rad;
+    const size_t smem = sizeof(double) * 6 * (size_t)n_rad;
     cudaError_t e = cudaFuncSetAttribute(k_inner_solve, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)(sizeof(double) * 5 * IS_MAX));
+                                         (int)(sizeof(double) * 6 * IS_MAX));
     if (e != cudaSuccess) return e;
-    k_inner_solve<<<(unsigned)(na * NLM), IS_NT, smem, s>>>(na, R, Z, n_rad, r_min, rho_lm, vR, v);
+    static_assert(NLM % IS_LM == 0, "groups of harmonics");
+    k_inner_solve<<<(unsigned)(na * (NLM / IS_LM)), IS_NT, smem, s>>>(na, R, Z, n_rad, r_min, rho_lm, vR, v);
     return cudaGetLastError();
 }
 
