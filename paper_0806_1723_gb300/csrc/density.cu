@@ -29,13 +29,11 @@ namespace lasto {
 // ---------------------------------------------------------------- harmonics table
 static __constant__ Mono c_mono[N_MONO_TERMS];
 
-// double-float copies for the FP32-pair deposit
-struct MonoF {
-    int lm, a, b, c;
-    float h, l;
-};
-static __constant__ MonoF c_mono_f[N_MONO_TERMS];
-static __constant__ float c_exp_h[64], c_exp_l[64];   // 2^(-j/64) as double-floats
+constexpr int EXP_N = 2048;   // entries of the exponential's table: a power of two
+// ln 2 / EXP_N, also as a double-float
+constexpr double LN2_N = 0.69314718055994530942 / EXP_N;
+constexpr float LN2_H = (float)LN2_N, LN2_L = (float)(LN2_N - (double)LN2_H);
+static __device__ float2 g_exp_tab[EXP_N];   // 2^(-j/EXP_N) as double-floats
 
 void host_monomials(Mono* o)
 {
@@ -84,6 +82,36 @@ void host_solid_harmonics(double x, double y, double z, double* S)
     for (int i = 0; i < N_MONO_TERMS; i++) S[t[i].lm] += t[i].coef * px[t[i].a] * py[t[i].b] * pz[t[i].c];
 }
 
+// ---------------------------------------------------------------- sphere records
+// rec[i][*]: 0-2 pos, 3 R, 4-6 W_k, 7-9 zeta_k, 10-12 A_k, 13-15 B_k, 16-18 (a, b, c),
+// 19 q, 20 rho0(R), 21 rho0'(R), 22-23: x y z R^2 as four floats, 24-78 float forms for the
+// FP32-pair deposit (pairs are double-floats): the position as three floats per axis (exact), W
+// pairs, zeta, EXP_N zeta / ln 2 pairs, which zeta are twice zeta_0, 2 A and 2 B pairs, 1/R^2,
+// zeta_1^3 / (8 pi), and the nonspherical polynomial sum_lm c_lm / R^l S_lm: a pair per monomial
+// x^a y^b z^c of degree 0 to 4 (the constant is 0) in the order of its Horner evaluation, a = 4..0,
+// b = 4-a..0, c = 4-a-b..0
+enum { RX = 0, RR = 3, RW = 4, RZ = 7, RA = 10, RB = 13, RC = 16, RQ = 19, RRHO = 20, RDRHO = 21, RXF = 22, RF = 24 };
+enum { FP = 0, FW = 9, FZ = 15, FC = 18, F2 = 24, FA = 26, FB = 32, FR = 38, FN = 40, FH = 42 };   // floats from RF
+constexpr int POLY_N = 35;
+static_assert(RF + (FH + 2 * POLY_N + 1) / 2 <= SPHERE_REC_DOUBLES, "sphere record");
+
+// place of x^a y^b z^c in the Horner order
+__host__ __device__ constexpr int poly_slot(int a, int b, int c)
+{
+    int s = 0;
+    for (int q = 4; q > a; q--) s += (5 - q) * (6 - q) / 2;
+    for (int q = 4 - a; q > b; q--) s += 5 - a - q;
+    return s + (4 - a - b) - c;
+}
+
+// the monomials of each place: S_lm's coefficients there (lm 0: none; the constant is left out)
+constexpr int POLY_TERMS = 4;
+struct PolyTerm {
+    int lm;
+    double coef;
+};
+static __device__ PolyTerm g_poly[POLY_N][POLY_TERMS];
+
 // Constant tables are per device: each device gets its own upload, once, with that device
 // current (a flag per device, so alternating devices uploads nothing again).
 constexpr int MAX_DEVICES = 64;
@@ -103,25 +131,24 @@ static cudaError_t ensure_monomials()
     host_monomials(t);
     e = cudaMemcpyToSymbol(c_mono, t, sizeof(t));
     if (e != cudaSuccess) return e;
-    MonoF tf[N_MONO_TERMS];
-    for (int i = 0; i < N_MONO_TERMS; i++) {
-        tf[i].lm = t[i].lm;
-        tf[i].a = t[i].a;
-        tf[i].b = t[i].b;
-        tf[i].c = t[i].c;
-        tf[i].h = (float)t[i].coef;
-        tf[i].l = (float)(t[i].coef - (double)tf[i].h);
+    PolyTerm pt[POLY_N][POLY_TERMS] = {};
+    for (int q = 1; q < N_MONO_TERMS; q++) {
+        PolyTerm* o = pt[poly_slot(t[q].a, t[q].b, t[q].c)];
+        int k = 0;
+        while (k < POLY_TERMS && o[k].lm != 0) k++;
+        if (k == POLY_TERMS) return cudaErrorInvalidValue;
+        o[k].lm = t[q].lm;
+        o[k].coef = t[q].coef;
     }
-    e = cudaMemcpyToSymbol(c_mono_f, tf, sizeof(tf));
+    e = cudaMemcpyToSymbol(g_poly, pt, sizeof(pt));
     if (e != cudaSuccess) return e;
-    float eh[64], el[64];
-    for (int j = 0; j < 64; j++) {
-        const double v = std::exp2(-j / 64.0);
-        eh[j] = (float)v;
-        el[j] = (float)(v - (double)eh[j]);
+    static float2 ex[EXP_N];   // (under the lock)
+    for (int j = 0; j < EXP_N; j++) {
+        const double v = std::exp2(-j / (double)EXP_N);
+        ex[j].x = (float)v;
+        ex[j].y = (float)(v - (double)ex[j].x);
     }
-    e = cudaMemcpyToSymbol(c_exp_h, eh, sizeof(eh));
-    if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_exp_l, el, sizeof(el));
+    e = cudaMemcpyToSymbol(g_exp_tab, ex, sizeof(ex));
     if (e == cudaSuccess) g_mono_uploaded[dev] = true;
     return e;
 }
@@ -145,12 +172,6 @@ __device__ __forceinline__ void solid_harmonics(double x, double y, double z, do
     }
 }
 
-// ---------------------------------------------------------------- sphere records
-// rec[i][*]: 0-2 pos, 3 R, 4-6 W_k, 7-9 zeta_k, 10-12 A_k, 13-15 B_k, 16-18 (a, b, c),
-// 19 q, 20 rho0(R), 21 rho0'(R), 22-23: x y z R^2 as four floats, 24-47: c_lm / R^l as 24
-// double-floats (float pairs)
-enum { RX = 0, RR = 3, RW = 4, RZ = 7, RA = 10, RB = 13, RC = 16, RQ = 19, RRHO = 20, RDRHO = 21, RXF = 22, RNS = 24 };
-
 struct SphArgs {
     int na;
     const double *pos, *Z, *R, *w, *zeta, *clm;
@@ -160,6 +181,17 @@ struct SphArgs {
     double *q, *rhoR, *drhoR, *coef;
     int* status;
 };
+
+using dfa::df;
+
+// x as the sum of three floats (72 bits: exact over any range of exponents that matters here)
+__device__ __forceinline__ void three_floats(double x, float* o)
+{
+    o[0] = (float)x;
+    x -= (double)o[0];
+    o[1] = (float)x;
+    o[2] = (float)(x - (double)o[1]);
+}
 
 constexpr int SPH_NT = 128;
 
@@ -222,6 +254,15 @@ __global__ void __launch_bounds__(SPH_NT) k_sphere_params(SphArgs a)
         r[RZ + k] = z;
         r[RA + k] = A;
         r[RB + k] = B;
+        float* f = reinterpret_cast<float*>(r + RF);
+        const df Wf = dfa::from_double(W), cf = dfa::from_double(z * (1.0 / LN2_N));
+        f[FW + 2 * k] = Wf.h;
+        f[FW + 2 * k + 1] = Wf.l;
+        f[FZ + k] = (float)z;
+        f[FC + 2 * k] = cf.h;
+        f[FC + 2 * k + 1] = cf.l;
+        if (k == 0)
+            f[F2] = __int_as_float((a.zeta[3 * i + 1] == 2.0 * z ? 1 : 0) | (a.zeta[3 * i + 2] == 2.0 * z ? 2 : 0));
         const double zR = z * Ri, eR = exp(-zR), sh = sinh(zR), ch = cosh(zR);
         own[0][k] = W * eR + 2.0 * A * sh / Ri - 2.0 * B * ch;
         own[1][k] = -z * W * eR + 2.0 * A * (z * ch / Ri - sh / (Ri * Ri)) - 2.0 * B * z * sh;
@@ -230,14 +271,33 @@ __global__ void __launch_bounds__(SPH_NT) k_sphere_params(SphArgs a)
         const double I1 = Ri * ch / z - sh / (z * z);                                   // int r sinh
         const double I2 = Ri * Ri * sh / z - 2.0 * Ri * ch / (z * z) + 2.0 * sh / (z * z * z);  // int r^2 cosh
         own[2][k] = in + 4.0 * PI * (2.0 * A * I1 - 2.0 * B * I2);
-    } else if (tid >= 32 && tid < 32 + NLM - 1) {
-        const int lm = tid - 31;
-        double iRl = 1.0;
-        for (int l = 0; l < l_of_lm(lm); l++) iRl /= Ri;
-        const double v = a.clm[24 * (size_t)i + lm - 1] * iRl;
-        float* ns = reinterpret_cast<float*>(r + RNS);
-        ns[2 * (lm - 1)] = (float)v;
-        ns[2 * (lm - 1) + 1] = (float)(v - (double)(float)v);
+        const df A2 = dfa::from_double(2.0 * A), B2 = dfa::from_double(2.0 * B);
+        f[FA + 2 * k] = A2.h;
+        f[FA + 2 * k + 1] = A2.l;
+        f[FB + 2 * k] = B2.h;
+        f[FB + 2 * k + 1] = B2.l;
+        if (k == 0) {
+            const df n1 = dfa::from_double(z * z * z / (8.0 * PI));
+            f[FN] = n1.h;
+            f[FN + 1] = n1.l;
+        }
+    } else if (tid >= 32 && tid < 64) {
+        // the nonspherical polynomial's coefficients, two per thread
+        const double iR = 1.0 / Ri;
+        for (int slot = tid - 32; slot < POLY_N; slot += 32) {
+            double v = 0.0;
+#pragma unroll
+            for (int t = 0; t < POLY_TERMS; t++) {
+                const int lm = g_poly[slot][t].lm;
+                const double iR2 = iR * iR;
+                const double iRl = lm >= 16 ? iR2 * iR2 : lm >= 9 ? iR2 * iR : lm >= 4 ? iR2 : iR;
+                if (lm > 0) v = fma(g_poly[slot][t].coef * iRl, a.clm[24 * (size_t)i + lm - 1], v);
+            }
+            const df c = dfa::from_double(v);
+            float* f = reinterpret_cast<float*>(r + RF) + FH + 2 * slot;
+            f[0] = c.h;
+            f[1] = c.l;
+        }
     } else if (tid == 64) {
         r[RX] = xi;
         r[RX + 1] = yi;
@@ -248,6 +308,12 @@ __global__ void __launch_bounds__(SPH_NT) k_sphere_params(SphArgs a)
         xf[1] = (float)yi;
         xf[2] = (float)zi;
         xf[3] = (float)(Ri * Ri);
+        const df iR2 = dfa::from_double(1.0 / (Ri * Ri));
+        float* f = reinterpret_cast<float*>(r + RF) + FR;
+        f[0] = iR2.h;
+        f[1] = iR2.l;
+    } else if (tid >= 96 && tid < 99) {
+        three_floats(a.pos[3 * i + tid - 96], reinterpret_cast<float*>(r + RF) + FP + 3 * (tid - 96));
     }
     __syncthreads();
     if (tid != 0) return;
@@ -282,6 +348,8 @@ cudaError_t launch_sphere_params(const lasto_cluster& cl, const double* ax0, con
                                  double* rec, double* q, double* rhoR, double* drhoR, double* coef, int* status,
                                  cudaStream_t s)
 {
+    const cudaError_t em = ensure_monomials();
+    if (em != cudaSuccess) return em;
     SphArgs a;
     a.na = cl.n_atoms;
     a.pos = cl.pos;
@@ -316,26 +384,26 @@ struct DepArgs {
     int* status;
 };
 
-// FP32-pair deposit, per atom floats: {D(x,y,z) rounded to FP32, R^2}, {W_k rounded to FP32, 0},
-// then the double-float D(x,y,z) and W_k pairs (D = atom - tile origin)
-constexpr int SAF = 20;
 __global__ void k_deposit_df(DepArgs a);
 
 // per-atom fields staged in shared memory
 constexpr int SA = 14;  // x y z R^2 W0 W1 W2 A0 A1 A2 B0 B1 B2 R
 constexpr int DEP_NT = 256;
-constexpr int DT_X = 8, DT_Y = 8, DT_Z = 4;   // FP32-pair deposit: one 8 x 8 x 4 tile of nodes per block
-static_assert(DT_X * DT_Y * DT_Z == DEP_NT, "deposit tile = one block");
 constexpr double EXP_CUT = 40.0;   // e^{-40} * max W < 1e-14 absolute; skipped terms are below FP64 rounding of n_e
-// FP32-pair deposit: Slater terms with zeta r > FAR_T in plain FP32.  FP32 carries a relative
-// error of a few 1e-6 in e^{-zeta r} there (the FP32 distance and exponent); at 20 the node-wise
-// deposit error stays near 1e-10 of the local density, while 16 (measured) raises it to ~4e-9.
-constexpr float FAR_T = 20.0f;
-// FP32-pair deposit: Slater terms with zeta r > DF_EXP_CUT are dropped, and atoms beyond
-// DF_EXP_CUT / zeta_min of a tile's bounding box for the whole tile.  Measured against the
-// oracle on the small test clusters (Pd13 graded 33^3 and uniform 65^3, Pd2): the largest
-// node-wise error where the density exceeds 1e-3 of its maximum is 2e-11 to 6e-11 of the local
-// density at 37 (FP32 far field included); at 34 it was 3.6e-10.
+// FP32-pair deposit: where a pair's precision changes, in units of 1/zeta_min.  A Slater term is
+// summed with an absolute error far below that of the density it adds to, so a term that is small
+// at its distance needs fewer bits: from NEAR_T on (e^-9 of its weight) about 35 relative bits
+// do, from MID_T on an FP32 exponential of an accurate exponent (relative error 3e-7), from FAR_T
+// on plain FP32 (a few 1e-6 in e^{-zeta r}: the FP32 distance and exponent).  The far limit was 20
+// with no class before it but the double-float one: an error four times as large, where three
+// equal exponents add up (1.1e-10 of the density node by node), at 2.6 times the time.
+constexpr float NEAR_T = 9.0f;
+constexpr float MID_T = 18.0f;
+constexpr float FAR_T = 22.0f;
+// Slater terms with zeta r > DF_EXP_CUT are dropped, and atoms beyond DF_EXP_CUT / zeta_min of a
+// tile's bounding box for the whole tile.  Measured against the oracle on the small test clusters
+// (Pd13 graded 33^3 and uniform 65^3, Pd2): the largest node-wise error where the density exceeds
+// 1e-3 of its maximum is 2e-11 to 6e-11 of the local density at 37; at 34 it was 3.6e-10.
 constexpr float DF_EXP_CUT = 37.0f;
 
 __device__ __forceinline__ double nonspherical(const double* __restrict__ c, double dx, double dy, double dz,
@@ -431,6 +499,11 @@ __global__ void __launch_bounds__(DEP_NT) k_deposit64(DepArgs a)
 }
 
 
+// FP32-pair deposit: one 8 x 8 x 8 tile of nodes per block, two nodes (four planes apart) per thread
+constexpr int DT_X = 8, DT_Y = 8, DT_Z = 8;
+static_assert(DT_X * DT_Y * DT_Z == 2 * DEP_NT, "deposit tile = one block");
+constexpr int DF_MAX_ATOMS = 2431;   // most atoms the FP32-pair form takes (four index lists in shared memory)
+
 cudaError_t launch_deposit(const lasto_cluster& cl, const double* rec, int precision, double* b, int* owner,
                            const double* /*xm_tab*/, double* /*row_mom*/, int* status, cudaStream_t s)
 {
@@ -450,12 +523,11 @@ cudaError_t launch_deposit(const lasto_cluster& cl, const double* rec, int preci
     const size_t N = (size_t)cl.n[0] * cl.n[1] * cl.n[2];
     const size_t smem = sizeof(double) * SA * (size_t)cl.n_atoms;
     if (precision == LASTO_PREC_MIXED) {
-        const size_t smf = sizeof(float) * (128 + SAF * (size_t)cl.n_atoms) + sizeof(int) * (size_t)cl.n_atoms;
-        if (smf > 200 * 1024) return cudaErrorInvalidValue;
+        if (cl.n_atoms > DF_MAX_ATOMS) return cudaErrorInvalidValue;
         const dim3 grid((unsigned)((cl.n[0] + DT_X - 1) / DT_X), (unsigned)((cl.n[1] + DT_Y - 1) / DT_Y),
                         (unsigned)((cl.n[2] + DT_Z - 1) / DT_Z));
         if (grid.y > 65535 || grid.z > 65535) return cudaErrorInvalidValue;
-        k_deposit_df<<<grid, DEP_NT, smf, s>>>(a);
+        k_deposit_df<<<grid, DEP_NT, sizeof(int) * 4 * (size_t)cl.n_atoms, s>>>(a);
         return cudaGetLastError();
     }
     if (smem > 200 * 1024) return cudaErrorInvalidValue;
@@ -464,8 +536,6 @@ cudaError_t launch_deposit(const lasto_cluster& cl, const double* rec, int preci
 }
 
 // ---------------------------------------------------------------- deposit (FP32 pairs)
-using dfa::df;
-
 __device__ __forceinline__ bool inside_fp64(const DepArgs& a, double x, double y, double z, int t)
 {
     const double* r = a.rec + (size_t)SPHERE_REC_DOUBLES * t;
@@ -473,283 +543,558 @@ __device__ __forceinline__ bool inside_fp64(const DepArgs& a, double x, double y
     return fma(dx, dx, fma(dy, dy, dz * dz)) < r[RR] * r[RR];
 }
 
-// The FP32-pair deposit works on 8 x 8 x 4 tiles of nodes (a warp covers 8 x 4 x 1): a compact
-// footprint lets a whole warp agree more often on which branch an atom takes (double-float,
-// plain FP32 far field, beyond the cut-off), and lets the block drop, once, every atom whose
-// distance from the tile's bounding box exceeds the cut-off (each node would skip it anyway).
+constexpr float ROUND_MAGIC = 12582912.0f;   // 1.5 * 2^23: adding it rounds to an integer in the low bits
 
-__global__ void __launch_bounds__(DEP_NT) k_deposit_df(DepArgs a)
+// the power of two 2^-floor(k / EXP_N) from the bits of k + ROUND_MAGIC
+__device__ __forceinline__ float pow2_of(int ki)
 {
-    extern __shared__ float sf[];
-    __shared__ int s_cnt[DEP_NT / 32];
-    __shared__ float s_off[2 * (DT_X + DT_Y + DT_Z)];   // node coordinate - tile origin, double-float
-    float* th = sf;
-    float* tl = sf + 64;
-    float* sat = sf + 128;
-    int* list = reinterpret_cast<int*>(sat + SAF * (size_t)a.na);
-    const int i0 = blockIdx.x * DT_X, j0 = blockIdx.y * DT_Y, k0 = blockIdx.z * DT_Z;
-    const int i = i0 + (threadIdx.x & 7), j = j0 + ((threadIdx.x >> 3) & 7), k = k0 + (threadIdx.x >> 6);
-    const bool valid = i < a.n[0] && j < a.n[1] && k < a.n[2];
-    // tile origin: its first node; offsets from it keep the pairs' magnitudes small
-    const double ox = a.ax[0][i0], oy = a.ax[1][j0], oz = a.ax[2][k0];
-    for (int t = threadIdx.x; t < 64; t += DEP_NT) {
-        th[t] = c_exp_h[t];
-        tl[t] = c_exp_l[t];
-    }
-    if (threadIdx.x < DT_X + DT_Y + DT_Z) {
-        const int t = threadIdx.x;
-        const int d = t < DT_X ? 0 : t < DT_X + DT_Y ? 1 : 2;
-        const int o = t - (d == 0 ? 0 : d == 1 ? DT_X : DT_X + DT_Y);
-        const int first = d == 0 ? i0 : d == 1 ? j0 : k0;
-        const double org = d == 0 ? ox : d == 1 ? oy : oz;
-        const df v = dfa::from_double(a.ax[d][min(first + o, a.n[d] - 1)] - org);
-        s_off[2 * t] = v.h;
-        s_off[2 * t + 1] = v.l;
-    }
-    df zt[3];
-    float zmin = 1e30f;
+    return __int_as_float(0x3f800000 - (ki & ~(EXP_N - 1)) * ((1 << 23) / EXP_N));
+}
+
+// r = r0 + r1 of a squared distance h + l (h >= 0): the FP32 root by the approximate reciprocal
+// square root and one Newton correction, relative error about 2^-46
+__device__ __forceinline__ df root(float h, float l)
+{
+    const float s = h > 0.0f ? rsqrtf(h) : 0.0f;
+    const float r0 = h * s;
+    return {r0, (fmaf(-r0, r0, h) + l) * (0.5f * s)};
+}
+
+// y = c r in units of ln 2 / EXP_N (c = EXP_N zeta / ln 2 as a double-float), unevaluated
+__device__ __forceinline__ df exponent(df r, float ch, float cl)
+{
+    const float y0 = r.h * ch;
+    return {y0, fmaf(r.l, ch, fmaf(r.h, cl, fmaf(r.h, ch, -y0)))};
+}
+
+// e^{-y ln2/EXP_N} to double-float accuracy: k = round(y), 2^(-k/EXP_N) from the table (Tang's
+// table-driven reduction) times 1 + g, |g| <= 1.7e-4: g's linear term as a double-float, its
+// quadratic and cubic terms in FP32
+__device__ __forceinline__ df exp_pair(df y, const float2* __restrict__ T)
+{
+    const float km = y.h + ROUND_MAGIC;
+    const df f = dfa::fast_two_sum(y.h - (km - ROUND_MAGIC), y.l);
+    const int ki = __float_as_int(km);
+    const float2 t = T[ki & (EXP_N - 1)];
+    const float gh = -LN2_H * f.h;
+    float gl = fmaf(-LN2_H, f.h, -gh);
+    gl = fmaf(-LN2_L, f.h, gl);
+    gl = fmaf(-LN2_H, f.l, gl);
+    gl = fmaf(gh * gh, fmaf(gh, 1.0f / 6.0f, 0.5f), gl);
+    const float p = t.x * gh;
+    const float lo = fmaf(t.x, gh, -p) + fmaf(t.x, gl, fmaf(t.y, gh, t.y));
+    const float e = t.x + p;
+    const float sc = pow2_of(ki);
+    return {e * sc, (((t.x - e) + p) + lo) * sc};
+}
+
+// the same to about 35 bits (an error below 4e-11; four times that with 512 entries): 1 + g with g in FP32, the pair left unevaluated
+__device__ __forceinline__ df exp_mid(df y, const float2* __restrict__ T)
+{
+    constexpr float C1 = -LN2_H, C2 = 0.5f * LN2_H * LN2_H, C3 = -LN2_H * LN2_H * LN2_H / 6.0f;
+    const float km = y.h + ROUND_MAGIC;
+    const float f = (y.h - (km - ROUND_MAGIC)) + y.l;
+    const int ki = __float_as_int(km);
+    const float2 t = T[ki & (EXP_N - 1)];
+    const float g = f * fmaf(f, fmaf(f, C3, C2), C1);
+    const float sc = pow2_of(ki);
+    return {t.x * sc, fmaf(t.x, g, t.y) * sc};
+}
+
+// s += w e, the sum left as an unevaluated pair
+__device__ __forceinline__ void add_product(df& s, float wh, float wl, df e)
+{
+    const float p = wh * e.h;
+    const float l = fmaf(wh, e.h, -p) + fmaf(wh, e.l, wl * e.h);
+    const df t = dfa::two_sum(s.h, p);
+    s.h = t.h;
+    s.l += t.l + l;
+}
+
+// e^{-x ln 2}
+__device__ __forceinline__ float ex2_neg(float x)
+{
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(-x));
+    return r;
+}
+
+// p - o of two three-float numbers, to double-float accuracy of the difference
+__device__ __forceinline__ df diff3(const float* p, const float* o)
+{
+    const df s = dfa::two_sum(p[0], -o[0]), t = dfa::two_sum(p[1], -o[1]);
+    df u = dfa::two_sum(s.l, t.h);
+    u.l += t.l + (p[2] - o[2]);
+    df w = dfa::two_sum(s.h, u.h);
+    w.l += u.l;
+    return dfa::fast_two_sum(w.h, w.l);
+}
+
+struct DfExps {
+    float ch[3], cl[3];   // EXP_N zeta / ln 2
+    bool twice[3];        // zeta_q exactly twice zeta_0
+};
+
+// s = s x + c in double-floats
+__device__ __forceinline__ df mul_add(df s, df x, df c)
+{
+    const float p = s.h * x.h;
+    const float e = fmaf(s.h, x.h, -p) + fmaf(s.h, x.l, s.l * x.h);
+    df t = dfa::two_sum(p, c.h);
+    t.l += e + c.l;
+    return dfa::fast_two_sum(t.h, t.l);
+}
+
+// n_e's monopole swap and nonspherical part at a node inside its sphere, added to the neighbours'
+// Slater sum s: s - N_i(r) + rho_ns + pseudo-density.  d: node - centre.  The nonspherical part is
+// its polynomial in d by nested Horner steps (34 multiply-adds where the sum over the harmonics'
+// 55 monomials took four products each); the pseudo-density, ten times the result in places, is
+// FP64.
+__device__ __noinline__ double inside_value(df s, const double* __restrict__ rc, df dx, df dy, df dz, DfExps ex,
+                                            const float2* __restrict__ T)
+{
+    const float2* f2 = reinterpret_cast<const float2*>(reinterpret_cast<const float*>(rc + RF));
+    auto pair = [&](int o) {
+        const float2 v = f2[o >> 1];
+        return df{v.x, v.y};
+    };
+    const df r2 = dfa::add(dfa::add(dfa::sqr(dx), dfa::sqr(dy)), dfa::sqr(dz));
+    const df rr = root(r2.h, r2.l), r = dfa::fast_two_sum(rr.h, rr.l);
+    df nbr = {0.0f, 0.0f}, e1 = {1.0f, 0.0f};
+#pragma unroll 1
     for (int q = 0; q < 3; q++) {
-        zt[q] = dfa::from_double(a.rec[RZ + q]);
-        zmin = fminf(zmin, zt[q].h);
+        const float ch = q == 0 ? ex.ch[0] : q == 1 ? ex.ch[1] : ex.ch[2];
+        const float cl = q == 0 ? ex.cl[0] : q == 1 ? ex.cl[1] : ex.cl[2];
+        const df y = exponent(r, ch, cl);
+        const df em = exp_pair(y, T), ep = exp_pair(dfa::neg(y), T);
+        if (q == 0) e1 = em;
+        const df A2 = pair(FA + 2 * q), B2 = pair(FB + 2 * q);
+        df shr;   // 2 sinh(zeta r) / r
+        if (y.h > 1e-3f / LN2_H) {
+            shr = dfa::div(dfa::add(ep, dfa::neg(em)), r);
+        } else {
+            const df zt = dfa::from_double(rc[RZ + q]);
+            const float zr = zt.h * r.h;
+            shr = dfa::mul(df{2.0f * zt.h, 2.0f * zt.l}, dfa::add_f(df{1.0f, 0.0f}, zr * zr * (1.0f / 6.0f)));
+        }
+        const df t = dfa::add(dfa::mul(A2, shr), dfa::neg(dfa::mul(B2, dfa::add(ep, em))));
+        nbr = dfa::add(nbr, df{0.5f * t.h, 0.5f * t.l});
     }
-    const float cut = DF_EXP_CUT / zmin;
-    const float cut2 = cut * cut * (1.0f + 1e-5f);
-    int nkept, nnear;
-    // Atoms within the cut-off of the tile's bounding box, in ascending order, tested in FP32
-    // on the records' float copies of the positions: first those that may come within
-    // FAR_T / zeta_min of a node of the tile (near candidates), then those farther than that
-    // from every node (far-only).  The margins 1e-3 on the squared distances cover the
-    // rounding of these tests (~1e-6 relative) and of a node's own FP32 distance tests, so an
-    // atom dropped here fails the cut-off test, and a far-only atom passes the far test, at
-    // every node of the tile.
-    const float far_box2 = (FAR_T / zmin) * (FAR_T / zmin) * (1.0f + 1e-3f);
+    // nonspherical part: slater(zeta_1, r) (1 - r^2/R^2)^2 sum c_lm (r/R)^l y_lm
+    df ang = {0.0f, 0.0f};
+#pragma unroll
+    for (int a = 4; a >= 0; a--) {
+        df qy = {0.0f, 0.0f};
+#pragma unroll
+        for (int b = 4 - a; b >= 0; b--) {
+            df qz = pair(FH + 2 * poly_slot(a, b, 4 - a - b));
+#pragma unroll
+            for (int c = 3 - a - b; c >= 0; c--) qz = mul_add(qz, dz, pair(FH + 2 * poly_slot(a, b, c)));
+            qy = b == 4 - a ? qz : mul_add(qy, dy, qz);
+        }
+        ang = a == 4 ? qy : mul_add(ang, dx, qy);
+    }
+    const df tt = dfa::add_f(dfa::neg(dfa::mul(r2, pair(FR))), 1.0f);
+    const df radial = dfa::mul(dfa::mul(pair(FN), e1), dfa::sqr(tt));
+    s = dfa::add(dfa::add(s, dfa::neg(nbr)), dfa::mul(radial, ang));
+    const double rsq = dfa::to_double(r2);
+    return dfa::to_double(s) + fma(fma(rc[RC + 2], rsq, rc[RC + 1]), rsq, rc[RC]);
+}
+
+// The FP32-pair deposit works on 8 x 8 x 8 tiles of nodes (a warp covers 8 x 4 x 1, each thread
+// two nodes four planes apart).  Once per block, every atom is dropped (beyond the cut-off of the
+// tile's bounding box) or sorted by its distance from that box into four lists, each taken
+// through a loop of its own in which every lane does the same work:
+//   near    the double-float sum, with the test for the node inside the atom's sphere;
+//   mid     every node beyond NEAR_T / zeta_min of the atom: e^{-zeta r} to about 35 bits;
+//   outer   every node beyond MID_T / zeta_min: the FP32 exponential of the accurate exponent;
+//   far     every node beyond FAR_T / zeta_min: plain FP32.
+// Near, mid and outer atoms are staged as the squares of the 24 coordinate differences of the tile's
+// planes, so that a pair's squared distance costs two or four additions per node instead of three
+// double-float subtractions, squares and sums: near as double-floats, the others as a multiple of a
+// common power of two plus a remainder, whose high parts add exactly.  Bound: instruction issue.
+// Before this form (three branches inside one loop over the atoms, 8 x 8 x 4 tiles): Pd147 161^3
+// 1308 us, Pd561 385^3 29.7 ms, Pd55 129^3 461 us; now 479 us, 10.8 ms and 175 us (0.81 of the issue
+// rate), with a quarter of the error (Pd147: 5.8e-13 -> 1.6e-13 of the 2-norm).
+constexpr int DF_CH = 32;    // near or mid atoms staged at a time
+constexpr int DF_FCH = 128;  // far atoms staged at a time
+constexpr int DF_ROWS = DT_X + DT_Y + DT_Z;
+
+__global__ void __launch_bounds__(DEP_NT, 3) k_deposit_df(DepArgs a)
+{
+    extern __shared__ int lists[];                 // near, mid, outer, far atom indices [4][na]
+    __shared__ unsigned long long s_cnt[DEP_NT / 32];   // four 16-bit counts
+    __shared__ float2 s_off[DF_ROWS];              // node coordinate - tile origin, double-float
+    __shared__ float2 s_T[EXP_N];
+    __shared__ float2 s_D[DF_CH][3];               // atom - tile origin
+    __shared__ __align__(16) float2 s_sq[DF_CH][DF_ROWS];
+    __shared__ __align__(16) float s_w[DF_CH][8];  // W pairs, R^2, -
+    __shared__ __align__(16) float s_far[DF_FCH][8];
+    __shared__ int s_queued;
+    __shared__ float s_org[3][3], s_box[3][2];     // the tile origin as three floats, the tile's bounds
+    const int tid = threadIdx.x, na = a.na;
+    const int i0 = blockIdx.x * DT_X, j0 = blockIdx.y * DT_Y, k0 = blockIdx.z * DT_Z;
+    const int li = tid & 7, lj = (tid >> 3) & 7, lk = tid >> 6;
+    if (tid == 0) s_queued = 0;
+    for (int t = tid; t < EXP_N; t += DEP_NT) s_T[t] = g_exp_tab[t];
+    // tile origin: its first node; offsets from it keep the pairs' magnitudes small.  (FP64 work
+    // is kept to these two warps and to what a node's own sphere needs: the pipe is narrow enough
+    // that conversions and differences per atom in every tile kept it 46 % busy and cost a third
+    // of the kernel's time; the sphere records hold float forms instead.)
+    if (tid < DF_ROWS) {
+        const int d = tid >> 3, o = tid & 7, first = d == 0 ? i0 : d == 1 ? j0 : k0;
+        const df v = dfa::from_double(a.ax[d][min(first + o, a.n[d] - 1)] - a.ax[d][first]);
+        s_off[tid] = make_float2(v.h, v.l);
+    } else if (tid >= 32 && tid < 35) {
+        const int d = tid - 32, first = d == 0 ? i0 : d == 1 ? j0 : k0;
+        three_floats(a.ax[d][first], s_org[d]);
+        s_box[d][0] = s_org[d][0];
+        s_box[d][1] = (float)a.ax[d][min(first + 7, a.n[d] - 1)];
+    }
+    // the exponents are the same on every atom (checked by the sphere kernel)
+    const float* f0 = reinterpret_cast<const float*>(a.rec + RF);
+    const int twice = __float_as_int(f0[F2]);
+    float zt[3], zmin = 1e30f;
+    DfExps ex;
+#pragma unroll
+    for (int q = 0; q < 3; q++) {
+        zt[q] = f0[FZ + q];
+        zmin = fminf(zmin, zt[q]);
+        ex.ch[q] = f0[FC + 2 * q];
+        ex.cl[q] = f0[FC + 2 * q + 1];
+        ex.twice[q] = q > 0 && (twice >> (q - 1) & 1);
+    }
+    __syncthreads();
+    const float cut = DF_EXP_CUT / zmin, cut2 = cut * cut * (1.0f + 1e-5f);
+    // Sort the atoms in ascending order, tested in FP32 on the records' float copies of the
+    // positions.  The margins 1e-3 on the squared distances cover the rounding of these tests
+    // (~1e-6 relative): an atom dropped here is beyond the cut-off at every node of the tile, and
+    // a mid or far atom is beyond its limit, and beyond its own sphere, at every node.
+    int count[4] = {0, 0, 0, 0};
     {
-        const float bx0 = (float)ox, bx1 = (float)a.ax[0][min(i0 + DT_X - 1, a.n[0] - 1)];
-        const float by0 = (float)oy, by1 = (float)a.ax[1][min(j0 + DT_Y - 1, a.n[1] - 1)];
-        const float bz0 = (float)oz, bz1 = (float)a.ax[2][min(k0 + DT_Z - 1, a.n[2] - 1)];
         const float lim = cut2 * (1.0f + 1e-3f);
-        const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-        int total = 0;
-        for (int pass = 0; pass < 2; pass++) {
-            if (pass == 1) nnear = total;
-            for (int base = 0; base < a.na; base += DEP_NT) {
-                const int t = base + threadIdx.x;
-                bool keep = false;
-                if (t < a.na) {
-                    const float4 c = *reinterpret_cast<const float4*>(a.rec + (size_t)SPHERE_REC_DOUBLES * t + RXF);
-                    const float ex = fmaxf(fmaxf(bx0 - c.x, c.x - bx1), 0.0f);
-                    const float ey = fmaxf(fmaxf(by0 - c.y, c.y - by1), 0.0f);
-                    const float ez = fmaxf(fmaxf(bz0 - c.z, c.z - bz1), 0.0f);
-                    const float d2 = fmaf(ex, ex, fmaf(ey, ey, ez * ez));
-                    keep = d2 <= lim && ((d2 > far_box2) == (pass == 1));
-                }
-                const unsigned m = __ballot_sync(0xffffffffu, keep);
-                if (l == 0) s_cnt[w] = __popc(m);
-                __syncthreads();
-                int off = total, sum = 0;
-                for (int q = 0; q < DEP_NT / 32; q++) {
-                    off += q < w ? s_cnt[q] : 0;
-                    sum += s_cnt[q];
-                }
-                if (keep) list[off + __popc(m & ((1u << l) - 1u))] = t;
-                __syncthreads();
-                total += sum;
+        const float near2 = (NEAR_T / zmin) * (NEAR_T / zmin) * (1.0f + 1e-3f);
+        const float mid2 = (MID_T / zmin) * (MID_T / zmin) * (1.0f + 1e-3f);
+        const float far2 = (FAR_T / zmin) * (FAR_T / zmin) * (1.0f + 1e-3f);
+        const float bx0 = s_box[0][0], bx1 = s_box[0][1], by0 = s_box[1][0], by1 = s_box[1][1];
+        const float bz0 = s_box[2][0], bz1 = s_box[2][1];
+        const int w = tid >> 5, l = tid & 31;
+        for (int base = 0; base < na; base += DEP_NT) {
+            const int t = base + tid;
+            int cls = 4;
+            if (t < na) {
+                const float4 c = *reinterpret_cast<const float4*>(a.rec + (size_t)SPHERE_REC_DOUBLES * t + RXF);
+                const float dx = fmaxf(fmaxf(bx0 - c.x, c.x - bx1), 0.0f);
+                const float dy = fmaxf(fmaxf(by0 - c.y, c.y - by1), 0.0f);
+                const float dz = fmaxf(fmaxf(bz0 - c.z, c.z - bz1), 0.0f);
+                const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+                // (comparisons that a NaN position or exponent fails: such an atom is near)
+                cls = !(d2 > c.w * (1.0f + 1e-3f)) ? 0
+                      : d2 > lim                   ? 4
+                      : d2 > far2                  ? 3
+                      : d2 > mid2                  ? 2
+                      : d2 > near2                 ? 1
+                                                   : 0;
             }
-        }
-        // stage the kept atoms' fields in list order (far-only atoms: offsets and weights only,
-        // {D(x,y,z), W_0} and {W_1, W_2}, the layout of their loop below)
-        for (int q = threadIdx.x; q < total; q += DEP_NT) {
-            const double* r = a.rec + (size_t)SPHERE_REC_DOUBLES * list[q];
-            float* o = sat + SAF * q;
-            if (q >= nnear) {
-                o[0] = (float)(r[RX] - ox);
-                o[1] = (float)(r[RX + 1] - oy);
-                o[2] = (float)(r[RX + 2] - oz);
-                o[3] = (float)r[RW];
-                o[4] = (float)r[RW + 1];
-                o[5] = (float)r[RW + 2];
-                continue;
-            }
-            const df Dx = dfa::from_double(r[RX] - ox), Dy = dfa::from_double(r[RX + 1] - oy),
-                     Dz = dfa::from_double(r[RX + 2] - oz);
-            o[0] = Dx.h; o[1] = Dy.h; o[2] = Dz.h;
-            o[3] = reinterpret_cast<const float*>(r + RXF)[3];
-            o[8] = Dx.h; o[9] = Dx.l; o[10] = Dy.h; o[11] = Dy.l; o[12] = Dz.h; o[13] = Dz.l;
-            for (int c = 0; c < 3; c++) {
-                const df W = dfa::from_double(r[RW + c]);
-                o[4 + c] = W.h;
-                o[14 + 2 * c] = W.h;
-                o[15 + 2 * c] = W.l;
-            }
-            o[7] = 0.0f;
-        }
-        __syncthreads();
-        nkept = total;
-    }
-    if (!valid) return;
-    const size_t P = ((size_t)k * a.n[1] + j) * a.n[0] + i;
-    const double x = a.ax[0][i], y = a.ax[1][j], z = a.ax[2][k];
-    const int li = threadIdx.x & 7, lj = DT_X + ((threadIdx.x >> 3) & 7), lk = DT_X + DT_Y + (threadIdx.x >> 6);
-    const df px = {s_off[2 * li], s_off[2 * li + 1]}, py = {s_off[2 * lj], s_off[2 * lj + 1]},
-             pz = {s_off[2 * lk], s_off[2 * lk + 1]};
-    bool twice[3];   // zeta_q exactly twice zeta_0 (both parts of the double-float)
+            unsigned mine = 0;   // lanes of this lane's class
+            unsigned long long cnt = 0;
 #pragma unroll
-    for (int q = 0; q < 3; q++) twice[q] = q > 0 && zt[q].h == 2.0f * zt[0].h && zt[q].l == 2.0f * zt[0].l;
-    // beyond zeta_min r = FAR_T every Slater term is below e^-20 of its weight: plain FP32
-    // (relative error ~1e-7 of terms that small is ~1e-16 of the node's density scale)
-    const float far = FAR_T / zmin;
-    const float far2 = far * far * (1.0f + 1e-4f);
-    df s = {0.0f, 0.0f};
-    // the Slater terms beyond zeta r = FAR_T (each below e^-20 of its weight) summed in plain
-    // FP32 and added to the double-float sum once: their total is below 1e-6 of the node's
-    // density wherever that density matters, so FP32 rounding of it stays below 1e-13
-    float sfar = 0.0f;
-    int own = -1;
-    df orr2 = {0.0f, 0.0f}, odx = s, ody = s, odz = s;
-    for (int q0 = 0; q0 < nnear; q0++) {
-        const float* o = sat + SAF * q0;
-        // the pair's distance in FP32 from the FP32 roundings of the two offsets (one subtraction
-        // per axis): the atom's offset is at most r + the tile's extent, so r carries a relative
-        // error of ~1.5e-7 wherever the far field applies (r >= FAR_T / zeta_max)
-        const float4 A = *reinterpret_cast<const float4*>(o);
-        const float fx = px.h - A.x, fy = py.h - A.y, fz = pz.h - A.z;
-        const float r2f = fmaf(fx, fx, fmaf(fy, fy, fz * fz));
-        if (r2f > cut2) continue;
-        if (r2f > far2) {
-            // far pair: every term is below e^-FAR_T of its weight; the ~1.5e-7 relative error of
-            // r is ~3e-6 in e^{-zeta r} at zeta r = 20, the fast reciprocal square root and
-            // exponential add errors of the same size, and e^{-zeta_q r} for zeta_q = 2 zeta_0
-            // is the square of e^{-zeta_0 r}.  Terms beyond zeta r = DF_EXP_CUT are dropped.
-            const float4 W = *reinterpret_cast<const float4*>(o + 4);
-            const float rf = r2f * rsqrtf(r2f);
-            const float e0 = __expf(-zt[0].h * rf);
-            sfar = fmaf(W.x, e0, sfar);
-            if (twice[1]) {
-                sfar = fmaf(W.y, e0 * e0, sfar);
-            } else {
-                const float e = zt[1].h * rf;
-                if (e < DF_EXP_CUT) sfar = fmaf(W.y, __expf(-e), sfar);
+            for (int q = 0; q < 4; q++) {
+                const unsigned m = __ballot_sync(0xffffffffu, cls == q);
+                if (cls == q) mine = m;
+                cnt |= (unsigned long long)__popc(m) << (16 * q);
             }
-            if (twice[2]) {
-                sfar = fmaf(W.z, e0 * e0, sfar);
-            } else {
-                const float e = zt[2].h * rf;
-                if (e < DF_EXP_CUT) sfar = fmaf(W.z, __expf(-e), sfar);
+            if (l == 0) s_cnt[w] = cnt;
+            __syncthreads();
+            unsigned long long before = 0, all = 0;
+            for (int v = 0; v < DEP_NT / 32; v++) {
+                if (v == w) before = all;
+                all += s_cnt[v];
             }
-            continue;
-        }
-        const df dx = dfa::add(px, df{-o[8], -o[9]});
-        const df dy = dfa::add(py, df{-o[10], -o[11]});
-        const df dz = dfa::add(pz, df{-o[12], -o[13]});
-        const df r2 = dfa::add(dfa::add(dfa::sqr(dx), dfa::sqr(dy)), dfa::sqr(dz));
-        if (r2.h > cut2) continue;
-        if (r2.h < A.w * (1.0f + 2e-6f)) {
-            const int t = list[q0];
-            const bool in = (r2.h < A.w * (1.0f - 2e-6f)) ? true : inside_fp64(a, x, y, z, t);
-            if (in) {
-                own = t;
-                orr2 = r2;
-                odx = dx;
-                ody = dy;
-                odz = dz;
-                continue;
+            if (cls < 4) {
+                const int c0 = cls == 0 ? count[0] : cls == 1 ? count[1] : cls == 2 ? count[2] : count[3];
+                lists[cls * na + c0 + (int)(before >> (16 * cls) & 0xffff) + __popc(mine & ((1u << l) - 1u))] = t;
             }
-        }
-        const df r = dfa::sqrt_df(r2);
-        df e0 = {0.0f, 0.0f};   // e^{-zeta_0 r} when it was taken in double-float
-        bool have0 = false;
+            __syncthreads();
 #pragma unroll
-        for (int q = 0; q < 3; q++) {
-            const df tq = dfa::mul(r, zt[q]);
-            if (tq.h >= DF_EXP_CUT) continue;
-            if (tq.h > FAR_T) {
-                sfar = fmaf(o[14 + 2 * q], expf(-tq.h), sfar);
-            } else {
-                // zeta_q = 2 zeta_0 (as in the density model's 1.5, 3.0): e^{-zeta_q r} = (e^{-zeta_0 r})^2
-                const df eq = (q > 0 && twice[q] && have0) ? dfa::sqr(e0) : dfa::exp_neg(tq, th, tl);
-                if (q == 0) {
-                    e0 = eq;
-                    have0 = true;
-                }
-                s = dfa::add(s, dfa::mul(df{o[14 + 2 * q], o[15 + 2 * q]}, eq));
-            }
+            for (int q = 0; q < 4; q++) count[q] += (int)(all >> (16 * q) & 0xffff);
         }
     }
-    // far-only atoms: every node of the tile is beyond FAR_T / zeta_min of them, so only the
-    // far-field terms remain, and a term whose exponent exceeds DF_EXP_CUT at that distance
-    // (zeta_q >= zeta_min DF_EXP_CUT / FAR_T) is dropped for all of them at once
+    const int i = i0 + li, j = j0 + lj, kA = k0 + lk, kB = kA + 4;
+    const bool okA = i < a.n[0] && j < a.n[1] && kA < a.n[2], okB = okA && kB < a.n[2];
+    df sA = {0.0f, 0.0f}, sB = {0.0f, 0.0f};   // the double-float sums
+    float fA = 0.0f, fB = 0.0f;                // the outer and far atoms' FP32 sums
+    int ownA = -1, ownB = -1;
+
+    // ---- near, mid and outer atoms, DF_CH at a time
+    // high parts of the mid and outer squares: multiples of g = 2^(e - 23) with 2^e >= 4 cut^2, rounded by
+    // adding 1.5 * 2^23 g; three of them add exactly for distances up to twice the cut-off
+    const float grid_magic = __int_as_float(((__float_as_int(4.0f * cut2) >> 23) + 1) << 23) * 1.5f;
+    for (int pass = 0; pass < 3; pass++) {
+        const int cnt = pass == 0 ? count[0] : pass == 1 ? count[1] : count[2];
+        const int* list = lists + pass * na;
+        for (int c0 = 0; c0 < cnt; c0 += DF_CH) {
+            const int ch = min(DF_CH, cnt - c0);
+            __syncthreads();
+            for (int t = tid; t < ch * 8; t += DEP_NT) {
+                const int q = t >> 3, f = t & 7;
+                const double* r = a.rec + (size_t)SPHERE_REC_DOUBLES * list[c0 + q];
+                const float* fr = reinterpret_cast<const float*>(r + RF);
+                if (f < 3) {
+                    const df D = diff3(fr + FP + 3 * f, s_org[f]);
+                    s_D[q][f] = make_float2(D.h, D.l);
+                } else if (f < 6) {
+                    s_w[q][2 * (f - 3)] = fr[FW + 2 * (f - 3)];
+                    s_w[q][2 * (f - 3) + 1] = fr[FW + 2 * (f - 3) + 1];
+                } else if (f == 6) {
+                    s_w[q][6] = reinterpret_cast<const float*>(r + RXF)[3];
+                }
+            }
+            __syncthreads();
+            for (int t = tid; t < ch * DF_ROWS; t += DEP_NT) {
+                const int q = t / DF_ROWS, c = t - q * DF_ROWS;
+                const float2 o = s_off[c], D = s_D[q][c >> 3];
+                df d = dfa::sqr(dfa::add(df{o.x, o.y}, df{-D.x, -D.y}));
+                if (pass > 0) {
+                    const float hi = (d.h + grid_magic) - grid_magic;
+                    d.l += d.h - hi;
+                    d.h = hi;
+                }
+                s_sq[q][c] = make_float2(d.h, d.l);
+            }
+            __syncthreads();
+            if (pass == 0) {
+                for (int q = 0; q < ch; q++) {
+                    const float2 X = s_sq[q][li], Y = s_sq[q][DT_X + lj];
+                    const float4 W01 = *reinterpret_cast<const float4*>(&s_w[q][0]);
+                    const float4 W2R = *reinterpret_cast<const float4*>(&s_w[q][4]);
+                    const df xy = dfa::add(df{X.x, X.y}, df{Y.x, Y.y});
+#pragma unroll
+                    for (int n = 0; n < 2; n++) {
+                        const float2 Z = s_sq[q][DT_X + DT_Y + lk + 4 * n];
+                        const df r2 = dfa::add(xy, df{Z.x, Z.y});
+                        if (r2.h > cut2) continue;
+                        if (r2.h < W2R.z * (1.0f + 2e-6f)) {
+                            const int t = list[c0 + q];
+                            const bool in = (r2.h < W2R.z * (1.0f - 2e-6f)) ||
+                                            inside_fp64(a, a.ax[0][min(i, a.n[0] - 1)], a.ax[1][min(j, a.n[1] - 1)],
+                                                        a.ax[2][min(n ? kB : kA, a.n[2] - 1)], t);
+                            if (in) {
+                                if (n) ownB = t;
+                                else ownA = t;
+                                continue;
+                            }
+                        }
+                        const df r = root(r2.h, r2.l);
+                        df& s = n ? sB : sA;
+                        df e0 = {0.0f, 0.0f};
+#pragma unroll
+                        for (int v = 0; v < 3; v++) {
+                            if (zt[v] * r.h >= DF_EXP_CUT) continue;
+                            df e;
+                            if (v > 0 && ex.twice[v] && zt[0] * r.h < DF_EXP_CUT) {
+                                e = dfa::sqr(e0);   // e^{-2 zeta_0 r}
+                            } else {
+                                e = exp_pair(exponent(r, ex.ch[v], ex.cl[v]), s_T);
+                            }
+                            if (v == 0) e0 = e;
+                            add_product(s, v == 0 ? W01.x : v == 1 ? W01.z : W2R.x,
+                                        v == 0 ? W01.y : v == 1 ? W01.w : W2R.y, e);
+                        }
+                    }
+                }
+            } else if (pass == 1) {
+                // a term that is beyond the cut-off at every mid distance is dropped for all of
+                // them; nodes of a mid atom beyond 2^-120 are held there (the exponent's range)
+                const float rmin = NEAR_T / zmin, ymax = 120.0f * EXP_N;
+                const bool on0 = zt[0] * rmin < DF_EXP_CUT, on1 = zt[1] * rmin < DF_EXP_CUT,
+                           on2 = zt[2] * rmin < DF_EXP_CUT;
+                if (on0 && on1 && ex.twice[1] && !on2) {
+                    // (W0 + W1 e) e, e = e^{-zeta_0 r}
+                    for (int q = 0; q < ch; q++) {
+                        const float2 X = s_sq[q][li], Y = s_sq[q][DT_X + lj];
+                        const float4 W = *reinterpret_cast<const float4*>(&s_w[q][0]);
+                        const float xh = X.x + Y.x, xl = X.y + Y.y;
+#pragma unroll
+                        for (int n = 0; n < 2; n++) {
+                            const float2 Z = s_sq[q][DT_X + DT_Y + lk + 4 * n];
+                            df y = exponent(root(xh + Z.x, xl + Z.y), ex.ch[0], ex.cl[0]);
+                            y.h = fminf(y.h, ymax);
+                            const df e = exp_mid(y, s_T);
+                            const float p = W.z * e.h;
+                            df v = dfa::two_sum(W.x, p);
+                            v.l += W.y + (fmaf(W.z, e.h, -p) + fmaf(W.z, e.l, W.w * e.h));
+                            add_product(n ? sB : sA, v.h, v.l, e);
+                        }
+                    }
+                } else {
+                    for (int q = 0; q < ch; q++) {
+                        const float2 X = s_sq[q][li], Y = s_sq[q][DT_X + lj];
+                        const float xh = X.x + Y.x, xl = X.y + Y.y;
+#pragma unroll
+                        for (int n = 0; n < 2; n++) {
+                            const float2 Z = s_sq[q][DT_X + DT_Y + lk + 4 * n];
+                            const df r = root(xh + Z.x, xl + Z.y);
+#pragma unroll
+                            for (int v = 0; v < 3; v++) {
+                                if (!(v == 0 ? on0 : v == 1 ? on1 : on2)) continue;
+                                df y = exponent(r, ex.ch[v], ex.cl[v]);
+                                y.h = fminf(y.h, ymax);
+                                add_product(n ? sB : sA, s_w[q][2 * v], s_w[q][2 * v + 1], exp_mid(y, s_T));
+                            }
+                        }
+                    }
+                }
+            } else {
+                // e^{-zeta r} = 2^-y0 (1 - y1 ln 2), y0 + y1 = zeta r / ln 2
+                const float rmin = MID_T / zmin;
+                const bool on0 = zt[0] * rmin < DF_EXP_CUT, on1 = zt[1] * rmin < DF_EXP_CUT,
+                           on2 = zt[2] * rmin < DF_EXP_CUT;
+                constexpr float LN2 = 0.693147181f, S = 1.0f / EXP_N;
+                if (on0 && (!on1 || ex.twice[1]) && !on2) {
+                    const float ch0 = ex.ch[0] * S, cl0 = ex.cl[0] * S;
+                    for (int q = 0; q < ch; q++) {
+                        const float2 X = s_sq[q][li], Y = s_sq[q][DT_X + lj];
+                        const float4 W = *reinterpret_cast<const float4*>(&s_w[q][0]);
+                        const float xh = X.x + Y.x, xl = X.y + Y.y, w1 = on1 ? W.z : 0.0f;
+#pragma unroll
+                        for (int n = 0; n < 2; n++) {
+                            const float2 Z = s_sq[q][DT_X + DT_Y + lk + 4 * n];
+                            const df y = exponent(root(xh + Z.x, xl + Z.y), ch0, cl0);
+                            const float e0 = ex2_neg(y.h), e = fmaf(-LN2 * y.l, e0, e0);
+                            float& f = n ? fB : fA;
+                            f = fmaf(fmaf(w1, e, W.x), e, f);
+                        }
+                    }
+                } else {
+                    for (int q = 0; q < ch; q++) {
+                        const float2 X = s_sq[q][li], Y = s_sq[q][DT_X + lj];
+                        const float xh = X.x + Y.x, xl = X.y + Y.y;
+#pragma unroll
+                        for (int n = 0; n < 2; n++) {
+                            const float2 Z = s_sq[q][DT_X + DT_Y + lk + 4 * n];
+                            const df r = root(xh + Z.x, xl + Z.y);
+#pragma unroll
+                            for (int v = 0; v < 3; v++) {
+                                if (!(v == 0 ? on0 : v == 1 ? on1 : on2)) continue;
+                                const df y = exponent(r, ex.ch[v] * S, ex.cl[v] * S);
+                                const float e0 = ex2_neg(y.h);
+                                float& f = n ? fB : fA;
+                                f = fmaf(s_w[q][2 * v], fmaf(-LN2 * y.l, e0, e0), f);
+                            }
+                        }
+                    }
+                }
+            }
+        }
+    }
+
+    // ---- far atoms: their terms, each below e^-FAR_T of its weight, in plain FP32 and added to
+    // the double-float sum once.  The distance comes from the FP32 roundings of the two offsets
+    // (one subtraction per axis): the atom's offset is at most r plus the tile's extent, so r
+    // carries a relative error of ~1.5e-7.  A term that is beyond the cut-off at every far
+    // distance is dropped for all of them.
     {
-        bool qf[3];
+        const bool on0 = zt[0] * (FAR_T / zmin) < DF_EXP_CUT, on1 = zt[1] * (FAR_T / zmin) < DF_EXP_CUT,
+                   on2 = zt[2] * (FAR_T / zmin) < DF_EXP_CUT;
+        const float l2e = 1.44269504f;
+        const float c0f = zt[0] * l2e, c1f = zt[1] * l2e, c2f = zt[2] * l2e;
+        const float pxf = s_off[li].x, pyf = s_off[DT_X + lj].x;
+        const float pzA = s_off[DT_X + DT_Y + lk].x, pzB = s_off[DT_X + DT_Y + lk + 4].x;
+        for (int c0 = 0; c0 < count[3]; c0 += DF_FCH) {
+            const int ch = min(DF_FCH, count[3] - c0);
+            __syncthreads();
+            for (int t = tid; t < ch; t += DEP_NT) {
+                const float* fr = reinterpret_cast<const float*>(
+                    a.rec + (size_t)SPHERE_REC_DOUBLES * lists[3 * na + c0 + t] + RF);
+                float D[3];
 #pragma unroll
-        for (int q = 0; q < 3; q++) qf[q] = zt[q].h * (FAR_T / zmin) < DF_EXP_CUT;
-        const float z0 = zt[0].h, z1 = zt[1].h, z2 = zt[2].h;
-        for (int q0 = nnear; q0 < nkept; q0++) {
-            const float* o = sat + SAF * q0;
-            const float4 A = *reinterpret_cast<const float4*>(o);
-            const float fx = px.h - A.x, fy = py.h - A.y, fz = pz.h - A.z;
-            const float r2f = fmaf(fx, fx, fmaf(fy, fy, fz * fz));
-            const float rf = r2f * rsqrtf(r2f);
-            if (qf[0]) sfar = fmaf(A.w, __expf(-z0 * rf), sfar);
-            if (qf[1]) sfar = fmaf(o[4], __expf(-z1 * rf), sfar);
-            if (qf[2]) sfar = fmaf(o[5], __expf(-z2 * rf), sfar);
-        }
-    }
-    if (own >= 0) {
-        const double* rc = a.rec + (size_t)SPHERE_REC_DOUBLES * own;
-        const df r = dfa::sqrt_df(orr2);
-        df nbr = {0.0f, 0.0f}, e1 = {1.0f, 0.0f};
-#pragma unroll
-        for (int q = 0; q < 3; q++) {
-            const df zr = dfa::mul(r, zt[q]);
-            const df em = dfa::exp_neg(zr, th, tl), ep = dfa::exp_neg(dfa::neg(zr), th, tl);
-            if (q == 0) e1 = em;
-            df shr;   // sinh(zeta r) / r
-            if (zr.h > 1e-3f) {
-                df sh = dfa::add(ep, dfa::neg(em));
-                sh.h *= 0.5f;
-                sh.l *= 0.5f;
-                shr = dfa::div(sh, r);
-            } else {
-                shr = dfa::mul(zt[q], dfa::add_f(df{1.0f, 0.0f}, zr.h * zr.h * (1.0f / 6.0f)));
+                for (int d = 0; d < 3; d++)
+                    D[d] = (fr[FP + 3 * d] - s_org[d][0]) + (fr[FP + 3 * d + 1] - s_org[d][1]);
+                *reinterpret_cast<float4*>(&s_far[t][0]) = make_float4(D[0], D[1], D[2], fr[FW]);
+                s_far[t][4] = fr[FW + 2];
+                s_far[t][5] = fr[FW + 4];
             }
-            df ch = dfa::add(ep, em);
-            ch.h *= 0.5f;
-            ch.l *= 0.5f;
-            const df A2 = dfa::from_double(2.0 * rc[RA + q]), B2 = dfa::from_double(2.0 * rc[RB + q]);
-            nbr = dfa::add(nbr, dfa::add(dfa::mul(A2, shr), dfa::neg(dfa::mul(B2, ch))));
+            __syncthreads();
+            if (on0 && !on1 && !on2) {
+#pragma unroll 4
+                for (int q = 0; q < ch; q++) {
+                    const float4 A = *reinterpret_cast<const float4*>(&s_far[q][0]);
+                    const float fx = pxf - A.x, fy = pyf - A.y, za = pzA - A.z, zb = pzB - A.z;
+                    const float xy = fmaf(fx, fx, fy * fy);
+                    const float ra = fmaf(za, za, xy), rb = fmaf(zb, zb, xy);
+                    fA = fmaf(A.w, ex2_neg(c0f * (ra * rsqrtf(ra))), fA);
+                    fB = fmaf(A.w, ex2_neg(c0f * (rb * rsqrtf(rb))), fB);
+                }
+            } else {
+                for (int q = 0; q < ch; q++) {
+                    const float4 A = *reinterpret_cast<const float4*>(&s_far[q][0]);
+                    const float fx = pxf - A.x, fy = pyf - A.y, za = pzA - A.z, zb = pzB - A.z;
+                    const float xy = fmaf(fx, fx, fy * fy);
+                    const float ra2 = fmaf(za, za, xy), rb2 = fmaf(zb, zb, xy);
+                    const float ra = ra2 * rsqrtf(ra2), rb = rb2 * rsqrtf(rb2);
+                    if (on0) {
+                        fA = fmaf(A.w, ex2_neg(c0f * ra), fA);
+                        fB = fmaf(A.w, ex2_neg(c0f * rb), fB);
+                    }
+                    if (on1) {
+                        fA = fmaf(s_far[q][4], ex2_neg(c1f * ra), fA);
+                        fB = fmaf(s_far[q][4], ex2_neg(c1f * rb), fB);
+                    }
+                    if (on2) {
+                        fA = fmaf(s_far[q][5], ex2_neg(c2f * ra), fA);
+                        fB = fmaf(s_far[q][5], ex2_neg(c2f * rb), fB);
+                    }
+                }
+            }
         }
-        const df ca = dfa::from_double(rc[RC]), cb = dfa::from_double(rc[RC + 1]), cc = dfa::from_double(rc[RC + 2]);
-        const df pseudo = dfa::add(ca, dfa::mul(orr2, dfa::add(cb, dfa::mul(orr2, cc))));
-        // nonspherical part: slater(zeta_1, r) (1 - r^2/R^2)^2 sum c_lm (r/R)^l y_lm
-        const float* ns = reinterpret_cast<const float*>(rc + RNS);
-        df pxs[5], pys[5], pzs[5];
-        pxs[0] = pys[0] = pzs[0] = df{1.0f, 0.0f};
-        for (int p = 1; p < 5; p++) {
-            pxs[p] = dfa::mul(pxs[p - 1], odx);
-            pys[p] = dfa::mul(pys[p - 1], ody);
-            pzs[p] = dfa::mul(pzs[p - 1], odz);
-        }
-        df ang = {0.0f, 0.0f};
-        for (int t = 1; t < N_MONO_TERMS; t++) {
-            const MonoF m = c_mono_f[t];
-            const df term = dfa::mul(dfa::mul(df{m.h, m.l}, df{ns[2 * (m.lm - 1)], ns[2 * (m.lm - 1) + 1]}),
-                                     dfa::mul(dfa::mul(pxs[m.a], pys[m.b]), pzs[m.c]));
-            ang = dfa::add(ang, term);
-        }
-        const double R = rc[RR];
-        const df invR2 = dfa::from_double(1.0 / (R * R));
-        const df tt = dfa::add_f(dfa::neg(dfa::mul(orr2, invR2)), 1.0f);
-        const double z1 = rc[RZ];
-        const df radial = dfa::mul(dfa::mul(dfa::from_double(z1 * z1 * z1 / (8.0 * PI)), e1), dfa::sqr(tt));
-        const df nsv = dfa::mul(radial, ang);
-        s = dfa::add(dfa::add(s, dfa::neg(nbr)), dfa::add(pseudo, nsv));
     }
-    s = dfa::add_f(s, sfar);
+
+    // nodes outside every sphere are done; the others' sums go to a queue that full warps take
+    // (one to ten lanes of a warp are inside a sphere where any are)
+    auto store = [&](int P, double bv) {
+        a.b[P] = bv;
+        // (infinities and NaN by the exponent's bits)
+        if ((__double2hiint(bv) & 0x7ff00000) == 0x7ff00000 && a.status) atomicMax(a.status, (int)LASTO_ERR_NONFINITE);
+    };
     const df fourpi = dfa::from_double(4.0 * PI);
-    const double bv = dfa::to_double(dfa::mul(fourpi, s));
-    a.b[P] = bv;
-    if (a.owner) a.owner[P] = own;
-    if (!isfinite(bv) && a.status) atomicMax(a.status, (int)LASTO_ERR_NONFINITE);
+    __syncthreads();   // the staged atoms are not needed any more: their memory holds the queue
+    float2* q_sum = &s_sq[0][0];
+    int* q_node = reinterpret_cast<int*>(&s_far[0][0]);   // place in the tile, then the atom
+    static_assert(sizeof(s_sq) >= 2 * DEP_NT * sizeof(float2) && sizeof(s_far) >= 4 * DEP_NT * sizeof(int), "queue");
+#pragma unroll
+    for (int n = 0; n < 2; n++) {
+        if (!(n ? okB : okA)) continue;
+        const int own = n ? ownB : ownA;
+        df s = n ? sB : sA;
+        s = dfa::add_f(dfa::fast_two_sum(s.h, s.l), n ? fB : fA);
+        const int P = ((n ? kB : kA) * a.n[1] + j) * a.n[0] + i;   // (grids hold fewer than 2^31 nodes)
+        if (a.owner) a.owner[P] = own;
+        if (own < 0) {
+            store(P, dfa::to_double(dfa::mul(fourpi, s)));
+        } else {
+            const int e = atomicAdd(&s_queued, 1);
+            q_sum[e] = make_float2(s.h, s.l);
+            q_node[2 * e] = tid | n << 8;
+            q_node[2 * e + 1] = own;
+        }
+    }
+    __syncthreads();
+    for (int e = tid; e < s_queued; e += DEP_NT) {
+        const int node = q_node[2 * e];
+        const int ni = node & 7, nj = node >> 3 & 7, nk = (node >> 6 & 3) + 4 * (node >> 8);
+        const double* rc = a.rec + (size_t)SPHERE_REC_DOUBLES * q_node[2 * e + 1];
+        const float* fr = reinterpret_cast<const float*>(rc + RF) + FP;
+        df d[3];
+#pragma unroll
+        for (int v = 0; v < 3; v++) {
+            const df D = diff3(fr + 3 * v, s_org[v]);
+            const float2 o = s_off[v == 0 ? ni : v == 1 ? DT_X + nj : DT_X + DT_Y + nk];
+            d[v] = dfa::add(df{o.x, o.y}, dfa::neg(D));
+        }
+        const double v = inside_value(df{q_sum[e].x, q_sum[e].y}, rc, d[0], d[1], d[2], ex, s_T);
+        store(((k0 + nk) * a.n[1] + j0 + nj) * a.n[0] + i0 + ni, 4.0 * PI * v);
+    }
 }
 
 void init_device_constants()
