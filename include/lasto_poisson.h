@@ -316,7 +316,7 @@ int lasto_op_deposit(const lasto_cluster* cl, int precision, double* b, int* own
  * owned by another framework's allocator, a real-time loop that forbids allocation).
  * The paper has no counterpart: this is a property of the library, not of the method.
  * Same arguments, kernels and results as lasto_op_deposit; the per-sphere records live
- * in one file-scope device array sized for 1024 atoms (640 KiB, held by every device
+ * in one file-scope device array sized for 1024 atoms (928 KiB, held by every device
  * that loads the library until exit) instead of allocator scratch.  No cudaMalloc,
  * cudaFree or allocating library routine is called.
  * b (and owner, when given) must hold N = n0 n1 n2 elements: the entry point takes no

@@ -33,6 +33,7 @@ constexpr int EXP_N = 2048;   // entries of the exponential's table: a power of 
 // ln 2 / EXP_N, also as a double-float
 constexpr double LN2_N = 0.69314718055994530942 / EXP_N;
 constexpr float LN2_H = (float)LN2_N, LN2_L = (float)(LN2_N - (double)LN2_H);
+static __device__ double g_exp_tab64[EXP_N];
 static __device__ float2 g_exp_tab[EXP_N];   // 2^(-j/EXP_N) as double-floats
 
 void host_monomials(Mono* o)
@@ -89,11 +90,11 @@ void host_solid_harmonics(double x, double y, double z, double* S)
 // pairs, zeta, EXP_N zeta / ln 2 pairs, which zeta are twice zeta_0, 2 A and 2 B pairs, 1/R^2,
 // zeta_1^3 / (8 pi), and the nonspherical polynomial sum_lm c_lm / R^l S_lm: a pair per monomial
 // x^a y^b z^c of degree 0 to 4 (the constant is 0) in the order of its Horner evaluation, a = 4..0,
-// b = 4-a..0, c = 4-a-b..0
-enum { RX = 0, RR = 3, RW = 4, RZ = 7, RA = 10, RB = 13, RC = 16, RQ = 19, RRHO = 20, RDRHO = 21, RXF = 22, RF = 24 };
+// b = 4-a..0, c = 4-a-b..0; from 80 the same coefficients in FP64
+enum { RX = 0, RR = 3, RW = 4, RZ = 7, RA = 10, RB = 13, RC = 16, RQ = 19, RRHO = 20, RDRHO = 21, RXF = 22, RF = 24, RP = 80 };
 enum { FP = 0, FW = 9, FZ = 15, FC = 18, F2 = 24, FA = 26, FB = 32, FR = 38, FN = 40, FH = 42 };   // floats from RF
 constexpr int POLY_N = 35;
-static_assert(RF + (FH + 2 * POLY_N + 1) / 2 <= SPHERE_REC_DOUBLES, "sphere record");
+static_assert(RF + (FH + 2 * POLY_N + 1) / 2 <= RP && RP + POLY_N <= SPHERE_REC_DOUBLES, "sphere record");
 
 // place of x^a y^b z^c in the Horner order
 __host__ __device__ constexpr int poly_slot(int a, int b, int c)
@@ -143,11 +144,15 @@ static cudaError_t ensure_monomials()
     e = cudaMemcpyToSymbol(g_poly, pt, sizeof(pt));
     if (e != cudaSuccess) return e;
     static float2 ex[EXP_N];   // (under the lock)
+    static double ex64[EXP_N];
     for (int j = 0; j < EXP_N; j++) {
         const double v = std::exp2(-j / (double)EXP_N);
+        ex64[j] = v;
         ex[j].x = (float)v;
         ex[j].y = (float)(v - (double)ex[j].x);
     }
+    e = cudaMemcpyToSymbol(g_exp_tab64, ex64, sizeof(ex64));
+    if (e != cudaSuccess) return e;
     e = cudaMemcpyToSymbol(g_exp_tab, ex, sizeof(ex));
     if (e == cudaSuccess) g_mono_uploaded[dev] = true;
     return e;
@@ -297,6 +302,7 @@ __global__ void __launch_bounds__(SPH_NT) k_sphere_params(SphArgs a)
             float* f = reinterpret_cast<float*>(r + RF) + FH + 2 * slot;
             f[0] = c.h;
             f[1] = c.l;
+            r[RP + slot] = v;
         }
     } else if (tid == 64) {
         r[RX] = xi;
@@ -372,7 +378,7 @@ cudaError_t launch_sphere_params(const lasto_cluster& cl, const double* ax0, con
     return cudaGetLastError();
 }
 
-// ---------------------------------------------------------------- deposit (FP64)
+// ---------------------------------------------------------------- deposit
 struct DepArgs {
     int na;
     int n[3];
@@ -386,8 +392,6 @@ struct DepArgs {
 
 __global__ void k_deposit_df(DepArgs a);
 
-// per-atom fields staged in shared memory
-constexpr int SA = 14;  // x y z R^2 W0 W1 W2 A0 A1 A2 B0 B1 B2 R
 constexpr int DEP_NT = 256;
 constexpr double EXP_CUT = 40.0;   // e^{-40} * max W < 1e-14 absolute; skipped terms are below FP64 rounding of n_e
 // FP32-pair deposit: where a pair's precision changes, in units of 1/zeta_min.  A Slater term is
@@ -406,100 +410,9 @@ constexpr float FAR_T = 22.0f;
 // 1e-3 of its maximum is 2e-11 to 6e-11 of the local density at 37; at 34 it was 3.6e-10.
 constexpr float DF_EXP_CUT = 37.0f;
 
-__device__ __forceinline__ double nonspherical(const double* __restrict__ c, double dx, double dy, double dz,
-                                               double r, double R, double z1)
-{
-    double S[NLM];
-    solid_harmonics(dx, dy, dz, S);
-    const double iR = 1.0 / R;
-    double ang = 0.0, Rl = iR;
-    int l = 1;
-    for (int lm = 1; lm < NLM; lm++) {
-        const int ll = l_of_lm(lm);
-        if (ll != l) {
-            Rl *= iR;
-            l = ll;
-        }
-        ang = fma(c[lm - 1] * Rl, S[lm], ang);
-    }
-    const double t = 1.0 - r * r * iR * iR;
-    return z1 * z1 * z1 / (8.0 * PI) * exp(-z1 * r) * t * t * ang;
-}
-
-__global__ void __launch_bounds__(DEP_NT) k_deposit64(DepArgs a)
-{
-    extern __shared__ double sat[];
-    // the exponents are the same on every atom (checked by the sphere kernel): take atom 0's
-    const double z0 = a.rec[RZ], z1 = a.rec[RZ + 1], z2 = a.rec[RZ + 2];
-    for (int t = threadIdx.x; t < a.na; t += DEP_NT) {
-        const double* r = a.rec + (size_t)SPHERE_REC_DOUBLES * t;
-        double* o = sat + SA * t;
-        o[0] = r[RX];
-        o[1] = r[RX + 1];
-        o[2] = r[RX + 2];
-        o[3] = r[RR] * r[RR];
-        for (int k = 0; k < 3; k++) {
-            o[4 + k] = r[RW + k];
-            o[7 + k] = r[RA + k];
-            o[10 + k] = r[RB + k];
-        }
-        o[13] = r[RR];
-    }
-    __syncthreads();
-    const size_t N = (size_t)a.n[0] * a.n[1] * a.n[2];
-    const size_t P = blockIdx.x * (size_t)DEP_NT + threadIdx.x;
-    if (P >= N) return;
-    const size_t nxy = (size_t)a.n[0] * a.n[1];
-    const int k = (int)(P / nxy);
-    const int j = (int)((P - (size_t)k * nxy) / a.n[0]);
-    const int i = (int)(P - (size_t)k * nxy - (size_t)j * a.n[0]);
-    const double x = a.ax[0][i], y = a.ax[1][j], z = a.ax[2][k];
-    const double zz[3] = {z0, z1, z2};
-    double s = 0.0;
-    int own = -1;
-    double ox = 0, oy = 0, oz = 0, or2 = 0;
-    for (int t = 0; t < a.na; t++) {
-        const double* o = sat + SA * t;
-        const double dx = x - o[0], dy = y - o[1], dz = z - o[2];
-        const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-        if (r2 < o[3]) {
-            own = t;
-            ox = dx;
-            oy = dy;
-            oz = dz;
-            or2 = r2;
-            continue;
-        }
-        const double r = sqrt(r2);
-#pragma unroll
-        for (int q = 0; q < 3; q++) {
-            const double e = zz[q] * r;
-            if (e < EXP_CUT) s = fma(o[4 + q], exp(-e), s);
-        }
-    }
-    if (own >= 0) {
-        const double* o = sat + SA * own;
-        const double* rc = a.rec + (size_t)SPHERE_REC_DOUBLES * own;
-        const double r = sqrt(or2);
-        double nbr = 0.0;
-#pragma unroll
-        for (int q = 0; q < 3; q++) {
-            const double zr = zz[q] * r;
-            const double shr = (zr > 1e-6) ? sinh(zr) / r : zz[q] * (1.0 + zr * zr / 6.0);
-            nbr += 2.0 * o[7 + q] * shr - 2.0 * o[10 + q] * cosh(zr);
-        }
-        const double pseudo = fma(fma(rc[RC + 2], or2, rc[RC + 1]), or2, rc[RC]);
-        const double ns = nonspherical(a.clm + 24 * (size_t)own, ox, oy, oz, r, o[13], z0);
-        s = s - nbr + ns + pseudo;
-    }
-    const double bv = 4.0 * PI * s;
-    a.b[P] = bv;
-    if (a.owner) a.owner[P] = own;
-    if (!isfinite(bv) && a.status) atomicMax(a.status, (int)LASTO_ERR_NONFINITE);
-}
-
-
-// FP32-pair deposit: one 8 x 8 x 8 tile of nodes per block, two nodes (four planes apart) per thread
+// one 8 x 8 x 8 tile of nodes per block, two nodes (four planes apart) per thread
+__global__ void k_deposit64(DepArgs a);
+constexpr int DEP64_MAX_ATOMS = 1828;   // most atoms the FP64 form takes (two index lists in shared memory)
 constexpr int DT_X = 8, DT_Y = 8, DT_Z = 8;
 static_assert(DT_X * DT_Y * DT_Z == 2 * DEP_NT, "deposit tile = one block");
 constexpr int DF_MAX_ATOMS = 2431;   // most atoms the FP32-pair form takes (four index lists in shared memory)
@@ -520,22 +433,18 @@ cudaError_t launch_deposit(const lasto_cluster& cl, const double* rec, int preci
     a.b = b;
     a.owner = owner;
     a.status = status;
-    const size_t N = (size_t)cl.n[0] * cl.n[1] * cl.n[2];
-    const size_t smem = sizeof(double) * SA * (size_t)cl.n_atoms;
-    if (precision == LASTO_PREC_MIXED) {
-        if (cl.n_atoms > DF_MAX_ATOMS) return cudaErrorInvalidValue;
-        const dim3 grid((unsigned)((cl.n[0] + DT_X - 1) / DT_X), (unsigned)((cl.n[1] + DT_Y - 1) / DT_Y),
-                        (unsigned)((cl.n[2] + DT_Z - 1) / DT_Z));
-        if (grid.y > 65535 || grid.z > 65535) return cudaErrorInvalidValue;
+    const bool mixed = precision == LASTO_PREC_MIXED;
+    if (cl.n_atoms > (mixed ? DF_MAX_ATOMS : DEP64_MAX_ATOMS)) return cudaErrorInvalidValue;
+    const dim3 grid((unsigned)((cl.n[0] + DT_X - 1) / DT_X), (unsigned)((cl.n[1] + DT_Y - 1) / DT_Y),
+                    (unsigned)((cl.n[2] + DT_Z - 1) / DT_Z));
+    if (grid.y > 65535 || grid.z > 65535) return cudaErrorInvalidValue;
+    if (mixed)
         k_deposit_df<<<grid, DEP_NT, sizeof(int) * 4 * (size_t)cl.n_atoms, s>>>(a);
-        return cudaGetLastError();
-    }
-    if (smem > 200 * 1024) return cudaErrorInvalidValue;
-    k_deposit64<<<(unsigned)((N + DEP_NT - 1) / DEP_NT), DEP_NT, smem, s>>>(a);
+    else
+        k_deposit64<<<grid, DEP_NT, sizeof(int) * 2 * (size_t)cl.n_atoms, s>>>(a);
     return cudaGetLastError();
 }
 
-// ---------------------------------------------------------------- deposit (FP32 pairs)
 __device__ __forceinline__ bool inside_fp64(const DepArgs& a, double x, double y, double z, int t)
 {
     const double* r = a.rec + (size_t)SPHERE_REC_DOUBLES * t;
@@ -543,6 +452,260 @@ __device__ __forceinline__ bool inside_fp64(const DepArgs& a, double x, double y
     return fma(dx, dx, fma(dy, dy, dz * dz)) < r[RR] * r[RR];
 }
 
+// ---------------------------------------------------------------- deposit (FP64)
+constexpr double ROUND_MAGIC64 = 6755399441055744.0;   // 1.5 * 2^52
+
+// r of a squared distance: the hardware's approximate reciprocal square root (about 20 bits, not
+// on the FP64 pipe) and one third-order step, t (1 - h)^(-1/2) = t (1 + h/2 + 3 h^2/8 + O(h^3))
+__device__ __forceinline__ double root64(double r2)
+{
+    double s;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(s) : "d"(r2));
+    const double t = r2 * s, h = fma(-t, s, 1.0);
+    return fma(t * h, fma(h, 0.375, 0.5), t);
+}
+
+// e^{-zeta r}, c = EXP_N zeta / ln 2: k = round(c r), 2^(-k/EXP_N) from the table times 1 + p,
+// p = e^x - 1 to third order (|x| <= 1.7e-4: the fourth is 3.5e-17): seven FP64 operations.  k at
+// least kmax: returns false without the last four.
+__device__ __forceinline__ bool exp64(double r, double c, int kmax, const double* __restrict__ T, double* e)
+{
+    constexpr double C1 = -LN2_N, C2 = 0.5 * LN2_N * LN2_N, C3 = -LN2_N * LN2_N * LN2_N / 6.0;
+    const double y = fma(r, c, ROUND_MAGIC64);
+    // (the bits of y grow with it, also beyond the range of a 32-bit k)
+    if (__double_as_longlong(y) - 0x4338000000000000ll >= kmax) return false;
+    const int k = __double2loint(y);
+    const double f = fma(r, c, -(y - ROUND_MAGIC64));
+    const double t = T[k & (EXP_N - 1)];
+    const double v = fma(t, f * fma(f, fma(f, C3, C2), C1), t);
+    *e = __hiloint2double(__double2hiint(v) - (k & ~(EXP_N - 1)) * ((1 << 20) / EXP_N), __double2loint(v));
+    return true;
+}
+
+// FP64 form of inside_value below: s - N_i(r) + rho_ns + pseudo-density at the offset d
+__device__ __noinline__ double inside_value64(double s, const double* __restrict__ rc, double dx, double dy, double dz,
+                                              const double* __restrict__ T)
+{
+    const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+    const double r = r2 > 0.0 ? root64(r2) : 0.0, ir = r > 0.0 ? 1.0 / r : 0.0;
+    double nbr = 0.0, e1 = 1.0;
+#pragma unroll 1
+    for (int q = 0; q < 3; q++) {
+        const double z = rc[RZ + q], c = z * (1.0 / LN2_N), zr = z * r;
+        double em = 0.0, ep = 0.0;
+        exp64(r, c, 0x7fffffff, T, &em);
+        exp64(r, -c, 0x7fffffff, T, &ep);
+        if (q == 0) e1 = em;
+        double shr;   // sinh(zeta r) / r
+        if (zr > 0.3) {
+            shr = 0.5 * (ep - em) * ir;
+        } else {      // its series to (zeta r)^10
+            const double x2 = zr * zr;
+            shr = z * fma(x2, fma(x2, fma(x2, fma(x2, fma(x2, 1.0 / 39916800.0, 1.0 / 362880.0), 1.0 / 5040.0), 1.0 / 120.0),
+                                  1.0 / 6.0), 1.0);
+        }
+        nbr += fma(2.0 * rc[RA + q], shr, -rc[RB + q] * (ep + em));
+    }
+    double ang = 0.0;
+#pragma unroll
+    for (int a = 4; a >= 0; a--) {
+        double qy = 0.0;
+#pragma unroll
+        for (int b = 4 - a; b >= 0; b--) {
+            double qz = rc[RP + poly_slot(a, b, 4 - a - b)];
+#pragma unroll
+            for (int c = 3 - a - b; c >= 0; c--) qz = fma(qz, dz, rc[RP + poly_slot(a, b, c)]);
+            qy = b == 4 - a ? qz : fma(qy, dy, qz);
+        }
+        ang = a == 4 ? qy : fma(ang, dx, qy);
+    }
+    const double iR = 1.0 / rc[RR], tt = fma(-r2 * iR, iR, 1.0), z1 = rc[RZ];
+    const double ns = z1 * z1 * z1 / (8.0 * PI) * e1 * tt * tt * ang;
+    return s - nbr + ns + fma(fma(rc[RC + 2], r2, rc[RC + 1]), r2, rc[RC]);
+}
+
+// The FP64 deposit on the tiles of the FP32-pair form: atoms beyond the cut-off of a tile's
+// bounding box dropped, the others sorted into those close enough for every term and for the test
+// of the node inside the sphere (within 40 / the largest zeta, or their own radius), and the rest,
+// whose largest-zeta terms are all dropped; the squares of the coordinate differences staged.  A
+// pair takes 16 FP64 operations (two additions, five for the root, seven for e^{-zeta_0 r}, two
+// for (W0 + W1 e) e) where a distance, a correctly rounded root and a library exponential per
+// term took about 50; nodes inside spheres are queued for full warps.  Bound: FP64 issue (0.595 T
+// per second here): Pd55 129^3 9912 -> 3356 us, Pd13 65^3 463 -> 210 us.
+constexpr int D64_CH = 32;
+__global__ void __launch_bounds__(DEP_NT) k_deposit64(DepArgs a)
+{
+    extern __shared__ int lists[];                  // [2][na]
+    constexpr int ROWS = DT_X + DT_Y + DT_Z;
+    __shared__ unsigned s_cnt[DEP_NT / 32];
+    __shared__ int s_queued;
+    __shared__ double s_x[ROWS];                    // node coordinates
+    __shared__ double s_T[EXP_N];
+    __shared__ __align__(16) double s_sq[D64_CH][ROWS];
+    __shared__ __align__(16) double s_w[D64_CH][4];  // W, R^2
+    const int tid = threadIdx.x, na = a.na;
+    const int i0 = blockIdx.x * DT_X, j0 = blockIdx.y * DT_Y, k0 = blockIdx.z * DT_Z;
+    const int li = tid & 7, lj = (tid >> 3) & 7, lk = tid >> 6;
+    if (tid == 0) s_queued = 0;
+    for (int t = tid; t < EXP_N; t += DEP_NT) s_T[t] = g_exp_tab64[t];
+    if (tid < ROWS) {
+        const int d = tid >> 3, first = d == 0 ? i0 : d == 1 ? j0 : k0;
+        s_x[tid] = a.ax[d][min(first + (tid & 7), a.n[d] - 1)];
+    }
+    // the exponents are the same on every atom (checked by the sphere kernel)
+    const float* f0 = reinterpret_cast<const float*>(a.rec + RF);
+    const bool twice1 = __float_as_int(f0[F2]) & 1, twice2 = __float_as_int(f0[F2]) & 2;
+    const float zf[3] = {f0[FZ], f0[FZ + 1], f0[FZ + 2]};
+    const float zmin = fminf(fminf(zf[0], zf[1]), zf[2]), zmax = fmaxf(fmaxf(zf[0], zf[1]), zf[2]);
+    const double c[3] = {a.rec[RZ] * (1.0 / LN2_N), a.rec[RZ + 1] * (1.0 / LN2_N), a.rec[RZ + 2] * (1.0 / LN2_N)};
+    const int kcut = (int)(EXP_CUT / LN2_N);
+    __syncthreads();
+    // margins 1e-3 on the squared distances cover the rounding of the FP32 tests
+    int count[2] = {0, 0};
+    {
+        const float cut = (float)EXP_CUT * (1.0f + 1e-3f);
+        const float lim = (cut / zmin) * (cut / zmin), near2 = (cut / zmax) * (cut / zmax);
+        const int w = tid >> 5, l = tid & 31;
+        for (int base = 0; base < na; base += DEP_NT) {
+            const int t = base + tid;
+            int cls = 2;
+            if (t < na) {
+                const float4 p = *reinterpret_cast<const float4*>(a.rec + (size_t)SPHERE_REC_DOUBLES * t + RXF);
+                const float dx = fmaxf(fmaxf((float)s_x[0] - p.x, p.x - (float)s_x[DT_X - 1]), 0.0f);
+                const float dy = fmaxf(fmaxf((float)s_x[DT_X] - p.y, p.y - (float)s_x[DT_X + DT_Y - 1]), 0.0f);
+                const float dz = fmaxf(fmaxf((float)s_x[DT_X + DT_Y] - p.z, p.z - (float)s_x[ROWS - 1]), 0.0f);
+                const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+                // (comparisons that a NaN position or exponent fails: such an atom is near)
+                cls = !(d2 > p.w * (1.0f + 1e-3f)) || !(d2 > near2) ? 0 : d2 > lim ? 2 : 1;
+            }
+            const unsigned m0 = __ballot_sync(0xffffffffu, cls == 0), m1 = __ballot_sync(0xffffffffu, cls == 1);
+            if (l == 0) s_cnt[w] = __popc(m0) | __popc(m1) << 16;
+            __syncthreads();
+            unsigned before = 0, all = 0;
+            for (int v = 0; v < DEP_NT / 32; v++) {
+                if (v == w) before = all;
+                all += s_cnt[v];
+            }
+            if (cls < 2)
+                lists[cls * na + (cls ? count[1] + (int)(before >> 16) : count[0] + (int)(before & 0xffff)) +
+                      __popc((cls ? m1 : m0) & ((1u << l) - 1u))] = t;
+            __syncthreads();
+            count[0] += (int)(all & 0xffff);
+            count[1] += (int)(all >> 16);
+        }
+    }
+    const int i = i0 + li, j = j0 + lj, kA = k0 + lk, kB = kA + 4;
+    const bool okA = i < a.n[0] && j < a.n[1] && kA < a.n[2], okB = okA && kB < a.n[2];
+    double sA = 0.0, sB = 0.0;
+    int ownA = -1, ownB = -1;
+    // terms that a distant atom keeps: zeta_q below the largest
+    const bool on0 = zf[0] < zmax, on1 = zf[1] < zmax, on2 = zf[2] < zmax;
+    for (int pass = 0; pass < 2; pass++) {
+        const int cnt = count[pass];
+        const int* list = lists + pass * na;
+        for (int c0 = 0; c0 < cnt; c0 += D64_CH) {
+            const int ch = min(D64_CH, cnt - c0);
+            __syncthreads();
+            for (int t = tid; t < ch * ROWS; t += DEP_NT) {
+                const int q = t / ROWS, r = t - q * ROWS;
+                const double d = s_x[r] - a.rec[(size_t)SPHERE_REC_DOUBLES * list[c0 + q] + RX + (r >> 3)];
+                s_sq[q][r] = d * d;
+            }
+            for (int t = tid; t < ch * 4; t += DEP_NT) {
+                const double* r = a.rec + (size_t)SPHERE_REC_DOUBLES * list[c0 + (t >> 2)];
+                s_w[t >> 2][t & 3] = (t & 3) < 3 ? r[RW + (t & 3)] : r[RR] * r[RR];
+            }
+            __syncthreads();
+            if (pass == 0) {
+                for (int q = 0; q < ch; q++) {
+                    const double xy = s_sq[q][li] + s_sq[q][DT_X + lj];
+                    const double w0 = s_w[q][0], w1 = s_w[q][1], w2 = s_w[q][2], R2 = s_w[q][3];
+#pragma unroll
+                    for (int n = 0; n < 2; n++) {
+                        const double r2 = xy + s_sq[q][DT_X + DT_Y + lk + 4 * n];
+                        if (r2 < R2 * (1.0 + 1e-14)) {   // decided on the unrounded differences near the surface
+                            const int t = list[c0 + q];
+                            if (r2 < R2 * (1.0 - 1e-14) ||
+                                inside_fp64(a, s_x[li], s_x[DT_X + lj], s_x[DT_X + DT_Y + lk + 4 * n], t)) {
+                                if (n) ownB = t;
+                                else ownA = t;
+                                continue;
+                            }
+                        }
+                        const double r = r2 > 0.0 ? root64(r2) : 0.0;
+                        double& s = n ? sB : sA;
+                        double e0 = 0.0, e = 0.0;
+                        const bool in0 = exp64(r, c[0], kcut, s_T, &e0);
+                        if (in0) s = fma(w0, e0, s);
+                        if (twice1) s = fma(w1, e0 * e0, s);
+                        else if (exp64(r, c[1], kcut, s_T, &e)) s = fma(w1, e, s);
+                        if (twice2) s = fma(w2, e0 * e0, s);
+                        else if (exp64(r, c[2], kcut, s_T, &e)) s = fma(w2, e, s);
+                    }
+                }
+            } else if (on0 && on1 && twice1 && !on2) {
+                for (int q = 0; q < ch; q++) {
+                    const double xy = s_sq[q][li] + s_sq[q][DT_X + lj];
+                    const double w0 = s_w[q][0], w1 = s_w[q][1];
+#pragma unroll
+                    for (int n = 0; n < 2; n++) {
+                        double e;
+                        if (exp64(root64(xy + s_sq[q][DT_X + DT_Y + lk + 4 * n]), c[0], kcut, s_T, &e)) {
+                            double& s = n ? sB : sA;
+                            s = fma(fma(w1, e, w0), e, s);
+                        }
+                    }
+                }
+            } else {
+                for (int q = 0; q < ch; q++) {
+                    const double xy = s_sq[q][li] + s_sq[q][DT_X + lj];
+#pragma unroll
+                    for (int n = 0; n < 2; n++) {
+                        const double r = root64(xy + s_sq[q][DT_X + DT_Y + lk + 4 * n]);
+                        double& s = n ? sB : sA;
+                        double e;
+                        if (on0 && exp64(r, c[0], kcut, s_T, &e)) s = fma(s_w[q][0], e, s);
+                        if (on1 && exp64(r, c[1], kcut, s_T, &e)) s = fma(s_w[q][1], e, s);
+                        if (on2 && exp64(r, c[2], kcut, s_T, &e)) s = fma(s_w[q][2], e, s);
+                    }
+                }
+            }
+        }
+    }
+    auto store = [&](int P, double bv) {
+        a.b[P] = bv;
+        if ((__double2hiint(bv) & 0x7ff00000) == 0x7ff00000 && a.status) atomicMax(a.status, (int)LASTO_ERR_NONFINITE);
+    };
+    __syncthreads();   // the staged squares are not needed any more: their memory holds the queue
+    double* q_sum = &s_sq[0][0];
+    __shared__ int q_node[2 * DEP_NT][2];
+    static_assert(sizeof(s_sq) >= 2 * DEP_NT * sizeof(double), "queue");
+#pragma unroll
+    for (int n = 0; n < 2; n++) {
+        if (!(n ? okB : okA)) continue;
+        const int own = n ? ownB : ownA, P = ((n ? kB : kA) * a.n[1] + j) * a.n[0] + i;   // (fewer than 2^31 nodes)
+        if (a.owner) a.owner[P] = own;
+        if (own < 0) {
+            store(P, 4.0 * PI * (n ? sB : sA));
+        } else {
+            const int e = atomicAdd(&s_queued, 1);
+            q_sum[e] = n ? sB : sA;
+            q_node[e][0] = tid | n << 8;
+            q_node[e][1] = own;
+        }
+    }
+    __syncthreads();
+    for (int e = tid; e < s_queued; e += DEP_NT) {
+        const int node = q_node[e][0];
+        const int ni = node & 7, nj = node >> 3 & 7, nk = (node >> 6 & 3) + 4 * (node >> 8);
+        const double* rc = a.rec + (size_t)SPHERE_REC_DOUBLES * q_node[e][1];
+        const double v = inside_value64(q_sum[e], rc, s_x[ni] - rc[RX], s_x[DT_X + nj] - rc[RX + 1],
+                                        s_x[DT_X + DT_Y + nk] - rc[RX + 2], s_T);
+        store(((k0 + nk) * a.n[1] + j0 + nj) * a.n[0] + i0 + ni, 4.0 * PI * v);
+    }
+}
+
+// ---------------------------------------------------------------- deposit (FP32 pairs)
 constexpr float ROUND_MAGIC = 12582912.0f;   // 1.5 * 2^23: adding it rounds to an integer in the low bits
 
 // the power of two 2^-floor(k / EXP_N) from the bits of k + ROUND_MAGIC

@@ -14,7 +14,7 @@
 namespace {
 
 // Largest cluster the allocation-free deposit accepts.  The array below is
-// LASTO_NOALLOC_MAX_ATOMS * 80 doubles = 640 KiB, held by every device that loads the
+// LASTO_NOALLOC_MAX_ATOMS * 116 doubles = 928 KiB, held by every device that loads the
 // library until the process exits.
 constexpr int LASTO_NOALLOC_MAX_ATOMS = 1024;
 
