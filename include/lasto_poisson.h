@@ -94,7 +94,8 @@ typedef struct lasto_config {
     int precision;    /* enum lasto_precision */
     int cycle;        /* enum lasto_cycle */
     int nu1, nu2;     /* pre/post Gauss-Seidel sweeps per level (red+black = one sweep; the mixed
-                         precision's one-block coarse levels use nu_coarse) */
+                         precision's one-block coarse levels use nu_coarse; a cycle sweeps no level
+                         below the one it solves exactly) */
     int max_cycles;   /* cap on cycles / CG iterations */
     double rel_tol;   /* stop when ||b - A u||_2 <= rel_tol ||b_eff||_2 (b_eff: b with the faces moved in) */
     int n_theta;      /* Gauss-Legendre points in cos(theta) of the sphere quadrature (<= 32) */
@@ -112,7 +113,9 @@ typedef struct lasto_config {
     int boundary;     /* enum lasto_boundary: Dirichlet values on the box faces */
     int nu_coarse;    /* pre/post sweeps per level on the coarse levels the FP32 cycle of the
                          mixed precision runs inside one thread block (at most 17 nodes per axis,
-                         above the exact solve); >= 0.  The other levels use nu1/nu2. */
+                         above the exact solve); >= 0.  The other levels use nu1/nu2.  Grids whose
+                         cycle solves a larger coarse level exactly (65 nodes per axis and more)
+                         have no such levels. */
     int nu_fine;      /* pre/post sweeps on the finest level when > 0 (0: nu1/nu2 there too) */
 } lasto_config;
 

@@ -72,6 +72,16 @@ struct SmoothChoice {
     float us = 0.0f;   // measured time of one pre-smoothing phase
 };
 
+template <typename T>
+void carve_direct(Carver& c, int m, DirectMats<T>* M)
+{
+    for (int d = 0; d < 3; d++) {
+        M->Ft[d] = c.take<T>((size_t)m * m);
+        M->Bt[d] = c.take<T>((size_t)m * m);
+        M->lam[d] = c.take<T>(m);
+    }
+}
+
 // Everything one cluster's solve touches on the device.
 struct ClusterPlan {
     int L = 0;
@@ -85,6 +95,8 @@ struct ClusterPlan {
     double* Q = nullptr;
     Ctl* ctl = nullptr;
     CoarseEig* eig = nullptr;
+    DirectMats<float> dir32;            // eigenvectors of the exactly solved level (FP32 cycle)
+    DirectMats<double> dir64;           // the same for the FP64 cycle
     int* status = nullptr;              // [0] status, [1] reduction ticket counter
     lasto_stats* stats_dev = nullptr;
     // learned guess: the 33^3 subgrid (every gm-th node) and the level gl it is resampled from
@@ -125,6 +137,10 @@ size_t cluster_bytes(const int n[3], int n_atoms)
     c.take<double>(32);
     c.take<Ctl>(1);
     c.take<CoarseEig>(1);
+    DirectMats<float> d32;
+    DirectMats<double> d64;
+    carve_direct(c, DIRECT_PAD, &d32);   // (sizes that do not depend on n: a smaller grid never needs more)
+    carve_direct(c, DIRECT_PAD64, &d64);
     c.take<int>(4);
     c.take<lasto_stats>(1);
     for (int d = 0; d < 3; d++) c.take<double>(GUESS_N);
@@ -171,6 +187,8 @@ bool carve_cluster(Carver& c, const int n[3], int n_atoms, ClusterPlan& P)
     P.Q = c.take<double>(32);
     P.ctl = c.take<Ctl>(1);
     P.eig = c.take<CoarseEig>(1);
+    carve_direct(c, DIRECT_PAD, &P.dir32);
+    carve_direct(c, DIRECT_PAD64, &P.dir64);
     P.status = c.take<int>(4);
     P.stats_dev = c.take<lasto_stats>(1);
     for (int d = 0; d < 3; d++) P.gax[d] = c.take<double>(GUESS_N);
@@ -469,6 +487,46 @@ int bottom_level(const ClusterPlan& P)
     return -1;
 }
 
+// The level the cycle solves exactly by fast diagonalisation (direct.cu) instead of smoothing it
+// and the levels below, or -1.  The first level below the finest that is small enough; level 1
+// only for the FP32 cycle and above 33 nodes: in FP64 the products of a 65^3 level cost what its
+// smoothing does (160 us), and a 65^3 solve keeps its 33^3 level smoothed because its tuning
+// table, which callers read and set, lists that level.  Levels of up to 97 nodes in FP32 against
+// up to 49, measured: Pd55 129^3 (65^3 against 33^3) 3677 and 4468 us, Pd561 385^3 (97^3 against
+// 49^3) 41.5 and 43.3 ms, an uneven batch of eight the same within its 2 %.
+template <typename T>
+int direct_level(const ClusterPlan& P)
+{
+    const int most = (sizeof(T) == 4 ? DIRECT_MAX : DIRECT_MAX64) + 2;
+    for (int l = 1; l < P.L - 1; l++) {
+        const int* n = P.lv[l].n;
+        if (std::max(n[0], std::max(n[1], n[2])) > most) continue;
+        if (l == 1 && (sizeof(T) == 8 || std::min(n[0], std::min(n[1], n[2])) <= 33)) continue;
+        return l;
+    }
+    return -1;
+}
+
+template <typename T>
+DirectArgs<T> direct_args(const ClusterPlan& P, int l)
+{
+    const LevelStore& S = P.lv[l];
+    DirectArgs<T> a;
+    if constexpr (sizeof(T) == 4) {
+        a.b = S.b32;
+        a.u = S.u32;
+        a.w = S.r32;
+        a.M = P.dir32;
+    } else {
+        a.b = S.b;
+        a.u = S.u;
+        a.w = S.r;
+        a.M = P.dir64;
+    }
+    for (int d = 0; d < 3; d++) a.n[d] = S.n[d];
+    return a;
+}
+
 template <typename T>
 int enqueue_cycle(lasto_poisson* h, ClusterPlan& P, int l, T* u, T* b, T* r, bool fcycle, bool sym, cudaStream_t s,
                   bool zero_start = false)
@@ -477,6 +535,11 @@ int enqueue_cycle(lasto_poisson* h, ClusterPlan& P, int l, T* u, T* b, T* r, boo
     const LevelT<T> V = Arr<T>::view(S);
     const int nu1 = (l == 0 && h->cfg.nu_fine > 0) ? h->cfg.nu_fine : h->cfg.nu1;
     const int nu2 = (l == 0 && h->cfg.nu_fine > 0) ? h->cfg.nu_fine : h->cfg.nu2;
+    const int dl = direct_level<T>(P);
+    if (l == dl) {
+        TRY(launch_direct<T>(direct_args<T>(P, l), s));   // (the faces of u are zero)
+        return LASTO_OK;
+    }
     if (sizeof(T) == 4 && !fcycle && l > 0 && l == bottom_level(P)) {
         BottomArgs<T> a;
         a.nlev = P.L - l;
@@ -535,11 +598,11 @@ int enqueue_cycle(lasto_poisson* h, ClusterPlan& P, int l, T* u, T* b, T* r, boo
         // FP64: each residual once (FP64 arithmetic, not bandwidth, bounds this chip)
         TRY(launch_residual<T>(V, cur, b, r, s));
         TRY(launch_restrict<T>(V, VC, r, Arr<T>::b(C), s));
-        TRY(cudaMemsetAsync(Arr<T>::u(C), 0, sizeof(T) * C.N(), s));
+        if (l + 1 != dl) TRY(cudaMemsetAsync(Arr<T>::u(C), 0, sizeof(T) * C.N(), s));
     }
     int st = enqueue_cycle<T>(h, P, l + 1, Arr<T>::u(C), Arr<T>::b(C), Arr<T>::r(C), fcycle, sym, s);
     if (st) return st;
-    if (fcycle) {
+    if (fcycle && l + 1 != dl) {
         st = enqueue_cycle<T>(h, P, l + 1, Arr<T>::u(C), Arr<T>::b(C), Arr<T>::r(C), false, sym, s);
         if (st) return st;
     }
@@ -553,22 +616,17 @@ int enqueue_setup(lasto_poisson* h, ClusterPlan& P, const lasto_cluster& cl, cud
 {
     // the FP64 smoother (plain preconditioner, stationary cycles) reads a stored inverse diagonal
     const bool fp64 = h->cfg.precision == LASTO_PREC_FP64 || h->cfg.cycle != LASTO_CYCLE_PCG;
-    for (int l = 0; l < P.L; l++) {
-        const double* src[3];
-        int stride;
-        if (l == 0) {
-            src[0] = cl.x;
-            src[1] = cl.y;
-            src[2] = cl.z;
-            stride = 1;
-        } else {
-            for (int d = 0; d < 3; d++) src[d] = P.lv[l - 1].ax[d].c;
-            stride = 2;
-        }
-        TRY(launch_level_tables(P.lv[l], nullptr, src, stride, s));
-        if (fp64 && l < P.L - 1) TRY(launch_inv_diag(P.lv[l], s));
+    const double* const src[3] = {cl.x, cl.y, cl.z};
+    TRY(launch_hierarchy_tables(P.lv, P.L, src, s));
+    const int dl = fp64 ? direct_level<double>(P) : direct_level<float>(P);
+    if (dl < 0) {
+        TRY(launch_coarse_eig(P.lv[P.L - 1], P.eig, s));
+    } else if (fp64) {
+        TRY(launch_direct_eig<double>(P.lv[dl], P.dir64, s));
+    } else {
+        TRY(launch_direct_eig<float>(P.lv[dl], P.dir32, s));
     }
-    TRY(launch_coarse_eig(P.lv[P.L - 1], P.eig, s));
+    for (int l = 0; fp64 && l < (dl < 0 ? P.L - 1 : dl); l++) TRY(launch_inv_diag(P.lv[l], s));
     return LASTO_OK;
 }
 
@@ -748,7 +806,10 @@ int tune_plans(lasto_poisson* h, const lasto_cluster* cls, int nc, cudaStream_t 
     for (int c = 0; c < nc; c++) {
         ClusterPlan& P = h->plans[c];
         int last = P.L - 2;
-        if (f32) {
+        const int dl = f32 ? direct_level<float>(P) : direct_level<double>(P);
+        if (dl > 0) {
+            last = dl - 1;
+        } else if (f32) {
             const int bl = bottom_level(P);
             if (bl > 0) last = bl - 1;
         }
@@ -782,6 +843,10 @@ int enqueue_start(lasto_poisson* h, ClusterPlan& P, cudaGraphConditionalHandle c
     TRY(launch_bnorm(V, F.u, F.b, P.red(FIN_BNORM), s));
     const double tol = h->cfg.rel_tol;
     const bool dc = is_defect_correction(h);
+    // the exactly solved level's solution has zero faces (the guess uses the array before this)
+    if (!dc)
+        if (const int dl = direct_level<double>(P); dl > 0)
+            TRY(cudaMemsetAsync(P.lv[dl].u, 0, sizeof(double) * P.lv[dl].N(), s));
     TRY(launch_ctl_init(P.ctl, tol, (cyc == LASTO_CYCLE_PCG && !dc) ? 0.5 * tol : tol, h->cfg.max_cycles, s));
     if (cyc == LASTO_CYCLE_FV) {
         int st = enqueue_cycle<double>(h, P, 0, F.u, F.b, F.r, true, false, s);
@@ -926,7 +991,15 @@ int count_kernels(cudaGraph_t g)
 // Clusters of a defect-correction batch whose hierarchies have the same shape and storage run
 // their iterations in lockstep: each kernel is launched once for the whole group.
 constexpr size_t LOCKSTEP_MAX = BAT_MAX;   // members per lockstep group
-static_assert(sizeof(BatPack<BatLevel>) < 32000 && sizeof(BatPack<BatVec>) < 32000, "kernel parameter size");
+static_assert(sizeof(BatPack<BatLevel>) < 32000 && sizeof(BatPack<BatVec>) < 32000 && sizeof(BatPack<BatDirect>) < 32000,
+              "kernel parameter size");
+
+// the level that the FP32 cycle hands to the exact solve or to the one-block kernel
+int coarse_start(const ClusterPlan& P)
+{
+    const int dl = direct_level<float>(P);
+    return dl > 0 ? dl : bottom_level(P);
+}
 
 std::vector<std::vector<int>> lockstep_groups(const lasto_poisson* h, int nc)
 {
@@ -935,7 +1008,7 @@ std::vector<std::vector<int>> lockstep_groups(const lasto_poisson* h, int nc)
     std::map<std::array<int, 4>, std::vector<int>> by;
     for (int c = 0; c < nc; c++) {
         const ClusterPlan& P = h->plans[c];
-        if (P.L < 2 || bottom_level(P) < 1) continue;   // the group's coarsest levels run in one block
+        if (P.L < 2 || coarse_start(P) < 1) continue;   // the group's coarse levels run in their own launches
         by[{P.lv[0].n[0], P.lv[0].n[1], P.lv[0].n[2], P.lv[0].split32 ? 1 : 0}].push_back(c);
     }
     for (auto& kv : by)
@@ -951,8 +1024,10 @@ std::vector<std::vector<int>> lockstep_groups(const lasto_poisson* h, int nc)
 struct BatLayout {
     std::vector<BatPack<BatLevel>> lev;
     BatPack<BatVec> vec;
+    BatPack<BatDirect> dir;
     size_t bot = 0, ctls = 0;
     int bl = 0;
+    bool direct = false;   // level bl: solved exactly, or the one-block kernel's first
 };
 
 BottomArgs<float> bottom_args(const lasto_poisson* h, const ClusterPlan& P, int l, bool sym)
@@ -987,7 +1062,9 @@ int upload_bat_args(lasto_poisson* h, const std::vector<std::vector<int>>& group
         const int nm = (int)g.size();
         BatLayout& L = lay[gi];
         if (nm > BAT_MAX) return fail(h, LASTO_ERR_INVALID_ARG, "lockstep group too large");
-        L.bl = bottom_level(h->plans[g[0]]);
+        L.bl = coarse_start(h->plans[g[0]]);
+        L.direct = direct_level<float>(h->plans[g[0]]) > 0;
+        std::memset(&L.dir, 0, sizeof(L.dir));
         L.lev.assign(L.bl, BatPack<BatLevel>());
         std::memset(L.lev.data(), 0, sizeof(BatPack<BatLevel>) * L.lev.size());
         for (int l = 0; l < L.bl; l++) {
@@ -1009,8 +1086,13 @@ int upload_bat_args(lasto_poisson* h, const std::vector<std::vector<int>>& group
         for (int q = 0; q < nm; q++) {
             const ClusterPlan& P = h->plans[g[q]];
             const LevelStore& F = P.lv[0];
-            bb[q].a = bottom_args(h, P, L.bl, true);
-            bb[q].ctl = P.ctl;
+            if (L.direct) {
+                L.dir.m[q].a = direct_args<float>(P, L.bl);
+                L.dir.m[q].ctl = P.ctl;
+            } else {
+                bb[q].a = bottom_args(h, P, L.bl, true);
+                bb[q].ctl = P.ctl;
+            }
             BatVec& a = L.vec.m[q];
             a.V32 = F.view32();
             a.V64 = F.view64();
@@ -1065,8 +1147,11 @@ int enqueue_cycle_bat(lasto_poisson* h, const std::vector<int>& g, const BatLayo
         // after nu1 >= 1 sweeps that end on the black half sweep the black residuals are zero
         TRY(launch_resid_restrict_bat(V, VC, lev(l), nm, nu1 > 0, s));
     }
-    TRY(launch_bottom_bat(bottom_args(h, P, L.bl, true), reinterpret_cast<const BatBottom*>(h->bat_args + L.bot), nm,
-                          s));
+    if (L.direct)
+        TRY(launch_direct_bat(P.lv[L.bl].n, L.dir, nm, s));
+    else
+        TRY(launch_bottom_bat(bottom_args(h, P, L.bl, true), reinterpret_cast<const BatBottom*>(h->bat_args + L.bot), nm,
+                              s));
     for (int l = L.bl - 1; l >= 0; l--) {
         const LevelT<float> V = P.lv[l].view32(), VC = P.lv[l + 1].view32();
         const int nu2 = nu_of(l, h->cfg.nu2), nt = nt_of(l);
@@ -1737,8 +1822,8 @@ struct OpLevel {
             p += axis_pool_doubles(n[d]);
         }
         S.inv_diag = inv ? p : nullptr;
-        const double* src[3] = {x, y, z};
-        launch_level_tables(S, nullptr, src, 1, s);
+        const double* const src[3] = {x, y, z};
+        launch_hierarchy_tables(&S, 1, src, s);
         if (inv) launch_inv_diag(S, s);
     }
     bool ok() const { return mem.p != nullptr; }

@@ -1272,6 +1272,7 @@ void init_device_constants()
     cudaFuncSetAttribute(k_deposit64, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     cudaFuncSetAttribute(k_deposit_df, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     init_mg_attributes();
+    init_direct_attributes();
     init_slab_attributes();
     init_wave_attributes();
     std::lock_guard<std::mutex> lock(g_constants_mutex);

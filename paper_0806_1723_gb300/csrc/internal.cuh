@@ -217,6 +217,24 @@ struct CoarseEig {
     int ok[3];
 };
 
+// Exact solve of a coarse level (direct.cu): transposed forward [i][p] and backward [p][i] matrices,
+// padded with zeros, and eigenvalues per axis, interior nodes n - 2 <= DIRECT_MAX.
+constexpr int DIRECT_MAX = 95;
+constexpr int DIRECT_MAX64 = 47;     // FP64 (its products are bound by the FP64 pipe)
+constexpr int DIRECT_PAD = 96, DIRECT_PAD64 = 64;   // largest padded sizes
+template <typename T>
+struct DirectMats {
+    T *Ft[3], *Bt[3], *lam[3];
+};
+template <typename T>
+struct DirectArgs {
+    const T* b;   // right-hand side (natural storage, faces included)
+    T* u;         // solution: the interior is written
+    T* w;         // scratch, interior nodes
+    DirectMats<T> M;
+    int n[3];
+};
+
 int num_levels(const int n[3], int* coarse_n = nullptr);
 size_t axis_pool_doubles(int n);     // doubles needed by one AxisStore of n nodes
 void carve_axis(AxisStore* a, int n, double* pool);
@@ -225,10 +243,16 @@ void carve_axis(AxisStore* a, int n, double* pool);
 // mesh.cu
 cudaError_t launch_mesh_axis(int n, double c, double L, double h_min, double h_max, double p_max, double* x,
                              double* info, cudaStream_t s);
-cudaError_t launch_level_tables(const LevelStore& fine, const LevelStore* coarse, const double* src_coords[3],
-                                int src_stride, cudaStream_t s);
 cudaError_t launch_inv_diag(const LevelStore& L, cudaStream_t s);
+cudaError_t launch_hierarchy_tables(const LevelStore* lv, int L, const double* const src[3], cudaStream_t s);
 cudaError_t launch_coarse_eig(const LevelStore& L, CoarseEig* eig, cudaStream_t s);
+
+// direct.cu
+template <typename T>
+cudaError_t launch_direct_eig(const LevelStore& L, const DirectMats<T>& out, cudaStream_t s);
+template <typename T>
+cudaError_t launch_direct(const DirectArgs<T>& a, cudaStream_t s);
+void init_direct_attributes();   // shared-memory opt-in; call outside capture
 
 // mg.cu
 // nt: threads per block of the flat kernels (32 .. 512), 0 for one warp (colour-split storage)
@@ -451,6 +475,10 @@ struct BatVec {              // one member's finest-level vectors, partials and 
     Ctl* ctl;
     int* status;             // the member's solve status (bounded waits of the staged kernels)
 };
+struct BatDirect {           // one member's exactly solved level
+    DirectArgs<float> a;
+    const Ctl* ctl;
+};
 struct BatBottom {           // one member's one-block bottom levels
     BottomArgs<float> a;
     const Ctl* ctl;
@@ -472,6 +500,7 @@ cudaError_t launch_resid_restrict_bat(const LevelT<float>& F0, const LevelT<floa
                                       int nm, bool red_only, cudaStream_t s);
 cudaError_t launch_prolong_add_bat(const LevelT<float>& F0, const LevelT<float>& C0, const BatPack<BatLevel>& m,
                                    int nm, cudaStream_t s);
+cudaError_t launch_direct_bat(const int n[3], const BatPack<BatDirect>& m, int nm, cudaStream_t s);   // direct.cu
 cudaError_t launch_bottom_bat(const BottomArgs<float>& a0, const BatBottom* m, int nm, cudaStream_t s);
 // finest-level steps; `op` the reduction's scalar step (FinOp)
 cudaError_t launch_zero_bat(const BatPack<BatVec>& m, int nm, size_t n, int which, int mode, cudaStream_t s);

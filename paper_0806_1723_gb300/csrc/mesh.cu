@@ -148,19 +148,20 @@ cudaError_t launch_mesh_axis(int n, double c, double L, double h_min, double h_m
 }
 
 // ---------------------------------------------------------------- level tables
+// Levels first .. first + gridDim.z - 1 of a hierarchy in one launch: level l holds every 2^l-th
+// node of the finest axis.
 struct TabArgs {
-    AxisStore ax[3];
+    AxisStore ax[MAX_LEVELS][3];
     const double* src[3];
-    int stride;
 };
 
-__global__ void k_level_tables(TabArgs a)
+__global__ void k_level_tables(const __grid_constant__ TabArgs a)
 {
     const int d = blockIdx.y;
-    const AxisStore& A = a.ax[d];
+    const AxisStore& A = a.ax[blockIdx.z][d];
     const int n = A.n;
     const double* src = a.src[d];
-    const int st = a.stride;
+    const int st = 1 << blockIdx.z;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         auto C = [&](int t) { return src[(size_t)st * t]; };
         const double ci = C(i);
@@ -212,17 +213,15 @@ __global__ void k_level_tables(TabArgs a)
     }
 }
 
-cudaError_t launch_level_tables(const LevelStore& lv, const LevelStore* /*coarse*/, const double* src_coords[3],
-                                int src_stride, cudaStream_t s)
+cudaError_t launch_hierarchy_tables(const LevelStore* lv, int L, const double* const src[3], cudaStream_t s)
 {
     TabArgs a;
     for (int d = 0; d < 3; d++) {
-        a.ax[d] = lv.ax[d];
-        a.src[d] = src_coords[d];
+        a.src[d] = src[d];
+        for (int l = 0; l < L; l++) a.ax[l][d] = lv[l].ax[d];
     }
-    a.stride = src_stride;
-    const int nmax = std::max(lv.n[0], std::max(lv.n[1], lv.n[2]));
-    k_level_tables<<<dim3((nmax + 127) / 128, 3), 128, 0, s>>>(a);
+    const int nmax = std::max(lv[0].n[0], std::max(lv[0].n[1], lv[0].n[2]));
+    k_level_tables<<<dim3((nmax + 127) / 128, 3, L), 128, 0, s>>>(a);
     return cudaGetLastError();
 }
 
