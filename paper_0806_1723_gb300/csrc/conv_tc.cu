@@ -1,9 +1,11 @@
 // 3x3x3 convolution of the learned-guess network on the fifth-generation tensor cores
 // (tcgen05): an implicit GEMM, M = 128 nodes per CTA, N = cout, K = 27 taps x cin, issued as
 // K = 16 steps (one tap, 16 input channels) of tcgen05.mma kind::f16 (BF16 x BF16 -> FP32)
-// with the accumulator in tensor memory.
+// with the accumulator in tensor memory.  Two forms: over the grids as one padded sequence
+// (k_conv_seq, nearly all calls), and with gathered rows (k_conv_tc: tap groups split over CTAs,
+// and rows too long for the first).
 //
-// A (128 x 16 per step) is gathered by the CTA's 128 threads, one node row each (the
+// In the second, A (128 x 16 per step) is gathered by the CTA's 128 threads, one node row each (the
 // neighbour's 16 channels, zero outside the grid), into shared memory in the no-swizzle
 // K-major core-matrix layout: 8 rows x 16 bytes per core matrix, the two K halves 128 bytes
 // apart (leading byte offset), consecutive 8-row groups 256 bytes apart (stride byte
@@ -16,6 +18,8 @@
 // bias, ReLU and the output conversions.  Every mbarrier wait is bounded: on a timeout the
 // kernel records an error, stops issuing, frees its tensor memory and returns.
 #include <cuda_bf16.h>
+
+#include <algorithm>
 
 #include "internal.cuh"
 
@@ -235,6 +239,231 @@ __global__ void __launch_bounds__(TC_M) k_conv_tc(Grid g, int cin, const bf16* _
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(NCOL) : "memory");
 }
 
+// ---------------------------------------------------------------- grids as one padded sequence
+// The nodes of all grids in one sequence of positions with a zero column after every row, a zero
+// row after every plane and a zero plane after every grid: position ((b (D+1) + z)(H+1) + y)(W+1) +
+// x.  Every neighbour of a node is then at a constant distance (a pad where the grid ends), so a
+// tap's operand for 128 consecutive positions is the staged sequence read from another start: 16
+// bytes (8 channels) per position, 8 positions to a core matrix, whatever the shift.  A tile reads
+// its input from L2 once per z neighbour instead of once per tap.
+struct Seq {
+    int W, H, D;
+    int pitch, plane;       // W + 1, (W + 1)(H + 1)
+    int total;              // positions
+    DivMagic dp, dh, dd;    // division by W + 1, H + 1, D + 1
+};
+
+inline bool make_seq(const Grid& g, Seq* q)
+{
+    const size_t total = (size_t)g.nb * (g.D + 1) * (g.H + 1) * (g.W + 1);
+    if (total >= (size_t(1) << 30)) return false;
+    q->W = g.W;
+    q->H = g.H;
+    q->D = g.D;
+    q->pitch = g.W + 1;
+    q->plane = (g.W + 1) * (g.H + 1);
+    q->total = (int)total;
+    q->dp = div_magic((unsigned)g.W + 1);
+    q->dh = div_magic((unsigned)g.H + 1);
+    q->dd = div_magic((unsigned)g.D + 1);
+    return true;
+}
+
+// node at position p, or -1 (a pad, or outside the sequence)
+__device__ __forceinline__ int seq_node(const Seq& q, int p)
+{
+    if ((unsigned)p >= (unsigned)q.total) return -1;
+    const int q1 = (int)div_by((unsigned)p, q.dp), x = p - q1 * q.pitch;
+    const int q2 = (int)div_by((unsigned)q1, q.dh), y = q1 - q2 * (q.H + 1);
+    const int b = (int)div_by((unsigned)q2, q.dd), z = q2 - b * (q.D + 1);
+    return x == q.W || y == q.H || z == q.D ? -1 : ((b * q.D + z) * q.H + y) * q.W + x;
+}
+
+// shared-memory matrix descriptor without swizzle, byte offsets lbo and sbo
+__device__ __forceinline__ uint64_t make_desc_any(uint32_t saddr, uint32_t lbo, uint32_t sbo)
+{
+    return (uint64_t)((saddr & 0x3FFFF) >> 4) | (uint64_t)(lbo >> 4) << 16 | (uint64_t)(sbo >> 4) << 32 | (uint64_t)1 << 46;
+}
+
+// Issued by a whole warp in uniform control flow, one elected lane executing: 21 cycles per MMA at
+// M = 64, N = 16 and 36 at M = 128, against 44 and more from a branch on the thread's index, where
+// every descriptor has to be moved to the uniform registers.
+__device__ __forceinline__ void mma_f16(uint32_t tmem, uint64_t ad, uint64_t bd, uint32_t idesc, int accumulate)
+{
+    asm volatile(
+        "{\n.reg .pred p, q;\nelect.sync _|q, 0xffffffff;\nsetp.ne.b32 p, %4, 0;\n"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
+        "l"(ad), "l"(bd), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
+__device__ __forceinline__ void mma_commit(uint32_t mbar)
+{
+    asm volatile(
+        "{\n.reg .pred q;\nelect.sync _|q, 0xffffffff;\n"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(mbar)
+        : "memory");
+}
+
+__device__ __forceinline__ void copy16(uint32_t dst, const void* src, bool in)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(in ? 16u : 0u) : "memory");
+}
+
+// y = act(conv(x, w) + bias) for 256 positions per CTA: two M = 128 accumulators.  The channels go
+// through shared memory 16 at a time (two buffers where there are more): the three z neighbours'
+// segments of 256 + 2 (W + 2) positions and the 27 taps' weight tiles; then 2 x 27 MMAs, K = 16,
+// issued by a ninth warp while the other eight load.  Bound: 3 TB/s of 32-byte pieces from L2, the
+// weights a third to a half of them (a sixth of the time is MMAs; more warps, one buffer and more
+// CTAs per SM, or an x neighbour triple per MMA change nothing).  8 grids of 33^3, against the kernel
+// above, which gathers every tap's neighbour rows from L2 (745 MB at 48 channels), a K step per
+// barrier: 48 -> 16 channels 204 -> 53 us, 16 -> 48 87 -> 33 us, 64 -> 64 336 -> 108 us.
+constexpr int SQ_NT = 256, SQ_M = 256;
+__host__ __device__ constexpr int sq_seg(int W) { return SQ_M + 2 * (W + 2); }
+inline size_t sq_smem(int W, int cin, int cout)
+{
+    return (cin > 16 ? 2 : 1) * ((size_t)6 * sq_seg(W) * 16 + (size_t)27 * 32 * cout);
+}
+
+template <int COUT>
+__global__ void __launch_bounds__(SQ_NT + 32) k_conv_seq(Seq q, int cin, int cout, const bf16* __restrict__ x, const uint4* __restrict__ wpk,
+                                                    const float* __restrict__ bias, int relu, float* __restrict__ y32,
+                                                    int ldy32, int off32, bf16* __restrict__ y16, int ldy16, int off16,
+                                                    int* __restrict__ err)
+{
+    constexpr int NCOL = 2 * COUT <= 32 ? 32 : 2 * COUT <= 64 ? 64 : 2 * COUT <= 128 ? 128 : 256;
+    extern __shared__ __align__(1024) unsigned char sq_raw[];
+    __shared__ __align__(8) unsigned long long mbar[2];
+    __shared__ uint32_t tmem_slot;
+    const int tid = threadIdx.x, warp = tid >> 5;
+    bool bad = false;   // a wait ran out
+    const int seg = sq_seg(q.W), p0 = blockIdx.x * SQ_M, cpt = cin / 16;
+    const int n0 = blockIdx.y * COUT;   // the CTA's output channels n0 .. n0 + COUT - 1
+    const uint32_t a_bytes = 6 * seg * 16, buf_bytes = a_bytes + 27 * 32 * COUT, base = smem_u32(sq_raw);
+    if (tid == 0) {
+        for (int s = 0; s < 2; s++)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&mbar[s])) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(&tmem_slot)),
+                     "r"(NCOL)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    const uint32_t tmem = tmem_slot;
+    const uint32_t idesc = make_idesc(COUT);
+
+    // channels 16 c .. 16 c + 15 into buffer c & 1 (after the MMAs that last read it): a lane pair
+    // per position, 32 contiguous bytes
+    auto load = [&](int c) {
+        if (c >= 2 && !mbar_wait(smem_u32(&mbar[c % 2]), (uint32_t)((c / 2 - 1) & 1))) bad = true;
+        const uint32_t buf = base + (c % 2) * buf_bytes;
+        const int h = tid & 1;
+        for (int t = tid >> 1; t < 3 * seg; t += SQ_NT / 2) {
+            const int dz = t >= 2 * seg ? 2 : t >= seg ? 1 : 0;
+            const int nd = seq_node(q, p0 + (dz - 1) * q.plane - (q.pitch + 1) + t - dz * seg);
+            copy16(buf + (h * 3 * seg + t) * 16, x + (size_t)(nd < 0 ? 0 : nd) * cin + c * 16 + h * 8, nd >= 0);
+        }
+        for (int t = tid; t < 27 * 2 * COUT; t += SQ_NT) {
+            const int tap = t / (2 * COUT), r = t - tap * 2 * COUT;
+            copy16(buf + a_bytes + t * 16, wpk + (size_t)(tap * cpt + c) * 2 * cout + 2 * n0 + r, true);
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+    if (tid < SQ_NT) load(0);
+    for (int c = 0; c < cpt; c++) {
+        asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");   // visible to the tensor core
+        bad = __syncthreads_or(bad);
+        if (bad) break;
+        if (__shfl_sync(0xffffffffu, warp, 0) == SQ_NT / 32) {
+            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+            const uint32_t buf = base + (c % 2) * buf_bytes;
+            const uint64_t a0 = make_desc_any(buf, 3 * seg * 16, 128);
+            const uint64_t b0 = make_desc(buf + a_bytes);
+#pragma unroll
+            for (int dz = 0; dz < 3; dz++) {
+#pragma unroll
+                for (int t = 0; t < 9; t++) {
+                    // (positions from -(pitch + 1) on; addresses in units of 16 bytes)
+                    const uint64_t ad = a0 + (uint32_t)(dz * seg + (t / 3) * q.pitch + t % 3);
+                    const uint64_t bd = b0 + (dz * 9 + t) * 2 * COUT;
+#pragma unroll
+                    for (int m = 0; m < 2; m++) mma_f16(tmem + m * COUT, ad + m * 128, bd, idesc, c > 0 || dz > 0 || t > 0);
+                }
+            }
+            mma_commit(smem_u32(&mbar[c % 2]));
+        }
+        if (tid < SQ_NT && c + 1 < cpt) load(c + 1);   // while these are issued
+    }
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    if (!bad) {   // the last commit (they complete in issue order)
+        const int c = cpt - 1;
+        if (!mbar_wait(smem_u32(&mbar[c % 2]), (uint32_t)((c / 2) & 1))) bad = true;
+    }
+    bad = __syncthreads_or(bad);
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    if (!bad) {
+        // warp w: accumulator w / 4, tensor-memory lanes 32 (w % 4) ..; the rows leave through shared
+        // memory (idle now), so that a warp stores consecutive channels of consecutive nodes
+        if (tid < SQ_NT) {
+            constexpr int LD = COUT + 4, Q = COUT / 4;
+            const int nd = seq_node(q, p0 + tid), lane = tid & 31;
+            const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * COUT);
+            float* stage = reinterpret_cast<float*>(sq_raw) + warp * 32 * LD;
+#pragma unroll
+            for (int c0 = 0; c0 < COUT; c0 += 16) {
+                float v[16];
+                tmem_ld16(lane_base + (uint32_t)c0, v);
+                asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+#pragma unroll
+                for (int j = 0; j < 16; j++) {
+                    v[j] += bias ? bias[n0 + c0 + j] : 0.0f;
+                    if (relu) v[j] = fmaxf(v[j], 0.0f);
+                }
+#pragma unroll
+                for (int j = 0; j < 16; j += 4)
+                    *reinterpret_cast<float4*>(stage + lane * LD + c0 + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+            }
+            __syncwarp();
+            const bool v32 = ((ldy32 | off32) & 3) == 0 && ((uintptr_t)y32 & 15) == 0;
+            const bool v16 = ((ldy16 | off16) & 3) == 0 && ((uintptr_t)y16 & 7) == 0;
+            for (int e = lane; e < 32 * Q; e += 32) {
+                const int r = e / Q, c = (e - r * Q) * 4, node = __shfl_sync(0xffffffffu, nd, r);
+                const float4 v = *reinterpret_cast<const float4*>(stage + r * LD + c);
+                if (node < 0) continue;
+                if (y32) {
+                    float* o = y32 + (size_t)node * ldy32 + off32 + n0 + c;
+                    if (v32) {
+                        *reinterpret_cast<float4*>(o) = v;
+                    } else {
+                        o[0] = v.x, o[1] = v.y, o[2] = v.z, o[3] = v.w;
+                    }
+                }
+                if (y16) {
+                    bf16* o = y16 + (size_t)node * ldy16 + off16 + n0 + c;
+                    const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+                    if (v16) {
+                        *reinterpret_cast<uint2*>(o) =
+                            make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+                    } else {
+                        o[0] = lo.x, o[1] = lo.y, o[2] = hi.x, o[3] = hi.y;
+                    }
+                }
+            }
+        }
+    } else if (tid == 0 && err) {
+        atomicExch(err, 1);
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(NCOL) : "memory");
+}
+
 // Pack w [27][cin][cout] into the per-step B tiles: step k = tap * (cin/16) + c0/16 holds
 // element (n = output channel, kk = input channel c0 + kk) at byte
 // ((n/8)*2 + kk/8)*128 + (n%8)*16 + (kk%8)*2 of its cout*32-byte tile.
@@ -441,6 +670,149 @@ __global__ void __launch_bounds__(TC_M) k_conv_wgrad_tc(Grid g, GridDiv gd, int 
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(NCOL) : "memory");
 }
 
+// The same GEMM over the padded sequence: per stage 128 positions of dy and the three z neighbours'
+// segments of x (CG channels), both channel group by channel group, 16 bytes per position, which is
+// the MN-major operand layout (8 positions x 8 channels to a core matrix) for every shift.  One
+// M = 64 MMA (64 channel rows, those beyond CG unused) per tap and 16 positions.  Up to 16 output
+// channels the three x neighbours share one: dw[dz, dy, dx] = sum_p x[p + dz, dy] dy[p - dx], with dy
+// staged at the three shifts (an MMA costs 21 cycles at 16 columns, 26 at 48, 43 at 96: at 16
+// channels 62 against 79 us, at 48 140 against 131).  Every tap has its own columns of tensor memory,
+// so the input is staged once for all taps of the CTA.  Stages alternate between two buffers, filled
+// by eight warps while a ninth issues; a CTA takes every gridDim.x-th one, and adds its sums to dw
+// with vector reductions at the end.  Bound: 32-byte pieces from L2 (3 to 4 TB/s; three or four
+// buffers, or 16 loading warps, change nothing).  8 grids of 33^3, against the kernel above (27
+// gathered rows per node): 48 x 16 channels 330 -> 57 us.
+constexpr int WS_K = 128, WS_NT = 256;
+__host__ __device__ constexpr int ws_dx(int cout) { return cout <= 16 ? 3 : 1; }
+__host__ __device__ constexpr int ws_seg(int W) { return WS_K + 2 * (W + 2); }
+// groups of ws_dx taps whose columns fit in tensor memory
+__host__ __device__ constexpr int ws_groups(int cout) { return cout <= 16 ? 9 : cout <= 32 ? 14 : cout <= 48 ? 9 : cout <= 64 ? 7 : cout <= 96 ? 5 : 4; }
+inline size_t ws_smem(int W, int cg, int cout)
+{
+    // two buffers, and what the unused rows of the second one's operand read beyond it
+    return 2 * ((size_t)cg / 8 * 3 * ws_seg(W) * 16 + (size_t)ws_dx(cout) * cout / 8 * WS_K * 16) + (size_t)(64 - cg) / 8 * 3 * ws_seg(W) * 16;
+}
+
+template <int COUT>
+__global__ void __launch_bounds__(WS_NT + 32) k_conv_wgrad_seq(Seq q, int cin, int cg, const bf16* __restrict__ x,
+                                                          const bf16* __restrict__ dy, float* __restrict__ dw,
+                                                          int* __restrict__ err)
+{
+    constexpr int DX = ws_dx(COUT), N = DX * COUT, TAPS = ws_groups(COUT), USED = TAPS * N;   // a group: DX taps
+    constexpr int NCOL = USED <= 128 ? 128 : USED <= 256 ? 256 : 512;
+    extern __shared__ __align__(1024) unsigned char ws_raw[];
+    __shared__ __align__(8) unsigned long long mbar[2];
+    __shared__ uint32_t tmem_slot;
+    bool bad = false;   // a wait ran out
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int seg = ws_seg(q.W), groups = cin / cg;
+    const int tap0 = (int)blockIdx.y / groups * TAPS, c0 = (int)blockIdx.y % groups * cg, ntap = min(TAPS, 27 / DX - tap0);
+    const int nchunk = (q.total + WS_K - 1) / WS_K;
+    const int nk = ((int)blockIdx.x < nchunk) ? (nchunk - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
+    const uint32_t a_bytes = (uint32_t)cg / 8 * 3 * seg * 16, b_bytes = N / 8 * WS_K * 16;
+    // both B buffers, then both A buffers
+    const uint32_t baseA = smem_u32(ws_raw) + 2 * b_bytes, baseB = smem_u32(ws_raw);
+    if (tid == 0) {
+        for (int s = 0; s < 2; s++)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&mbar[s])) : "memory");
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(&tmem_slot)),
+                     "r"(NCOL)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    const uint32_t tmem = tmem_slot;
+    // M = 64, A and B MN-major
+    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((uint32_t)(N >> 3) << 17) | (4u << 24);
+
+    auto load = [&](int k) {
+        const int s = k & 1, p0 = ((int)blockIdx.x + k * (int)gridDim.x) * WS_K;
+        if (k >= 2 && !mbar_wait(smem_u32(&mbar[s]), (uint32_t)((k / 2 - 1) & 1))) bad = true;
+        const int h = tid & 1;
+        for (int t = tid >> 1; t < 3 * seg; t += WS_NT / 2) {
+            const int dz = t >= 2 * seg ? 2 : t >= seg ? 1 : 0;
+            const int nd = seq_node(q, p0 + (dz - 1) * q.plane - (q.pitch + 1) + t - dz * seg);
+            const bf16* src = x + (size_t)(nd < 0 ? 0 : nd) * cin + c0;
+            for (int c = h; c < cg / 8; c += 2) copy16(baseA + s * a_bytes + (c * 3 * seg + t) * 16, src + c * 8, nd >= 0);
+        }
+        for (int t = tid >> 1; t < DX * WS_K; t += WS_NT / 2) {
+            const int dx = t / WS_K, i = t - dx * WS_K;   // dy at p0 + i - (dx - 1)
+            const int nd = seq_node(q, p0 + i - (DX == 3 ? dx - 1 : 0));
+            const bf16* src = dy + (size_t)(nd < 0 ? 0 : nd) * COUT;
+#pragma unroll
+            for (int c = 0; c < COUT / 16; c++)
+                copy16(baseB + s * b_bytes + ((dx * (COUT / 8) + 2 * c + h) * WS_K + i) * 16, src + (2 * c + h) * 8, nd >= 0);
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+    if (nk > 0 && tid < WS_NT) load(0);
+    for (int k = 0; k < nk; k++) {
+        asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+        bad = __syncthreads_or(bad);
+        if (bad) break;
+        if (__shfl_sync(0xffffffffu, warp, 0) == WS_NT / 32) {
+            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+            const uint64_t a0 = make_desc_any(baseA + (k & 1) * a_bytes, 128, 3 * seg * 16);
+            const uint64_t b0 = make_desc_any(baseB + (k & 1) * b_bytes, 128, WS_K * 16);
+#pragma unroll
+            for (int t = 0; t < TAPS; t++) {
+                const int tap = (tap0 + t) * DX;   // its start in a segment set, in positions
+                const uint64_t ad = a0 + (uint32_t)(tap / 9 * seg + (tap / 3) % 3 * q.pitch + (DX == 3 ? 1 : tap % 3));
+                if (t < ntap) {
+#pragma unroll
+                    for (int j = 0; j < WS_K / 16; j++) mma_f16(tmem + t * N, ad + j * 16, b0 + j * 16, idesc, k > 0 || j > 0);
+                }
+            }
+            mma_commit(smem_u32(&mbar[k & 1]));
+        }
+        if (tid < WS_NT && k + 1 < nk) load(k + 1);   // while these are issued
+    }
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    if (!bad && nk > 0) {
+        const int k = nk - 1;
+        if (!mbar_wait(smem_u32(&mbar[k & 1]), (uint32_t)((k / 2) & 1))) bad = true;
+    }
+    bad = __syncthreads_or(bad);
+    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+    if (!bad && nk > 0) {
+        // an M = 64 accumulator: row r in tensor-memory lane 32 (r / 16) + r % 16
+        const int row = (warp & 3) * 16 + (lane & 15);
+        const bool live = lane < 16 && row < cg, vec = ((uintptr_t)dw & 15) == 0;
+        const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+        for (int t = tid < WS_NT ? warp >> 2 : ntap * DX; t < ntap * DX; t += WS_NT / 128) {
+            float* dst = dw + ((size_t)(tap0 * DX + t) * cin + c0 + row) * COUT;
+#pragma unroll
+            for (int c = 0; c < COUT; c += 16) {
+                float v[16];
+                __syncwarp();
+                tmem_ld16(lane_base + (uint32_t)(t * COUT + c), v);
+                asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+                if (!live) continue;
+                if (vec) {
+#pragma unroll
+                    for (int j = 0; j < 16; j += 4)
+                        asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};\n" ::"l"(dst + c + j), "f"(v[j]),
+                                     "f"(v[j + 1]), "f"(v[j + 2]), "f"(v[j + 3])
+                                     : "memory");
+                } else {
+                    for (int j = 0; j < 16; j++) atomicAdd(dst + c + j, v[j]);
+                }
+            }
+        }
+    } else if (bad && tid == 0 && err) {
+        atomicExch(err, 1);
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    __syncthreads();
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(NCOL) : "memory");
+}
+
 }  // namespace tc
 
 cudaError_t launch_pack_weights(int cin, int cout, const void* w, void* wpk, cudaStream_t s)
@@ -470,6 +842,32 @@ int conv_fwd_tc(int nb, const int dims[3], int cin, int cout, const void* x, con
     const bf16* X = (const bf16*)x;
     const uint4* W = (const uint4*)wpk;
     bf16* Y16 = (bf16*)y16;
+    // the padded sequence where a tile's segments fit in shared memory (rows of up to about 800
+    // nodes).  Many channels on few tiles are better
+    // split over CTAs by taps (128 -> 64 channels: 6 tiles 23.3 against 18.8 us, 16 tiles 23.8
+    // against 25.4; 64 -> 64 on 3 tiles 15.1 against 14.8, 16 -> 16 7.1 against 12.6), if there is
+    // room for their sums (without: 97 us).
+    Seq q;
+    const int half = cout > 64 ? 2 : 1;   // 96 and 128 output channels as two CTAs' work
+    const size_t sm = sq_smem(g.W, cin, cout / half);
+    if (make_seq(g, &q) && (!scratch || cin <= 64 || q.total / SQ_M >= cin / 8) && sm <= 200 * 1024) {
+        const dim3 tiles((unsigned)((q.total + SQ_M - 1) / SQ_M), (unsigned)half);
+#define LASTO_SQ_CASE(C)                                                                                            \
+    case C:                                                                                                         \
+        if (cudaFuncSetAttribute(k_conv_seq<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) !=         \
+            cudaSuccess)                                                                                            \
+            return LASTO_ERR_CUDA;                                                                                  \
+        k_conv_seq<C><<<tiles, SQ_NT + 32, sm, s>>>(q, cin, cout, X, W, bias, relu, y32, ldy32, off32, Y16, ldy16, off16, err); \
+        break;
+        switch (cout / half) {
+            LASTO_SQ_CASE(16)
+            LASTO_SQ_CASE(32)
+            LASTO_SQ_CASE(48)
+            LASTO_SQ_CASE(64)
+        }
+#undef LASTO_SQ_CASE
+        return cudaGetLastError() == cudaSuccess ? LASTO_OK : LASTO_ERR_CUDA;
+    }
 #define LASTO_TC_CASE(C)                                                                                           \
     case C:                                                                                                        \
         k_conv_tc<C><<<grid, TC_M, 0, s>>>(g, cin, X, W, bias, relu, y32, ldy32, off32, Y16, ldy16, off16, part, err); \
@@ -508,6 +906,34 @@ int conv_wgrad_tc(int nb, const int dims[3], int cin, int cout, const void* x, c
     const dim3 grid((unsigned)((g.nodes() + WG_CHUNK - 1) / WG_CHUNK), (unsigned)((27 + tpt - 1) / tpt));
     const bf16* X = (const bf16*)x;
     const bf16* DY = (const bf16*)dy16;
+    // the padded sequence with the largest group of channels whose buffers fit (rows of up to about
+    // 450 nodes); one CTA per SM: its accumulators fill the tensor memory
+    Seq q;
+    int cg = 64;
+    while (cg > 16 && (cin % cg || ws_smem(g.W, cg, cout) > 220 * 1024)) cg -= 16;
+    if (make_seq(g, &q) && cin % cg == 0 && ws_smem(g.W, cg, cout) <= 220 * 1024) {
+        const size_t sm = std::max(ws_smem(g.W, cg, cout), (size_t)116 * 1024);
+        const int per = ws_groups(cout) * ws_dx(cout);
+        const int ny = (27 + per - 1) / per * (cin / cg), nchunk = (q.total + WS_K - 1) / WS_K;
+        const dim3 grid((unsigned)std::min(nchunk, std::max(1, 152 / ny)), (unsigned)ny);
+#define LASTO_WS_CASE(C)                                                                                              \
+    case C:                                                                                                           \
+        if (cudaFuncSetAttribute(k_conv_wgrad_seq<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) !=     \
+            cudaSuccess)                                                                                              \
+            return LASTO_ERR_CUDA;                                                                                    \
+        k_conv_wgrad_seq<C><<<grid, WS_NT + 32, sm, s>>>(q, cin, cg, X, DY, dw, err);                                       \
+        break;
+        switch (cout) {
+            LASTO_WS_CASE(16)
+            LASTO_WS_CASE(32)
+            LASTO_WS_CASE(48)
+            LASTO_WS_CASE(64)
+            LASTO_WS_CASE(96)
+            LASTO_WS_CASE(128)
+        }
+#undef LASTO_WS_CASE
+        return cudaGetLastError() == cudaSuccess ? LASTO_OK : LASTO_ERR_CUDA;
+    }
 #define LASTO_WG_CASE(C)                                                                                 \
     case C:                                                                                              \
         if (cudaFuncSetAttribute(k_conv_wgrad_tc<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, wg_smem(C)) != \
