@@ -557,7 +557,7 @@ int enqueue_cycle(lasto_poisson* h, ClusterPlan& P, int l, T* u, T* b, T* r, boo
     }
     if (l == P.L - 1) {
         if (l == 0) {
-            TRY(launch_residual<T>(V, u, b, r, s));
+            TRY(launch_residual<T>(V, u, b, r, false, s));
             TRY(launch_coarse_apply<T>(V, P.eig, r, u, true, s));
         } else {
             TRY(launch_coarse_apply<T>(V, P.eig, b, u, false, s));
@@ -573,9 +573,11 @@ int enqueue_cycle(lasto_poisson* h, ClusterPlan& P, int l, T* u, T* b, T* r, boo
         if (ch.nt == RBGS_STAGED) ch.nt = 0;   // natural storage: one block per row
     }
     T* cur = u;   // fused passes move the iterate between u and the partner array
-    if (zero_start && sizeof(T) == 4 && nu1 >= 1 && (ch.fused == 0 || ch.fused == 3)) {
+    if (zero_start && nu1 >= 1 && (ch.fused == 0 || ch.fused == 3)) {
         // from u = 0 (faces zero) the first red half sweep is a point update
-        if constexpr (sizeof(T) == 4) {
+        if constexpr (sizeof(T) == 8) {
+            TRY(launch_first_red64(V, u, b, s));
+        } else {
             if (V.lsh && ch.nt == RBGS_STAGED)
                 TRY(launch_split_stage_first_red(V, u, b, P.status, s));
             else
@@ -595,12 +597,12 @@ int enqueue_cycle(lasto_poisson* h, ClusterPlan& P, int l, T* u, T* b, T* r, boo
         TRY(launch_resid_restrict<T>(V, VC, cur, b, Arr<T>::b(C), Arr<T>::u(C), nu1 > 0, s, V.lsh ? r : nullptr,
                                      P.status));
     } else {
-        // FP64: each residual once (FP64 arithmetic, not bandwidth, bounds this chip)
-        TRY(launch_residual<T>(V, cur, b, r, s));
-        TRY(launch_restrict<T>(V, VC, r, Arr<T>::b(C), s));
-        if (l + 1 != dl) TRY(cudaMemsetAsync(Arr<T>::u(C), 0, sizeof(T) * C.N(), s));
+        // FP64: each residual once (FP64 arithmetic, not bandwidth, bounds this chip); the black
+        // ones are zero up to rounding after a black half sweep, and only correct the cycle
+        TRY(launch_residual<T>(V, cur, b, r, nu1 > 0, s));
+        TRY(launch_restrict<T>(V, VC, r, Arr<T>::b(C), l + 1 != dl ? Arr<T>::u(C) : nullptr, nu1 > 0, s));
     }
-    int st = enqueue_cycle<T>(h, P, l + 1, Arr<T>::u(C), Arr<T>::b(C), Arr<T>::r(C), fcycle, sym, s);
+    int st = enqueue_cycle<T>(h, P, l + 1, Arr<T>::u(C), Arr<T>::b(C), Arr<T>::r(C), fcycle, sym, s, sizeof(T) == 8);
     if (st) return st;
     if (fcycle && l + 1 != dl) {
         st = enqueue_cycle<T>(h, P, l + 1, Arr<T>::u(C), Arr<T>::b(C), Arr<T>::r(C), false, sym, s);
@@ -751,7 +753,8 @@ int enqueue_guess_in(lasto_poisson* h, ClusterPlan& P, const lasto_cluster& cl, 
     const int G[3] = {GUESS_N, GUESS_N, GUESS_N};
     for (int d = 0; d < 3; d++) TRY(launch_axis_stride(ax[d], P.gm[d], GUESS_N, P.gax[d], s));
     for (int l = 0; l < P.gl; l++)
-        TRY(launch_restrict<double>(P.lv[l].view64(), P.lv[l + 1].view64(), P.lv[l].b, P.lv[l + 1].b, s));
+        TRY(launch_restrict<double>(P.lv[l].view64(), P.lv[l + 1].view64(), P.lv[l].b, P.lv[l + 1].b,
+                                    (double*)nullptr, false, s));
     const LevelStore& S = P.lv[P.gl];
     TRY(launch_resample(S.n, S.ax[0].c, S.ax[1].c, S.ax[2].c, S.b, G, P.gax[0], P.gax[1], P.gax[2], P.bG, 0, s));
     // faces (and a zero interior) from the fine grid's first iterate: copies at shared nodes
@@ -870,7 +873,7 @@ int enqueue_iteration(lasto_poisson* h, ClusterPlan& P, cudaGraphConditionalHand
         return LASTO_OK;
     }
     TRY(cudaMemsetAsync(P.z, 0, sizeof(double) * F.N(), s));
-    int st = enqueue_cycle<double>(h, P, 0, P.z, F.r, P.q, false, true, s);
+    int st = enqueue_cycle<double>(h, P, 0, P.z, F.r, P.q, false, true, s, true);
     if (st) return st;
     TRY(launch_dot_rz(V, F.r, P.z, P.red(FIN_BETA), s));
     TRY(launch_update_p(V, P.ctl, P.z, P.p, s));
@@ -1940,7 +1943,7 @@ int lasto_op_residual(const int n[3], const double* x, const double* y, const do
     cudaStream_t s = (cudaStream_t)stream;
     OpLevel L(n, x, y, z, false, s);
     if (!L.ok()) return LASTO_ERR_NO_MEMORY;
-    return op_status(launch_residual<double>(L.S.view64(), u, b, r, s));
+    return op_status(launch_residual<double>(L.S.view64(), u, b, r, false, s));
 }
 
 int lasto_op_smooth(const int n[3], const double* x, const double* y, const double* z, double* u, const double* b,
@@ -2069,7 +2072,7 @@ int lasto_op_restrict(const int n[3], const double* x, const double* y, const do
     if (!L.ok()) return LASTO_ERR_NO_MEMORY;
     LevelT<double> C = L.S.view64();
     set_dims(C, (n[0] + 1) / 2, (n[1] + 1) / 2, (n[2] + 1) / 2);
-    return op_status(launch_restrict<double>(L.S.view64(), C, r, bc, s));
+    return op_status(launch_restrict<double>(L.S.view64(), C, r, bc, (double*)nullptr, false, s));
 }
 
 int lasto_op_prolong_add(const int n[3], const double* x, const double* y, const double* z, const double* ec,

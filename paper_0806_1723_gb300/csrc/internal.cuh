@@ -82,6 +82,31 @@ __device__ __forceinline__ float rb_point32(float acc, float dsum)
     return acc * r;
 }
 
+// A point update's right-hand side less its six neighbour terms (order x-, x+, y-, y+, z-, z+).
+// FP64 subtracts them from b one by one: six operations where the sum first takes seven, and the
+// FP64 pipe bounds every kernel that forms it.
+template <typename T>
+__device__ __forceinline__ T rhs_less_neighbours(T b, T cmx, T xm, T cpx, T xp, T cmy, T ym, T cpy, T yp, T cmz, T zm,
+                                                 T cpz, T zp)
+{
+    if constexpr (sizeof(T) == 8) {
+        T t = fma(-cmx, xm, b);
+        t = fma(-cpx, xp, t);
+        t = fma(-cmy, ym, t);
+        t = fma(-cpy, yp, t);
+        t = fma(-cmz, zm, t);
+        return fma(-cpz, zp, t);
+    } else {
+        T t = cmx * xm;
+        t = fma(cpx, xp, t);
+        t = fma(cmy, ym, t);
+        t = fma(cpy, yp, t);
+        t = fma(cmz, zm, t);
+        t = fma(cpz, zp, t);
+        return b - t;
+    }
+}
+
 // ---------------------------------------------------------------- block reductions
 template <int NT>
 __device__ __forceinline__ double block_sum(double v, double* smem)
@@ -263,6 +288,7 @@ template <typename T>
 cudaError_t launch_rbgs(const LevelT<T>& L, T* u, const T* b, int colour, cudaStream_t s, int nt = 256,
                         int* status = nullptr);
 // the first red FP32 half sweep from u = 0 (either storage order; faces of u already zero)
+cudaError_t launch_first_red64(const LevelT<double>& L, double* u, const double* b, cudaStream_t s);
 cudaError_t launch_first_red32(const LevelT<float>& L, float* u, const float* b, cudaStream_t s);
 // stage.cu
 cudaError_t launch_split_stage(const LevelT<float>& L, float* u, const float* b, int colour, int* status, cudaStream_t s);
@@ -274,11 +300,12 @@ cudaError_t launch_prolong_stage(const LevelT<float>& F, const LevelT<float>& C,
 bool split_stage_ok(int nx, int ny, int nz);
 void init_stage_attributes();
 template <typename T>
-cudaError_t launch_residual(const LevelT<T>& L, const T* u, const T* b, T* r, cudaStream_t s);
+cudaError_t launch_residual(const LevelT<T>& L, const T* u, const T* b, T* r, bool red_only, cudaStream_t s);
 template <typename T>
 cudaError_t launch_apply(const LevelT<T>& L, const T* u, T* Au, cudaStream_t s);
 template <typename T>
-cudaError_t launch_restrict(const LevelT<T>& fine, const LevelT<T>& coarse, const T* r, T* bc, cudaStream_t s);
+cudaError_t launch_restrict(const LevelT<T>& fine, const LevelT<T>& coarse, const T* r, T* bc, T* uc, bool red_only,
+                            cudaStream_t s);
 template <typename T>
 cudaError_t launch_prolong_add(const LevelT<T>& fine, const LevelT<T>& coarse, const T* ec, T* u, cudaStream_t s,
                                int* status = nullptr);

@@ -8,6 +8,7 @@
 // (per-block partials, then one block in a fixed order), so every norm and dot is
 // bitwise reproducible.
 #include <algorithm>
+#include <type_traits>
 
 #include "internal.cuh"
 #include "ctl.cuh"
@@ -69,6 +70,20 @@ __device__ __forceinline__ T offdiag(const LevelT<T>& L, const T* __restrict__ u
     }
 }
 
+// b less those terms (rhs_less_neighbours)
+template <int LS = 0, typename T>
+__device__ __forceinline__ T rhs_less_offdiag(const LevelT<T>& L, T b, const T* __restrict__ u, size_t P, int i, int j, int k)
+{
+    if constexpr (LS == 0) {
+        const int sy = L.nx, sz = L.nx * L.ny;
+        const T* __restrict__ c = u + P;
+        return rhs_less_neighbours(b, L.ax[0].cm[i], c[-1], L.ax[0].cp[i], c[1], L.ax[1].cm[j], c[-sy], L.ax[1].cp[j],
+                                   c[sy], L.ax[2].cm[k], c[-sz], L.ax[2].cp[k], c[sz]);
+    } else {
+        return b - offdiag<LS>(L, u, P, i, j, k);
+    }
+}
+
 // storage position of node P for a compile-time storage order
 template <int LS, typename T>
 __device__ __forceinline__ unsigned pos(const LevelT<T>& L, size_t P)
@@ -96,7 +111,7 @@ __device__ __forceinline__ void k_rbgs_body(LevelT<T> L, T* __restrict__ u, cons
     node_ijk(P, L, i, j, k);
     if (is_face(L, i, j, k)) return;
     const unsigned Q = pos<LS>(L, P);
-    const T acc = b[Q] - offdiag<LS>(L, u, P, i, j, k);
+    const T acc = rhs_less_offdiag<LS>(L, b[Q], u, P, i, j, k);
     if constexpr (sizeof(T) == 8) {
         u[Q] = acc * L.inv_diag[P];
     } else {
@@ -150,6 +165,25 @@ cudaError_t launch_first_red32(const LevelT<float>& L, float* u, const float* b,
     return cudaGetLastError();
 }
 
+// The same in FP64: the half sweep's update from u = 0 is b times the stored inverse diagonal, bitwise
+// (one operation per node instead of seven; 129^3: 17.7 -> 7.7 us)
+__global__ void __launch_bounds__(256) k_first_red64(LevelT<double> L, double* __restrict__ u, const double* __restrict__ b,
+                                                     unsigned nred)
+{
+    const unsigned t = blockIdx.x * 256u + threadIdx.x;
+    if (t >= nred) return;
+    int i, j, k;
+    node_ijk(2 * (size_t)t, L, i, j, k);
+    if (!is_face(L, i, j, k)) u[2 * (size_t)t] = b[2 * (size_t)t] * L.inv_diag[2 * (size_t)t];
+}
+
+cudaError_t launch_first_red64(const LevelT<double>& L, double* u, const double* b, cudaStream_t s)
+{
+    const unsigned nred = (unsigned)((L.N() + 1) / 2);
+    k_first_red64<<<(nred + 255u) / 256u, 256, 0, s>>>(L, u, b, nred);
+    return cudaGetLastError();
+}
+
 template <typename T, int LS>
 __global__ void __launch_bounds__(512) k_rbgs(LevelT<T> L, T* __restrict__ u, const T* __restrict__ b, int colour, size_t nhalf)
 {
@@ -167,7 +201,7 @@ __global__ void __launch_bounds__(512) k_rbgs_row(LevelT<T> L, T* __restrict__ u
     if (i == 0 || i >= L.nx - 1) return;
     const unsigned P = ((unsigned)k * L.ny + j) * L.nx + i;   // nodes < 2^31
     const unsigned Q = pos<LS>(L, P);
-    const T acc = b[Q] - offdiag<LS>(L, u, P, i, j, k);
+    const T acc = rhs_less_offdiag<LS>(L, b[Q], u, P, i, j, k);
     if constexpr (sizeof(T) == 8) {
         u[Q] = acc * L.inv_diag[P];
     } else {
@@ -339,20 +373,50 @@ cudaError_t launch_rbgs(const LevelT<T>& L, T* u, const T* b, int colour, cudaSt
 }
 
 // ---------------------------------------------------------------- residual / apply
-template <typename T>
+// One warp per (j, k) row, a pair of nodes (one of each colour) per lane and step.  Bound in FP64:
+// the pipe (0.6 T operations/s here), 8 per node (six neighbours, the diagonal's sum with the row's
+// y and z part, its product) where the flat form spent 10.  RED: the iterate's last half sweep was
+// black, so the black residuals are zero up to rounding and are written as zeros, half the work.
+// FP64: 129 x 97 x 113 nodes 27.4 -> 22.7 us;
+// red only at 129^3 39.6 -> 19.0 us.
+constexpr int RS_V = 2;
+
+template <typename T, int RED>
 __global__ void __launch_bounds__(NT) k_residual(LevelT<T> L, const T* __restrict__ u, const T* __restrict__ b,
                                                 T* __restrict__ r)
 {
-    const size_t P = blockIdx.x * (size_t)NT + threadIdx.x;
-    if (P >= L.N()) return;
-    int i, j, k;
-    node_ijk(P, L, i, j, k);
-    if (is_face(L, i, j, k)) {
-        r[P] = T(0);
+    const int nx = L.nx, row = (int)(blockIdx.x * (NT / 32) + (threadIdx.x >> 5));
+    if (row >= L.ny * L.nz) return;
+    const int k = row / L.ny, j = row - k * L.ny, lane = threadIdx.x & 31;
+    const size_t P0 = (size_t)row * nx, sz = (size_t)nx * L.ny;
+    if (j == 0 || k == 0 || j == L.ny - 1 || k == L.nz - 1) {
+        for (int i = lane; i < nx; i += 32) r[P0 + i] = T(0);
         return;
     }
-    const T Au = fma(-dsum(L, i, j, k), u[P], offdiag(L, u, P, i, j, k));
-    r[P] = b[P] - Au;
+    const T cmy = L.ax[1].cm[j], cpy = L.ax[1].cp[j], cmz = L.ax[2].cm[k], cpz = L.ax[2].cp[k];
+    const T dyz = L.ax[1].dg[j] + L.ax[2].dg[k];
+    for (int m0 = lane; 2 * m0 < nx; m0 += 32 * RS_V) {
+        T v[RS_V][2];
+#pragma unroll
+        for (int q = 0; q < RS_V; q++)
+#pragma unroll
+            for (int t = 0; t < 2; t++) {   // t = 0: the red node of the pair
+                const int i = 2 * (m0 + 32 * q) + ((j + k + t) & 1);
+                v[q][t] = T(0);
+                if ((RED && t) || i < 1 || i > nx - 2) continue;
+                const T* c = u + P0 + i;
+                v[q][t] = fma(L.ax[0].dg[i] + dyz, c[0],
+                              rhs_less_neighbours(b[P0 + i], L.ax[0].cm[i], c[-1], L.ax[0].cp[i], c[1], cmy,
+                                                  c[-(ptrdiff_t)nx], cpy, c[nx], cmz, c[-(ptrdiff_t)sz], cpz, c[sz]));
+            }
+#pragma unroll
+        for (int q = 0; q < RS_V; q++)
+#pragma unroll
+            for (int t = 0; t < 2; t++) {
+                const int i = 2 * (m0 + 32 * q) + ((j + k + t) & 1);
+                if (i < nx) r[P0 + i] = v[q][t];
+            }
+    }
 }
 
 template <typename T>
@@ -365,11 +429,16 @@ __global__ void __launch_bounds__(NT) k_apply(LevelT<T> L, const T* __restrict__
     Au[P] = is_face(L, i, j, k) ? T(0) : fma(-dsum(L, i, j, k), u[P], offdiag(L, u, P, i, j, k));
 }
 
+// (red_only: u's last half sweep was black)
 template <typename T>
-cudaError_t launch_residual(const LevelT<T>& L, const T* u, const T* b, T* r, cudaStream_t s)
+cudaError_t launch_residual(const LevelT<T>& L, const T* u, const T* b, T* r, bool red_only, cudaStream_t s)
 {
     if (L.lsh) return cudaErrorInvalidValue;   // natural storage only
-    k_residual<T><<<(unsigned)((L.N() + NT - 1) / NT), NT, 0, s>>>(L, u, b, r);
+    const unsigned g = (unsigned)(((size_t)L.ny * L.nz + NT / 32 - 1) / (NT / 32));
+    if (red_only)
+        k_residual<T, 1><<<g, NT, 0, s>>>(L, u, b, r);
+    else
+        k_residual<T, 0><<<g, NT, 0, s>>>(L, u, b, r);
     return cudaGetLastError();
 }
 
@@ -382,75 +451,160 @@ cudaError_t launch_apply(const LevelT<T>& L, const T* u, T* Au, cudaStream_t s)
 }
 
 // ---------------------------------------------------------------- transfers
-// bc = Vc^-1 P^T Vf r: the 27-point stencil factorises into per-axis weights.
-template <typename T>
-__global__ void __launch_bounds__(NT) k_restrict(LevelT<T> F, LevelT<T> C, const T* __restrict__ r,
-                                                T* __restrict__ bc)
+// Both as marches along z, a thread per coarse column (or column of cells) and tk coarse planes:
+// the per-axis weights are applied one axis after the other, and a plane's x and y part is shared by
+// the coarse planes on both sides of it.  Blocks: 32 x 4 columns, numbered x first.  tk: 4 where that
+// still gives every SM two blocks, else 1 (the smaller levels wait for their loads: 65^3 to 33^3
+// 9.8 us with marches of 4, 5.3 with 1).
+constexpr int TR_TX = 32, TR_TY = 4;
+
+struct March {
+    int I, J, K0, K1;
+};
+
+__device__ __forceinline__ March march_of(int mx, int my, int mz, int tk)
 {
-    const size_t t = blockIdx.x * (size_t)NT + threadIdx.x;
-    if (t >= C.N()) return;
-    int I, J, K;
-    node_ijk(t, C, I, J, K);
-    if (is_face(C, I, J, K)) {
-        bc[t] = T(0);
-        return;
-    }
-    const T* wx = F.ax[0].rw + 3 * I;
-    const T* wy = F.ax[1].rw + 3 * J;
-    const T* wz = F.ax[2].rw + 3 * K;
-    const size_t sy = F.nx, sz = (size_t)F.nx * F.ny;
-    const T* base = r + (size_t)(2 * K - 1) * sz + (size_t)(2 * J - 1) * sy + (2 * I - 1);
-    T acc = T(0);
+    const int gx = (mx + TR_TX - 1) / TR_TX, gy = (my + TR_TY - 1) / TR_TY;
+    const int bz = (int)blockIdx.x / (gx * gy), rem = (int)blockIdx.x - bz * gx * gy, by = rem / gx, bx = rem - by * gx;
+    March m;
+    m.I = bx * TR_TX + (int)threadIdx.x % TR_TX;
+    m.J = by * TR_TY + (int)threadIdx.x / TR_TX;
+    m.K0 = bz * tk;
+    m.K1 = min(m.K0 + tk, mz);
+    return m;
+}
+
+static unsigned march_grid(int mx, int my, int mz, int* tk)
+{
+    const size_t cols = (size_t)((mx + TR_TX - 1) / TR_TX) * ((my + TR_TY - 1) / TR_TY);
+    *tk = cols * ((mz + 3) / 4) >= 2 * 152 ? 4 : 1;
+    return (unsigned)(cols * ((mz + *tk - 1) / *tk));
+}
+
+// bc = Vc^-1 P^T Vf r: the 27-point stencil factorises into per-axis weights.  uc (optional): the
+// coarse correction, zeroed for the recursion.  RED: the black values of r are zero (13 of the 27 are
+// read).  Bound in FP64: the pipe, 27 operations per coarse node (18 with RED) where a row-by-row
+// sum of the products takes 45.  FP64: 129 x 97 x 113 fine nodes 18.0 -> 15.2 us; RED at
+// 129^3 24.8 -> 14.5 us.
+template <typename T, int RED>
+__global__ void __launch_bounds__(TR_TX * TR_TY) k_restrict(LevelT<T> F, LevelT<T> C, const T* __restrict__ r,
+                                                            T* __restrict__ bc, T* __restrict__ uc, int tk)
+{
+    March m = march_of(C.nx - 2, C.ny - 2, C.nz, tk);
+    if (m.I >= C.nx - 2 || m.J >= C.ny - 2) return;
+    m.I++, m.J++;   // interior columns; the ones next to a face write the face's too
+    const size_t csz = (size_t)C.nx * C.ny, fsz = (size_t)F.nx * F.ny;
+    const size_t col = (size_t)m.J * C.nx + m.I;
+    T* out = bc + col;
+    for (int dj = m.J == 1 ? -1 : 0; dj <= (m.J == C.ny - 2 ? 1 : 0); dj++)
+        for (int di = m.I == 1 ? -1 : 0; di <= (m.I == C.nx - 2 ? 1 : 0); di++)
+            for (int K = m.K0; K < m.K1; K++) {
+                const size_t P = (size_t)(K * (ptrdiff_t)csz + (ptrdiff_t)col + dj * C.nx + di);
+                if (uc) uc[P] = T(0);
+                if (di || dj) bc[P] = T(0);
+            }
+    T wx[3], wy[3];
 #pragma unroll
-    for (int c = 0; c < 3; c++)
+    for (int q = 0; q < 3; q++) wx[q] = F.ax[0].rw[3 * m.I + q], wy[q] = F.ax[1].rw[3 * m.J + q];
+    const T* base = r + (size_t)(2 * m.J - 1) * F.nx + (2 * m.I - 1);
+    // the plane's weighted 3 x 3 sum; odd: an odd fine plane (the red nodes of its rows change places)
+    auto plane = [&](int k, auto odd) {
+        const T* p = base + (size_t)k * fsz;
+        T sum = T(0);
 #pragma unroll
-        for (int bb = 0; bb < 3; bb++) {
-            const T* row = base + c * sz + bb * sy;
-            const T s = fma(wx[0], row[0], fma(wx[1], row[1], wx[2] * row[2]));
-            acc = fma(wz[c] * wy[bb], s, acc);
+        for (int q = 0; q < 3; q++) {
+            const T* row = p + (size_t)q * F.nx;
+            constexpr int O = decltype(odd)::value;
+            T x;
+            if (RED && (q + O) % 2 == 0)
+                x = wx[0] * row[0] + wx[2] * row[2];
+            else if (RED)
+                x = wx[1] * row[1];
+            else
+                x = fma(wx[0], row[0], fma(wx[1], row[1], wx[2] * row[2]));
+            sum = q ? fma(wy[q], x, sum) : wy[q] * x;
         }
-    bc[t] = acc;
+        return sum;
+    };
+    const std::integral_constant<int, 0> EVEN{};
+    const std::integral_constant<int, 1> ODD{};
+    T below = m.K0 > 0 ? plane(2 * m.K0 - 1, ODD) : T(0);
+    for (int K = m.K0; K < m.K1; K++) {
+        if (K == C.nz - 1) {
+            out[K * csz] = T(0);
+            break;
+        }
+        const T above = plane(2 * K + 1, ODD);
+        if (K == 0) {
+            out[0] = T(0);
+        } else {
+            const T* wz = F.ax[2].rw + 3 * K;
+            out[K * csz] = fma(wz[0], below, fma(wz[1], plane(2 * K, EVEN), wz[2] * above));
+        }
+        below = above;
+    }
 }
 
 template <typename T>
-cudaError_t launch_restrict(const LevelT<T>& F, const LevelT<T>& C, const T* r, T* bc, cudaStream_t s)
+cudaError_t launch_restrict(const LevelT<T>& F, const LevelT<T>& C, const T* r, T* bc, T* uc, bool red_only, cudaStream_t s)
 {
     if (F.lsh || C.lsh) return cudaErrorInvalidValue;
-    k_restrict<T><<<(unsigned)((C.N() + NT - 1) / NT), NT, 0, s>>>(F, C, r, bc);
+    int tk;
+    const unsigned g = march_grid(C.nx - 2, C.ny - 2, C.nz, &tk);
+    if (red_only)
+        k_restrict<T, 1><<<g, TR_TX * TR_TY, 0, s>>>(F, C, r, bc, uc, tk);
+    else
+        k_restrict<T, 0><<<g, TR_TX * TR_TY, 0, s>>>(F, C, r, bc, uc, tk);
     return cudaGetLastError();
 }
 
 // u += P ec: per axis an even fine node sits on a coarse node (weight 1), an odd one
-// between two (weights pl, pr in physical coordinates).
-template <typename T, int LS>
-__global__ void __launch_bounds__(NT) k_prolong_add(LevelT<T> F, LevelT<T> C, const T* __restrict__ ec,
-                                                   T* __restrict__ u)
+// between two (weights pl, pr in physical coordinates).  A thread takes the eight fine nodes of a
+// cell per step: interpolated along x, then y, then z, 3.25 FP64 operations per fine node with
+// the addition, where a node by itself takes 8 (and 10 in a warp of mixed parities).  129^3 in FP64:
+// 44.7 -> 17.5 us.
+__global__ void __launch_bounds__(TR_TX * TR_TY) k_prolong_cells(LevelT<double> F, LevelT<double> C,
+                                                                 const double* __restrict__ ec, double* __restrict__ u, int tk)
 {
-    const size_t P = blockIdx.x * (size_t)NT + threadIdx.x;
-    if (P >= F.N()) return;
-    int i, j, k;
-    node_ijk(P, F, i, j, k);
-    if (is_face(F, i, j, k)) return;
-    const int I = i >> 1, J = j >> 1, K = k >> 1;
-    const int ni = (i & 1) ? 2 : 1, nj = (j & 1) ? 2 : 1, nk = (k & 1) ? 2 : 1;
-    const T wx[2] = {F.ax[0].pl[i], F.ax[0].pr[i]};
-    const T wy[2] = {F.ax[1].pl[j], F.ax[1].pr[j]};
-    const T wz[2] = {F.ax[2].pl[k], F.ax[2].pr[k]};
-    const size_t sy = C.nx, sz = (size_t)C.nx * C.ny;
-    const T* base = ec + (size_t)K * sz + (size_t)J * sy + I;
-    T e = T(0);
-    for (int c = 0; c < nk; c++)
-        for (int bb = 0; bb < nj; bb++) {
-            const T* row = base + c * sz + bb * sy;
-            const T s = (ni == 2) ? fma(wx[0], row[0], wx[1] * row[1]) : row[0];
-            e = fma(wz[c] * wy[bb], s, e);
+    const March m = march_of(C.nx - 1, C.ny - 1, C.nz - 1, tk);
+    if (m.I >= C.nx - 1 || m.J >= C.ny - 1) return;
+    const double wx0 = F.ax[0].pl[2 * m.I + 1], wx1 = F.ax[0].pr[2 * m.I + 1];
+    const double wy0 = F.ax[1].pl[2 * m.J + 1], wy1 = F.ax[1].pr[2 * m.J + 1];
+    const size_t csz = (size_t)C.nx * C.ny, fsz = (size_t)F.nx * F.ny;
+    const double* base = ec + (size_t)m.J * C.nx + m.I;
+    struct Quad {
+        double v[2][2];   // [y][x]: on the coarse node, half way
+    };
+    auto plane = [&](int K) {
+        const double* p = base + K * csz;
+        const double a = p[0], b = p[1], c = p[C.nx], d = p[C.nx + 1];
+        const double ab = fma(wx0, a, wx1 * b), cd = fma(wx0, c, wx1 * d);
+        return Quad{{{a, ab}, {fma(wy0, a, wy1 * c), fma(wy0, ab, wy1 * cd)}}};
+    };
+    const bool onx[2] = {m.I > 0, true}, ony[2] = {m.J > 0, true};
+    Quad lo = plane(m.K0);
+    for (int K = m.K0; K < m.K1; K++) {
+        const Quad hi = plane(K + 1);
+        const double wz0 = F.ax[2].pl[2 * K + 1], wz1 = F.ax[2].pr[2 * K + 1];
+        double* f = u + (size_t)(2 * K) * fsz + (size_t)(2 * m.J) * F.nx + 2 * m.I;
+        double v[2][2][2];
+#pragma unroll
+        for (int t = 0; t < 8; t++) {
+            const int z = t >> 2, y = (t >> 1) & 1, x = t & 1;
+            v[z][y][x] = onx[x] && ony[y] && (z || K > 0) ? f[z * fsz + (size_t)y * F.nx + x] : 0.0;
         }
-    u[pos<LS>(F, P)] += e;
+#pragma unroll
+        for (int t = 0; t < 8; t++) {
+            const int z = t >> 2, y = (t >> 1) & 1, x = t & 1;
+            const double e = z ? fma(wz0, lo.v[y][x], wz1 * hi.v[y][x]) : lo.v[y][x];
+            if (onx[x] && ony[y] && (z || K > 0)) f[z * fsz + (size_t)y * F.nx + x] = v[z][y][x] + e;
+        }
+        lo = hi;
+    }
 }
 
 // The same in FP32 with one warp per interior fine (j, k) row, lanes along the row's red nodes and
-// its black ones: the row's y and z weights and coarse rows once per warp, no index division; the
-// node expression is k_prolong_add's, so the two are bitwise equal.  A lane takes PU nodes of each
+// its black ones: the row's y and z weights and coarse rows once per warp, no index division.  A lane takes PU nodes of each
 // colour run (64 fine nodes apart) per step and loads all their fine values before the first
 // update, so 2 PU loads of the iterate are in flight per lane rather than one.
 constexpr int PU = 3;
@@ -564,24 +718,21 @@ cudaError_t launch_prolong_add(const LevelT<T>& F, const LevelT<T>& C, const T* 
         // are padded to 256 bytes, so ec is readable to the next 16 bytes past its end
         if (F.lsh && split_stage_ok(F.nx, F.ny, F.nz) && !((uintptr_t)u & 15u) && !((uintptr_t)ec & 15u))
             return launch_prolong_stage(F, C, ec, u, status, s);
-        if (F.ny >= 3 && F.nz >= 3) {
-            const unsigned g = (unsigned)(((size_t)(F.ny - 2) * (F.nz - 2) + 7) / 8);
-            int pf = 0;
-            const cudaError_t e = F.lsh ? prolong_rows_pf<1>(F, &pf) : prolong_rows_pf<0>(F, &pf);
-            if (e != cudaSuccess) return e;
-            if ((uintptr_t)u & 15u) pf = 0;
-            if (F.lsh)
-                k_prolong_add_rows<1><<<g, 256, 0, s>>>(F, C, ec, u, pf);
-            else
-                k_prolong_add_rows<0><<<g, 256, 0, s>>>(F, C, ec, u, pf);
-            return cudaGetLastError();
-        }
+        const unsigned g = (unsigned)(((size_t)(F.ny - 2) * (F.nz - 2) + 7) / 8);   // (every axis has 3 nodes or more)
+        int pf = 0;
+        const cudaError_t e = F.lsh ? prolong_rows_pf<1>(F, &pf) : prolong_rows_pf<0>(F, &pf);
+        if (e != cudaSuccess) return e;
+        if ((uintptr_t)u & 15u) pf = 0;
+        if (F.lsh)
+            k_prolong_add_rows<1><<<g, 256, 0, s>>>(F, C, ec, u, pf);
+        else
+            k_prolong_add_rows<0><<<g, 256, 0, s>>>(F, C, ec, u, pf);
+    } else {
+        if (F.lsh) return cudaErrorInvalidValue;
+        int tk;
+        const unsigned g = march_grid(C.nx - 1, C.ny - 1, C.nz - 1, &tk);
+        k_prolong_cells<<<g, TR_TX * TR_TY, 0, s>>>(F, C, ec, u, tk);
     }
-    const unsigned g = (unsigned)((F.N() + NT - 1) / NT);
-    if (F.lsh)
-        k_prolong_add<T, 1><<<g, NT, 0, s>>>(F, C, ec, u);
-    else
-        k_prolong_add<T, 0><<<g, NT, 0, s>>>(F, C, ec, u);
     return cudaGetLastError();
 }
 
@@ -941,7 +1092,7 @@ __device__ __forceinline__ void bot_point(const LevelT<T>& L, T* __restrict__ u,
     const int i = 2 * sl + ((colour + j + k) & 1);
     if (i < 1 || i > L.nx - 2) return;
     const size_t P = ((size_t)k * L.ny + j) * L.nx + i;
-    const T acc = b[P] - offdiag(L, u, P, i, j, k);
+    const T acc = rhs_less_offdiag(L, b[P], u, P, i, j, k);
     if constexpr (sizeof(T) == 8) u[P] = acc * L.inv_diag[P];
     else u[P] = rb_point32(acc, dsum(L, i, j, k));
 }
@@ -1137,11 +1288,6 @@ constexpr int RED_BLOCKS = 1216;   // 152 SMs x 8
 
 int reduce_blocks(const LevelT<double>& L) { return (int)std::min<size_t>((L.N() + NT - 1) / NT, RED_BLOCKS); }
 static unsigned red_grid(size_t N) { return (unsigned)std::min<size_t>((N + NT - 1) / NT, RED_BLOCKS); }
-
-__device__ __forceinline__ double vol(const LevelT<double>& L, int i, int j, int k)
-{
-    return L.ax[0].dual[i] * L.ax[1].dual[j] * L.ax[2].dual[k];
-}
 
 // FP32 warp sums, one FP64 value per warp, FP64 across the block's warps
 __device__ __forceinline__ double block_sum_f32(float v, double* sm)
@@ -1377,13 +1523,9 @@ __device__ __forceinline__ void k_resid_norm_body(LevelT<double> L, const double
                 v[q] = 0.0;
                 if (!frow && i >= 1 && i <= nx - 2) {
                     const double* c = u + P0 + i;
-                    double t = L.ax[0].cm[i] * c[-1];
-                    t = fma(L.ax[0].cp[i], c[1], t);
-                    t = fma(cmy, c[-(ptrdiff_t)sy], t);
-                    t = fma(cpy, c[sy], t);
-                    t = fma(cmz, c[-(ptrdiff_t)sz], t);
-                    t = fma(cpz, c[sz], t);
-                    v[q] = b[P0 + i] - fma(-(L.ax[0].dg[i] + dyz), c[0], t);
+                    v[q] = fma(L.ax[0].dg[i] + dyz, c[0],
+                               rhs_less_neighbours(b[P0 + i], L.ax[0].cm[i], c[-1], L.ax[0].cp[i], c[1], cmy,
+                                                   c[-(ptrdiff_t)sy], cpy, c[sy], cmz, c[-(ptrdiff_t)sz], cpz, c[sz]));
                 }
             }
 #pragma unroll
@@ -1412,22 +1554,47 @@ __global__ void __launch_bounds__(NT) k_resid_norm(LevelT<double> L, const doubl
     k_resid_norm_body(L, u, b, r, r32, h32, red);
 }
 
-// q = A p and <p, q>_vol
+// q = A p and <p, q>_vol: rows as in k_resid_norm, the row's part of the volume applied to the row's
+// sum.  10 FP64 operations per node instead of 13: 129^3 58.9 -> 49.7 us (53.1 with a
+// warp per row: the last block waits for every block's ticket).
 __global__ void __launch_bounds__(NT) k_apply_dot(LevelT<double> L, const double* __restrict__ p,
                                                  double* __restrict__ q, Red red)
 {
     __shared__ double sm[32];
     double acc = 0.0;
-    GRID_STRIDE(P, L.N())
-    {
-        int i, j, k;
-        node_ijk(P, L, i, j, k);
-        double v = 0.0;
-        if (!is_face(L, i, j, k)) {
-            v = fma(-dsum(L, i, j, k), p[P], offdiag(L, p, P, i, j, k));
-            acc = fma(vol(L, i, j, k) * p[P], v, acc);
+    const int nx = L.nx, rows = L.ny * L.nz, lane = threadIdx.x & 31;
+    const size_t sz = (size_t)nx * L.ny;
+    for (int row = (int)(blockIdx.x * (NT / 32) + (threadIdx.x >> 5)); row < rows; row += (int)(gridDim.x * (NT / 32))) {
+        const int k = row / L.ny, j = row - k * L.ny;
+        const bool frow = j == 0 || k == 0 || j == L.ny - 1 || k == L.nz - 1;
+        const size_t P0 = (size_t)row * nx;
+        double cmy = 0.0, cpy = 0.0, cmz = 0.0, cpz = 0.0, dyz = 0.0, racc = 0.0;
+        if (!frow) {
+            cmy = L.ax[1].cm[j], cpy = L.ax[1].cp[j], cmz = L.ax[2].cm[k], cpz = L.ax[2].cp[k];
+            dyz = L.ax[1].dg[j] + L.ax[2].dg[k];
         }
-        q[P] = v;
+        for (int i0 = lane; i0 < nx; i0 += 32 * RN_V) {
+            double v[RN_V];
+#pragma unroll
+            for (int t = 0; t < RN_V; t++) {
+                const int i = i0 + 32 * t;
+                v[t] = 0.0;
+                if (frow || i < 1 || i > nx - 2) continue;
+                const double* c = p + P0 + i;
+                v[t] = L.ax[0].cm[i] * c[-1];
+                v[t] = fma(L.ax[0].cp[i], c[1], v[t]);
+                v[t] = fma(cmy, c[-(ptrdiff_t)nx], v[t]);
+                v[t] = fma(cpy, c[nx], v[t]);
+                v[t] = fma(cmz, c[-(ptrdiff_t)sz], v[t]);
+                v[t] = fma(cpz, c[sz], v[t]);
+                v[t] = fma(-(L.ax[0].dg[i] + dyz), c[0], v[t]);
+                racc = fma(L.ax[0].dual[i] * c[0], v[t], racc);
+            }
+#pragma unroll
+            for (int t = 0; t < RN_V; t++)
+                if (i0 + 32 * t < nx) q[P0 + i0 + 32 * t] = v[t];
+        }
+        if (!frow) acc = fma(L.ax[1].dual[j] * L.ax[2].dual[k], racc, acc);
     }
     reduce_finish(block_sum<NT>(acc, sm), red, sm);
 }
@@ -1453,16 +1620,31 @@ __global__ void __launch_bounds__(NT) k_update_ur(LevelT<double> L, const Ctl* _
     reduce_finish(block_sum<NT>(acc, sm), red, sm);
 }
 
+// <r, z>_vol over the interior rows, as above: 2 FP64 operations per node instead of 4 (129^3:
+// 26.7 -> 17.7 us; 23.0 with a warp per row)
 __global__ void __launch_bounds__(NT) k_dot_rz(LevelT<double> L, const double* __restrict__ r,
                                               const double* __restrict__ z, Red red)
 {
     __shared__ double sm[32];
     double acc = 0.0;
-    GRID_STRIDE(P, L.N())
-    {
-        int i, j, k;
-        node_ijk(P, L, i, j, k);
-        if (!is_face(L, i, j, k)) acc = fma(vol(L, i, j, k) * r[P], z[P], acc);
+    const int nx = L.nx, my = L.ny - 2, rows = my * (L.nz - 2), lane = threadIdx.x & 31;
+    for (int row = (int)(blockIdx.x * (NT / 32) + (threadIdx.x >> 5)); row < rows; row += (int)(gridDim.x * (NT / 32))) {
+        const int k = row / my + 1, j = row - (k - 1) * my + 1;
+        const size_t P0 = ((size_t)k * L.ny + j) * nx;
+        double racc = 0.0;
+        for (int i0 = 1 + lane; i0 < nx - 1; i0 += 32 * RN_V) {
+            double rv[RN_V], zv[RN_V];
+#pragma unroll
+            for (int t = 0; t < RN_V; t++) {
+                const bool in = i0 + 32 * t < nx - 1;
+                rv[t] = in ? r[P0 + i0 + 32 * t] : 0.0;
+                zv[t] = in ? z[P0 + i0 + 32 * t] : 0.0;
+            }
+#pragma unroll
+            for (int t = 0; t < RN_V; t++)
+                if (i0 + 32 * t < nx - 1) racc = fma(L.ax[0].dual[i0 + 32 * t] * rv[t], zv[t], racc);
+        }
+        acc = fma(L.ax[1].dual[j] * L.ax[2].dual[k], racc, acc);
     }
     reduce_finish(block_sum<NT>(acc, sm), red, sm);
 }
@@ -1973,7 +2155,7 @@ cudaError_t launch_resid_norm(const LevelT<double>& L, const double* u, const do
 }
 cudaError_t launch_apply_dot(const LevelT<double>& L, const double* p, double* q, const Red& red, cudaStream_t s)
 {
-    k_apply_dot<<<RGRID(L)>>>(L, p, q, red);
+    k_apply_dot<<<std::min(resid_rows_grid(L), (unsigned)VEC_BLOCKS), NT, 0, s>>>(L, p, q, red);
     return cudaGetLastError();
 }
 cudaError_t launch_update_ur(const LevelT<double>& L, const Ctl* ctl, const double* p, const double* q, double* u,
@@ -1984,7 +2166,7 @@ cudaError_t launch_update_ur(const LevelT<double>& L, const Ctl* ctl, const doub
 }
 cudaError_t launch_dot_rz(const LevelT<double>& L, const double* r, const double* z, const Red& red, cudaStream_t s)
 {
-    k_dot_rz<<<RGRID(L)>>>(L, r, z, red);
+    k_dot_rz<<<std::min(resid_rows_grid(L), (unsigned)VEC_BLOCKS), NT, 0, s>>>(L, r, z, red);
     return cudaGetLastError();
 }
 cudaError_t launch_update_p(const LevelT<double>& L, const Ctl* ctl, const double* z, double* p, cudaStream_t s)
@@ -2566,9 +2748,9 @@ void init_bat_attributes()
                                                   bool, cudaStream_t, T*, int*);                            \
     template cudaError_t launch_bottom<T>(const BottomArgs<T>&, cudaStream_t);                              \
     template cudaError_t launch_rbgs<T>(const LevelT<T>&, T*, const T*, int, cudaStream_t, int, int*);               \
-    template cudaError_t launch_residual<T>(const LevelT<T>&, const T*, const T*, T*, cudaStream_t);        \
+    template cudaError_t launch_residual<T>(const LevelT<T>&, const T*, const T*, T*, bool, cudaStream_t);      \
     template cudaError_t launch_apply<T>(const LevelT<T>&, const T*, T*, cudaStream_t);                     \
-    template cudaError_t launch_restrict<T>(const LevelT<T>&, const LevelT<T>&, const T*, T*, cudaStream_t); \
+    template cudaError_t launch_restrict<T>(const LevelT<T>&, const LevelT<T>&, const T*, T*, T*, bool, cudaStream_t); \
     template cudaError_t launch_prolong_add<T>(const LevelT<T>&, const LevelT<T>&, const T*, T*, cudaStream_t, int*); \
     template cudaError_t launch_coarse_apply<T>(const LevelT<T>&, const CoarseEig*, const T*, T*, bool, cudaStream_t);
 INST(double)

@@ -103,15 +103,10 @@ __global__ void __launch_bounds__(SLAB_NT) k_rb_slab(LevelT<T> L, const T* __res
                     const int i = ia + ((c - ia - j - q) & 1) + 2 * (e - jr * mc);
                     if (i > ib) continue;
                     const int o = (j - gy) * RX + (i - gx);
-                    // the six neighbour terms in the fixed order x-, x+, y-, y+, z-, z+
-                    T t = L.ax[0].cm[i] * pc[o - 1];
-                    t = fma(L.ax[0].cp[i], pc[o + 1], t);
-                    t = fma(L.ax[1].cm[j], pc[o - RX], t);
-                    t = fma(L.ax[1].cp[j], pc[o + RX], t);
-                    t = fma(cmz, pm[o], t);
-                    t = fma(cpz, pp[o], t);
                     const size_t P = (size_t)q * sz + (size_t)j * sy + i;
-                    const T acc = b[P] - t;
+                    const T acc = rhs_less_neighbours(b[P], L.ax[0].cm[i], pc[o - 1], L.ax[0].cp[i], pc[o + 1],
+                                                      L.ax[1].cm[j], pc[o - RX], L.ax[1].cp[j], pc[o + RX], cmz, pm[o],
+                                                      cpz, pp[o]);
                     if constexpr (sizeof(T) == 8) {
                         pc[o] = acc * L.inv_diag[P];
                     } else {
@@ -253,27 +248,16 @@ __device__ __forceinline__ void col_sweep(const LevelT<T>& L, const T* __restric
             const int q = p - 1;
             if (q >= max(1, k0 - 1) && q <= min(nz - 2, k1) && (red_a ? int_a : int_b)) {
                 const T* zc = ZC + 3 * (q - k0 + 2);
-                T t;
                 if (red_a) {
-                    t = cmxa * A[oA - 1];
-                    t = fma(cpxa, ub[r1], t);
-                    t = fma(cmy, A[oA - AX], t);
-                    t = fma(cpy, A[oA + AX], t);
-                    t = fma(zc[0], ua[r2], t);
-                    t = fma(zc[1], ua[r0], t);
-                    const T acc = ba[r1] - t;
+                    const T acc = rhs_less_neighbours(ba[r1], cmxa, A[oA - 1], cpxa, ub[r1], cmy, A[oA - AX], cpy, A[oA + AX],
+                                                      zc[0], ua[r2], zc[1], ua[r0]);
                     if constexpr (sizeof(T) == 8)
                         ua[r1] = acc * va[r1];
                     else
                         ua[r1] = rb_point32(acc, dga + dgy + zc[2]);
                 } else {
-                    t = cmxb * ua[r1];
-                    t = fma(cpxb, A[oA + 2], t);
-                    t = fma(cmy, A[oA + 1 - AX], t);
-                    t = fma(cpy, A[oA + 1 + AX], t);
-                    t = fma(zc[0], ub[r2], t);
-                    t = fma(zc[1], ub[r0], t);
-                    const T acc = bb[r1] - t;
+                    const T acc = rhs_less_neighbours(bb[r1], cmxb, ua[r1], cpxb, A[oA + 2], cmy, A[oA + 1 - AX], cpy, A[oA + 1 + AX],
+                                                      zc[0], ub[r2], zc[1], ub[r0]);
                     if constexpr (sizeof(T) == 8)
                         ub[r1] = acc * vb[r1];
                     else
@@ -285,27 +269,16 @@ __device__ __forceinline__ void col_sweep(const LevelT<T>& L, const T* __restric
             const int q2 = p - 2;
             if (q2 >= max(1, k0) && q2 <= min(nz - 2, k1 - 1) && (blk_a ? (int_a && wa) : (int_b && wb))) {
                 const T* zc = ZC + 3 * (q2 - k0 + 2);
-                T t;
                 if (blk_a) {
-                    t = cmxa * Bp[oB - 1];
-                    t = fma(cpxa, ub[r2], t);
-                    t = fma(cmy, Bp[oB - BX], t);
-                    t = fma(cpy, Bp[oB + BX], t);
-                    t = fma(zc[0], ua[r3], t);
-                    t = fma(zc[1], ua[r1], t);
-                    const T acc = ba[r2] - t;
+                    const T acc = rhs_less_neighbours(ba[r2], cmxa, Bp[oB - 1], cpxa, ub[r2], cmy, Bp[oB - BX], cpy, Bp[oB + BX],
+                                                      zc[0], ua[r3], zc[1], ua[r1]);
                     if constexpr (sizeof(T) == 8)
                         ua[r2] = acc * va[r2];
                     else
                         ua[r2] = rb_point32(acc, dga + dgy + zc[2]);
                 } else {
-                    t = cmxb * ua[r2];
-                    t = fma(cpxb, Bp[oB + 2], t);
-                    t = fma(cmy, Bp[oB + 1 - BX], t);
-                    t = fma(cpy, Bp[oB + 1 + BX], t);
-                    t = fma(zc[0], ub[r3], t);
-                    t = fma(zc[1], ub[r1], t);
-                    const T acc = bb[r2] - t;
+                    const T acc = rhs_less_neighbours(bb[r2], cmxb, ua[r2], cpxb, Bp[oB + 2], cmy, Bp[oB + 1 - BX], cpy, Bp[oB + 1 + BX],
+                                                      zc[0], ub[r3], zc[1], ub[r1]);
                     if constexpr (sizeof(T) == 8)
                         ub[r2] = acc * vb[r2];
                     else
