@@ -682,11 +682,10 @@ int enqueue_rhs(lasto_poisson* h, ClusterPlan& P, const lasto_cluster& cl, const
         TRY(launch_deposit(cl, P.rec, h->cfg.precision, F.b, nullptr, nullptr, nullptr, P.status, s));
     }
     double* tabs = P.mom;
-    double* rowm = tabs + 5 * ((size_t)n[0] + n[1] + n[2]);
-    double* plane = rowm + 5 * (size_t)n[1] * n[2];
+    double* plane = tabs + 5 * ((size_t)n[0] + n[1] + n[2]);
     TRY(cudaMemsetAsync(F.u, 0, sizeof(double) * F.N(), s));
     if (h->cfg.boundary == LASTO_BC_MULTIPOLE) {
-        TRY(launch_multipoles(n, cl.x, cl.y, cl.z, F.b, cl.centre, tabs, rowm, plane, P.Q, s));
+        TRY(launch_multipoles(n, cl.x, cl.y, cl.z, F.b, cl.centre, tabs, plane, P.Q, s));
         TRY(launch_boundary_fill(n, cl.x, cl.y, cl.z, cl.centre[0], cl.centre[1], cl.centre[2], P.Q, F.u, s));
     } else if (h->cfg.boundary == LASTO_BC_EXACT) {
         TRY(launch_boundary_exact(cl, tabs, F.u, s));   // the multipole scratch holds the moments
@@ -756,10 +755,14 @@ int enqueue_guess_in(lasto_poisson* h, ClusterPlan& P, const lasto_cluster& cl, 
         TRY(launch_restrict<double>(P.lv[l].view64(), P.lv[l + 1].view64(), P.lv[l].b, P.lv[l + 1].b,
                                     (double*)nullptr, false, s));
     const LevelStore& S = P.lv[P.gl];
-    TRY(launch_resample(S.n, S.ax[0].c, S.ax[1].c, S.ax[2].c, S.b, G, P.gax[0], P.gax[1], P.gax[2], P.bG, 0, s));
-    // faces (and a zero interior) from the fine grid's first iterate: copies at shared nodes
+    // (level gl is the subgrid itself where it has 33 nodes per axis: a copy, exactly)
+    if (std::equal(G, G + 3, S.n))
+        TRY(launch_copy_strided(S.n, S.b, G, P.bG, 0, s));
+    else
+        TRY(launch_resample(S.n, S.ax[0].c, S.ax[1].c, S.ax[2].c, S.b, G, P.gax[0], P.gax[1], P.gax[2], P.bG, 0, s));
+    // faces (and a zero interior) from the fine grid's first iterate, at the shared nodes
     const LevelStore& F = P.lv[0];
-    TRY(launch_resample(F.n, F.ax[0].c, F.ax[1].c, F.ax[2].c, F.u, G, P.gax[0], P.gax[1], P.gax[2], P.fG, 0, s));
+    TRY(launch_copy_strided(F.n, F.u, G, P.fG, 0, s));
     const float* sc = guess_net_scales(h->net);
     if (lasto_nn_guess_features(G, P.bG, P.fG, P.gax[0], P.gax[1], P.gax[2], sc[0], sc[1], sc[2],
                                 guess_net_features(h->net, P.gslot), s) != LASTO_OK)
@@ -780,14 +783,14 @@ int enqueue_guess_out(lasto_poisson* h, ClusterPlan& P, const lasto_cluster& cl,
     const LevelStore& F = P.lv[0];
     double* tgt = gl == 0 ? P.lv[0].u : S.u;
     // coarse levels: the fine grid's faces and zero interior (copies at shared nodes)
-    if (gl > 0)
-        TRY(launch_resample(F.n, F.ax[0].c, F.ax[1].c, F.ax[2].c, F.u, S.n, S.ax[0].c, S.ax[1].c, S.ax[2].c, tgt, 0, s));
-    TRY(launch_resample(G, P.gax[0], P.gax[1], P.gax[2], P.uG, S.n, S.ax[0].c, S.ax[1].c, S.ax[2].c, tgt, 1, s));
+    if (gl > 0) TRY(launch_copy_strided(F.n, F.u, S.n, tgt, 0, s));
+    if (std::equal(G, G + 3, S.n))
+        TRY(launch_copy_strided(G, P.uG, S.n, tgt, 1, s));
+    else
+        TRY(launch_resample(G, P.gax[0], P.gax[1], P.gax[2], P.uG, S.n, S.ax[0].c, S.ax[1].c, S.ax[2].c, tgt, 1, s));
     for (int l = gl - 1; l >= 0; l--) {
         LevelStore& Fl = P.lv[l];
-        if (l > 0)
-            TRY(launch_resample(F.n, F.ax[0].c, F.ax[1].c, F.ax[2].c, F.u, Fl.n, Fl.ax[0].c, Fl.ax[1].c, Fl.ax[2].c,
-                                Fl.u, 0, s));
+        if (l > 0) TRY(launch_copy_strided(F.n, F.u, Fl.n, Fl.u, 0, s));
         TRY(launch_prolong_add<double>(Fl.view64(), P.lv[l + 1].view64(), P.lv[l + 1].u, Fl.u, s));
     }
     (void)cl;
@@ -1899,9 +1902,8 @@ int lasto_op_multipoles(const int n[3], const double* x, const double* y, const 
     Scratch m(sizeof(double) * multipole_scratch_doubles(n), s);
     if (!m.p) return LASTO_ERR_NO_MEMORY;
     double* tabs = m.as<double>();
-    double* rowm = tabs + 5 * ((size_t)n[0] + n[1] + n[2]);
-    double* plane = rowm + 5 * (size_t)n[1] * n[2];
-    return op_status(launch_multipoles(n, x, y, z, b, centre, tabs, rowm, plane, Q, s));
+    double* plane = tabs + 5 * ((size_t)n[0] + n[1] + n[2]);
+    return op_status(launch_multipoles(n, x, y, z, b, centre, tabs, plane, Q, s));
 }
 
 int lasto_op_boundary_fill(const int n[3], const double* x, const double* y, const double* z, const double centre[3],

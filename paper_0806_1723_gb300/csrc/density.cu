@@ -1282,128 +1282,177 @@ void init_device_constants()
 // ---------------------------------------------------------------- boundary multipoles
 // Q_lm = sum (b/4pi) vol S_lm(node - centre).  S_lm is a polynomial of degree l in
 // (x, y, z) and vol a product of per-axis dual lengths, so the sum factorises:
-// per-row x-moments (5 FMAs per node), then y and z contractions over the rows,
-// then the monomial expansion of each S_lm.
-constexpr int MOM_NT = 128;
+// per-column y-moments (5 FMAs per node), then x and z contractions, then the monomial
+// expansion of each S_lm.
 
-// xm[a][i] = (x_i - cx)^a * dual_i, a = 0..4
-__global__ void k_moment_table(const double* __restrict__ x, int n, double c, double* __restrict__ tab)
+// tab[axis][a][i] = (x_i - c)^a * dual_i, a = 0..4 (blockIdx.y: the axis)
+__global__ void k_moment_tables(const double* __restrict__ x, const double* __restrict__ y, const double* __restrict__ z,
+                                int nx, int ny, int nz, double cx, double cy, double cz, double* __restrict__ tab)
 {
+    const int d = blockIdx.y, n = d == 0 ? nx : d == 1 ? ny : nz;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const double dual = (i == 0) ? 0.5 * (x[1] - x[0]) : (i == n - 1) ? 0.5 * (x[n - 1] - x[n - 2])
-                                                                  : 0.5 * (x[i + 1] - x[i - 1]);
-    const double d = x[i] - c;
-    double p = dual;
-    for (int a = 0; a < 5; a++) {
-        tab[(size_t)a * n + i] = p;
-        p *= d;
+    const double* a = d == 0 ? x : d == 1 ? y : z;
+    const double c = d == 0 ? cx : d == 1 ? cy : cz;
+    double* out = tab + 5 * (size_t)(d == 0 ? 0 : d == 1 ? nx : nx + ny);
+    double p = (i == 0) ? 0.5 * (a[1] - a[0]) : (i == n - 1) ? 0.5 * (a[n - 1] - a[n - 2]) : 0.5 * (a[i + 1] - a[i - 1]);
+    const double e = a[i] - c;
+    for (int q = 0; q < 5; q++) {
+        out[(size_t)q * n + i] = p;
+        p *= e;
     }
-}
-
-// row_mom[a][row] = sum_i xm[a][i] b[row, i],  row = k*ny + j: one thread per row, sequential
-// FP64 sums (no shuffle trees: FP64 adds are scarce on this GPU).
-__global__ void __launch_bounds__(MOM_NT) k_row_moments(const double* __restrict__ b, int nx, size_t nrows,
-                                                       const double* __restrict__ xm, double* __restrict__ row_mom)
-{
-    const size_t row = blockIdx.x * (size_t)MOM_NT + threadIdx.x;
-    if (row >= nrows) return;
-    const double* br = b + row * nx;
-    double acc[5] = {0, 0, 0, 0, 0};
-    for (int i = 0; i < nx; i++) {
-        const double v = br[i];
-#pragma unroll
-        for (int q = 0; q < 5; q++) acc[q] = fma(xm[(size_t)q * nx + i], v, acc[q]);
-    }
-#pragma unroll
-    for (int q = 0; q < 5; q++) row_mom[(size_t)q * nrows + row] = acc[q];
 }
 
 // pairs (a, b) with a + b <= 4, in a fixed order
 __constant__ int c_ab[15][2] = {{0, 0}, {0, 1}, {0, 2}, {0, 3}, {0, 4}, {1, 0}, {1, 1}, {1, 2}, {1, 3},
                                 {2, 0}, {2, 1}, {2, 2}, {3, 0}, {3, 1}, {4, 0}};
 
-// plane[ab][k] = sum_j ym[b][j] row_mom[a][k*ny + j]: one thread per (ab, k)
-__global__ void __launch_bounds__(MOM_NT) k_plane_moments(const double* __restrict__ row_mom, int ny, int nz,
-                                                         const double* __restrict__ ym, double* __restrict__ plane)
+// plane[ab][k] = sum_ij xm[a][i] ym[b][j] b[k, j, i]: one block per plane.  A thread sums the five
+// y-moments of a column i over one of JG ranges of j (consecutive lanes read consecutive nodes; a
+// sum along x would need a shuffle tree per row, and FP64 additions are scarce on this GPU), the
+// block adds the ranges and contracts the columns.  Columns in tiles of MOM_T.  Bound: 5 FP64
+// operations per node (129^3: 18 us).  With the tables and the z contraction 129^3 100 -> 41 us (before:
+// a thread per row, uncoalesced, then a thread per plane and pair), 385^3 710 -> 624 us.
+constexpr int MOM_T = 1024;
+
+__global__ void __launch_bounds__(MOM_T) k_plane_moments(const double* __restrict__ b, int nx, int ny, int nz, int JG,
+                                                        const double* __restrict__ xm, const double* __restrict__ ym,
+                                                        double* __restrict__ plane)
 {
-    const int t = blockIdx.x * MOM_NT + threadIdx.x;
-    if (t >= 15 * nz) return;
-    const int ab = t / nz, k = t - ab * nz;
-    const int A = c_ab[ab][0], B = c_ab[ab][1];
-    const size_t nrows = (size_t)ny * nz;
-    const double* rm = row_mom + (size_t)A * nrows + (size_t)k * ny;
-    const double* yb = ym + (size_t)B * ny;
-    double acc = 0.0;
-    for (int j = 0; j < ny; j++) acc = fma(yb[j], rm[j], acc);
-    plane[(size_t)ab * nz + k] = acc;
+    extern __shared__ double s_col[];   // [5][JG][columns of a tile]
+    __shared__ double s_ab[15];
+    const int k = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+    const int jl = (ny + JG - 1) / JG;
+    if (tid < 15) s_ab[tid] = 0.0;
+    for (int i0 = 0; i0 < nx; i0 += MOM_T) {
+        const int ni = min(MOM_T, nx - i0);
+        for (int e = tid; e < ni * JG; e += blockDim.x) {
+            const int g = e / ni, i = e - g * ni, j1 = min(ny, (g + 1) * jl);
+            const double* col = b + (size_t)k * ny * nx + i0 + i;
+            double acc[5] = {0, 0, 0, 0, 0};
+#pragma unroll 4
+            for (int j = g * jl; j < j1; j++) {
+                const double v = col[(size_t)j * nx];
+#pragma unroll
+                for (int q = 0; q < 5; q++) acc[q] = fma(__ldg(ym + (size_t)q * ny + j), v, acc[q]);
+            }
+#pragma unroll
+            for (int q = 0; q < 5; q++) s_col[(q * JG + g) * ni + i] = acc[q];
+        }
+        __syncthreads();
+        for (int e = tid; e < 5 * ni; e += blockDim.x) {   // the ranges' sums into the first one's place
+            const int q = e / ni, i = e - q * ni;
+            double v = s_col[q * JG * ni + i];
+            for (int g = 1; g < JG; g++) v += s_col[(q * JG + g) * ni + i];
+            s_col[q * JG * ni + i] = v;
+        }
+        __syncthreads();
+        for (int ab = warp; ab < 15; ab += nw) {
+            const double* xa = xm + (size_t)c_ab[ab][0] * nx + i0;
+            const double* cb = s_col + c_ab[ab][1] * JG * ni;
+            double acc = 0.0;
+            for (int i = lane; i < ni; i += 32) acc = fma(xa[i], cb[i], acc);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+            if (lane == 0) s_ab[ab] += acc;
+        }
+        __syncthreads();
+    }
+    if (tid < 15) plane[(size_t)tid * nz + k] = s_ab[tid];
 }
 
-// M[a][b][c] = sum_k zm[c][k] plane[ab][k] (one thread per monomial); Q_lm = sum_terms coef M / (4 pi)
-__global__ void __launch_bounds__(64) k_final_moments(const double* __restrict__ plane, int nz,
-                                                     const double* __restrict__ zm, double* __restrict__ Q)
+// M[a][b][c] = sum_k zm[c][k] plane[ab][k] (a warp per monomial); Q_lm = sum_terms coef M / (4 pi)
+__global__ void __launch_bounds__(1024) k_final_moments(const double* __restrict__ plane, int nz,
+                                                       const double* __restrict__ zm, double* __restrict__ Q)
 {
     __shared__ double M[5][5][5];
-    const int t = threadIdx.x;
-    if (t < 35) {
-        // monomial t -> (ab, c) in the order of c_ab with c = 0 .. 4 - a - b
-        int idx = 0, ab = 0, C = 0;
-        for (int q = 0; q < 15; q++) {
-            const int room = 5 - c_ab[q][0] - c_ab[q][1];
-            if (t < idx + room) {
-                ab = q;
-                C = t - idx;
-                break;
-            }
-            idx += room;
-        }
-        double acc = 0.0;
+    const int t = threadIdx.x, lane = t & 31;
+    for (int mono = t >> 5; mono < 35; mono += 32) {
+        // the monomial -> (ab, c) in the order of c_ab with c = 0 .. 4 - a - b
+        int idx = 0, ab = 0;
+        while (mono >= idx + 5 - c_ab[ab][0] - c_ab[ab][1]) idx += 5 - c_ab[ab][0] - c_ab[ab][1], ab++;
+        const int C = mono - idx;
         const double* pl = plane + (size_t)ab * nz;
         const double* zc = zm + (size_t)C * nz;
-        for (int k = 0; k < nz; k++) acc = fma(zc[k], pl[k], acc);
-        M[c_ab[ab][0]][c_ab[ab][1]][C] = acc;
+        double acc = 0.0;
+        for (int k = lane; k < nz; k += 32) acc = fma(zc[k], pl[k], acc);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+        if (lane == 0) M[c_ab[ab][0]][c_ab[ab][1]][C] = acc;
+    }
+    __syncthreads();
+    // a term per thread, then a harmonic's sum per thread (in the terms' order)
+    __shared__ double s_term[N_MONO_TERMS];
+    __shared__ int s_lm[N_MONO_TERMS];
+    if (t < N_MONO_TERMS) {
+        const Mono mo = c_mono[t];
+        s_lm[t] = mo.lm;
+        s_term[t] = mo.coef * M[mo.a][mo.b][mo.c];
     }
     __syncthreads();
     if (t < NLM) {
         double q = 0.0;
-        for (int m = 0; m < N_MONO_TERMS; m++) {
-            const Mono mo = c_mono[m];
-            if (mo.lm == t) q = fma(mo.coef, M[mo.a][mo.b][mo.c], q);
-        }
+#pragma unroll 8
+        for (int m = 0; m < N_MONO_TERMS; m++)
+            if (s_lm[m] == t) q += s_term[m];
         Q[t] = q / (4.0 * PI);
     }
 }
 
 cudaError_t launch_multipoles(const int n[3], const double* x, const double* y, const double* z, const double* b,
-                              const double centre[3], double* tabs, double* row_mom, double* plane, double* Q,
-                              cudaStream_t s)
+                              const double centre[3], double* tabs, double* plane, double* Q, cudaStream_t s)
 {
     cudaError_t e = ensure_monomials();
     if (e != cudaSuccess) return e;
-    double* xm = tabs;
-    double* ym = xm + 5 * (size_t)n[0];
-    double* zm = ym + 5 * (size_t)n[1];
-    k_moment_table<<<(n[0] + 127) / 128, 128, 0, s>>>(x, n[0], centre[0], xm);
-    k_moment_table<<<(n[1] + 127) / 128, 128, 0, s>>>(y, n[1], centre[1], ym);
-    k_moment_table<<<(n[2] + 127) / 128, 128, 0, s>>>(z, n[2], centre[2], zm);
-    const size_t nrows = (size_t)n[1] * n[2];
-    k_row_moments<<<(unsigned)((nrows + MOM_NT - 1) / MOM_NT), MOM_NT, 0, s>>>(b, n[0], nrows, xm, row_mom);
-    k_plane_moments<<<(15 * n[2] + MOM_NT - 1) / MOM_NT, MOM_NT, 0, s>>>(row_mom, n[1], n[2], ym, plane);
-    k_final_moments<<<1, 64, 0, s>>>(plane, n[2], zm, Q);
+    const int nm = std::max(n[0], std::max(n[1], n[2])), ni = std::min(n[0], MOM_T), JG = std::min(n[1], MOM_T / ni);
+    const unsigned nt = (unsigned)(ni * JG + 31) / 32 * 32;
+    const double *xm = tabs, *ym = xm + 5 * (size_t)n[0], *zm = ym + 5 * (size_t)n[1];
+    k_moment_tables<<<dim3((nm + 127) / 128, 3), 128, 0, s>>>(x, y, z, n[0], n[1], n[2], centre[0], centre[1], centre[2],
+                                                              tabs);
+    k_plane_moments<<<(unsigned)n[2], nt, sizeof(double) * 5 * ni * JG, s>>>(b, n[0], n[1], n[2], JG, xm, ym, plane);
+    k_final_moments<<<1, 1024, 0, s>>>(plane, n[2], zm, Q);
     return cudaGetLastError();
 }
 
+// (the exact faces' five moments per atom use the same array)
 size_t multipole_scratch_doubles(const int n[3])
 {
     return 5 * ((size_t)n[0] + n[1] + n[2]) + 5 * (size_t)n[1] * n[2] + 15 * (size_t)n[2];
 }
 
 // ---------------------------------------------------------------- Dirichlet faces
-// u = -sum_lm 4 pi/(2l+1) Q_lm S_lm(d) / r^(2l+1), d = node - centre (Eq. 2.7 decay).
+// slot of x^a y^b z^c (a + b + c = l, 1 <= l <= 4): degree offset + s(s+1)/2 + c, s = b + c
+__host__ __device__ constexpr int ex_slot(int l, int b, int c)
+{
+    return (l == 1 ? 0 : l == 2 ? 3 : l == 3 ? 9 : 19) + (b + c) * (b + c + 1) / 2 + c;
+}
+
+// u = -sum_lm 4 pi/(2l+1) Q_lm S_lm(d) / r^(2l+1), d = node - centre (Eq. 2.7 decay).  S_lm is
+// homogeneous of degree l, so with e = d / r^2 this is P(e) / r, one polynomial of degree 4 whose 35
+// coefficients each block forms first: about 55 FP64 operations per node where the harmonics one by
+// one take 300.  129^3 63.6 -> 18.1 us, 385^3 465 -> 109 us.
 __global__ void k_boundary_fill(int nx, int ny, int nz, const double* __restrict__ x, const double* __restrict__ y,
                                 const double* __restrict__ z, double cx, double cy, double cz,
                                 const double* __restrict__ Q, double* __restrict__ u)
 {
+    // the coefficients: a term of a harmonic per thread, then a coefficient's sum per thread
+    __shared__ double s_cf[35], s_term[N_MONO_TERMS];
+    __shared__ int s_slot[N_MONO_TERMS];
+    if (threadIdx.x < N_MONO_TERMS) {
+        const Mono mo = c_mono[threadIdx.x];
+        const int l = mo.a + mo.b + mo.c;
+        s_slot[threadIdx.x] = l == 0 ? 0 : 1 + ex_slot(l, mo.b, mo.c);
+        s_term[threadIdx.x] = -4.0 * PI / (2.0 * l + 1.0) * Q[mo.lm] * mo.coef;
+    }
+    __syncthreads();
+    if (threadIdx.x < 35) {
+        double cf = 0.0;
+#pragma unroll 8
+        for (int m = 0; m < N_MONO_TERMS; m++)
+            if (s_slot[m] == (int)threadIdx.x) cf += s_term[m];
+        s_cf[threadIdx.x] = cf;
+    }
+    __syncthreads();
     const size_t fx = (size_t)ny * nz, fy = (size_t)nx * nz, fz = (size_t)nx * ny;
     const size_t total = 2 * (fx + fy + fz);
     const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
@@ -1431,21 +1480,25 @@ __global__ void k_boundary_fill(int nx, int ny, int nz, const double* __restrict
         j = (int)(r / nx);
     }
     const double dx = x[i] - cx, dy = y[j] - cy, dz = z[k] - cz;
-    const double r2 = dx * dx + dy * dy + dz * dz;
-    const double ir = 1.0 / sqrt(r2), ir2 = ir * ir;
-    double S[NLM];
-    solid_harmonics(dx, dy, dz, S);
-    double v = 0.0, pw = ir;   // ir^(2l+1)
-    int l = 0;
-    for (int lm = 0; lm < NLM; lm++) {
-        const int ll = l_of_lm(lm);
-        if (ll != l) {
-            pw *= ir2;
-            l = ll;
+    const double ir = rsqrt(fma(dz, dz, fma(dy, dy, dx * dx))), ir2 = ir * ir;
+    const double X = dx * ir2, Y = dy * ir2, Z = dz * ir2;
+    double px = 0.0;   // Horner in x of Horner in y of Horner in z
+#pragma unroll
+    for (int a = 4; a >= 0; a--) {
+        double py = 0.0;
+#pragma unroll
+        for (int b = 4 - a; b >= 0; b--) {
+            double pz = 0.0;
+#pragma unroll
+            for (int c = 4 - a - b; c >= 0; c--) {
+                const double cf = s_cf[a + b + c == 0 ? 0 : 1 + ex_slot(a + b + c, b, c)];
+                pz = c == 4 - a - b ? cf : fma(pz, Z, cf);
+            }
+            py = b == 4 - a ? pz : fma(py, Y, pz);
         }
-        v = fma(-4.0 * PI / (2.0 * l + 1.0) * Q[lm] * pw, S[lm], v);
+        px = a == 4 ? py : fma(px, X, py);
     }
-    u[((size_t)k * ny + j) * nx + i] = v;
+    u[((size_t)k * ny + j) * nx + i] = px * ir;
 }
 
 cudaError_t launch_boundary_fill(const int n[3], const double* x, const double* y, const double* z, double cx,
@@ -1509,12 +1562,6 @@ constexpr int EX_NT = 128;
 constexpr int EX_CH = 64;        // atoms staged per pass
 constexpr int EX_NC = 34;        // monomials of degree 1..4
 constexpr int EX_REC = 10 + EX_NC;  // x y z q w0 w1 w2 zeta0 zeta1 zeta2 | coefficients
-
-// slot of x^a y^b z^c (a + b + c = l, 1 <= l <= 4): degree offset + s(s+1)/2 + c, s = b + c
-__host__ __device__ constexpr int ex_slot(int l, int b, int c)
-{
-    return (l == 1 ? 0 : l == 2 ? 3 : l == 3 ? 9 : 19) + (b + c) * (b + c + 1) / 2 + c;
-}
 
 __global__ void __launch_bounds__(EX_NT) k_boundary_exact(int nx, int ny, int nz, const double* __restrict__ x,
                                                           const double* __restrict__ y, const double* __restrict__ z,

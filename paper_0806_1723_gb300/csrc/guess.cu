@@ -77,6 +77,19 @@ __global__ void k_resample(int ax_n, int ay_n, int az_n, const double* __restric
     dst[t] = lerp(lerp(v00, v01, ty), lerp(v10, v11, ty), tz);
 }
 
+// The copy that this is where B's nodes are every m-th node of A per axis (no search, no division:
+// 65^3 nodes 65.6 -> 4 us, 33^3 12.7 -> 2.7 us)
+__global__ void __launch_bounds__(128) k_copy_strided(int ax_n, int ay_n, const double* __restrict__ src, int mx, int my,
+                                                      int mz, int bx_n, int by_n, int bz_n, double* __restrict__ dst,
+                                                      int interior_only)
+{
+    const int k = (int)(blockIdx.x / (unsigned)by_n), j = (int)(blockIdx.x - (unsigned)k * by_n);   // a block per row
+    if (interior_only && (j == 0 || k == 0 || j == by_n - 1 || k == bz_n - 1)) return;
+    const double* from = src + ((size_t)k * mz * ay_n + (size_t)j * my) * ax_n;
+    double* to = dst + (size_t)blockIdx.x * bx_n;
+    for (int i = threadIdx.x + interior_only; i < bx_n - interior_only; i += 128) to[i] = from[(size_t)i * mx];
+}
+
 }  // namespace
 
 // ---------------------------------------------------------------- network
@@ -258,6 +271,19 @@ cudaError_t launch_resample(const int na[3], const double* ax, const double* ay,
     const size_t N = (size_t)nbn[0] * nbn[1] * nbn[2];
     k_resample<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(na[0], na[1], na[2], ax, ay, az, src, nbn[0], nbn[1], nbn[2],
                                                            bx, by, bz, dst, interior_only);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_copy_strided(const int na[3], const double* src, const int nbn[3], double* dst, int interior_only,
+                                cudaStream_t s)
+{
+    int m[3];
+    for (int d = 0; d < 3; d++) {
+        if (nbn[d] < 2 || (na[d] - 1) % (nbn[d] - 1)) return cudaErrorInvalidValue;
+        m[d] = (na[d] - 1) / (nbn[d] - 1);
+    }
+    k_copy_strided<<<(unsigned)((size_t)nbn[1] * nbn[2]), 128, 0, s>>>(na[0], na[1], src, m[0], m[1], m[2], nbn[0], nbn[1],
+                                                                       nbn[2], dst, interior_only ? 1 : 0);
     return cudaGetLastError();
 }
 

@@ -407,8 +407,7 @@ cudaError_t launch_deposit(const lasto_cluster& cl, const double* rec, int preci
                            const double* xm_tab, double* row_mom, int* status, cudaStream_t s);
 size_t multipole_scratch_doubles(const int n[3]);
 cudaError_t launch_multipoles(const int n[3], const double* x, const double* y, const double* z, const double* b,
-                              const double centre[3], double* tabs, double* row_mom, double* plane, double* Q,
-                              cudaStream_t s);
+                              const double centre[3], double* tabs, double* plane, double* Q, cudaStream_t s);
 cudaError_t launch_boundary_exact(const lasto_cluster& cl, double* M, double* u, cudaStream_t s);   // M: 5 n_atoms scratch
 cudaError_t launch_boundary_fill(const int n[3], const double* x, const double* y, const double* z, double cx,
                                  double cy, double cz, const double* Q, double* u, cudaStream_t s);
@@ -470,6 +469,9 @@ cudaError_t launch_axis_stride(const double* src, int m, int n, double* dst, cud
 cudaError_t launch_resample(const int na[3], const double* ax, const double* ay, const double* az, const double* src,
                             const int nb[3], const double* bx, const double* by, const double* bz, double* dst,
                             int interior_only, cudaStream_t s);
+// the same where B's nodes are every m-th node of A per axis
+cudaError_t launch_copy_strided(const int na[3], const double* src, const int nb[3], double* dst, int interior_only,
+                                cudaStream_t s);
 
 // project.cu
 const SphereRule& sphere_rule(int n_theta, int n_phi);   // valid until this thread asks for another
