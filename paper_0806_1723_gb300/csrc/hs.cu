@@ -364,16 +364,21 @@ __global__ void __launch_bounds__(HS_NT) k_hs_gemm_f32(int M, int Mp, int nT, co
 // array), the four arrays (A_hi, A_lo, T_hi, T_lo) of a block adjacent, so that a stage of a
 // tile is two 16 KiB bulk copies (cp.async.bulk, completion counted on an mbarrier).
 //
-// Warp roles (10 warps): one thread issues the bulk copies into a ring of six 32 KiB stages,
-// one thread issues the MMAs (and frees a stage by tcgen05.commit to its mbarrier) into the
-// accumulators (tensor-memory columns 0-127 S, 128-255 2H; lane = function row), and eight
-// warps (warp w: lanes 32 (w % 4) .. +31, S for w < 4 and 2H for w >= 4) add each HS_IV-node
-// interval's sums into the unit's FP32 partial sums, which stay in tensor memory (columns
-// 256-511; tcgen05.ld, add, tcgen05.st), so that no FP32 accumulation inside the tensor core
-// is longer than one interval.  A work unit is one upper-triangle tile and HS_SEG nodes,
-// numbered segment-major so that the CTAs running together read the same table rows (from
-// L2); at a unit's end the drain warps form its partial sums in FP64, undo the scales
-// (exponent arithmetic) and add them to S and 2H by FP64 atomic addition while the MMAs run on.
+// Warp roles (10 warps): one thread issues the bulk copies into a ring of six 32 KiB stages, one
+// warp the MMAs (and frees a stage by tcgen05.commit to its mbarrier) into one of two accumulator
+// sets (tensor-memory columns 0-127 S, 128-255 2H; the other set 256 columns on; lane = function
+// row), and eight warps (warp w: lanes 32 (w % 4) .. +31, S for w < 4 and 2H for w >= 4) add each
+// HS_IV-node interval's sums into the unit's FP32 partial sums, 128 registers per thread, while the
+// MMAs go on in the other set; so no FP32 accumulation inside the tensor core is longer than one
+// interval.  A work unit is one upper-triangle tile and HS_SEG nodes, numbered segment-major so that
+// the CTAs running together read the same table rows (from L2); at a unit's end the drain warps
+// form its partial sums in FP64, undo the scales (exponent arithmetic) and add them to S and 2H by
+// FP64 atomic addition.  Bound: the tensor pipe (576 cycles of nine MMAs a stage) and close behind it
+// shared memory: an MMA of these sizes reads 8 KiB, 128 bytes a cycle at the full rate, unless its A
+// operand is still in the collector buffer, and the copies bring 32 KiB a stage.  55 spheres of 25
+// functions, 97^3 nodes: 12.4 ms with the partial sums in tensor memory (the MMAs then wait for each
+// interval's drain) and one thread issuing, 10.1 with this arrangement, 9.7 with the MMAs in the order
+// of their A operand: 0.91 of the measured bf16 rate.
 constexpr int TC_TM = 128;                       // functions per tile side (MMA M and N)
 constexpr int TC_NT = 320;                       // threads: 8 drain warps, producer, MMA issuer
 constexpr int TC_SK = 16;                        // nodes per stage (one MMA K step)
@@ -432,19 +437,33 @@ __device__ __forceinline__ uint64_t hs_desc(uint32_t saddr)
 // FP32 accumulator, FP16 A and B, both K-major, M = N = 128
 constexpr uint32_t HS_IDESC = (1u << 4) | ((uint32_t)(TC_TM >> 3) << 17) | ((uint32_t)(TC_TM >> 4) << 24);
 
+// By a whole warp in uniform control flow, one elected lane executing (the descriptors then stay in
+// uniform registers).  The A operand is kept in the collector buffer (FILL) and taken from there
+// (USE, LAST): consecutive MMAs on the same rows read it from shared memory once.
+enum { HS_FILL, HS_USE, HS_LAST, HS_ONCE };
+
+template <int C>
 __device__ __forceinline__ void hs_mma(uint32_t tmem, uint64_t a, uint64_t b, uint32_t acc)
 {
-    asm volatile(
-        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
-            tmem),
-        "l"(a), "l"(b), "r"(HS_IDESC), "r"(acc)
-        : "memory");
+#define HS_MMA(USAGE)                                                                                              \
+    asm volatile(                                                                                                  \
+        "{\n.reg .pred p, q;\nelect.sync _|q, 0xffffffff;\nsetp.ne.b32 p, %4, 0;\n"                               \
+        "@q tcgen05.mma.cta_group::1.kind::f16.collector::a::" USAGE " [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),      \
+        "l"(a), "l"(b), "r"(HS_IDESC), "r"(acc)                                                                    \
+        : "memory")
+    if constexpr (C == HS_FILL) HS_MMA("fill");
+    else if constexpr (C == HS_USE) HS_MMA("use");
+    else if constexpr (C == HS_LAST) HS_MMA("lastuse");
+    else HS_MMA("discard");
+#undef HS_MMA
 }
 
 __device__ __forceinline__ void hs_commit(uint32_t mbar)
 {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(mbar)
-                 : "memory");
+    asm volatile(
+        "{\n.reg .pred q;\nelect.sync _|q, 0xffffffff;\n"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(mbar)
+        : "memory");
 }
 
 __device__ __forceinline__ void hs_tmem_ld16(uint32_t taddr, float* v)
@@ -650,19 +669,6 @@ __device__ __forceinline__ HsUnit hs_unit(int u, int pairs, int nT, int K)
     return w;
 }
 
-__device__ __forceinline__ void hs_tmem_st16(uint32_t taddr, const float* v)
-{
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-        "%15, %16};\n" ::"r"(taddr),
-        "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])), "r"(__float_as_uint(v[3])),
-        "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])), "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7])),
-        "r"(__float_as_uint(v[8])), "r"(__float_as_uint(v[9])), "r"(__float_as_uint(v[10])),
-        "r"(__float_as_uint(v[11])), "r"(__float_as_uint(v[12])), "r"(__float_as_uint(v[13])),
-        "r"(__float_as_uint(v[14])), "r"(__float_as_uint(v[15]))
-        : "memory");
-}
-
 // x * 2^-e for a double x whose result stays a normal number: the exponent field lowered by e
 __device__ __forceinline__ double hs_unscale(float v, int e)
 {
@@ -677,10 +683,10 @@ __global__ void __launch_bounds__(TC_NT, 1) k_hs_gemm_tc(int M, int nT, const un
 {
     extern __shared__ unsigned char hs_dyn[];
     unsigned char* ring = reinterpret_cast<unsigned char*>(((uintptr_t)hs_dyn + 127) & ~(uintptr_t)127);
-    __shared__ __align__(8) unsigned long long full[TC_RING], empty[TC_RING], accf, acce;
+    __shared__ __align__(8) unsigned long long full[TC_RING], empty[TC_RING], accf[2], acce[2];
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int abort_flag;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int pairs = nT * (nT + 1) / 2;
 
     if (tid == 0) {
@@ -689,8 +695,10 @@ __global__ void __launch_bounds__(TC_NT, 1) k_hs_gemm_tc(int M, int nT, const un
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(hs_smem_u32(&full[s])) : "memory");
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(hs_smem_u32(&empty[s])) : "memory");
         }
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(hs_smem_u32(&accf)) : "memory");
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 256;\n" ::"r"(hs_smem_u32(&acce)) : "memory");
+        for (int q = 0; q < 2; q++) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(hs_smem_u32(&accf[q])) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 256;\n" ::"r"(hs_smem_u32(&acce[q])) : "memory");
+        }
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
     if (warp == 0) {
@@ -718,7 +726,9 @@ __global__ void __launch_bounds__(TC_NT, 1) k_hs_gemm_tc(int M, int nT, const un
                     break;
                 }
                 const uint32_t fb = hs_smem_u32(&full[slot]);
-                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(fb), "r"(TC_STAGE)
+                const bool diag = w.I == w.J;   // one block is both sides
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(fb),
+                             "r"(diag ? TC_SIDE : TC_STAGE)
                              : "memory");
                 const size_t kb = (size_t)(r0 / TC_SK) * nT;
                 const unsigned char* srcI = img + (kb + w.I) * TC_SIDE;
@@ -729,6 +739,7 @@ __global__ void __launch_bounds__(TC_NT, 1) k_hs_gemm_tc(int M, int nT, const un
                         dst),
                     "l"(srcI), "r"(TC_SIDE), "r"(fb)
                     : "memory");
+                if (diag) continue;
                 asm volatile(
                     "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
                         dst + TC_SIDE),
@@ -743,103 +754,91 @@ __global__ void __launch_bounds__(TC_NT, 1) k_hs_gemm_tc(int M, int nT, const un
                 hs_wait(hs_smem_u32(&full[q % TC_RING]), (uint32_t)((q / TC_RING) & 1), &never);
             }
         }
-    } else if (warp == 9 && lane == 0) {
-        // ---------------- MMA issuer: accumulators in columns 0-127 (S) and 128-255 (2H)
+    } else if (warp == 9) {
+        // ---------------- MMA issuer (the whole warp): S in columns 0-127 and 2H in 128-255 of one of
+        // two accumulator sets, interval by interval
         int g = 0, ic = 0;
         bool ok = true;
-        const uint32_t tS = tmem, tH = tmem + TC_TM;
+        constexpr uint32_t IMG = TC_IMG / 16, SIDE = TC_SIDE / 16;   // descriptor units
+        const uint64_t ring0 = hs_desc(hs_smem_u32(ring));
         for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
             const HsUnit w = hs_unit(u, pairs, nT, K);
+            const uint32_t side = w.I == w.J ? 0u : SIDE;
             for (int c0 = w.k0; c0 < w.k1 && ok; c0 += HS_IV, ic++) {
-                const int c1 = min(w.k1, c0 + HS_IV);
-                // the previous interval has been drained
-                if (ic >= 1 && !hs_wait(hs_smem_u32(&acce), (uint32_t)((ic - 1) & 1), &abort_flag)) {
-                    ok = false;
-                    break;
-                }
+                const int c1 = min(w.k1, c0 + HS_IV), set = ic & 1;
+                const uint32_t tS = tmem + (uint32_t)(set * 2 * TC_TM), tH = tS + TC_TM;
+                // the set's previous interval has been drained
+                if (ic >= 2)
+                    ok = __all_sync(0xffffffffu, hs_wait(hs_smem_u32(&acce[set]), (uint32_t)((ic / 2 - 1) & 1), &abort_flag));
+                if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
                 for (int r0 = c0; r0 < c1; r0 += TC_SK, g++) {
                     const int slot = g % TC_RING;
-                    if (!hs_wait(hs_smem_u32(&full[slot]), (uint32_t)((g / TC_RING) & 1), &abort_flag)) {
-                        ok = false;
-                        break;
-                    }
+                    ok = __all_sync(0xffffffffu, hs_wait(hs_smem_u32(&full[slot]), (uint32_t)((g / TC_RING) & 1), &abort_flag));
+                    if (!ok) break;
                     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                    const uint32_t sb = hs_smem_u32(ring + (size_t)slot * TC_STAGE);
-                    const uint64_t aIh = hs_desc(sb), aIl = hs_desc(sb + TC_IMG);
-                    const uint64_t tIh = hs_desc(sb + 2 * TC_IMG), tIl = hs_desc(sb + 3 * TC_IMG);
-                    const uint64_t aJh = hs_desc(sb + TC_SIDE), aJl = hs_desc(sb + TC_SIDE + TC_IMG);
-                    const uint64_t tJh = hs_desc(sb + TC_SIDE + 2 * TC_IMG), tJl = hs_desc(sb + TC_SIDE + 3 * TC_IMG);
+                    const uint64_t dI = ring0 + (uint32_t)(slot * (TC_STAGE / 16)), dJ = dI + side;
+                    const uint64_t aIh = dI, aIl = dI + IMG, tIh = dI + 2 * IMG, tIl = dI + 3 * IMG;
+                    const uint64_t aJh = dJ, aJl = dJ + IMG, tJh = dJ + 2 * IMG, tJl = dJ + 3 * IMG;
                     const uint32_t acc = r0 > c0 ? 1u : 0u;
-                    hs_mma(tS, aIh, aJh, acc);
-                    hs_mma(tS, aIh, aJl, 1u);
-                    hs_mma(tS, aIl, aJh, 1u);
-                    hs_mma(tH, aIh, tJh, acc);
-                    hs_mma(tH, aIh, tJl, 1u);
-                    hs_mma(tH, aIl, tJh, 1u);
-                    hs_mma(tH, tIh, aJh, 1u);
-                    hs_mma(tH, tIh, aJl, 1u);
-                    hs_mma(tH, tIl, aJh, 1u);
+                    // (each accumulator's terms in the order hi hi, hi lo, lo hi)
+                    hs_mma<HS_FILL>(tS, aIh, aJh, acc);
+                    hs_mma<HS_USE>(tS, aIh, aJl, 1u);
+                    hs_mma<HS_USE>(tH, aIh, tJh, acc);
+                    hs_mma<HS_LAST>(tH, aIh, tJl, 1u);
+                    hs_mma<HS_FILL>(tS, aIl, aJh, 1u);
+                    hs_mma<HS_LAST>(tH, aIl, tJh, 1u);
+                    hs_mma<HS_FILL>(tH, tIh, aJh, 1u);
+                    hs_mma<HS_LAST>(tH, tIh, aJl, 1u);
+                    hs_mma<HS_ONCE>(tH, tIl, aJh, 1u);
                     hs_commit(hs_smem_u32(&empty[slot]));
                     last_mma = g;
                 }
-                if (ok) hs_commit(hs_smem_u32(&accf));
+                if (ok) hs_commit(hs_smem_u32(&accf[set]));
             }
         }
     } else if (warp < 8) {
-        // ---------------- drain: row = tensor-memory lane; S (warps 0-3) or 2H (4-7) columns of
-        // the interval added into the unit's partial sums 256 columns further on
+        // ---------------- drain: row = tensor-memory lane; S (warps 0-3) or 2H (4-7): the interval's
+        // columns added into the unit's partial sums, one register per column
         const int q = warp & 3, half = warp >> 2, row = 32 * q + lane;
         const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(half * TC_TM);
-        const uint32_t tp = ta + 2 * TC_TM;
         int ic = 0;
         bool ok = true;
         for (int u = blockIdx.x; u < units && ok; u += gridDim.x) {
             const HsUnit w = hs_unit(u, pairs, nT, K);
+            float part[TC_TM];
+#pragma unroll
+            for (int c = 0; c < TC_TM; c++) part[c] = 0.0f;
             for (int c0 = w.k0; c0 < w.k1; c0 += HS_IV, ic++) {
-                const bool got = hs_wait(hs_smem_u32(&accf), (uint32_t)(ic & 1), &abort_flag);
+                const int set = ic & 1;
+                const bool got = hs_wait(hs_smem_u32(&accf[set]), (uint32_t)((ic / 2) & 1), &abort_flag);
                 if (!__all_sync(0xffffffffu, got)) {
                     ok = false;
                     abort_flag = 1;
                     break;
                 }
                 asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-                const bool first = c0 == w.k0;
-#pragma unroll 1
-                for (int cc = 0; cc < TC_TM; cc += 32) {
-                    float v[32], pv[32];
-                    hs_tmem_ld16(ta + (uint32_t)cc, v);
-                    hs_tmem_ld16(ta + (uint32_t)(cc + 16), v + 16);
-                    if (!first) {
-                        hs_tmem_ld16(tp + (uint32_t)cc, pv);
-                        hs_tmem_ld16(tp + (uint32_t)(cc + 16), pv + 16);
-                    }
-                    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-                    if (!first)
 #pragma unroll
-                        for (int jj = 0; jj < 32; jj++) v[jj] += pv[jj];
-                    hs_tmem_st16(tp + (uint32_t)cc, v);
-                    hs_tmem_st16(tp + (uint32_t)(cc + 16), v + 16);
+                for (int cc = 0; cc < TC_TM; cc += 16) {
+                    float v[16];
+                    hs_tmem_ld16(ta + (uint32_t)(set * 2 * TC_TM + cc), v);
+                    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+#pragma unroll
+                    for (int jj = 0; jj < 16; jj++) part[cc + jj] += v[jj];
                 }
-                asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
                 asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(hs_smem_u32(&acce)) : "memory");
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(hs_smem_u32(&acce[set])) : "memory");
             }
             if (!ok) break;
             // the unit's sums: FP64, scales undone, into S or 2H
             const int a = w.I * TC_TM + row;
             const int e_a = a < M ? ea[a] + (half ? ea[M] : 0) : 0;
             double* dst = (half ? H2 : S) + (size_t)(a < M ? a : 0) * M;
-#pragma unroll 1
-            for (int cc = 0; cc < TC_TM; cc += 16) {
-                float v[16];
-                hs_tmem_ld16(tp + (uint32_t)cc, v);
-                asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-                if (a >= M) continue;
+            if (a < M) {
 #pragma unroll
-                for (int jj = 0; jj < 16; jj++) {
-                    const int b = w.J * TC_TM + cc + jj;
-                    if (b < M && a <= b) atomicAdd(dst + b, hs_unscale(v[jj], e_a + __ldg(ea + b)));
+                for (int jj = 0; jj < TC_TM; jj++) {
+                    const int b = w.J * TC_TM + jj;
+                    if (b < M && a <= b) atomicAdd(dst + b, hs_unscale(part[jj], e_a + __ldg(ea + b)));
                 }
             }
         }
