@@ -191,21 +191,32 @@ __global__ void __launch_bounds__(CT) k_conv_wgrad(Grid g, int cin, const bf16* 
 }
 
 // dbias[co] += sum over nodes of dy[node][co] (FP32 gradient): each block sums a span of node
-// rows with the threads along the row (coalesced), reduces per channel in shared memory and
-// adds its partial with one atomic per channel
-constexpr int BG_ROWS = 128;    // node rows per block
-__global__ void __launch_bounds__(256) k_bias_grad(size_t N, int cout, const float* __restrict__ dy,
+// rows with the threads along the row (coalesced, V channels per thread), reduces per channel in
+// shared memory and adds its partial with one atomic per channel.  Bound: the read of dy (from L2
+// after the pass that wrote it) and, with many blocks, the atomics on the few channels: 16 floats of
+// 288k nodes 12.6 us with one channel per thread and 128 rows per block, 9.4 us with four and 512.
+template <int V>
+__global__ void __launch_bounds__(256) k_bias_grad(size_t N, int cout, int rows, const float* __restrict__ dy,
                                                    float* __restrict__ db)
 {
-    __shared__ float sm[256];
-    const int per = 256 / cout;                      // rows in flight per block step
-    const int t = threadIdx.x, c = t % cout, r0 = t / cout;
-    float acc = 0.0f;
+    __shared__ float sm[256 * V];
+    const int cols = cout / V, per = 256 / cols;     // threads per row, rows in flight per block step
+    const int t = threadIdx.x, c = t % cols, r0 = t / cols;
+    float acc[V] = {};
     if (r0 < per) {
-        const size_t first = (size_t)blockIdx.x * BG_ROWS, last = min(first + BG_ROWS, N);
-        for (size_t n = first + r0; n < last; n += per) acc += dy[n * cout + c];
+        const size_t first = (size_t)blockIdx.x * rows, last = min(first + rows, N);
+#pragma unroll 4
+        for (size_t n = first + r0; n < last; n += per) {
+            if constexpr (V == 4) {
+                const float4 v = *reinterpret_cast<const float4*>(dy + n * cout + 4 * c);
+                acc[0] += v.x, acc[1] += v.y, acc[2] += v.z, acc[3] += v.w;
+            } else {
+                acc[0] += dy[n * cout + c];
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < V; q++) sm[r0 * cout + V * c + q] = acc[q];
     }
-    sm[t] = acc;
     __syncthreads();
     if (t < cout) {
         float s = 0.0f;
@@ -227,14 +238,29 @@ __global__ void k_flip_weights(int cin, int cout, const bf16* __restrict__ w, bf
 }
 
 // ---------------------------------------------------------------- elementwise
-__global__ void k_relu_grad(size_t n, const float* __restrict__ y, const float* __restrict__ dy, float* __restrict__ dx,
-                            bf16* __restrict__ dx16)
+// dx = dy where y > 0, else 0, as FP32 and BF16 (either may be absent; dx may be dy).  Bound: 14 bytes
+// per value.  V values per thread: 4.6M values 24.4 us with one, 11.2 us with four.
+template <int V>
+__global__ void __launch_bounds__(256) k_relu_grad(size_t n, const float* __restrict__ y, const float* dy, float* dx,
+                                                   bf16* __restrict__ dx16)
 {
-    const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+    const size_t t = (blockIdx.x * (size_t)blockDim.x + threadIdx.x) * V;
     if (t >= n) return;
-    const float v = y[t] > 0.0f ? dy[t] : 0.0f;
-    if (dx) dx[t] = v;
-    if (dx16) dx16[t] = __float2bfloat16(v);
+    if constexpr (V == 4) {
+        const float4 a = *reinterpret_cast<const float4*>(y + t), g = *reinterpret_cast<const float4*>(dy + t);
+        const float4 v = make_float4(a.x > 0.0f ? g.x : 0.0f, a.y > 0.0f ? g.y : 0.0f, a.z > 0.0f ? g.z : 0.0f,
+                                     a.w > 0.0f ? g.w : 0.0f);
+        if (dx) *reinterpret_cast<float4*>(dx + t) = v;
+        if (dx16) {
+            const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+            *reinterpret_cast<uint2*>(dx16 + t) =
+                make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+        }
+    } else {
+        const float v = y[t] > 0.0f ? dy[t] : 0.0f;
+        if (dx) dx[t] = v;
+        if (dx16) dx16[t] = __float2bfloat16(v);
+    }
 }
 
 __global__ void k_to_bf16(size_t n, const float* __restrict__ a, bf16* __restrict__ b)
@@ -439,6 +465,15 @@ __global__ void k_guess_grid(size_t N, int nx, int ny, int nz, const float* __re
 
 inline unsigned blocks(size_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
+void launch_bias_grad(size_t N, int cout, const float* dy, float* db, cudaStream_t s)
+{
+    // (four channels per thread where rows are whole 16-byte pieces)
+    if (cout % 4 == 0 && !((uintptr_t)dy & 15u))
+        k_bias_grad<4><<<blocks(N, 512), 256, 0, s>>>(N, cout, 512, dy, db);
+    else
+        k_bias_grad<1><<<blocks(N, 128), 256, 0, s>>>(N, cout, 128, dy, db);
+}
+
 }  // namespace nn
 }  // namespace lasto
 
@@ -537,7 +572,7 @@ int lasto_nn_conv3d_wgrad(int nb, const int dims[3], int cin, int cout, const vo
         case 64: k_conv_wgrad<64><<<grid, CT, 0, s>>>(g, cin, X, DY, dw); break;
         default: return LASTO_ERR_INVALID_ARG;
     }
-    if (db && dy32) k_bias_grad<<<blocks(g.nodes(), BG_ROWS), 256, 0, s>>>(g.nodes(), cout, dy32, db);
+    if (db && dy32) launch_bias_grad(g.nodes(), cout, dy32, db, s);
     return cudaGetLastError() == cudaSuccess ? LASTO_OK : LASTO_ERR_CUDA;
 }
 
@@ -563,14 +598,18 @@ int lasto_nn_conv3d_wgrad_tc(int nb, const int dims[3], int cin, int cout, const
     if (st) return st;
     if (db && dy32) {
         Grid g{nb, dims[2], dims[1], dims[0]};
-        k_bias_grad<<<blocks(g.nodes(), BG_ROWS), 256, 0, (cudaStream_t)stream>>>(g.nodes(), cout, dy32, db);
+        launch_bias_grad(g.nodes(), cout, dy32, db, (cudaStream_t)stream);
     }
     return cudaGetLastError() == cudaSuccess ? LASTO_OK : LASTO_ERR_CUDA;
 }
 
 int lasto_nn_relu_grad(size_t n, const float* y, const float* dy, float* dx, void* dx16, void* stream)
 {
-    k_relu_grad<<<blocks(n, 256), 256, 0, (cudaStream_t)stream>>>(n, y, dy, dx, (bf16*)dx16);
+    // (four values per thread where every array is in whole 16-byte pieces, the BF16 one in 8-byte ones)
+    if (n % 4 == 0 && !(((uintptr_t)y | (uintptr_t)dy | (uintptr_t)dx) & 15u) && !((uintptr_t)dx16 & 7u))
+        k_relu_grad<4><<<blocks(n / 4, 256), 256, 0, (cudaStream_t)stream>>>(n, y, dy, dx, (bf16*)dx16);
+    else
+        k_relu_grad<1><<<blocks(n, 256), 256, 0, (cudaStream_t)stream>>>(n, y, dy, dx, (bf16*)dx16);
     return cudaGetLastError() == cudaSuccess ? LASTO_OK : LASTO_ERR_CUDA;
 }
 

@@ -79,3 +79,41 @@ def test_weight_gradient(cin, cout, nb, dims):
         assert int(err.item()) == 0
         got = dw.double().cpu().numpy().reshape(27, cin, cout)
         assert np.abs(got - rdw).max() <= 2e-5 * np.abs(rdw).max()
+
+
+@pytest.mark.parametrize("n,shift", [(4096, 0), (4099, 0), (1024, 1), (8, 0), (1, 0)])
+def test_relu_gradient(n, shift):
+    import torch
+    B = need_gpu()
+    L = B.load()
+    g = torch.Generator(device="cuda").manual_seed(n)
+    y = torch.randn(n + 4, generator=g, device="cuda")[shift:shift + n]
+    y[0], y[-1] = 0.0, float("nan")
+    for inplace in (False, True):
+        dy = torch.randn(n + 4, generator=g, device="cuda")[shift:shift + n]
+        dx = dy if inplace else torch.empty_like(dy)
+        dx16 = torch.empty(n, dtype=torch.bfloat16, device="cuda")
+        ref = torch.where(y > 0, dy, torch.zeros_like(dy))
+        assert L.lasto_nn_relu_grad(n, B._ptr(y), B._ptr(dy), B._ptr(dx), B._ptr(dx16), B._stream()) == 0
+        assert torch.equal(dx, ref) and torch.equal(dx16, ref.to(torch.bfloat16))
+
+
+@pytest.mark.parametrize("cout,nb,dims,shift", [(16, 2, (33, 9, 11), 0), (16, 1, (5, 3, 2), 0), (48, 1, (13, 7, 9), 1),
+                                                (128, 1, (17, 5, 7), 0), (96, 3, (9, 9, 9), 0)])
+def test_bias_gradient(cout, nb, dims, shift):
+    import torch
+    B = need_gpu()
+    L = B.load()
+    W, H, D = dims
+    N = nb * D * H * W
+    g = torch.Generator(device="cuda").manual_seed(N)
+    dy = torch.randn(N * cout + 4, generator=g, device="cuda")[shift:shift + N * cout].view(N, cout)
+    x, dy16 = torch.zeros(N, 16, dtype=torch.bfloat16, device="cuda"), dy.to(torch.bfloat16)
+    dw, db = torch.zeros(27 * 16 * cout, device="cuda"), torch.ones(cout, device="cuda")
+    err = torch.zeros(1, dtype=torch.int32, device="cuda")
+    assert L.lasto_nn_conv3d_wgrad_tc(nb, (ctypes.c_int * 3)(*dims), 16, cout, B._ptr(x), B._ptr(dy16), B._ptr(dy),
+                                      B._ptr(dw), B._ptr(db), B._ptr(err), B._stream()) == 0
+    ref = 1.0 + dy.double().sum(0)
+    # FP32 sums: at most 64 terms per thread, 256 threads and N / 512 + 1 blocks one after another
+    tol = (64 + 256 + N / 128 + 2) * 2.0 ** -24 * (1.0 + dy.double().abs().sum(0))
+    assert bool(((db.double() - ref).abs() <= tol).all())
