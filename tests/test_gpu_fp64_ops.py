@@ -45,3 +45,28 @@ def test_residual(orc, n):
     h = min(np.diff(a).min() for a in (x, y, z))
     assert np.abs(r - ref).max() <= 2 * 12 * EPS * 12.0 / (h * h) * np.abs(u).max()
     assert (r[0] == 0).all() and (r[:, -1] == 0).all() and (r[:, :, 0] == 0).all()
+
+
+@pytest.mark.parametrize("n,scale", [((5, 5, 5), 1.0), ((65, 9, 11), 1e-3), ((33, 37, 29), 1e4), ((5, 9, 5), 1e-153),
+                                     ((5, 9, 5), 1e152)])
+def test_inverse_diagonal(n, scale):
+    """One red half sweep from zero with b = 1 returns the negated reciprocal of the diagonal."""
+    import torch
+    B = need_gpu()
+    x, y, z = [a * scale for a in _grid(n, 5)]
+    u = torch.zeros(n[::-1], dtype=torch.float64, device="cuda")
+    b = torch.ones(n[::-1], dtype=torch.float64, device="cuda")
+    B.lasto_op_smooth(dev(x), dev(y), dev(z), u, b, 1)
+    got = host(u)
+
+    def dg(a):
+        h = np.diff(a).astype(np.longdouble)
+        s = h[:-1] + h[1:]
+        return 2 / (s * h[:-1]) + 2 / (s * h[1:])
+
+    d = dg(z)[:, None, None] + dg(y)[None, :, None] + dg(x)[None, None, :]
+    k, j, i = np.indices(d.shape) + 1
+    red = (i + j + k) % 2 == 0
+    ref = -1 / d
+    # the diagonal's own six terms carry up to 4 roundings each and two additions, the reciprocal one
+    assert (np.abs(got[1:-1, 1:-1, 1:-1] - ref)[red] <= 8 * 2 * EPS * np.abs(ref)[red]).all()
