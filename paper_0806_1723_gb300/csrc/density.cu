@@ -206,7 +206,6 @@ constexpr int SPH_NT = 128;
 // before): 55 spheres 47.8 -> 22.6 us, 147 spheres 54.3 -> 29.0 us.
 __global__ void __launch_bounds__(SPH_NT) k_sphere_params(SphArgs a)
 {
-    __shared__ double sm[32];
     __shared__ double red[6], own[3][3];
     __shared__ int bad_geom, bad_zeta;
     const int i = blockIdx.x, tid = threadIdx.x;
@@ -242,7 +241,7 @@ __global__ void __launch_bounds__(SPH_NT) k_sphere_params(SphArgs a)
         }
     }
     for (int v = 0; v < 6; v++) {
-        const double s = block_sum<SPH_NT>(acc[v], sm);
+        const double s = block_sum<SPH_NT>(acc[v]);
         if (tid == 0) red[v] = s;
     }
     __syncthreads();

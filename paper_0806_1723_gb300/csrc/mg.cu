@@ -1404,21 +1404,21 @@ __device__ void fin_apply(Ctl& c, double s, int op, cudaGraphConditionalHandle c
 }
 
 // Block partial -> last block sums the partials in order and applies the scalar step.
-__device__ void reduce_finish(double block_total, const Red& r, double* sm)
+__device__ void reduce_finish(double block_total, const Red& r)
 {
     __shared__ int is_last;
     if (threadIdx.x == 0) {
+        // the ticket releases this block's partial sum and acquires the others'
         r.part[blockIdx.x] = block_total;
-        __threadfence();
-        const unsigned prev = atomicAdd(r.counter, 1u);
+        unsigned prev;
+        asm volatile("atom.add.acq_rel.gpu.u32 %0, [%1], 1;\n" : "=r"(prev) : "l"(r.counter) : "memory");
         is_last = (prev == gridDim.x - 1);
     }
     __syncthreads();
     if (!is_last) return;
-    __threadfence();
     double acc = 0.0;
     for (unsigned t = threadIdx.x; t < gridDim.x; t += NT) acc += __ldcg(r.part + t);
-    const double s = block_sum<NT>(acc, sm);
+    const double s = block_sum<NT>(acc);
     if (threadIdx.x == 0) {
         *r.counter = 0u;
         fin_apply(*r.ctl, s, r.op, r.cond, r.use_cond);
@@ -1461,7 +1461,6 @@ __device__ __noinline__ double bnorm_face_adjust(const LevelT<double>& L, const 
 __global__ void __launch_bounds__(NT, VEC_MIN_BLOCKS) k_bnorm(LevelT<double> L, const double* __restrict__ u,
                                                              const double* __restrict__ b, Red red)
 {
-    __shared__ double sm[32];
     double acc = 0.0;
     const size_t N = L.N();
     GRID_STRIDE_U(P0, N)
@@ -1488,7 +1487,7 @@ __global__ void __launch_bounds__(NT, VEC_MIN_BLOCKS) k_bnorm(LevelT<double> L, 
         for (int q = 0; q < VU; q++)
             if (on[q]) acc = fma(v[q], v[q], acc);
     }
-    reduce_finish(block_sum<NT>(acc, sm), red, sm);
+    reduce_finish(block_sum<NT>(acc), red);
 }
 
 // r = b - A u (written when r != nullptr, FP32 copy when r32 != nullptr, in colour-split
@@ -1501,7 +1500,6 @@ constexpr int RN_V = 4;
 
 __device__ __forceinline__ void k_resid_norm_body(LevelT<double> L, const double* __restrict__ u, const double* __restrict__ b, double* __restrict__ r, float* __restrict__ r32, unsigned h32, Red red)
 {
-    __shared__ double sm[32];
     double acc = 0.0;
     const int nx = L.nx, rows = L.ny * L.nz;
     const int lane = threadIdx.x & 31;
@@ -1539,7 +1537,7 @@ __device__ __forceinline__ void k_resid_norm_body(LevelT<double> L, const double
             }
         }
     }
-    reduce_finish(block_sum<NT>(acc, sm), red, sm);
+    reduce_finish(block_sum<NT>(acc), red);
 }
 
 // rows kernels' grid: one warp per row while the partials allow (one per ceil(N / 256) nodes)
@@ -1555,12 +1553,10 @@ __global__ void __launch_bounds__(NT) k_resid_norm(LevelT<double> L, const doubl
 }
 
 // q = A p and <p, q>_vol: rows as in k_resid_norm, the row's part of the volume applied to the row's
-// sum.  10 FP64 operations per node instead of 13: 129^3 58.9 -> 49.7 us (53.1 with a
-// warp per row: the last block waits for every block's ticket).
+// sum.  10 FP64 operations per node instead of 13: 129^3 58.9 -> 48.5 us.
 __global__ void __launch_bounds__(NT) k_apply_dot(LevelT<double> L, const double* __restrict__ p,
                                                  double* __restrict__ q, Red red)
 {
-    __shared__ double sm[32];
     double acc = 0.0;
     const int nx = L.nx, rows = L.ny * L.nz, lane = threadIdx.x & 31;
     const size_t sz = (size_t)nx * L.ny;
@@ -1596,36 +1592,53 @@ __global__ void __launch_bounds__(NT) k_apply_dot(LevelT<double> L, const double
         }
         if (!frow) acc = fma(L.ax[1].dual[j] * L.ax[2].dual[k], racc, acc);
     }
-    reduce_finish(block_sum<NT>(acc, sm), red, sm);
+    reduce_finish(block_sum<NT>(acc), red);
 }
 
-// u += alpha p; r -= alpha q; ||r||^2
-__global__ void __launch_bounds__(NT) k_update_ur(LevelT<double> L, const Ctl* __restrict__ ctl,
-                                                 const double* __restrict__ p, const double* __restrict__ q,
-                                                 double* __restrict__ u, double* __restrict__ r, Red red)
+// u += alpha p; r -= alpha q; ||r||^2 (VU nodes per thread and step, loads first).  Bound: 48 bytes
+// per node from L2.  129^3 23.4 -> 19.9 us, 65^3 11.9 -> 8.4 us.
+__global__ void __launch_bounds__(NT, VEC_MIN_BLOCKS) k_update_ur(LevelT<double> L, const Ctl* __restrict__ ctl,
+                                                                 const double* __restrict__ p,
+                                                                 const double* __restrict__ q, double* __restrict__ u,
+                                                                 double* __restrict__ r, Red red)
 {
-    __shared__ double sm[32];
     const double alpha = ctl->alpha;
     double acc = 0.0;
-    GRID_STRIDE(P, L.N())
+    const size_t N = L.N();
+    GRID_STRIDE_U(P0, N)
     {
-        int i, j, k;
-        node_ijk(P, L, i, j, k);
-        if (is_face(L, i, j, k)) continue;
-        u[P] = fma(alpha, p[P], u[P]);
-        const double rv = fma(-alpha, q[P], r[P]);
-        r[P] = rv;
-        acc = fma(rv, rv, acc);
+        double pv[VU], qv[VU], uv[VU], rv[VU];
+        bool on[VU];
+#pragma unroll
+        for (int t = 0; t < VU; t++) {
+            const size_t P = P0 + (size_t)t * NT;
+            on[t] = false;
+            if (P < N) {
+                int i, j, k;
+                node_ijk(P, L, i, j, k);
+                on[t] = !is_face(L, i, j, k);
+            }
+            if (on[t]) pv[t] = p[P], qv[t] = q[P], uv[t] = u[P], rv[t] = r[P];
+        }
+#pragma unroll
+        for (int t = 0; t < VU; t++) {
+            if (!on[t]) continue;
+            const size_t P = P0 + (size_t)t * NT;
+            u[P] = fma(alpha, pv[t], uv[t]);
+            const double v = fma(-alpha, qv[t], rv[t]);
+            r[P] = v;
+            acc = fma(v, v, acc);
+        }
     }
-    reduce_finish(block_sum<NT>(acc, sm), red, sm);
+    reduce_finish(block_sum<NT>(acc), red);
 }
 
 // <r, z>_vol over the interior rows, as above: 2 FP64 operations per node instead of 4 (129^3:
-// 26.7 -> 17.7 us; 23.0 with a warp per row)
+// 26.7 -> 16.4 us; 18.3 with a block per eight rows: every block ends with a
+// ticket)
 __global__ void __launch_bounds__(NT) k_dot_rz(LevelT<double> L, const double* __restrict__ r,
                                               const double* __restrict__ z, Red red)
 {
-    __shared__ double sm[32];
     double acc = 0.0;
     const int nx = L.nx, my = L.ny - 2, rows = my * (L.nz - 2), lane = threadIdx.x & 31;
     for (int row = (int)(blockIdx.x * (NT / 32) + (threadIdx.x >> 5)); row < rows; row += (int)(gridDim.x * (NT / 32))) {
@@ -1646,7 +1659,7 @@ __global__ void __launch_bounds__(NT) k_dot_rz(LevelT<double> L, const double* _
         }
         acc = fma(L.ax[1].dual[j] * L.ax[2].dual[k], racc, acc);
     }
-    reduce_finish(block_sum<NT>(acc, sm), red, sm);
+    reduce_finish(block_sum<NT>(acc), red);
 }
 
 __global__ void __launch_bounds__(NT) k_update_p(LevelT<double> L, const Ctl* __restrict__ ctl,
@@ -1710,7 +1723,7 @@ __device__ __forceinline__ void k_apply_dot32_body(LevelT<float> L, const float*
             q[Q[u]] = v;
         }
     }
-    reduce_finish(block_sum_f32(acc, sm), red, sm);
+    reduce_finish(block_sum_f32(acc, sm), red);
 }
 
 template <int LS>
@@ -1799,7 +1812,7 @@ __device__ __forceinline__ void k_apply_dot32_rows_body(LevelT<float> L, const f
             }
         }
     }
-    reduce_finish(block_sum_f32(acc, sm), red, sm);
+    reduce_finish(block_sum_f32(acc, sm), red);
 }
 
 template <int LS, int V>
@@ -1971,7 +1984,7 @@ __device__ __forceinline__ void k_apply_stage_body(const LevelT<float>& L, const
         }
     }
     // every block takes part in the reduction (a timed-out one with its partial sum so far)
-    reduce_finish(block_sum_f32(acc, sm), red, sm);
+    reduce_finish(block_sum_f32(acc, sm), red);
 }
 
 template <int V, int LS>
@@ -2021,7 +2034,7 @@ __device__ __forceinline__ void k_update_er32_body(LevelT<float> L, const Ctl* _
             acc = fmaf(rn, rn, acc);
         }
     }
-    reduce_finish(block_sum_f32(acc, sm), red, sm);
+    reduce_finish(block_sum_f32(acc, sm), red);
 }
 
 template <int LS>
@@ -2030,46 +2043,41 @@ __global__ void __launch_bounds__(NT, VEC_MIN_BLOCKS) k_update_er32(LevelT<float
     k_update_er32_body<LS>(L, ctl, p, q, e, r, red);
 }
 
-// <r, z>_vol, or ||r||^2 when z == nullptr (VU_DOT nodes per thread and step, twice the update
-// kernels': with two streams and no stores it needs more nodes in flight; measured on the warm
-// Pd561 385^3 solve, 0.2 ms less over its 16 dots)
-constexpr int VU_DOT = 8;
-#define GRID_STRIDE_UD(P0, N) \
-    for (size_t P0 = blockIdx.x * (size_t)(NT * VU_DOT) + threadIdx.x; P0 < (N); P0 += (size_t)gridDim.x * (NT * VU_DOT))
+// <r, z>_vol, or ||r||^2 when z == nullptr: one warp per interior row (grid-stride over rows), DOT_V
+// nodes per lane and step with their loads first, the row's part of the volume applied to its sum.
+// Bound: at 385^3 the two reads; the node-by-node form spent 45 instructions a node (index, face test,
+// three table entries) where this takes about 10.  385^3 116 -> 80 us, 129^3 10.1 -> 9.7 us (about
+// 4.5 of it the reduction's end).
+constexpr int DOT_V = 8;
+
 template <int LS>
 __device__ __forceinline__ void k_dot32_body(LevelT<float> L, const float* __restrict__ r, const float* __restrict__ z, Red red)
 {
     __shared__ double sm[32];
     float acc = 0.0f;
-    const size_t N = L.N();
-    GRID_STRIDE_UD(P0, N)
-    {
-        float rv[VU_DOT], zv[VU_DOT], w[VU_DOT];
-        bool on[VU_DOT];
+    const int nx = L.nx, my = L.ny - 2, rows = my * (L.nz - 2), lane = threadIdx.x & 31;
+    for (int row = (int)(blockIdx.x * (NT / 32) + (threadIdx.x >> 5)); row < rows; row += (int)(gridDim.x * (NT / 32))) {
+        const int k = row / my + 1, j = row - (k - 1) * my + 1;
+        const unsigned P0 = ((unsigned)k * (unsigned)L.ny + (unsigned)j) * (unsigned)nx;
+        float racc = 0.0f;
+        for (int m = 0; 64 * m + 1 < nx - 1; m += DOT_V / 2) {
+            float rv[DOT_V], zv[DOT_V], w[DOT_V];
 #pragma unroll
-        for (int u = 0; u < VU_DOT; u++) {
-            const size_t P = P0 + (size_t)u * NT;
-            on[u] = false;
-            rv[u] = zv[u] = w[u] = 0.0f;
-            if (P < N) {
-                int i, j, k;
-                node_ijk(P, L, i, j, k);
-                on[u] = !is_face(L, i, j, k);
-                if (on[u]) {
-                    const unsigned Q = pos<LS>(L, P);
-                    rv[u] = r[Q];
-                    if (z) {
-                        zv[u] = z[Q];
-                        w[u] = vol32(L, i, j, k);
-                    }
-                }
+            for (int s = 0; s < DOT_V; s++) {
+                // (the same nodes in either storage order, so that the sum is bitwise the same)
+                const int i = 1 + lane + 64 * m + 32 * s;
+                const bool in = i < nx - 1;
+                const unsigned Q = pos<LS>(L, P0 + (unsigned)i);
+                rv[s] = in ? r[Q] : 0.0f;
+                zv[s] = in && z ? z[Q] : 0.0f;
+                w[s] = in && z ? L.ax[0].dual[i] : 0.0f;
             }
-        }
 #pragma unroll
-        for (int u = 0; u < VU_DOT; u++)
-            if (on[u]) acc = z ? fmaf(w[u] * rv[u], zv[u], acc) : fmaf(rv[u], rv[u], acc);
+            for (int s = 0; s < DOT_V; s++) racc = z ? fmaf(w[s] * rv[s], zv[s], racc) : fmaf(rv[s], rv[s], racc);
+        }
+        acc = z ? fmaf(L.ax[1].dual[j] * L.ax[2].dual[k], racc, acc) : acc + racc;
     }
-    reduce_finish(block_sum_f32(acc, sm), red, sm);
+    reduce_finish(block_sum_f32(acc, sm), red);
 }
 
 template <int LS>
@@ -2161,7 +2169,7 @@ cudaError_t launch_apply_dot(const LevelT<double>& L, const double* p, double* q
 cudaError_t launch_update_ur(const LevelT<double>& L, const Ctl* ctl, const double* p, const double* q, double* u,
                              double* r, const Red& red, cudaStream_t s)
 {
-    k_update_ur<<<RGRID(L)>>>(L, ctl, p, q, u, r, red);
+    k_update_ur<<<vec_grid(L.N()), NT, 0, s>>>(L, ctl, p, q, u, r, red);
     return cudaGetLastError();
 }
 cudaError_t launch_dot_rz(const LevelT<double>& L, const double* r, const double* z, const Red& red, cudaStream_t s)

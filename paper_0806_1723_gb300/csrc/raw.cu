@@ -39,7 +39,6 @@ constexpr int RSP_NT = 128;
 __global__ void __launch_bounds__(RSP_NT) k_raw_sphere_params(RawArgs a, double* __restrict__ rec,
                                                               int* __restrict__ status)
 {
-    __shared__ double sm[32];
     const int i = blockIdx.x;
     const double Ri = a.R[i], rm = a.r_min;
     const int n = a.n_rad;
@@ -63,7 +62,7 @@ __global__ void __launch_bounds__(RSP_NT) k_raw_sphere_params(RawArgs a, double*
         if (!(cc - Ri >= a.ax[d][2] && cc + Ri <= a.ax[d][a.n[d] - 3])) bad = true;
     }
     if (bad && status) atomicMax(status, (int)LASTO_ERR_GEOMETRY);
-    const double sum = block_sum<RSP_NT>(part, sm);
+    const double sum = block_sum<RSP_NT>(part);
     if (threadIdx.x != 0) return;
     const double s4 = sqrt(4.0 * RAW_PI);
     const double q = s4 * fma(h / 24.0, sum, f[0] * rm * rm * rm / 3.0) - a.Z[i];
