@@ -69,7 +69,7 @@ struct SmoothChoice {
     int fused = 0;
     int nt = 256;
     SlabShape sh{0, 0, 0, 0};
-    float us = 0.0f;   // measured time of one pre-smoothing phase
+    float us = 0.0f;   // measured time of one pre-smoothing phase (finest FP32 level: and its transfers)
 };
 
 template <typename T>
@@ -385,9 +385,13 @@ SmoothChoice smooth_choice(const lasto_poisson* h, const LevelStore& S)
 }
 
 // Time the candidates on this level's own arrays (zeroed; the stream is idle and not being
-// captured) and keep the fastest pre-smoothing phase.
+// captured) and keep the fastest pre-smoothing phase.  Launched one by one a half sweep below
+// 129^3 costs the host's 4 us whatever it does, so the candidates within a third of the best are timed
+// again as a graph, which is how the solve runs them; the finest FP32 level with its residual,
+// restriction and prolongation, which its storage order changes too.  193^3 solve: 9.7 ms by the first
+// times alone (natural storage), 8.9 with these; 161^3 6.14 and 6.02, 129^3 3.41 and 3.29.  C: the next level.
 template <typename T>
-int tune_level(lasto_poisson* h, LevelStore& S, bool finest, cudaStream_t st)
+int tune_level(lasto_poisson* h, LevelStore& S, LevelStore* C, bool finest, cudaStream_t st)
 {
     const std::array<int, 4> key{S.n[0], S.n[1], S.n[2], (int)sizeof(T)};
     if (h->tune.count(key)) return LASTO_OK;
@@ -446,33 +450,67 @@ int tune_level(lasto_poisson* h, LevelStore& S, bool finest, cudaStream_t st)
     cudaEvent_t e0, e1;
     TRY(cudaEventCreate(&e0));
     TRY(cudaEventCreate(&e1));
-    SmoothChoice best;
-    best.us = 1e30f;
-    for (const SmoothChoice& c : cand) {
-        if (!choice_usable(h, c, sizeof(T))) continue;
-        T* cur = u;
-        const LevelT<T>& Vc = c.fused == 3 ? Vs : V;
-        cudaError_t e = smooth<T>(Vc, cur, partner, u, b, h->cfg.nu1, 0, c, nullptr, st);   // warm
+    constexpr int REPS = 3;
+    auto timed = [&](auto&& pass, float* us) {
+        cudaError_t e = pass();   // warm
         if (e == cudaSuccess) e = cudaEventRecord(e0, st);
-        for (int r = 0; r < 3 && e == cudaSuccess; r++)
-            e = smooth<T>(Vc, cur, partner, u, b, h->cfg.nu1, 0, c, nullptr, st);
+        for (int r = 0; r < REPS && e == cudaSuccess; r++) e = pass();
         if (e == cudaSuccess) e = cudaEventRecord(e1, st);
         if (e == cudaSuccess) e = cudaEventSynchronize(e1);
         float ms = 0.0f;
         if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
-        if (e != cudaSuccess) {
-            cudaEventDestroy(e0);
-            cudaEventDestroy(e1);
-            return set_cuda_error(&h->err, e, "smoother tuning");
+        *us = ms * 1000.0f / REPS;
+        return e;
+    };
+    auto phase = [&](const SmoothChoice& c, bool transfers, cudaStream_t q) {
+        T* cur = u;
+        const LevelT<T>& Vc = c.fused == 3 ? Vs : V;
+        cudaError_t e = smooth<T>(Vc, cur, partner, u, b, h->cfg.nu1, 0, c, nullptr, q);
+        if constexpr (sizeof(T) == 4) {
+            if (transfers && e == cudaSuccess) {
+                LevelT<T> VC = Arr<T>::view(*C);
+                e = launch_resid_restrict<T>(Vc, VC, cur, b, Arr<T>::b(*C), Arr<T>::u(*C), h->cfg.nu1 > 0, q,
+                                             c.fused == 3 ? Arr<T>::r(S) : nullptr, nullptr);
+                if (e == cudaSuccess) e = launch_prolong_add<T>(Vc, VC, Arr<T>::u(*C), cur, q, nullptr);
+            }
         }
-        const float us = ms * 1000.0f / 3.0f;
-        if (us < best.us) {
-            best = c;
-            best.us = us;
-        }
+        return e;
+    };
+    auto graphed = [&](const SmoothChoice& c, float* us) {
+        cudaGraph_t g = nullptr;
+        cudaGraphExec_t x = nullptr;
+        cudaError_t e = cudaStreamBeginCapture(h->cs2, cudaStreamCaptureModeThreadLocal);
+        if (e != cudaSuccess) return e;
+        e = phase(c, finest && C, h->cs2);
+        const cudaError_t e2 = cudaStreamEndCapture(h->cs2, &g);
+        if (e == cudaSuccess) e = e2;
+        if (e == cudaSuccess) e = cudaGraphInstantiate(&x, g, 0);
+        if (e == cudaSuccess) e = timed([&] { return cudaGraphLaunch(x, st); }, us);
+        if (x) cudaGraphExecDestroy(x);
+        if (g) cudaGraphDestroy(g);
+        return e;
+    };
+    cudaError_t e = cudaSuccess;
+    float least = 1e30f;
+    for (SmoothChoice& c : cand) {
+        c.us = 1e30f;
+        if (e != cudaSuccess || !choice_usable(h, c, sizeof(T))) continue;
+        e = timed([&] { return phase(c, false, st); }, &c.us);
+        least = std::min(least, c.us);
+    }
+    // colour-split storage costs the CG's vector kernels a little (129^3: phases of 72.2 us over split
+    // and 76.3 over natural storage give the same solve)
+    auto cost = [&](const SmoothChoice& c) { return c.fused == 3 ? 1.055f * c.us : c.us; };
+    SmoothChoice best;
+    best.us = 1e30f;
+    for (SmoothChoice& c : cand) {
+        if (e != cudaSuccess || c.us > 1.34f * least) continue;
+        e = graphed(c, &c.us);
+        if (e == cudaSuccess && cost(c) < cost(best)) best = c;
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
+    if (e != cudaSuccess) return set_cuda_error(&h->err, e, "smoother tuning");
     h->tune[key] = best;
     return LASTO_OK;
 }
@@ -826,7 +864,10 @@ int tune_plans(lasto_poisson* h, const lasto_cluster* cls, int nc, cudaStream_t 
         int st = enqueue_setup(h, P, cls[c], s);   // the level's own coefficients
         if (st) return st;
         for (int l = 0; l <= last && !st; l++)
-            st = f32 ? tune_level<float>(h, P.lv[l], l == 0, s) : tune_level<double>(h, P.lv[l], l == 0, s);
+        {
+            LevelStore* C = l + 1 < P.L ? &P.lv[l + 1] : nullptr;
+            st = f32 ? tune_level<float>(h, P.lv[l], C, l == 0, s) : tune_level<double>(h, P.lv[l], C, l == 0, s);
+        }
         if (st) return st;
     }
     // the finest level's FP32 storage order follows its choice (fixed for every kernel of the
