@@ -521,8 +521,8 @@ def main():
             "clocks": clk.summary(),
             "e2e": e2e,
             "gpu_launches": launches,
-            # the dominant kernel of the Pd561 solve is the deposit (about 39 % of a warm solve,
-            # ahead of the finest level's smoother at about 20 %): instruction-issue bound
+            # the dominant kernel of the Pd561 solve is the deposit (about a quarter of a warm
+            # solve, as is the finest level's smoother): instruction-issue bound
             "roofline": {"kernel": dep["kernel"], "bound": "alu", "achieved": dep.get("issue_ginst_s"),
                          "peak": dep.get("issue_peak_ginst_s"), "unit": "Ginst/s", "frac": dep.get("frac"),
                          "traffic": DEPOSIT_DRAM_BYTES, "ms_per_launch": dep["ms"],
@@ -844,7 +844,8 @@ def next_rows(B, synth, flush, stream, dev):
         "workload": cl.name,
         "inner_sphere_density": {"ms": t_sd, "unit": "Gpair/s",
                                  "achieved": na * n_rad * nq * na / (t_sd / 1e3) / 1e9,
-                                 "work": f"{na} spheres x {n_rad} radii x {nq} quadrature points x {na} atoms"},
+                                 "work": f"{na} spheres x {n_rad} radii x {nq} quadrature points x {na} atoms, the method's own "
+                                         "count (evaluated at 26 Chebyshev radii per sphere)"},
         "inner_solve": {"ms": t_in, "points": na * 25 * n_rad},
         "boundary_exact": {"ms": t_bx, "unit": "Gpair/s", "achieved": faces * na / (t_bx / 1e3) / 1e9,
                            "work": f"{faces} face nodes x {na} atoms"},
@@ -1028,8 +1029,8 @@ def smoother_roofline(B, stream, flush, dev, tuned, probes):
 def fp64_half_sweep(B, cl, axes, flush, stream, dev, peak, probes):
     """The plain form's FP64 red-black half sweep at 385^3, one block per row.  Algorithmic bytes
     per launch: 12 B per node (u read, the colour's b read and u written: 24 B per node per FP64
-    sweep).  FP64 work per updated node: one multiply, five FMAs, a subtraction and the multiply by
-    the stored 1/diagonal = 8 FP64 instructions (13 FLOP), against the FP64 FMA rate the probe
+    sweep).  FP64 work per updated node: six FMAs from b on and the multiply by the
+    stored 1/diagonal = 7 FP64 instructions (13 FLOP), against the FP64 FMA rate the probe
     measured (2 FLOP per FMA instruction)."""
     import torch
     n = cl.n
@@ -1059,7 +1060,7 @@ def fp64_half_sweep(B, cl, axes, flush, stream, dev, peak, probes):
     return {"kernel": "k_rbgs_row<double> (FP64 red-black half sweep, 385^3 graded)", "us_per_launch": t * 1e6,
             "achieved_gbs": bytes_per_launch / t / 1e9, "hbm_frac": bytes_per_launch / t / 1e9 / peak,
             "fp64_tflops": 13 * upd / t / 1e12, "fp64_fma_tflops_measured": fp64_peak,
-            "fp64_issue_frac": 8 * upd / t / (fp64_peak / 2 * 1e12), "bytes_per_launch": bytes_per_launch,
+            "fp64_issue_frac": 7 * upd / t / (fp64_peak / 2 * 1e12), "bytes_per_launch": bytes_per_launch,
             "traffic": DRAM_BYTES_257_F64 * (n / 257.0) ** 3}
 
 
@@ -1102,13 +1103,13 @@ def deposit_rate(B, synth, stream, flush, dev, probes):
 
 
 # One Pd561 385^3 deposit launch (k_deposit_df) under ncu (`bench.py --profile deposit`, second
-# launch): FP32 FLOP from the sass thread-instruction counts (2 per FFMA: 132.4 G, 1 per FADD:
-# 329.4 G and per FMUL: 89.9 G), the warp instructions issued (smsp__inst_executed.sum) and the
-# DRAM bytes (read 14.6 MB + written 850.7 MB); the launch issued 0.87 instructions per cycle per
-# scheduler.
-DEPOSIT_FP32_FLOP = 684.0e9
-DEPOSIT_WARP_INST = 32.623e9
-DEPOSIT_DRAM_BYTES = 865.3e6
+# launch; one single-pass capture per group of metrics): FP32 FLOP from the sass
+# thread-instruction counts (2 per FFMA: 52.8 G, 1 per FADD: 87.7 G and per FMUL: 58.9 G), the
+# warp instructions issued (smsp__inst_executed.sum) and the DRAM bytes (read 1.3 MB + written
+# 638.1 MB).
+DEPOSIT_FP32_FLOP = 252.2e9
+DEPOSIT_WARP_INST = 11.218e9
+DEPOSIT_DRAM_BYTES = 639.4e6
 MAX_SM_MHZ = 2070.0   # the GB300's maximum SM clock (the clock the timed runs hold)
 
 

@@ -158,25 +158,6 @@ static cudaError_t ensure_monomials()
     return e;
 }
 
-__device__ __forceinline__ void solid_harmonics(double x, double y, double z, double* S)
-{
-    double px[5], py[5], pz[5];
-    px[0] = py[0] = pz[0] = 1.0;
-#pragma unroll
-    for (int p = 1; p < 5; p++) {
-        px[p] = px[p - 1] * x;
-        py[p] = py[p - 1] * y;
-        pz[p] = pz[p - 1] * z;
-    }
-#pragma unroll
-    for (int q = 0; q < NLM; q++) S[q] = 0.0;
-#pragma unroll
-    for (int t = 0; t < N_MONO_TERMS; t++) {
-        const Mono m = c_mono[t];
-        S[m.lm] = fma(m.coef, px[m.a] * py[m.b] * pz[m.c], S[m.lm]);
-    }
-}
-
 struct SphArgs {
     int na;
     const double *pos, *Z, *R, *w, *zeta, *clm;

@@ -2147,7 +2147,6 @@ __global__ void k_to_f32(const double* __restrict__ a, float* __restrict__ b, si
     if (t < n) b[t] = (float)a[t];
 }
 
-#define RGRID(L) red_grid(L.N()), NT, 0, s
 #define GRID(L) (unsigned)((L.N() + NT - 1) / NT), NT, 0, s
 
 cudaError_t launch_bnorm(const LevelT<double>& L, const double* u, const double* b, const Red& red, cudaStream_t s)

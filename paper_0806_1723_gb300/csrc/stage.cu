@@ -304,7 +304,7 @@ cudaError_t launch_split_stage_first_red(const LevelT<float>& L, float* u, const
 // contiguous run -- kept in a ring of PS_NS slots with the next plane in flight (a coarse plane
 // serves two fine planes).  The fine values are read and written in place, the next fine
 // plane's rows brought into L2 by a bulk prefetch one plane ahead.  The node expression is
-// k_prolong_add's, so the two are bitwise equal.  ec must be readable up to the next multiple
+// k_prolong_add_rows's, so the two are bitwise equal.  ec must be readable up to the next multiple
 // of 4 floats past its end (the solver's arrays are padded to 256 bytes).
 namespace {
 
