@@ -194,7 +194,9 @@ __global__ void __launch_bounds__(CT) k_conv_wgrad(Grid g, int cin, const bf16* 
 // rows with the threads along the row (coalesced, V channels per thread), reduces per channel in
 // shared memory and adds its partial with one atomic per channel.  Bound: the read of dy (from L2
 // after the pass that wrote it) and, with many blocks, the atomics on the few channels: 16 floats of
-// 288k nodes 12.6 us with one channel per thread and 128 rows per block, 9.4 us with four and 512.
+// 288k nodes 12.6 us with one channel per thread and 128 rows per block, 9.4 us with four channels and
+// eight rows per thread (512 per block; fewer rows per block for more channels keep small grids'
+// sums short).
 template <int V>
 __global__ void __launch_bounds__(256) k_bias_grad(size_t N, int cout, int rows, const float* __restrict__ dy,
                                                    float* __restrict__ db)
@@ -468,10 +470,12 @@ inline unsigned blocks(size_t n, int t) { return (unsigned)((n + t - 1) / t); }
 void launch_bias_grad(size_t N, int cout, const float* dy, float* db, cudaStream_t s)
 {
     // (four channels per thread where rows are whole 16-byte pieces)
-    if (cout % 4 == 0 && !((uintptr_t)dy & 15u))
-        k_bias_grad<4><<<blocks(N, 512), 256, 0, s>>>(N, cout, 512, dy, db);
-    else
+    if (cout % 4 == 0 && !((uintptr_t)dy & 15u)) {
+        const int rows = 8 * (256 / (cout / 4));
+        k_bias_grad<4><<<blocks(N, rows), 256, 0, s>>>(N, cout, rows, dy, db);
+    } else {
         k_bias_grad<1><<<blocks(N, 128), 256, 0, s>>>(N, cout, 128, dy, db);
+    }
 }
 
 }  // namespace nn
