@@ -479,17 +479,16 @@ __device__ __forceinline__ void hs_tmem_ld16(uint32_t taddr, float* v)
     for (int i = 0; i < 16; i++) v[i] = __uint_as_float(r[i]);
 }
 
-// phi and phi~ (FP32, times sqrt(Vol)) of every function of atom `at` at listed node P:
+// phi and phi~ (FP32, times sqrt(Vol)) of every function of atom `at` at a listed node (px0, py0, pz0):
 // out(loc, phi, phi~) for loc in [0, per).  The 25 solid harmonics first (straight-line, the
 // same monomial terms in every lane), then per table entry its radial factors and its 2l+1
 // functions (a switch on l keeps the harmonic index a compile-time constant).
-template <typename Out>
-__device__ __forceinline__ void hs_eval_atom(const HsBasis& B, const HsGrid& g, int P, float w, float Vp, int at,
-                                             Out&& out)
+template <bool L4, typename Out>
+__device__ __forceinline__ void hs_eval_atom(const HsBasis& B, const HsGrid& g, double px0, double py0, double pz0, float w,
+                                             float Vp, int at, Out&& out)
 {
-    const int i = P % g.nx, j = (P / g.nx) % g.ny, k = P / (g.nx * g.ny);
-    const float dx = (float)(g.x[i] - g.pos[3 * at]), dy = (float)(g.y[j] - g.pos[3 * at + 1]),
-                dz = (float)(g.z[k] - g.pos[3 * at + 2]);
+    const float dx = (float)(px0 - g.pos[3 * at]), dy = (float)(py0 - g.pos[3 * at + 1]),
+                dz = (float)(pz0 - g.pos[3 * at + 2]);
     const float r = sqrtf(dx * dx + dy * dy + dz * dz);
     const float ir = 1.0f / r;
     float px[5], py[5], pz[5];
@@ -504,7 +503,7 @@ __device__ __forceinline__ void hs_eval_atom(const HsBasis& B, const HsGrid& g, 
 #pragma unroll
     for (int lm = 0; lm < NLM; lm++) sh[lm] = 0.0f;
 #define HS_ACC(i, LM, EA, EB, EC) \
-    if (i < HS_L3_TERMS || B.lmax >= 4) sh[LM] = fmaf(c_hs_coef[i], px[EA] * py[EB] * pz[EC], sh[LM]);
+    if (i < HS_L3_TERMS || L4) sh[LM] = fmaf(c_hs_coef[i], px[EA] * py[EB] * pz[EC], sh[LM]);
     HS_TERMS(HS_ACC)
 #undef HS_ACC
 #pragma unroll 1
@@ -526,8 +525,11 @@ __device__ __forceinline__ void hs_eval_atom(const HsBasis& B, const HsGrid& g, 
         case 2: HS_OUT(0, 4) HS_OUT(1, 5) HS_OUT(2, 6) HS_OUT(3, 7) HS_OUT(4, 8) break;
         case 3: HS_OUT(0, 9) HS_OUT(1, 10) HS_OUT(2, 11) HS_OUT(3, 12) HS_OUT(4, 13) HS_OUT(5, 14) HS_OUT(6, 15) break;
         default:
-            HS_OUT(0, 16) HS_OUT(1, 17) HS_OUT(2, 18) HS_OUT(3, 19) HS_OUT(4, 20) HS_OUT(5, 21) HS_OUT(6, 22)
-            HS_OUT(7, 23) HS_OUT(8, 24) break;
+            if constexpr (L4) {
+                HS_OUT(0, 16) HS_OUT(1, 17) HS_OUT(2, 18) HS_OUT(3, 19) HS_OUT(4, 20) HS_OUT(5, 21) HS_OUT(6, 22)
+                HS_OUT(7, 23) HS_OUT(8, 24)
+            }
+            break;
         }
 #undef HS_OUT
     }
@@ -614,44 +616,75 @@ __global__ void __launch_bounds__(1024) k_hs_bounds(HsBasis B, HsGrid g, const u
 }
 
 // (2'c) the FP16 operand images of one chunk: rows p in [0, K) are listed nodes p0 + p (zero
-// past n_list); functions past M keep the zeros the tables were cleared to.  Block: 32 nodes
-// (lanes) x 8 atoms (warps).  Each warp stages its atom's four FP16 arrays for its 32 nodes in
-// shared memory ([array][function][node]) and writes them out as 16-byte pieces (8 nodes of one
-// function), so that a warp store fills whole 128-byte lines (8 consecutive functions).
+// past n_list: weight 0 at the last listed node); functions past M keep the zeros the tables were
+// cleared to.  Block: 32 nodes (lanes), their coordinates, weights and potentials staged
+// once, and all atoms, eight (warps) at a time.  Each warp stages its atom's values for its 32 nodes in shared memory as
+// pairs ([high, low][function][node], A in the lower half of a word and T in the upper) and writes
+// them out as 16-byte pieces (8 nodes of one function), a quarter warp the four pieces of a function's
+// 32 nodes.  Bound: instruction issue (0.79 of the peak with four 16-bit stores per function, divisions
+// by the function count in the write-out and the index decomposed per atom: 2122 warp instructions per
+// 32 nodes and atom), then the write (2 GB per 190 656 nodes of 55 x 25 functions): 702 -> 481 us (575 with a block per eight atoms).
+template <bool L4>   // functions with l = 4
 __global__ void __launch_bounds__(256) k_hs_basis16(const __grid_constant__ HsBasis B, HsGrid g, int nT, const int* __restrict__ idx,
                                                     const float* __restrict__ sw, const double* __restrict__ V,
                                                     const int* __restrict__ ea, int p0, int n_list,
                                                     __half* __restrict__ img)
 {
-    extern __shared__ __align__(16) __half hs_stage[];   // [8 warps][4][per][32]
-    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5, at = blockIdx.y * 8 + wp;
-    if (at >= g.na) return;
-    __half* st = hs_stage + (size_t)wp * 4 * B.per * 32;
-    const int p = blockIdx.x * 32 + lane;   // row within the chunk
-    const bool live = p0 + p < n_list;
-    const int P = live ? idx[p0 + p] : 0;
-    const int ec = ea[g.na * B.per];
-    hs_eval_atom(B, g, P, live ? sw[p0 + p] : 0.0f, live ? (float)V[P] : 0.0f, at, [&](int loc, float ph, float pt) {
-        const int e = ea[at * B.per + loc];
-        const float a = live ? ph * __int_as_float((127 + e) << 23) : 0.0f;
-        const float t = live ? pt * __int_as_float((127 + e + ec) << 23) : 0.0f;
-        const __half ah = __float2half_rn(a), th = __float2half_rn(t);
-        st[(0 * B.per + loc) * 32 + lane] = ah;
-        st[(1 * B.per + loc) * 32 + lane] = __float2half_rn(a - __half2float(ah));
-        st[(2 * B.per + loc) * 32 + lane] = th;
-        st[(3 * B.per + loc) * 32 + lane] = __float2half_rn(t - __half2float(th));
-    });
-    __syncwarp();
-    // piece (array, function, kb, k half): 8 nodes = 16 bytes
-    const int kb0 = blockIdx.x * 2;
-    for (int t = lane; t < 4 * B.per * 4; t += 32) {
-        const int arr = t / (4 * B.per), rem = t - arr * 4 * B.per, loc = rem >> 2, kbh = rem & 3;
-        const int kb = kb0 + (kbh >> 1), kh = kbh & 1;
-        const int f = at * B.per + loc, fb = f >> 7, r = f & 127;
-        const uint4 v = *reinterpret_cast<const uint4*>(st + (arr * B.per + loc) * 32 + (kbh >> 1) * 16 + kh * 8);
-        __half* dst = img + ((size_t)kb * nT + fb) * (TC_SIDE / 2) + arr * (TC_IMG / 2) + (r >> 3) * 128 + kh * 64 +
-                      (r & 7) * 8;
-        *reinterpret_cast<uint4*>(dst) = v;
+    extern __shared__ __align__(16) unsigned hs_stage[];   // [8 warps][2][per][32]
+    __shared__ double s_c[3][32];
+    __shared__ float s_w[32], s_v[32], s_sc[8][HS_MAXF];
+    const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+    if (wp == 0) {
+        const int p = p0 + blockIdx.x * 32 + lane;
+        const int P = idx[min(p, n_list - 1)];
+        s_c[0][lane] = g.x[P % g.nx];
+        s_c[1][lane] = g.y[(P / g.nx) % g.ny];
+        s_c[2][lane] = g.z[P / (g.nx * g.ny)];
+        s_w[lane] = p < n_list ? sw[p] : 0.0f;
+        s_v[lane] = (float)V[P];
+    }
+    __syncthreads();
+    unsigned* st = hs_stage + (size_t)wp * 2 * B.per * 32;
+    const float c2 = __int_as_float((127 + ea[g.na * B.per]) << 23);
+    const double x = s_c[0][lane], y = s_c[1][lane], z = s_c[2][lane];
+    const float w = s_w[lane], v = s_v[lane];
+    const int kb = blockIdx.x * 2 + ((lane >> 1) & 1), kh = lane & 1;
+    __half* out = img + (size_t)kb * nT * (TC_SIDE / 2) + kh * 64 + (lane >> 2) * 8;
+    for (int at = wp; at < g.na; at += 8) {
+        for (int f = lane; f < B.per; f += 32) s_sc[wp][f] = __int_as_float((127 + ea[at * B.per + f]) << 23);
+        __syncwarp();
+        hs_eval_atom<L4>(B, g, x, y, z, w, v, at, [&](int loc, float ph, float pt) {
+            const float sc = s_sc[wp][loc];
+            const float a = ph * sc, t = pt * (sc * c2);
+            const __half2 hi = __floats2half2_rn(a, t);
+            const float2 back = __half22float2(hi);
+            const __half2 lo = __floats2half2_rn(a - back.x, t - back.y);
+            // (the fours of an odd function's row change places: the reads below then meet no bank twice)
+            unsigned* row = st + loc * 32 + (lane ^ ((loc & 1) << 2));
+            row[0] = *reinterpret_cast<const unsigned*>(&hi);
+            row[B.per * 32] = *reinterpret_cast<const unsigned*>(&lo);
+        });
+        __syncwarp();
+        // lane: nodes 8 (lane & 3) .. +7 (16-node block kb, half kh of it) of function f0 + lane / 4, f0 in
+        // whole groups of eight functions, so that a store fills 128-byte lines
+        const int first = at * B.per;
+        for (int f0 = first & ~7; f0 < first + B.per; f0 += 8) {
+            const int loc = f0 + (lane >> 2) - first, odd = (loc & 1) << 2;
+            if (loc < 0 || loc >= B.per) continue;
+            __half* dst = out + (size_t)(f0 >> 7) * (TC_SIDE / 2) + ((f0 & 127) >> 3) * 128;
+#pragma unroll
+            for (int h = 0; h < 2; h++) {   // high, low parts: images A_hi, A_lo, T_hi, T_lo
+                const unsigned* src = st + (h * B.per + loc) * 32 + 8 * (lane & 3);
+                const uint4 u = *reinterpret_cast<const uint4*>(src + odd), o = *reinterpret_cast<const uint4*>(src + 4 - odd);
+                *reinterpret_cast<uint4*>(dst + h * (TC_IMG / 2)) =
+                    make_uint4(__byte_perm(u.x, u.y, 0x5410), __byte_perm(u.z, u.w, 0x5410), __byte_perm(o.x, o.y, 0x5410),
+                               __byte_perm(o.z, o.w, 0x5410));
+                *reinterpret_cast<uint4*>(dst + (2 + h) * (TC_IMG / 2)) =
+                    make_uint4(__byte_perm(u.x, u.y, 0x7632), __byte_perm(u.z, u.w, 0x7632), __byte_perm(o.x, o.y, 0x7632),
+                               __byte_perm(o.z, o.w, 0x7632));
+            }
+        }
+        __syncwarp();
     }
 }
 
@@ -896,9 +929,10 @@ cudaError_t ensure_hs_attributes()
     std::lock_guard<std::mutex> lock(g_hs_mutex);
     if (g_hs_attr_device == dev) return cudaSuccess;
     e = cudaFuncSetAttribute(k_hs_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_hs_basis16, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(8 * 4 * HS_MAXF * 32 * sizeof(__half)));
+    for (auto* f : {k_hs_basis16<false>, k_hs_basis16<true>})
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)(8 * 4 * HS_MAXF * 32 * sizeof(__half)));
     if (e == cudaSuccess) g_hs_attr_device = dev;
     return e;
 }
@@ -1020,7 +1054,6 @@ int launch_interstitial_hs(const int n[3], const double* x, const double* y, con
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return LASTO_ERR_CUDA;
 
-    const unsigned ablocks = (unsigned)((na + 7) / 8);
     if (tensor && n_list > 0) {
         // per-function scales; operand images cleared once (the padding functions past M stay zero)
         e = cudaMemsetAsync(tables, 0, 8 * (size_t)Mp128 * Kmax, s);
@@ -1035,7 +1068,8 @@ int launch_interstitial_hs(const int n[3], const double* x, const double* y, con
         const int K = (int)std::min<size_t>(Kmax, ((size_t)(n_list - p0) + HS_KC - 1) / HS_KC * HS_KC);
         mark();
         if (tensor) {
-            k_hs_basis16<<<dim3((unsigned)(K / 32), ablocks), 256, (size_t)8 * 4 * per * 32 * sizeof(__half), s>>>(
+            auto* basis16 = B.lmax >= 4 ? k_hs_basis16<true> : k_hs_basis16<false>;
+            basis16<<<(unsigned)(K / 32), 256, (size_t)8 * 4 * per * 32 * sizeof(__half), s>>>(
                 B, g, nT, idx, sw, V, ea, p0, n_list, reinterpret_cast<__half*>(tables));
         } else {
             const size_t tot = (size_t)K * Mp;
