@@ -106,54 +106,109 @@ __device__ __forceinline__ double monopole_at(const double* __restrict__ f, int 
 
 // b = 4pi (ne - rho_00(r)/sqrt(4pi) + quartic(r)) inside sphere i (|x - X_i| < R_i), 4pi ne
 // outside.  Ownership: an FP32 distance test decides all nodes farther than 1e-4 R^2 from
-// a sphere surface; the rest are decided in FP64.
-__global__ void __launch_bounds__(256) k_raw_deposit(RawArgs a, const double* __restrict__ rec,
-                                                    double* __restrict__ b, int* __restrict__ owner,
-                                                    int* __restrict__ status)
+// a sphere surface; the rest are decided in FP64.  A block takes 32 x 8 x 4 nodes (lanes along x) and
+// first lists, in the atoms' order, the spheres that reach its nodes' box by that FP32 test (with room
+// for its rounding): most boxes meet none.  Nodes that pass the FP32 test of some sphere are queued
+// and finished together, so that the FP64 of the exact test and of the table (a logarithm, divisions)
+// runs in whole warps: it is the bound, 10 % of the nodes of Pd55 129^3.  167 us with every sphere
+// tested at every node and the inside nodes in place (214 with the lists alone) -> 119 us.
+constexpr int RD_X = 32, RD_Y = 8, RD_Z = 4;
+
+__global__ void __launch_bounds__(RD_X * RD_Y) k_raw_deposit(RawArgs a, const double* __restrict__ rec,
+                                                            double* __restrict__ b, int* __restrict__ owner,
+                                                            int* __restrict__ status)
 {
-    // per atom, once per block: the FP32 position and the FP32 sphere-test bound (the node loop
-    // then needs no FP64 conversion)
-    extern __shared__ float4 raw_at[];
-    for (int t = threadIdx.x; t < a.na; t += blockDim.x) {
-        const double* o = rec + (size_t)RAW_REC * t;
-        const float R2f = (float)(o[3] * o[3]);
-        raw_at[t] = make_float4((float)o[0], (float)o[1], (float)o[2], R2f * (1.0f + 1e-4f));
-    }
-    __syncthreads();
-    const unsigned N = (unsigned)a.n[0] * a.n[1] * a.n[2];   // < 2^31 (checked where grids are accepted)
-    const unsigned P = blockIdx.x * blockDim.x + threadIdx.x;
-    if (P >= N) return;
-    const unsigned nxy = (unsigned)a.n[0] * a.n[1];
-    const int k = (int)(P / nxy), j = (int)((P - (unsigned)k * nxy) / a.n[0]), i = (int)(P - (unsigned)k * nxy - (unsigned)j * a.n[0]);
-    const double x = a.ax[0][i], y = a.ax[1][j], z = a.ax[2][k];
-    const float xf = (float)x, yf = (float)y, zf = (float)z;
-    int own = -1;
-    double r = 0.0;
-    for (int t = 0; t < a.na; t++) {
-        const float4 c = raw_at[t];
-        const float dx = xf - c.x, dy = yf - c.y, dz = zf - c.z;
-        const float r2f = dx * dx + dy * dy + dz * dz;
-        if (r2f > c.w) continue;
-        const double* o = rec + (size_t)RAW_REC * t;
-        const double ex = x - o[0], ey = y - o[1], ez = z - o[2];
-        const double d = sqrt(ex * ex + ey * ey + ez * ez);
-        if (d < o[3]) {
-            own = t;
-            r = d;
-            break;
+    extern __shared__ int near_at[];   // [na]: atoms whose spheres reach the box
+    __shared__ int s_cnt[RD_Y], s_queued;
+    __shared__ unsigned s_queue[RD_X * RD_Y * RD_Z];   // node of the box | place in the list << 10
+    static_assert(RD_X * RD_Y * RD_Z == 1 << 10 && RD_X == 32 && RD_Y == 8, "queue entries and decoding");
+    const int gx = (a.n[0] + RD_X - 1) / RD_X, gy = (a.n[1] + RD_Y - 1) / RD_Y;
+    const int bz = (int)blockIdx.x / (gx * gy), rem = (int)blockIdx.x - bz * gx * gy;
+    const int lane = threadIdx.x % RD_X, wp = threadIdx.x / RD_X;
+    const int i0 = (rem % gx) * RD_X, j0 = (rem / gx) * RD_Y, k0 = bz * RD_Z;
+    // the box of the block's nodes, in FP32 as the test below sees them
+    float lo[3], hi[3];
+#pragma unroll
+    for (int d = 0; d < 3; d++) {
+        const int first = d == 0 ? i0 : d == 1 ? j0 : k0, len = d == 0 ? RD_X : d == 1 ? RD_Y : RD_Z;
+        const float c = (float)a.ax[d][min(first + min(lane, len - 1), a.n[d] - 1)];
+        lo[d] = hi[d] = c;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            lo[d] = fminf(lo[d], __shfl_xor_sync(0xffffffffu, lo[d], o));
+            hi[d] = fmaxf(hi[d], __shfl_xor_sync(0xffffffffu, hi[d], o));
         }
     }
-    double v = a.ne[P];
-    if (own >= 0) {
-        const double* o = rec + (size_t)RAW_REC * own;
-        const double rho0 = monopole_at(a.rho00 + (size_t)own * a.n_rad, a.n_rad, a.r_min, o[7], r) /
-                            sqrt(4.0 * RAW_PI);
-        v = v - rho0 + (o[4] + o[5] * r * r + o[6] * r * r * r * r);
+    int count = 0;
+    for (int base = 0; base < a.na; base += RD_X * RD_Y) {
+        const int t = base + (int)threadIdx.x;
+        bool in = false;
+        if (t < a.na) {
+            const double* o = rec + (size_t)RAW_REC * t;
+            float r2 = 0.0f;
+#pragma unroll
+            for (int d = 0; d < 3; d++) {
+                const float c = (float)o[d], e = fmaxf(fmaxf(lo[d] - c, c - hi[d]), 0.0f);
+                r2 += e * e;
+            }
+            in = !(r2 > (float)(o[3] * o[3]) * (1.0f + 1e-4f) * (1.0f + 1e-5f));
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, in);
+        __syncthreads();
+        if (lane == 0) s_cnt[wp] = __popc(m);
+        __syncthreads();
+        int at = count;
+        for (int q = 0; q < RD_Y; q++) {
+            at += q < wp ? s_cnt[q] : 0;
+            count += s_cnt[q];
+        }
+        if (in) near_at[at + __popc(m & ((1u << lane) - 1u))] = t;
     }
-    const double bv = 4.0 * RAW_PI * v;
-    b[P] = bv;
-    if (owner) owner[P] = own;
-    if (!isfinite(bv) && status) atomicMax(status, (int)LASTO_ERR_NONFINITE);
+    if (threadIdx.x == 0) s_queued = 0;
+    __syncthreads();
+    auto finish = [&](size_t P, double v, int own) {
+        const double bv = 4.0 * RAW_PI * v;
+        b[P] = bv;
+        if (owner) owner[P] = own;
+        if (!isfinite(bv) && status) atomicMax(status, (int)LASTO_ERR_NONFINITE);
+    };
+    const int i = i0 + lane, j = j0 + wp;
+    if (i < a.n[0] && j < a.n[1]) {
+        const float xf = (float)a.ax[0][i], yf = (float)a.ax[1][j];
+        for (int kk = 0; kk < min(RD_Z, a.n[2] - k0); kk++) {
+            const size_t P = ((size_t)(k0 + kk) * a.n[1] + j) * a.n[0] + i;
+            const float zf = (float)a.ax[2][k0 + kk];
+            int q = 0;
+            for (; q < count; q++) {
+                const double* o = rec + (size_t)RAW_REC * near_at[q];
+                const float dx = xf - (float)o[0], dy = yf - (float)o[1], dz = zf - (float)o[2];
+                if (!(dx * dx + dy * dy + dz * dz > (float)(o[3] * o[3]) * (1.0f + 1e-4f))) break;
+            }
+            if (q < count)
+                s_queue[atomicAdd(&s_queued, 1)] = (unsigned)(kk * 256 + (int)threadIdx.x) | (unsigned)q << 10;
+            else
+                finish(P, a.ne[P], -1);
+        }
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < s_queued; e += RD_X * RD_Y) {
+        const int node = (int)(s_queue[e] & 1023u), ni = i0 + (node & 31), nj = j0 + ((node >> 5) & 7), nk = k0 + (node >> 8);
+        const size_t P = ((size_t)nk * a.n[1] + nj) * a.n[0] + ni;
+        const double x = a.ax[0][ni], y = a.ax[1][nj], z = a.ax[2][nk];
+        double v = a.ne[P];
+        int own = -1;
+        for (int q = (int)(s_queue[e] >> 10); q < count && own < 0; q++) {
+            const double* o = rec + (size_t)RAW_REC * near_at[q];
+            const double ex = x - o[0], ey = y - o[1], ez = z - o[2];
+            const double r = sqrt(ex * ex + ey * ey + ez * ez);
+            if (!(r < o[3])) continue;
+            own = near_at[q];
+            const double rho0 = monopole_at(a.rho00 + (size_t)own * a.n_rad, a.n_rad, a.r_min, o[7], r) /
+                                sqrt(4.0 * RAW_PI);
+            v = v - rho0 + (o[4] + o[5] * r * r + o[6] * r * r * r * r);
+        }
+        finish(P, v, own);
+    }
 }
 
 }  // namespace
@@ -167,13 +222,15 @@ cudaError_t launch_raw_sphere_params(const RawArgs& a, double* rec, int* status,
 cudaError_t launch_raw_deposit(const RawArgs& a, const double* rec, double* b, int* owner, int* status, cudaStream_t s)
 {
     const size_t N = (size_t)a.n[0] * a.n[1] * a.n[2];
-    const size_t smem = sizeof(float4) * (size_t)a.na;
-    if (smem > 200 * 1024 || N >= (size_t(1) << 31)) return cudaErrorInvalidValue;
+    // (up to 12 800 atoms)
+    if (sizeof(float4) * (size_t)a.na > 200 * 1024 || N >= (size_t(1) << 31)) return cudaErrorInvalidValue;
+    const size_t smem = sizeof(int) * (size_t)a.na;
     if (smem > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(k_raw_deposit, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    k_raw_deposit<<<(unsigned)((N + 255) / 256), 256, smem, s>>>(a, rec, b, owner, status);
+    const size_t g = (size_t)((a.n[0] + RD_X - 1) / RD_X) * ((a.n[1] + RD_Y - 1) / RD_Y) * ((a.n[2] + RD_Z - 1) / RD_Z);
+    k_raw_deposit<<<(unsigned)g, RD_X * RD_Y, smem, s>>>(a, rec, b, owner, status);
     return cudaGetLastError();
 }
 
