@@ -156,8 +156,10 @@ typedef struct lasto_poisson lasto_poisson;   /* opaque; owns workspace, plans a
  * solve of each new batch layout times, per level shape and precision, the red-black
  * smoother as in-place half sweeps (128, 256 or 512 threads per block over the flat node
  * index, or one block per (j, k) row: threads = 0) and as fused passes of the z-slab and
- * register-column kernels (several tile shapes), and the cycle uses the fastest; all give
- * bitwise the same iterates.  lasto_poisson_tune_table writes the table as
+ * register-column kernels (several tile shapes), on the finest FP32 level also over
+ * colour-split storage, and the cycle uses the fastest; all give bitwise the same iterates.
+ * us: one pre-smoothing phase run as a graph (finest FP32 level: with its residual,
+ * restriction and prolongation).  lasto_poisson_tune_table writes the table as
  * text, one line per shape: "nx ny nz elem_bytes fused threads tx ty kz sweeps_per_pass us"
  * (NUL-terminated into buf when cap > 0) and returns its length, -1 for a null handle.
  * lasto_poisson_set_tune_table adds such lines (shapes it lists are then not timed);
