@@ -679,7 +679,9 @@ __global__ void __launch_bounds__(TC_M) k_conv_wgrad_tc(Grid g, GridDiv gd, int 
 // channels 62 against 79 us, at 48 140 against 131).  Every tap has its own columns of tensor memory,
 // so the input is staged once for all taps of the CTA.  Stages alternate between two buffers, filled
 // by eight warps while a ninth issues; a CTA takes every gridDim.x-th one, and adds its sums to dw
-// with vector reductions at the end.  Bound: 32-byte pieces from L2 (3 to 4 TB/s; three or four
+// with vector reductions, at the latest after `most` stages: the tensor core's FP32 accumulation
+// truncates, so its error grows with the length of a sum (positive values, 64 x 64 channels on 8 grids
+// of 33^3: 1.7e-5 of the largest with one sum per CTA, 3.6e-6 so, the gathered form's 3.8e-6).  Bound: 32-byte pieces from L2 (3 to 4 TB/s; three or four
 // buffers, or 16 loading warps, change nothing).  8 grids of 33^3, against the kernel above (27
 // gathered rows per node): 48 x 16 channels 330 -> 57 us.
 constexpr int WS_K = 128, WS_NT = 256;
@@ -694,7 +696,7 @@ inline size_t ws_smem(int W, int cg, int cout)
 }
 
 template <int COUT>
-__global__ void __launch_bounds__(WS_NT + 32) k_conv_wgrad_seq(Seq q, int cin, int cg, const bf16* __restrict__ x,
+__global__ void __launch_bounds__(WS_NT + 32) k_conv_wgrad_seq(Seq q, int cin, int cg, int most, const bf16* __restrict__ x,
                                                           const bf16* __restrict__ dy, float* __restrict__ dw,
                                                           int* __restrict__ err)
 {
@@ -709,6 +711,7 @@ __global__ void __launch_bounds__(WS_NT + 32) k_conv_wgrad_seq(Seq q, int cin, i
     const int tap0 = (int)blockIdx.y / groups * TAPS, c0 = (int)blockIdx.y % groups * cg, ntap = min(TAPS, 27 / DX - tap0);
     const int nchunk = (q.total + WS_K - 1) / WS_K;
     const int nk = ((int)blockIdx.x < nchunk) ? (nchunk - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
+    const int runs = (nk + most - 1) / most, run = nk > 0 ? (nk + runs - 1) / runs : 1;   // stages per accumulation
     const uint32_t a_bytes = (uint32_t)cg / 8 * 3 * seg * 16, b_bytes = N / 8 * WS_K * 16;
     // both B buffers, then both A buffers
     const uint32_t baseA = smem_u32(ws_raw) + 2 * b_bytes, baseB = smem_u32(ws_raw);
@@ -750,38 +753,8 @@ __global__ void __launch_bounds__(WS_NT + 32) k_conv_wgrad_seq(Seq q, int cin, i
         }
         asm volatile("cp.async.commit_group;\n" ::: "memory");
     };
-    if (nk > 0 && tid < WS_NT) load(0);
-    for (int k = 0; k < nk; k++) {
-        asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-        bad = __syncthreads_or(bad);
-        if (bad) break;
-        if (__shfl_sync(0xffffffffu, warp, 0) == WS_NT / 32) {
-            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-            const uint64_t a0 = make_desc_any(baseA + (k & 1) * a_bytes, 128, 3 * seg * 16);
-            const uint64_t b0 = make_desc_any(baseB + (k & 1) * b_bytes, 128, WS_K * 16);
-#pragma unroll
-            for (int t = 0; t < TAPS; t++) {
-                const int tap = (tap0 + t) * DX;   // its start in a segment set, in positions
-                const uint64_t ad = a0 + (uint32_t)(tap / 9 * seg + (tap / 3) % 3 * q.pitch + (DX == 3 ? 1 : tap % 3));
-                if (t < ntap) {
-#pragma unroll
-                    for (int j = 0; j < WS_K / 16; j++) mma_f16(tmem + t * N, ad + j * 16, b0 + j * 16, idesc, k > 0 || j > 0);
-                }
-            }
-            mma_commit(smem_u32(&mbar[k & 1]));
-        }
-        if (tid < WS_NT && k + 1 < nk) load(k + 1);   // while these are issued
-    }
-    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-    if (!bad && nk > 0) {
-        const int k = nk - 1;
-        if (!mbar_wait(smem_u32(&mbar[k & 1]), (uint32_t)((k / 2) & 1))) bad = true;
-    }
-    bad = __syncthreads_or(bad);
-    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    if (!bad && nk > 0) {
-        // an M = 64 accumulator: row r in tensor-memory lane 32 (r / 16) + r % 16
+    // the sums of a run into dw.  An M = 64 accumulator: row r in tensor-memory lane 32 (r / 16) + r % 16
+    auto drain = [&]() {
         const int row = (warp & 3) * 16 + (lane & 15);
         const bool live = lane < 16 && row < cg, vec = ((uintptr_t)dw & 15) == 0;
         const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
@@ -805,7 +778,42 @@ __global__ void __launch_bounds__(WS_NT + 32) k_conv_wgrad_seq(Seq q, int cin, i
                 }
             }
         }
-    } else if (bad && tid == 0 && err) {
+    };
+    if (nk > 0 && tid < WS_NT) load(0);
+    for (int k = 0, first = 0; k < nk; k++) {   // first: of the run
+        asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+        bad = __syncthreads_or(bad);
+        if (bad) break;
+        if (__shfl_sync(0xffffffffu, warp, 0) == WS_NT / 32) {
+            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+            const uint64_t a0 = make_desc_any(baseA + (k & 1) * a_bytes, 128, 3 * seg * 16);
+            const uint64_t b0 = make_desc_any(baseB + (k & 1) * b_bytes, 128, WS_K * 16);
+#pragma unroll
+            for (int t = 0; t < TAPS; t++) {
+                const int tap = (tap0 + t) * DX;   // its start in a segment set, in positions
+                const uint64_t ad = a0 + (uint32_t)(tap / 9 * seg + (tap / 3) % 3 * q.pitch + (DX == 3 ? 1 : tap % 3));
+                if (t < ntap) {
+#pragma unroll
+                    for (int j = 0; j < WS_K / 16; j++) mma_f16(tmem + t * N, ad + j * 16, b0 + j * 16, idesc, k > first || j > 0);
+                }
+            }
+            mma_commit(smem_u32(&mbar[k & 1]));
+        }
+        if (tid < WS_NT && k + 1 < nk) load(k + 1);   // while these are issued
+        if (k + 1 == nk || k + 1 == first + run) {
+            // (commits complete in issue order)
+            if (!mbar_wait(smem_u32(&mbar[k & 1]), (uint32_t)((k / 2) & 1))) bad = true;
+            bad = __syncthreads_or(bad);
+            if (bad) break;
+            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+            drain();
+            asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");   // (the next stage's barrier)
+            first = k + 1;
+        }
+    }
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    if (bad && tid == 0 && err) {
         atomicExch(err, 1);
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
@@ -916,12 +924,14 @@ int conv_wgrad_tc(int nb, const int dims[3], int cin, int cout, const void* x, c
         const int per = ws_groups(cout) * ws_dx(cout);
         const int ny = (27 + per - 1) / per * (cin / cg), nchunk = (q.total + WS_K - 1) / WS_K;
         const dim3 grid((unsigned)std::min(nchunk, std::max(1, 152 / ny)), (unsigned)ny);
+        // a sum of at most WG_CHUNK nodes, as in the gathered form (the pads add nothing)
+        const int most = (int)((size_t)WG_CHUNK * (size_t)q.total / g.nodes() / WS_K);
 #define LASTO_WS_CASE(C)                                                                                              \
     case C:                                                                                                           \
         if (cudaFuncSetAttribute(k_conv_wgrad_seq<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) !=     \
             cudaSuccess)                                                                                              \
             return LASTO_ERR_CUDA;                                                                                    \
-        k_conv_wgrad_seq<C><<<grid, WS_NT + 32, sm, s>>>(q, cin, cg, X, DY, dw, err);                                       \
+        k_conv_wgrad_seq<C><<<grid, WS_NT + 32, sm, s>>>(q, cin, cg, most, X, DY, dw, err);                                 \
         break;
         switch (cout) {
             LASTO_WS_CASE(16)

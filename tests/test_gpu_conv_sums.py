@@ -1,0 +1,54 @@
+"""The weight gradient where one sum is long: its error must not grow with the number of nodes that
+a block takes (the tensor core's FP32 accumulation truncates)."""
+import ctypes
+
+import pytest
+
+from gpu_common import need_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+def wgrad(B, x, dy, nb, dims, cin, cout):
+    import torch
+    dw = torch.zeros(27, cin, cout, device="cuda")
+    err = torch.zeros(1, dtype=torch.int32, device="cuda")
+    assert B.load().lasto_nn_conv3d_wgrad_tc(nb, (ctypes.c_int * 3)(*dims), cin, cout, B._ptr(x), B._ptr(dy), None, B._ptr(dw),
+                                             None, B._ptr(err), B._stream()) == 0
+    torch.cuda.synchronize()
+    assert int(err.item()) == 0
+    return dw
+
+
+def wgrad_ref(x, dy, nb, dims):
+    """The same in 64 bits: per tap, the rows of x at the neighbour against the rows of dy."""
+    import torch
+    W, H, D = dims
+    X, Y = x.double().view(nb, D, H, W, -1), dy.double().view(nb, D, H, W, -1)
+    here = lambda d, n: slice(max(0, -d), n - max(0, d))
+    there = lambda d, n: slice(max(0, d), n + min(0, d))
+    out = []
+    for dz in (-1, 0, 1):
+        for dy_ in (-1, 0, 1):
+            for dx in (-1, 0, 1):
+                a = X[:, there(dz, D), there(dy_, H), there(dx, W)].reshape(-1, X.shape[-1])
+                b = Y[:, here(dz, D), here(dy_, H), here(dx, W)].reshape(-1, Y.shape[-1])
+                out.append(a.T @ b)
+    return torch.stack(out)
+
+
+@pytest.mark.parametrize("cin,cout,nb,dims", [(64, 64, 8, (33, 33, 33)), (128, 128, 4, (33, 33, 33)), (128, 64, 6, (65, 17, 31)),
+                                              (96, 32, 12, (33, 33, 33))])
+def test_long_sums(cin, cout, nb, dims):
+    import torch
+    B = need_gpu()
+    g = torch.Generator(device="cuda").manual_seed(cin + cout)
+    N = nb * dims[0] * dims[1] * dims[2]
+    # (positive values: truncation then always errs to the same side)
+    x = torch.randn(N, cin, generator=g, device="cuda").abs().bfloat16()
+    dy = torch.randn(N, cout, generator=g, device="cuda").abs().bfloat16()
+    got, ref = wgrad(B, x, dy, nb, dims, cin, cout).double(), wgrad_ref(x, dy, nb, dims)
+    # sums of at most 2048 nodes, 16 per MMA, each truncated by up to 2^-23 of a partial sum that is
+    # half the whole on average; then one rounded FP32 addition (2^-24) per such sum
+    tol = 2.0 ** -24 * (2048 / 16 + N / 2048 + 1)
+    assert float(((got - ref) / ref).abs().max()) <= tol
