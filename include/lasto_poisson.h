@@ -422,6 +422,15 @@ int lasto_op_smooth_wave_f32(const int n[3], const double* x, const double* y, c
  * Asynchronous on the stream; the stream stays usable afterwards. */
 int lasto_selftest_bounded_wait(double seconds, int* status, void* stream);
 
+/* Self-test of what a convolution kernel does when such a wait runs out: the kernel that
+ * lasto_nn_conv3d_fwd_tc (which 0; m: packed weights, out: y32 with cout channels per node) or
+ * lasto_nn_conv3d_wgrad_tc (which 1; m: dy16, out: dw) launches for these sizes, with waits
+ * that run out at once.  A block that meets one (forward: 48 input channels and more) leaves
+ * `out` alone, waits for its copies and matrix instructions, gives its tensor memory back and
+ * sets *err.  Asynchronous on the stream; the stream stays usable. */
+int lasto_selftest_conv_wait(int which, int nb, const int dims[3], int cin, int cout, const void* x, const void* m,
+                             float* out, int* err, void* stream);
+
 /* Arithmetic throughput probe (the paper has no counterpart): `blocks` blocks of 256
  * threads, each thread 8 independent fused multiply-add chains of 16 * iters steps, in FP64
  * (precision 0) or FP32 (precision 1); out: device array of blocks * 256 elements of that

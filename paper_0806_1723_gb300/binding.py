@@ -56,7 +56,7 @@ EXPORTS = ["lasto_config_default", "lasto_poisson_create", "lasto_poisson_solve"
            "lasto_poisson_last_error", "lasto_poisson_kernel_counts", "lasto_mesh_axis", "lasto_op_sphere_params", "lasto_op_deposit",
            "lasto_op_deposit_noalloc",
            "lasto_op_multipoles", "lasto_op_boundary_fill", "lasto_op_boundary_exact", "lasto_op_apply", "lasto_op_residual", "lasto_op_smooth",
-           "lasto_op_smooth_f32", "lasto_op_smooth_split_f32", "lasto_op_smooth_slab", "lasto_op_smooth_slab_f32", "lasto_op_smooth_wave_f32", "lasto_selftest_bounded_wait",
+           "lasto_op_smooth_f32", "lasto_op_smooth_split_f32", "lasto_op_smooth_slab", "lasto_op_smooth_slab_f32", "lasto_op_smooth_wave_f32", "lasto_selftest_bounded_wait", "lasto_selftest_conv_wait",
            "lasto_probe_fma", "lasto_op_restrict", "lasto_op_prolong_add", "lasto_op_coarse_solve",
            "lasto_op_project", "lasto_op_sphere_density", "lasto_op_inner_solve", "lasto_op_interstitial_hs", "lasto_guess_param_count", "lasto_poisson_set_guess",
            "lasto_poisson_tune_table", "lasto_poisson_set_tune_table", "lasto_nn_conv3d_fwd", "lasto_nn_pack_weights", "lasto_nn_conv3d_fwd_tc", "lasto_nn_conv3d_dgrad", "lasto_nn_conv3d_wgrad", "lasto_nn_conv3d_dgrad_tc", "lasto_nn_conv3d_wgrad_tc",
@@ -103,6 +103,7 @@ def _declare(L):
         "lasto_op_smooth_slab_f32": (i, [ip, vp, vp, vp, vp, vp, vp, i, i, i, ip, vp]),
         "lasto_op_smooth_wave_f32": (i, [ip, vp, vp, vp, vp, vp, vp, i, i, i, i, vp]),
         "lasto_selftest_bounded_wait": (i, [d, vp, vp]),
+        "lasto_selftest_conv_wait": (i, [i, i, ip, i, i, vp, vp, vp, vp, vp]),
         "lasto_probe_fma": (i, [i, i, i, vp, vp]),
         "lasto_op_restrict": (i, [ip, vp, vp, vp, vp, vp, vp]),
         "lasto_op_prolong_add": (i, [ip, vp, vp, vp, vp, vp, vp]),

@@ -15,8 +15,10 @@
 // thread issues the MMA of a stage and commits it to the stage's mbarrier, which releases the
 // stage for the copies of the step five later.  After the last step every thread reads its node's row of the
 // accumulator (tcgen05.ld 32x32b: warp w owns tensor-memory lanes 32w .. 32w+31) and applies
-// bias, ReLU and the output conversions.  Every mbarrier wait is bounded: on a timeout the
-// kernel records an error, stops issuing, frees its tensor memory and returns.
+// bias, ReLU and the output conversions.  Every mbarrier wait is bounded (`limit` attempts inside
+// the loops): on a timeout the kernel records an error, stops issuing, waits (again bounded) for its
+// copies and for the last MMA it issued, which may still read its shared memory and write its
+// tensor memory, frees the latter and returns.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -57,9 +59,10 @@ __host__ __device__ constexpr uint32_t make_idesc(int n)
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(TC_M >> 4) << 24);
 }
 
-__device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity)
+// (a limit of 0: gives up at once)
+__device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, long long limit = TC_SPIN_LIMIT)
 {
-    for (long long it = 0; it < TC_SPIN_LIMIT; it++) {
+    for (long long it = 0; it < limit; it++) {
         uint32_t ok;
         asm volatile(
             "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
@@ -91,7 +94,7 @@ __global__ void __launch_bounds__(TC_M) k_conv_tc(Grid g, int cin, const bf16* _
                                                  const uint4* __restrict__ wpk, const float* __restrict__ bias,
                                                  int relu, float* __restrict__ y32, int ldy32, int off32,
                                                  bf16* __restrict__ y16, int ldy16, int off16,
-                                                 float* __restrict__ part, int* __restrict__ err)
+                                                 float* __restrict__ part, long long limit, int* __restrict__ err)
 {
     constexpr int A_BYTES = TC_M * 32;
     constexpr int B_BYTES = COUT * 32;
@@ -147,7 +150,7 @@ __global__ void __launch_bounds__(TC_M) k_conv_tc(Grid g, int cin, const bf16* _
     auto prefetch = [&](int k) {
         const int st = k % TC_STAGES;
         if (k >= TC_STAGES) {
-            if (!mbar_wait(smem_u32(&mbar[st]), (uint32_t)((k / TC_STAGES - 1) & 1))) abort_flag = 1;
+            if (!mbar_wait(smem_u32(&mbar[st]), (uint32_t)((k / TC_STAGES - 1) & 1), limit)) abort_flag = 1;
         }
         const int tap = tap_a + k / cpt, c0 = (k % cpt) * 16;
         const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
@@ -171,6 +174,7 @@ __global__ void __launch_bounds__(TC_M) k_conv_tc(Grid g, int cin, const bf16* _
         if (k < nk) prefetch(k);
         asm volatile("cp.async.commit_group;\n" ::: "memory");
     }
+    int issued = 0;   // steps
     for (int kc = 0; kc < nk; kc++) {
         const int s = kc % TC_STAGES;
         if (kc + TC_AHEAD < nk) prefetch(kc + TC_AHEAD);
@@ -192,12 +196,13 @@ __global__ void __launch_bounds__(TC_M) k_conv_tc(Grid g, int cin, const bf16* _
                              smem_u32(&mbar[s]))
                          : "memory");
         }
+        issued = kc + 1;
     }
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-    // wait for the last MMA (commits complete in issue order)
-    if (!abort_flag && nk > 0) {
-        const int s = (nk - 1) % TC_STAGES;
-        if (!mbar_wait(smem_u32(&mbar[s]), (uint32_t)(((nk - 1) / TC_STAGES) & 1))) abort_flag = 1;
+    // wait for the last MMA (commits complete in issue order), also in a block that gives up
+    if (issued > 0) {
+        const int s = (issued - 1) % TC_STAGES;
+        if (!mbar_wait(smem_u32(&mbar[s]), (uint32_t)(((issued - 1) / TC_STAGES) & 1))) abort_flag = 1;
     }
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
@@ -329,7 +334,7 @@ template <int COUT>
 __global__ void __launch_bounds__(SQ_NT + 32) k_conv_seq(Seq q, int cin, int cout, const bf16* __restrict__ x, const uint4* __restrict__ wpk,
                                                     const float* __restrict__ bias, int relu, float* __restrict__ y32,
                                                     int ldy32, int off32, bf16* __restrict__ y16, int ldy16, int off16,
-                                                    int* __restrict__ err)
+                                                    long long limit, int* __restrict__ err)
 {
     constexpr int NCOL = 2 * COUT <= 32 ? 32 : 2 * COUT <= 64 ? 64 : 2 * COUT <= 128 ? 128 : 256;
     extern __shared__ __align__(1024) unsigned char sq_raw[];
@@ -360,7 +365,10 @@ __global__ void __launch_bounds__(SQ_NT + 32) k_conv_seq(Seq q, int cin, int cou
     // channels 16 c .. 16 c + 15 into buffer c & 1 (after the MMAs that last read it): a lane pair
     // per position, 32 contiguous bytes
     auto load = [&](int c) {
-        if (c >= 2 && !mbar_wait(smem_u32(&mbar[c % 2]), (uint32_t)((c / 2 - 1) & 1))) bad = true;
+        if (c >= 2 && !mbar_wait(smem_u32(&mbar[c % 2]), (uint32_t)((c / 2 - 1) & 1), limit)) {
+            bad = true;
+            return;
+        }
         const uint32_t buf = base + (c % 2) * buf_bytes;
         const int h = tid & 1;
         for (int t = tid >> 1; t < 3 * seg; t += SQ_NT / 2) {
@@ -375,6 +383,7 @@ __global__ void __launch_bounds__(SQ_NT + 32) k_conv_seq(Seq q, int cin, int cou
         asm volatile("cp.async.commit_group;\n" ::: "memory");
     };
     if (tid < SQ_NT) load(0);
+    int issued = 0;   // channel chunks
     for (int c = 0; c < cpt; c++) {
         asm volatile("cp.async.wait_group 0;\n" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");   // visible to the tensor core
@@ -398,11 +407,12 @@ __global__ void __launch_bounds__(SQ_NT + 32) k_conv_seq(Seq q, int cin, int cou
             }
             mma_commit(smem_u32(&mbar[c % 2]));
         }
+        issued = c + 1;
         if (tid < SQ_NT && c + 1 < cpt) load(c + 1);   // while these are issued
     }
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-    if (!bad) {   // the last commit (they complete in issue order)
-        const int c = cpt - 1;
+    if (issued > 0) {   // the last commit (they complete in issue order), also in a block that gives up
+        const int c = issued - 1;
         if (!mbar_wait(smem_u32(&mbar[c % 2]), (uint32_t)((c / 2) & 1))) bad = true;
     }
     bad = __syncthreads_or(bad);
@@ -533,7 +543,7 @@ struct GridDiv {
 template <int COUT>
 __global__ void __launch_bounds__(TC_M) k_conv_wgrad_tc(Grid g, GridDiv gd, int cin, const bf16* __restrict__ x,
                                                        const bf16* __restrict__ dy, float* __restrict__ dw,
-                                                       int* __restrict__ err)
+                                                       long long limit, int* __restrict__ err)
 {
     constexpr int B_BYTES = COUT * 2 * WG_STEP;
     constexpr int NCOL = COUT <= 32 ? 32 : (COUT <= 64 ? 64 : 128);
@@ -579,7 +589,7 @@ __global__ void __launch_bounds__(TC_M) k_conv_wgrad_tc(Grid g, GridDiv gd, int 
     auto prefetch = [&](int k) {
         const int st = k % WG_STAGES;
         if (k >= WG_STAGES) {
-            if (!mbar_wait(smem_u32(&mbar[st]), (uint32_t)((k / WG_STAGES - 1) & 1))) abort_flag = 1;
+            if (!mbar_wait(smem_u32(&mbar[st]), (uint32_t)((k / WG_STAGES - 1) & 1), limit)) abort_flag = 1;
         }
         // A: piece p = (node kk, row group r8), r8 fastest (one node's row read contiguously)
         for (int p = tid; p < WG_STEP * r8n; p += TC_M) {
@@ -616,6 +626,7 @@ __global__ void __launch_bounds__(TC_M) k_conv_wgrad_tc(Grid g, GridDiv gd, int 
         if (k < nk) prefetch(k);
         asm volatile("cp.async.commit_group;\n" ::: "memory");
     }
+    int issued = 0;   // steps
     for (int kc = 0; kc < nk; kc++) {
         const int st = kc % WG_STAGES;
         if (kc + WG_AHEAD < nk) prefetch(kc + WG_AHEAD);
@@ -640,11 +651,12 @@ __global__ void __launch_bounds__(TC_M) k_conv_wgrad_tc(Grid g, GridDiv gd, int 
                              smem_u32(&mbar[st]))
                          : "memory");
         }
+        issued = kc + 1;
     }
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-    if (!abort_flag && nk > 0) {
-        const int st = (nk - 1) % WG_STAGES;
-        if (!mbar_wait(smem_u32(&mbar[st]), (uint32_t)(((nk - 1) / WG_STAGES) & 1))) abort_flag = 1;
+    if (issued > 0) {   // the last MMA, also in a block that gives up
+        const int st = (issued - 1) % WG_STAGES;
+        if (!mbar_wait(smem_u32(&mbar[st]), (uint32_t)(((issued - 1) / WG_STAGES) & 1))) abort_flag = 1;
     }
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
@@ -698,7 +710,7 @@ inline size_t ws_smem(int W, int cg, int cout)
 template <int COUT>
 __global__ void __launch_bounds__(WS_NT + 32) k_conv_wgrad_seq(Seq q, int cin, int cg, int most, const bf16* __restrict__ x,
                                                           const bf16* __restrict__ dy, float* __restrict__ dw,
-                                                          int* __restrict__ err)
+                                                          long long limit, int* __restrict__ err)
 {
     constexpr int DX = ws_dx(COUT), N = DX * COUT, TAPS = ws_groups(COUT), USED = TAPS * N;   // a group: DX taps
     constexpr int NCOL = USED <= 128 ? 128 : USED <= 256 ? 256 : 512;
@@ -735,7 +747,10 @@ __global__ void __launch_bounds__(WS_NT + 32) k_conv_wgrad_seq(Seq q, int cin, i
 
     auto load = [&](int k) {
         const int s = k & 1, p0 = ((int)blockIdx.x + k * (int)gridDim.x) * WS_K;
-        if (k >= 2 && !mbar_wait(smem_u32(&mbar[s]), (uint32_t)((k / 2 - 1) & 1))) bad = true;
+        if (k >= 2 && !mbar_wait(smem_u32(&mbar[s]), (uint32_t)((k / 2 - 1) & 1), limit)) {
+            bad = true;
+            return;
+        }
         const int h = tid & 1;
         for (int t = tid >> 1; t < 3 * seg; t += WS_NT / 2) {
             const int dz = t >= 2 * seg ? 2 : t >= seg ? 1 : 0;
@@ -780,6 +795,7 @@ __global__ void __launch_bounds__(WS_NT + 32) k_conv_wgrad_seq(Seq q, int cin, i
         }
     };
     if (nk > 0 && tid < WS_NT) load(0);
+    int issued = 0;   // stages
     for (int k = 0, first = 0; k < nk; k++) {   // first: of the run
         asm volatile("cp.async.wait_group 0;\n" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
@@ -800,10 +816,11 @@ __global__ void __launch_bounds__(WS_NT + 32) k_conv_wgrad_seq(Seq q, int cin, i
             }
             mma_commit(smem_u32(&mbar[k & 1]));
         }
+        issued = k + 1;
         if (tid < WS_NT && k + 1 < nk) load(k + 1);   // while these are issued
         if (k + 1 == nk || k + 1 == first + run) {
             // (commits complete in issue order)
-            if (!mbar_wait(smem_u32(&mbar[k & 1]), (uint32_t)((k / 2) & 1))) bad = true;
+            if (!mbar_wait(smem_u32(&mbar[k & 1]), (uint32_t)((k / 2) & 1), limit)) bad = true;
             bad = __syncthreads_or(bad);
             if (bad) break;
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
@@ -813,6 +830,7 @@ __global__ void __launch_bounds__(WS_NT + 32) k_conv_wgrad_seq(Seq q, int cin, i
         }
     }
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    if (bad && issued > 0) mbar_wait(smem_u32(&mbar[(issued - 1) & 1]), (uint32_t)(((issued - 1) / 2) & 1));
     if (bad && tid == 0 && err) {
         atomicExch(err, 1);
     }
@@ -832,9 +850,10 @@ cudaError_t launch_pack_weights(int cin, int cout, const void* w, void* wpk, cud
 
 int conv_fwd_tc(int nb, const int dims[3], int cin, int cout, const void* x, const void* wpk, const float* bias,
                 int relu, float* y32, int ldy32, int off32, void* y16, int ldy16, int off16, float* scratch,
-                size_t scratch_floats, int* err, void* stream)
+                size_t scratch_floats, int* err, void* stream, bool give_up)
 {
     using namespace tc;
+    const long long limit = give_up ? 0 : TC_SPIN_LIMIT;
     if (nb < 1 || !dims || cin % 16 || cin < 16 || !x || !wpk ||
         !(cout == 16 || cout == 32 || cout == 48 || cout == 64 || cout == 96 || cout == 128))
         return LASTO_ERR_INVALID_ARG;
@@ -865,7 +884,8 @@ int conv_fwd_tc(int nb, const int dims[3], int cin, int cout, const void* x, con
         if (cudaFuncSetAttribute(k_conv_seq<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) !=         \
             cudaSuccess)                                                                                            \
             return LASTO_ERR_CUDA;                                                                                  \
-        k_conv_seq<C><<<tiles, SQ_NT + 32, sm, s>>>(q, cin, cout, X, W, bias, relu, y32, ldy32, off32, Y16, ldy16, off16, err); \
+        k_conv_seq<C><<<tiles, SQ_NT + 32, sm, s>>>(q, cin, cout, X, W, bias, relu, y32, ldy32, off32, Y16, ldy16, off16,  \
+                                                    limit, err);                                                    \
         break;
         switch (cout / half) {
             LASTO_SQ_CASE(16)
@@ -878,7 +898,8 @@ int conv_fwd_tc(int nb, const int dims[3], int cin, int cout, const void* x, con
     }
 #define LASTO_TC_CASE(C)                                                                                           \
     case C:                                                                                                        \
-        k_conv_tc<C><<<grid, TC_M, 0, s>>>(g, cin, X, W, bias, relu, y32, ldy32, off32, Y16, ldy16, off16, part, err); \
+        k_conv_tc<C><<<grid, TC_M, 0, s>>>(g, cin, X, W, bias, relu, y32, ldy32, off32, Y16, ldy16, off16, part,   \
+                                           limit, err);                                                            \
         break;
     switch (cout) {
         LASTO_TC_CASE(16)
@@ -899,9 +920,10 @@ int conv_fwd_tc(int nb, const int dims[3], int cin, int cout, const void* x, con
 }
 
 int conv_wgrad_tc(int nb, const int dims[3], int cin, int cout, const void* x, const void* dy16, float* dw,
-                  int* err, void* stream)
+                  int* err, void* stream, bool give_up)
 {
     using namespace tc;
+    const long long limit = give_up ? 0 : TC_SPIN_LIMIT;
     if (nb < 1 || !dims || cin % 16 || cin < 16 || cin > 128 || !x || !dy16 || !dw ||
         !(cout == 16 || cout == 32 || cout == 48 || cout == 64 || cout == 96 || cout == 128))
         return LASTO_ERR_INVALID_ARG;
@@ -931,7 +953,7 @@ int conv_wgrad_tc(int nb, const int dims[3], int cin, int cout, const void* x, c
         if (cudaFuncSetAttribute(k_conv_wgrad_seq<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) !=     \
             cudaSuccess)                                                                                              \
             return LASTO_ERR_CUDA;                                                                                    \
-        k_conv_wgrad_seq<C><<<grid, WS_NT + 32, sm, s>>>(q, cin, cg, most, X, DY, dw, err);                                 \
+        k_conv_wgrad_seq<C><<<grid, WS_NT + 32, sm, s>>>(q, cin, cg, most, X, DY, dw, limit, err);                    \
         break;
         switch (cout) {
             LASTO_WS_CASE(16)
@@ -949,7 +971,7 @@ int conv_wgrad_tc(int nb, const int dims[3], int cin, int cout, const void* x, c
         if (cudaFuncSetAttribute(k_conv_wgrad_tc<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, wg_smem(C)) != \
             cudaSuccess)                                                                                 \
             return LASTO_ERR_CUDA;                                                                       \
-        k_conv_wgrad_tc<C><<<grid, TC_M, wg_smem(C), s>>>(g, gd, cin, X, DY, dw, err);                     \
+        k_conv_wgrad_tc<C><<<grid, TC_M, wg_smem(C), s>>>(g, gd, cin, X, DY, dw, limit, err);               \
         break;
     switch (cout) {
         LASTO_WG_CASE(16)

@@ -607,6 +607,16 @@ int lasto_nn_conv3d_wgrad_tc(int nb, const int dims[3], int cin, int cout, const
     return cudaGetLastError() == cudaSuccess ? LASTO_OK : LASTO_ERR_CUDA;
 }
 
+int lasto_selftest_conv_wait(int which, int nb, const int dims[3], int cin, int cout, const void* x, const void* m, float* out,
+                             int* err, void* stream)
+{
+    if ((which != 0 && which != 1) || !dims || !x || !m || !out || !err) return LASTO_ERR_INVALID_ARG;
+    if (which == 0)
+        return lasto::conv_fwd_tc(nb, dims, cin, cout, x, m, nullptr, 0, out, cout, 0, nullptr, 0, 0, nullptr, 0, err, stream,
+                                  true);
+    return lasto::conv_wgrad_tc(nb, dims, cin, cout, x, m, out, err, stream, true);
+}
+
 int lasto_nn_relu_grad(size_t n, const float* y, const float* dy, float* dx, void* dx16, void* stream)
 {
     // (four values per thread where every array is in whole 16-byte pieces, the BF16 one in 8-byte ones)
