@@ -103,13 +103,12 @@ __global__ void __launch_bounds__(TC_M) k_conv_tc(Grid g, int cin, const bf16* _
     __shared__ __align__(1024) unsigned char sB[TC_STAGES][B_BYTES];
     __shared__ __align__(8) unsigned long long mbar[TC_STAGES];
     __shared__ uint32_t tmem_slot;
-    __shared__ int abort_flag;
+    bool bad = false;   // a wait ran out
     const int tid = threadIdx.x, warp = tid >> 5;
     const size_t N = g.nodes();
     const size_t node0 = (size_t)blockIdx.x * TC_M;
 
     if (tid == 0) {
-        abort_flag = 0;
         for (int s = 0; s < TC_STAGES; s++)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&mbar[s])) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -150,7 +149,7 @@ __global__ void __launch_bounds__(TC_M) k_conv_tc(Grid g, int cin, const bf16* _
     auto prefetch = [&](int k) {
         const int st = k % TC_STAGES;
         if (k >= TC_STAGES) {
-            if (!mbar_wait(smem_u32(&mbar[st]), (uint32_t)((k / TC_STAGES - 1) & 1), limit)) abort_flag = 1;
+            if (!mbar_wait(smem_u32(&mbar[st]), (uint32_t)((k / TC_STAGES - 1) & 1), limit)) bad = true;
         }
         const int tap = tap_a + k / cpt, c0 = (k % cpt) * 16;
         const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
@@ -182,8 +181,8 @@ __global__ void __launch_bounds__(TC_M) k_conv_tc(Grid g, int cin, const bf16* _
         asm volatile("cp.async.wait_group %0;\n" ::"n"(TC_AHEAD) : "memory");   // step kc's copies have landed
         // make the shared-memory writes visible to the tensor core (async proxy)
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-        __syncthreads();
-        if (abort_flag) break;
+        bad = __syncthreads_or(bad);   // (every thread leaves at the same step)
+        if (bad) break;
         if (tid == 0) {
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
             const uint64_t ad = make_desc(smem_u32(sA[s])), bd = make_desc(smem_u32(sB[s]));
@@ -202,11 +201,11 @@ __global__ void __launch_bounds__(TC_M) k_conv_tc(Grid g, int cin, const bf16* _
     // wait for the last MMA (commits complete in issue order), also in a block that gives up
     if (issued > 0) {
         const int s = (issued - 1) % TC_STAGES;
-        if (!mbar_wait(smem_u32(&mbar[s]), (uint32_t)(((issued - 1) / TC_STAGES) & 1))) abort_flag = 1;
+        if (!mbar_wait(smem_u32(&mbar[s]), (uint32_t)(((issued - 1) / TC_STAGES) & 1))) bad = true;
     }
-    __syncthreads();
+    bad = __syncthreads_or(bad);
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    if (!abort_flag) {
+    if (!bad) {
         const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);
         float acc[COUT];
 #pragma unroll
@@ -552,7 +551,7 @@ __global__ void __launch_bounds__(TC_M) k_conv_wgrad_tc(Grid g, GridDiv gd, int 
     unsigned char* sB = wg_smem_raw + WG_STAGES * WG_A_BYTES;      // [WG_STAGES][B_BYTES]
     __shared__ __align__(8) unsigned long long mbar[WG_STAGES];
     __shared__ uint32_t tmem_slot;
-    __shared__ int abort_flag;
+    bool bad = false;   // a wait ran out
     const int tid = threadIdx.x, warp = tid >> 5;
     const size_t N = g.nodes();
     const size_t node0 = (size_t)blockIdx.x * WG_CHUNK;
@@ -565,7 +564,6 @@ __global__ void __launch_bounds__(TC_M) k_conv_wgrad_tc(Grid g, GridDiv gd, int 
     for (int t = tid; t < WG_STAGES * (WG_A_BYTES + B_BYTES) / 16; t += TC_M)
         reinterpret_cast<uint4*>(wg_smem_raw)[t] = make_uint4(0, 0, 0, 0);
     if (tid == 0) {
-        abort_flag = 0;
         for (int st = 0; st < WG_STAGES; st++)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&mbar[st])) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -589,7 +587,7 @@ __global__ void __launch_bounds__(TC_M) k_conv_wgrad_tc(Grid g, GridDiv gd, int 
     auto prefetch = [&](int k) {
         const int st = k % WG_STAGES;
         if (k >= WG_STAGES) {
-            if (!mbar_wait(smem_u32(&mbar[st]), (uint32_t)((k / WG_STAGES - 1) & 1), limit)) abort_flag = 1;
+            if (!mbar_wait(smem_u32(&mbar[st]), (uint32_t)((k / WG_STAGES - 1) & 1), limit)) bad = true;
         }
         // A: piece p = (node kk, row group r8), r8 fastest (one node's row read contiguously)
         for (int p = tid; p < WG_STEP * r8n; p += TC_M) {
@@ -633,8 +631,8 @@ __global__ void __launch_bounds__(TC_M) k_conv_wgrad_tc(Grid g, GridDiv gd, int 
         asm volatile("cp.async.commit_group;\n" ::: "memory");
         asm volatile("cp.async.wait_group %0;\n" ::"n"(WG_AHEAD) : "memory");
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-        __syncthreads();
-        if (abort_flag) break;
+        bad = __syncthreads_or(bad);   // (every thread leaves at the same step)
+        if (bad) break;
         if (tid == 0) {
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
 #pragma unroll
@@ -656,11 +654,11 @@ __global__ void __launch_bounds__(TC_M) k_conv_wgrad_tc(Grid g, GridDiv gd, int 
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
     if (issued > 0) {   // the last MMA, also in a block that gives up
         const int st = (issued - 1) % WG_STAGES;
-        if (!mbar_wait(smem_u32(&mbar[st]), (uint32_t)(((issued - 1) / WG_STAGES) & 1))) abort_flag = 1;
+        if (!mbar_wait(smem_u32(&mbar[st]), (uint32_t)(((issued - 1) / WG_STAGES) & 1))) bad = true;
     }
-    __syncthreads();
+    bad = __syncthreads_or(bad);
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    if (!abort_flag && nk > 0) {
+    if (!bad && nk > 0) {
         // thread tid owns accumulator row m = tid (tensor-memory lane tid)
         const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);
         float acc[COUT];
@@ -674,7 +672,7 @@ __global__ void __launch_bounds__(TC_M) k_conv_wgrad_tc(Grid g, GridDiv gd, int 
 #pragma unroll
             for (int c = 0; c < COUT; c++) atomicAdd(dst + c, acc[c]);
         }
-    } else if (abort_flag && tid == 0 && err) {
+    } else if (bad && tid == 0 && err) {
         atomicExch(err, 1);
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
