@@ -691,7 +691,8 @@ __global__ void __launch_bounds__(TC_M) k_conv_wgrad_tc(Grid g, GridDiv gd, int 
 // by eight warps while a ninth issues; a CTA takes every gridDim.x-th one, and adds its sums to dw
 // with vector reductions, at the latest after `most` stages: the tensor core's FP32 accumulation
 // truncates, so its error grows with the length of a sum (positive values, 64 x 64 channels on 8 grids
-// of 33^3: 1.7e-5 of the largest with one sum per CTA, 3.6e-6 so, the gathered form's 3.8e-6).  Bound: 32-byte pieces from L2 (3 to 4 TB/s; three or four
+// of 33^3: 1.7e-5 of the largest and 245 us with one sum per CTA, 3.6e-6 and 258 us so; 3.8e-6 in the
+// gathered form).  Bound: 32-byte pieces from L2 (3 to 4 TB/s; three or four
 // buffers, or 16 loading warps, change nothing).  8 grids of 33^3, against the kernel above (27
 // gathered rows per node): 48 x 16 channels 330 -> 57 us.
 constexpr int WS_K = 128, WS_NT = 256;
@@ -703,6 +704,22 @@ inline size_t ws_smem(int W, int cg, int cout)
 {
     // two buffers, and what the unused rows of the second one's operand read beyond it
     return 2 * ((size_t)cg / 8 * 3 * ws_seg(W) * 16 + (size_t)ws_dx(cout) * cout / 8 * WS_K * 16) + (size_t)(64 - cg) / 8 * 3 * ws_seg(W) * 16;
+}
+
+// One element's sum over the stages k0 .. k1 - 1 of a CTA from the nodes themselves: output node at
+// position p - e, input node one tap away.
+__device__ __noinline__ float ws_node_sum(const Seq& q, int k0, int k1, int e, int tap, const bf16* __restrict__ x, int cin,
+                                          const bf16* __restrict__ dy, int cout)
+{
+    const int shift = (tap / 9 - 1) * q.plane + (tap / 3 % 3 - 1) * q.pitch + tap % 3 - 1;
+    float s = 0.0f;
+    for (int k = k0; k < k1; k++)
+        for (int i = 0; i < WS_K; i++) {
+            const int p = ((int)blockIdx.x + k * (int)gridDim.x) * WS_K + i - e;
+            const int out = seq_node(q, p), in = seq_node(q, p + shift);
+            if (out >= 0 && in >= 0) s = fmaf(__bfloat162float(x[(size_t)in * cin]), __bfloat162float(dy[(size_t)out * cout]), s);
+        }
+    return s;
 }
 
 template <int COUT>
@@ -767,7 +784,9 @@ __global__ void __launch_bounds__(WS_NT + 32) k_conv_wgrad_seq(Seq q, int cin, i
         asm volatile("cp.async.commit_group;\n" ::: "memory");
     };
     // the sums of a run into dw.  An M = 64 accumulator: row r in tensor-memory lane 32 (r / 16) + r % 16
-    auto drain = [&]() {
+    // A NaN may come from a pad alone (its 0 times an infinity at the grid's edge): such elements are formed
+    // again without the pads.
+    auto drain = [&](int k0, int k1) {
         const int row = (warp & 3) * 16 + (lane & 15);
         const bool live = lane < 16 && row < cg, vec = ((uintptr_t)dw & 15) == 0;
         const uint32_t lane_base = tmem + ((uint32_t)((warp & 3) * 32) << 16);
@@ -780,7 +799,15 @@ __global__ void __launch_bounds__(WS_NT + 32) k_conv_wgrad_seq(Seq q, int cin, i
                 tmem_ld16(lane_base + (uint32_t)(t * COUT + c), v);
                 asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
                 if (!live) continue;
-                if (vec) {
+                bool nan = false;
+#pragma unroll
+                for (int j = 0; j < 16; j++) nan |= v[j] != v[j];
+                if (nan) {
+#pragma unroll 1
+                    for (int j = 0; j < 16; j++)
+                        atomicAdd(dst + c + j, ws_node_sum(q, k0, k1, DX == 3 ? t % 3 - 1 : 0, tap0 * DX + t, x + c0 + row, cin,
+                                                           dy + c + j, COUT));
+                } else if (vec) {
 #pragma unroll
                     for (int j = 0; j < 16; j += 4)
                         asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};\n" ::"l"(dst + c + j), "f"(v[j]),
@@ -822,7 +849,7 @@ __global__ void __launch_bounds__(WS_NT + 32) k_conv_wgrad_seq(Seq q, int cin, i
             bad = __syncthreads_or(bad);
             if (bad) break;
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-            drain();
+            drain(first, k + 1);
             asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");   // (the next stage's barrier)
             first = k + 1;
         }

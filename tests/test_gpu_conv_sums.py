@@ -52,3 +52,28 @@ def test_long_sums(cin, cout, nb, dims):
     # half the whole on average; then one rounded FP32 addition (2^-24) per such sum
     tol = 2.0 ** -24 * (2048 / 16 + N / 2048 + 1)
     assert float(((got - ref) / ref).abs().max()) <= tol
+
+
+@pytest.mark.parametrize("cin,cout,nb,dims", [(16, 16, 2, (7, 8, 9)), (48, 16, 2, (7, 8, 9)), (32, 32, 2, (7, 8, 9)),
+                                              (128, 64, 1, (5, 3, 4)), (32, 96, 1, (9, 5, 6)), (64, 64, 4, (33, 33, 33))])
+@pytest.mark.parametrize("where", ["x", "dy"])
+def test_infinities_at_the_edges(cin, cout, nb, dims, where):
+    """An infinity at a corner, an edge and a face of a grid reaches the taps that have a partner for it
+    inside the grid, and no others."""
+    import torch
+    B = need_gpu()
+    W, H, D = dims
+    g = torch.Generator(device="cuda").manual_seed(cin)
+    x = torch.randn(nb, D, H, W, cin, generator=g, device="cuda").bfloat16()
+    dy = torch.randn(nb, D, H, W, cout, generator=g, device="cuda").bfloat16()
+    t = x if where == "x" else dy
+    t[0, 0, 0, 0, 1] = float("inf")
+    t[nb - 1, D - 1, 1, W - 1, 2] = -float("inf")
+    t[0, 1, H - 1, 2, 3] = float("inf")
+    x, dy = x.view(-1, cin), dy.view(-1, cout)
+    got, ref = wgrad(B, x, dy, nb, dims, cin, cout).double(), wgrad_ref(x, dy, nb, dims)
+    assert bool(ref.isinf().any()) and bool(ref.isfinite().any())
+    assert torch.equal(got.isnan(), ref.isnan()) and torch.equal(got.isinf(), ref.isinf())
+    assert torch.equal(got[ref.isinf()], ref[ref.isinf()])
+    ok = ref.isfinite()
+    assert float((got[ok] - ref[ok]).abs().max()) <= 2e-5 * float(ref[ok].abs().max())
