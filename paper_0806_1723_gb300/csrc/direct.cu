@@ -21,12 +21,23 @@ namespace lasto {
 // Martin, Reinsch and Wilkinson, 1968) on S scaled by its largest element, in the precision of the
 // cycle it serves.  Q is a product of plane rotations, so it is orthogonal whatever the axis --
 // also for the near-degenerate pairs of an axis with two refined regions -- and e = Q D Q^T b stays
-// symmetric and definite whatever the rounding, which is all the conjugate gradients ask of their
-// preconditioner.  One lane runs the scalar chain (a rotation is about ten dependent operations)
+// symmetric whatever the rounding.  Definite, which the conjugate gradients also ask of their
+// preconditioner, it is because every eigenvalue is held at or below -8 / length^2: the operator is
+// exact for quadratics, so its inverse of -1 is (x - x_0)(x_1 - x) / 2 <= length^2 / 8, which bounds the
+// norm of the inverse.  QL's errors are a small multiple (0.2 to 2.5 seen) of eps times the largest
+// element, so a strongly graded axis, whose smallest eigenvalues FP32 would lose, is done in FP64
+// also for the FP32 cycle (EIG_WIDE; such solves take 100 iterations and more).
+// One lane runs the scalar chain (a rotation is about ten dependent operations)
 // and the other warps apply the rotations of the QL step before to Q, a component per thread.
 // Bound: that chain's latency; it runs beside the deposit.  Parallel cyclic Jacobi in the same
 // place took 697 us at m = 63; this 253 us (m = 95: 510 us; FP64: 279 us at m = 15, 900 us at m = 31).
 constexpr int EIG_NT = 128;
+// FP64 where FP32's eps times the largest element passes this part of the bound on the smallest
+// eigenvalue: below it that eigenvalue is right to about a seventh.  On 129 nodes over 80 bohr that is at a
+// ratio of spacings of 200, where both take 140 iterations (23.9 ms in FP32, 26.3 in FP64: 2.4 ms at
+// m = 63, 5.5 at 95); one axis with four cells 1000 times finer than the rest: FP32 diverges, FP64
+// 139 iterations (the smoothed hierarchy without this level: 148).
+constexpr double EIG_WIDE = 1.0 / 16;
 static_assert(DIRECT_MAX <= EIG_NT - 32, "a component of Q per applying thread");
 
 // the hardware's approximate reciprocal square root; FP64: about 20 bits of it and one third-order
@@ -45,29 +56,23 @@ __device__ __forceinline__ double inv_sqrt(double v)
     return fma(s * h, fma(h, 0.375, 0.5), s);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(EIG_NT) k_direct_eig(AxisStore ax0, AxisStore ax1, AxisStore ax2, DirectMats<T> out, int mp)
+// T: the precision of the iteration; big: S's largest element, low: the bound on its smallest
+template <typename T, typename O>
+__device__ __forceinline__ void direct_eig_axis(const AxisStore& A, T* Q, const DirectMats<O>& out, int dim, int mp, double big,
+                                                double low)
 {
-    extern __shared__ __align__(16) unsigned char eig_sm[];
     __shared__ T d[DIRECT_MAX + 1], e[DIRECT_MAX + 1], rc[2][DIRECT_MAX + 1], rs[2][DIRECT_MAX + 1];
-    __shared__ T s_scale;
     // per turn, in two buffers: rotations of columns (i, i + 1), i = hi - 1 .. lo, and whether it was the last
     __shared__ int r_hi[2], r_lo[2], s_done[2];
-    const int dim = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
-    const AxisStore& A = dim == 0 ? ax0 : dim == 1 ? ax1 : ax2;
+    const int tid = threadIdx.x, lane = tid & 31;
     const int m = A.n - 2, ld = m + 1 - (m & 1);
-    T* Q = reinterpret_cast<T*>(eig_sm);       // [m][ld]: row i holds eigenvector i
-    for (int t = tid; t < m * ld; t += EIG_NT) Q[t] = t / ld == t % ld ? (T)1 : (T)0;
-    if (tid == 0) {
-        double big = 0.0;
-        for (int i = 0; i < m; i++) big = fmax(big, A.dg[i + 1]);
-        s_scale = (T)big;
-        r_hi[0] = r_hi[1] = r_lo[0] = r_lo[1] = 0;
-    }
+    const T scale = (T)big;
+    for (int t = tid; t < m * ld; t += EIG_NT) Q[t] = t / ld == t % ld ? (T)1 : (T)0;   // [m][ld]: row i holds eigenvector i
+    if (tid == 0) r_hi[0] = r_hi[1] = r_lo[0] = r_lo[1] = 0;
     __syncthreads();
     for (int i = tid; i < m; i += EIG_NT) {
-        d[i] = (T)(-A.dg[i + 1] / (double)s_scale);
-        e[i] = i + 1 < m ? (T)(sqrt(A.cp[i + 1] * A.cm[i + 2]) / (double)s_scale) : (T)0;
+        d[i] = (T)(-A.dg[i + 1] / (double)scale);
+        e[i] = i + 1 < m ? (T)(sqrt(A.cp[i + 1] * A.cm[i + 2]) / (double)scale) : (T)0;
     }
     __syncthreads();
     const T eps = sizeof(T) == 4 ? (T)6e-8 : (T)1.1e-16;
@@ -154,10 +159,33 @@ __global__ void __launch_bounds__(EIG_NT) k_direct_eig(AxisStore ax0, AxisStore 
         const int p = t / mp, i = t - p * mp;
         const bool in = p < m && i < m;
         const T sv = in ? (T)sqrt(A.dual[i + 1]) : (T)1, v = in ? Q[p * ld + i] : (T)0;
-        out.Bt[dim][p * mp + i] = v / sv;
-        out.Ft[dim][i * mp + p] = v * sv;
+        out.Bt[dim][p * mp + i] = (O)(v / sv);
+        out.Ft[dim][i * mp + p] = (O)(v * sv);
     }
-    for (int p = tid; p < m; p += EIG_NT) out.lam[dim][p] = d[p] * s_scale;
+    for (int p = tid; p < m; p += EIG_NT) {
+        const O v = (O)(d[p] * scale), most = (O)-low;
+        out.lam[dim][p] = v > most ? most : v;   // (a NaN stays one)
+    }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(EIG_NT) k_direct_eig(AxisStore ax0, AxisStore ax1, AxisStore ax2, DirectMats<T> out, int mp)
+{
+    extern __shared__ __align__(16) unsigned char eig_sm[];
+    __shared__ double s_big;
+    const int dim = blockIdx.x;
+    const AxisStore& A = dim == 0 ? ax0 : dim == 1 ? ax1 : ax2;
+    if (threadIdx.x == 0) {
+        double big = 0.0;
+        for (int i = 1; i <= A.n - 2; i++) big = fmax(big, A.dg[i]);
+        s_big = big;
+    }
+    __syncthreads();
+    const double big = s_big, length = A.c[A.n - 1] - A.c[0], low = 8.0 / (length * length);
+    if (sizeof(T) == 4 && 6e-8 * big > EIG_WIDE * low)
+        direct_eig_axis(A, reinterpret_cast<double*>(eig_sm), out, dim, mp, big, low);
+    else
+        direct_eig_axis(A, reinterpret_cast<T*>(eig_sm), out, dim, mp, big, low);
 }
 
 // padded size of the transform matrices
@@ -171,7 +199,7 @@ template <typename T>
 cudaError_t launch_direct_eig(const LevelStore& L, const DirectMats<T>& out, cudaStream_t s)
 {
     const size_t m = (size_t)std::max(L.n[0], std::max(L.n[1], L.n[2])) - 2;
-    k_direct_eig<T><<<3, EIG_NT, sizeof(T) * m * (m + 1), s>>>(L.ax[0], L.ax[1], L.ax[2], out, direct_pad(L.n));
+    k_direct_eig<T><<<3, EIG_NT, sizeof(double) * m * (m + 1), s>>>(L.ax[0], L.ax[1], L.ax[2], out, direct_pad(L.n));
     return cudaGetLastError();
 }
 template cudaError_t launch_direct_eig<float>(const LevelStore&, const DirectMats<float>&, cudaStream_t);
