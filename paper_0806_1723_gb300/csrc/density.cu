@@ -397,6 +397,9 @@ constexpr int DT_X = 8, DT_Y = 8, DT_Z = 8;
 static_assert(DT_X * DT_Y * DT_Z == 2 * DEP_NT, "deposit tile = one block");
 constexpr int DF_MAX_ATOMS = 2431;   // most atoms the FP32-pair form takes (four index lists in shared memory)
 
+// bytes of a launch's index lists
+static size_t deposit_smem(bool mixed, int na) { return sizeof(int) * (mixed ? 4 : 2) * (size_t)na; }
+
 cudaError_t launch_deposit(const lasto_cluster& cl, const double* rec, int precision, double* b, int* owner,
                            const double* /*xm_tab*/, double* /*row_mom*/, int* status, cudaStream_t s)
 {
@@ -419,9 +422,9 @@ cudaError_t launch_deposit(const lasto_cluster& cl, const double* rec, int preci
                     (unsigned)((cl.n[2] + DT_Z - 1) / DT_Z));
     if (grid.y > 65535 || grid.z > 65535) return cudaErrorInvalidValue;
     if (mixed)
-        k_deposit_df<<<grid, DEP_NT, sizeof(int) * 4 * (size_t)cl.n_atoms, s>>>(a);
+        k_deposit_df<<<grid, DEP_NT, deposit_smem(true, a.na), s>>>(a);
     else
-        k_deposit64<<<grid, DEP_NT, sizeof(int) * 2 * (size_t)cl.n_atoms, s>>>(a);
+        k_deposit64<<<grid, DEP_NT, deposit_smem(false, a.na), s>>>(a);
     return cudaGetLastError();
 }
 
@@ -1248,15 +1251,19 @@ void init_device_constants()
         std::lock_guard<std::mutex> lock(g_constants_mutex);
         if (g_constants_done[dev]) return;
     }
-    ensure_monomials();
-    cudaFuncSetAttribute(k_deposit64, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    cudaFuncSetAttribute(k_deposit_df, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    // the index lists of the largest cluster.  (Dynamic and static memory share one limit: a request beyond
+    // it is refused, and the kernel keeps the default, 48 KiB for both.)
+    bool ok = ensure_monomials() == cudaSuccess;
+    ok = cudaFuncSetAttribute(k_deposit64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)deposit_smem(false, DEP64_MAX_ATOMS)) ==
+             cudaSuccess && ok;
+    ok = cudaFuncSetAttribute(k_deposit_df, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)deposit_smem(true, DF_MAX_ATOMS)) ==
+             cudaSuccess && ok;
     init_mg_attributes();
     init_direct_attributes();
     init_slab_attributes();
     init_wave_attributes();
     std::lock_guard<std::mutex> lock(g_constants_mutex);
-    g_constants_done[dev] = true;
+    g_constants_done[dev] = ok;   // (else the next call tries again)
 }
 
 // ---------------------------------------------------------------- boundary multipoles
