@@ -1132,6 +1132,10 @@ __global__ void __launch_bounds__(DEP_NT, 3) k_deposit_df(DepArgs a)
                     }
                 }
             }
+            // the low parts gather the terms below the high parts' last place: kept small, as their own
+            // rounding is FP32
+            sA = dfa::fast_two_sum(sA.h, sA.l);
+            sB = dfa::fast_two_sum(sB.h, sB.l);
         }
     }
 

@@ -15,14 +15,26 @@ def _lattice(na, k):
 # around the atoms whose lists fit beside the kernels' static memory in the default 48 KiB, and the most
 @pytest.mark.parametrize("precision,na,tol", [(1, 1276, 1e-11), (1, 1277, 1e-11), (1, 2431, 1e-11), (0, 1277, 1e-12),
                                               (0, 1828, 1e-12)])
-def test_deposit(orc, precision, na, tol):
+def test_deposit(precision, na, tol):
+    """Owners everywhere and the values outside the spheres, which are the Slater sums themselves,
+    against 64 bits."""
+    import torch
     B = need_gpu()
-    cl = synth.workloads.make_cluster("lattice", 1.25 * _lattice(na, 14) - 8.125, np.random.default_rng(na), n=17, half_width=12.0,
-                                      h_min=1.5, h_max=1.5)
-    cl.R[:] = 0.6
-    x = np.linspace(-12.0, 12.0, 17)
-    ref, rowner = orc.deposit(cl, x, x, x)
+    cl = synth.workloads.make_cluster("lattice", 1.5 * _lattice(na, 14) - 9.75, np.random.default_rng(na), n=33, half_width=12.0,
+                                      h_min=0.75, h_max=0.75)
+    cl.R[:] = 0.7
+    x = np.linspace(-12.0, 12.0, 33)
     b, owner, status = B.lasto_op_deposit(B.DeviceCluster(cl, axes=(x, x, x)), precision=precision)
-    assert host(status)[0] == 0
-    assert np.array_equal(host(owner), rowner)
-    assert np.abs(host(b) - ref).max() < tol * np.abs(ref).max()   # the bound of the deposit's own tests
+    assert host(status)[0] == 0 and bool(torch.isfinite(b).all())
+    t = torch.as_tensor(x, device="cuda")
+    ref, own = torch.zeros(33 ** 3, dtype=torch.float64, device="cuda"), torch.full((33 ** 3,), -1, dtype=torch.int32, device="cuda")
+    for a in range(na):
+        p = cl.pos[a]
+        r = ((t[None, None, :] - p[0]) ** 2 + (t[None, :, None] - p[1]) ** 2 + (t[:, None, None] - p[2]) ** 2).sqrt().view(-1)
+        own[r < cl.R[a]] = a
+        for w, z in zip(cl.slater_w[a], cl.slater_zeta[a]):
+            ref += 4 * np.pi * w * z ** 3 / (8 * np.pi) * torch.exp(-z * r)
+    assert torch.equal(owner.view(-1), own)
+    out = own < 0
+    # the bound of the deposit's own tests
+    assert float((b.view(-1)[out] - ref[out]).abs().max()) < tol * float(ref[out].max())
