@@ -392,10 +392,10 @@ constexpr float DF_EXP_CUT = 37.0f;
 
 // one 8 x 8 x 8 tile of nodes per block, two nodes (four planes apart) per thread
 __global__ void k_deposit64(DepArgs a);
-constexpr int DEP64_MAX_ATOMS = 1828;   // most atoms the FP64 form takes (two index lists in shared memory)
+constexpr int DEP64_MAX_ATOMS = 1828;   // most atoms the FP64 form takes (its two index lists: 14 KiB)
 constexpr int DT_X = 8, DT_Y = 8, DT_Z = 8;
 static_assert(DT_X * DT_Y * DT_Z == 2 * DEP_NT, "deposit tile = one block");
-constexpr int DF_MAX_ATOMS = 2431;   // most atoms the FP32-pair form takes (four index lists in shared memory)
+constexpr int DF_MAX_ATOMS = 2432;      // most atoms the FP32-pair form takes (its four index lists: 38 KiB)
 
 // bytes of a launch's index lists
 static size_t deposit_smem(bool mixed, int na) { return sizeof(int) * (mixed ? 4 : 2) * (size_t)na; }

@@ -13,7 +13,7 @@ def _lattice(na, k):
 
 
 # around the atoms whose lists fit beside the kernels' static memory in the default 48 KiB, and the most
-@pytest.mark.parametrize("precision,na,tol", [(1, 1276, 1e-11), (1, 1277, 1e-11), (1, 2431, 1e-11), (0, 1277, 1e-12),
+@pytest.mark.parametrize("precision,na,tol", [(1, 1276, 1e-11), (1, 1277, 1e-11), (1, 2431, 1e-11), (1, 2432, 1e-11), (0, 1277, 1e-12),
                                               (0, 1828, 1e-12)])
 def test_deposit(precision, na, tol):
     """Owners everywhere and the values outside the spheres, which are the Slater sums themselves,
@@ -38,3 +38,12 @@ def test_deposit(precision, na, tol):
     out = own < 0
     # the bound of the deposit's own tests
     assert float((b.view(-1)[out] - ref[out]).abs().max()) < tol * float(ref[out].max())
+
+
+@pytest.mark.parametrize("precision,na", [(0, 1829), (1, 2433)])
+def test_deposit_refuses_more(precision, na):
+    B = need_gpu()
+    cl = synth.workloads.make_cluster("lattice", 1.5 * _lattice(na, 14) - 9.75, np.random.default_rng(na), n=33, half_width=12.0,
+                                      h_min=0.75, h_max=0.75)
+    with pytest.raises(RuntimeError):
+        B.lasto_op_deposit(B.DeviceCluster(cl, axes=(np.linspace(-12.0, 12.0, 33),) * 3), precision=precision)
