@@ -113,6 +113,7 @@ __device__ __forceinline__ double monopole_at(const double* __restrict__ f, int 
 // runs in whole warps: it is the bound, 10 % of the nodes of Pd55 129^3.  167 us with every sphere
 // tested at every node and the inside nodes in place (214 with the lists alone) -> 119 us.
 constexpr int RD_X = 32, RD_Y = 8, RD_Z = 4;
+constexpr int RD_MAX_ATOMS = 12800;   // most atoms it takes (their list: 50 KiB)
 
 __global__ void __launch_bounds__(RD_X * RD_Y) k_raw_deposit(RawArgs a, const double* __restrict__ rec,
                                                             double* __restrict__ b, int* __restrict__ owner,
@@ -222,11 +223,13 @@ cudaError_t launch_raw_sphere_params(const RawArgs& a, double* rec, int* status,
 cudaError_t launch_raw_deposit(const RawArgs& a, const double* rec, double* b, int* owner, int* status, cudaStream_t s)
 {
     const size_t N = (size_t)a.n[0] * a.n[1] * a.n[2];
-    // (up to 12 800 atoms)
-    if (sizeof(float4) * (size_t)a.na > 200 * 1024 || N >= (size_t(1) << 31)) return cudaErrorInvalidValue;
+    if (a.na > RD_MAX_ATOMS || N >= (size_t(1) << 31)) return cudaErrorInvalidValue;
     const size_t smem = sizeof(int) * (size_t)a.na;
-    if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(k_raw_deposit, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (the default 48 KiB holds the static memory, 4 KiB, too; always the same request, whatever other
+    // threads ask for)
+    if (smem > 40 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(k_raw_deposit, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)(sizeof(int) * RD_MAX_ATOMS));
         if (e != cudaSuccess) return e;
     }
     const size_t g = (size_t)((a.n[0] + RD_X - 1) / RD_X) * ((a.n[1] + RD_Y - 1) / RD_Y) * ((a.n[2] + RD_Z - 1) / RD_Z);

@@ -47,3 +47,29 @@ def test_deposit_refuses_more(precision, na):
                                       h_min=0.75, h_max=0.75)
     with pytest.raises(RuntimeError):
         B.lasto_op_deposit(B.DeviceCluster(cl, axes=(np.linspace(-12.0, 12.0, 33),) * 3), precision=precision)
+
+
+# around the list that fits beside the static memory in the default 48 KiB and the one that fits alone
+@pytest.mark.parametrize("na", [10240, 11300, 12288, 12800])
+def test_raw_deposit(orc, na):
+    B = need_gpu()
+    rng = np.random.default_rng(na)
+    pos, Z, R = _lattice(na, 24) + 0.5, rng.uniform(1, 50, size=na), np.full(na, 0.4)
+    x = np.concatenate([[-0.3, -0.2], np.linspace(0.0, 24.0, 17), [24.2, 24.3]])
+    r = 0.4 * np.exp(np.linspace(np.log(1e-5 / 0.4), 0.0, 16))
+    rho00 = rng.uniform(1, 9, size=(na, 1)) * np.exp(-3.0 * r)[None]
+    ne = rng.uniform(0, 2, size=(21, 21, 21))
+    ref, rowner = orc.raw_deposit(pos, Z, R, x, x, x, ne, rho00)
+    b, owner, status = B.lasto_op_raw_deposit(B.RawCluster(pos, Z, R, x, x, x, (0, 0, 0), ne, rho00))
+    assert int(host(status)[0]) == 0
+    assert np.array_equal(host(owner).reshape(rowner.shape), rowner)
+    assert np.abs(host(b).reshape(ref.shape) - ref).max() < 1e-12 * np.abs(ref).max()   # the bound of the kernel's own test
+
+
+def test_raw_deposit_refuses_more():
+    B = need_gpu()
+    x = np.linspace(0.0, 24.0, 9)
+    rc = B.RawCluster(_lattice(12801, 24) + 0.5, np.ones(12801), np.full(12801, 0.4), x, x, x, (0, 0, 0), np.ones((9, 9, 9)),
+                      np.ones((12801, 16)))
+    with pytest.raises(RuntimeError):
+        B.lasto_op_raw_deposit(rc)
