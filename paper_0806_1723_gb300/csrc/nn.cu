@@ -221,9 +221,11 @@ __global__ void __launch_bounds__(256) k_bias_grad(size_t N, int cout, int rows,
     }
     __syncthreads();
     if (t < cout) {
-        float s = 0.0f;
-        for (int r = 0; r < per; r++) s += sm[r * cout + t];
-        atomicAdd(db + t, s);
+        float p[8] = {};   // (a serial sum of the up to 64 rows would round 64 times)
+        for (int r = 0; r < per; r += 8)
+#pragma unroll
+            for (int q = 0; q < 8; q++) p[q] += r + q < per ? sm[(r + q) * cout + t] : 0.0f;
+        atomicAdd(db + t, ((p[0] + p[1]) + (p[2] + p[3])) + ((p[4] + p[5]) + (p[6] + p[7])));
     }
 }
 

@@ -77,3 +77,29 @@ def test_infinities_at_the_edges(cin, cout, nb, dims, where):
     assert torch.equal(got[ref.isinf()], ref[ref.isinf()])
     ok = ref.isfinite()
     assert float((got[ok] - ref[ok]).abs().max()) <= 2e-5 * float(ref[ok].abs().max())
+
+
+def test_bias_gradient_sums_pairwise():
+    """64 rows of a block whose serial FP32 sum would round down by almost half a last place each time."""
+    import numpy as np
+    import torch
+    B = need_gpu()
+    v = [1.5]
+    s = np.float32(1.5)
+    for _ in range(63):
+        ulp = float(np.spacing(s + np.float32(1.25)))
+        x = 1.25
+        if ulp > 2.0 ** -22:
+            x += (ulp / 2 - 2.0 ** -23 - (float(s) + x) % ulp) % ulp
+        v.append(x)
+        s = np.float32(s + np.float32(x))
+    dy = torch.as_tensor(np.repeat(np.array(v, dtype=np.float32)[:, None], 16, 1)).cuda()
+    x16, dy16 = torch.zeros(64, 16, dtype=torch.bfloat16, device="cuda"), dy.bfloat16()
+    dw, db = torch.zeros(27, 16, 16, device="cuda"), torch.zeros(16, device="cuda")
+    err = torch.zeros(1, dtype=torch.int32, device="cuda")
+    assert B.load().lasto_nn_conv3d_wgrad_tc(1, (ctypes.c_int * 3)(4, 4, 4), 16, 16, B._ptr(x16), B._ptr(dy16), B._ptr(dy),
+                                             B._ptr(dw), B._ptr(db), B._ptr(err), B._stream()) == 0
+    torch.cuda.synchronize()
+    exact = sum(v)
+    # eight sums of eight rows and their three levels: ten roundings
+    assert float((db.double() - exact).abs().max()) <= 10 * 2.0 ** -24 * exact
