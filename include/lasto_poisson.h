@@ -113,17 +113,16 @@ typedef struct lasto_config {
     int boundary;     /* enum lasto_boundary: Dirichlet values on the box faces */
     int nu_coarse;    /* pre/post sweeps per level on the coarse levels the FP32 cycle of the
                          mixed precision runs inside one thread block (at most 17 nodes per axis,
-                         above the exact solve); >= 0.  The other levels use nu1/nu2.  Grids whose
-                         cycle solves a larger coarse level exactly (65 nodes per axis and more)
-                         have no such levels. */
+                         above the exact solve); >= 0.  The other levels use nu1/nu2.  Only grids
+                         of at most 33 nodes on every axis have such levels: the cycle of a
+                         larger one solves a larger coarse level exactly. */
     int nu_fine;      /* pre/post sweeps on the finest level when > 0 (0: nu1/nu2 there too) */
 } lasto_config;
 
 /* Fills cfg with the defaults: n_max 129, max_atoms 561, max_batch 1, FP64, PCG,
  * multipole faces, nu1 = nu2 = 4 (the fastest time to 1e-10 measured on GB300 for both precisions: more sweeps
- * per level cost less than the CG iterations and reductions they save), nu_coarse = 4 (1 keeps
- * the Pd55 129^3 iteration count and shortens each cycle, but costs iterations on smaller
- * grids), nu_fine = 0, 50 cycles, rel_tol 1e-10, 16 x 32 sphere points, graph launch. */
+ * per level cost less than the CG iterations and reductions they save), nu_coarse = 4,
+ * nu_fine = 0, 50 cycles, rel_tol 1e-10, 16 x 32 sphere points, graph launch. */
 void lasto_config_default(lasto_config* cfg);
 
 typedef struct lasto_cluster {
