@@ -112,6 +112,12 @@ struct ClusterPlan {
     }
 };
 
+// the multipoles' tables and planes, or the exact faces' five moments per atom
+size_t face_scratch_doubles(const int n[3], int n_atoms)
+{
+    return std::max(multipole_scratch_doubles(n), 5 * (size_t)std::max(n_atoms, 1));
+}
+
 size_t cluster_bytes(const int n[3], int n_atoms)
 {
     // generous upper bound computed by a dry run of the carver
@@ -132,7 +138,7 @@ size_t cluster_bytes(const int n[3], int n_atoms)
         for (int d = 0; d < 3; d++) nn[d] = (nn[d] + 1) / 2;
     }
     c.take<double>((size_t)SPHERE_REC_DOUBLES * std::max(n_atoms, 1));
-    c.take<double>(multipole_scratch_doubles(n));
+    c.take<double>(face_scratch_doubles(n, n_atoms));
     c.take<double>(((size_t)n[0] * n[1] * n[2] + 255) / 256 + 64);
     c.take<double>(32);
     c.take<Ctl>(1);
@@ -181,7 +187,7 @@ bool carve_cluster(Carver& c, const int n[3], int n_atoms, ClusterPlan& P)
         for (int d = 0; d < 3; d++) nn[d] = (nn[d] + 1) / 2;
     }
     P.rec = c.take<double>((size_t)SPHERE_REC_DOUBLES * std::max(n_atoms, 1));
-    P.mom = c.take<double>(multipole_scratch_doubles(n));
+    P.mom = c.take<double>(face_scratch_doubles(n, n_atoms));
     P.nparts = (int)(((size_t)n[0] * n[1] * n[2] + 255) / 256);
     P.part = c.take<double>((size_t)P.nparts + 64);
     P.Q = c.take<double>(32);
@@ -726,7 +732,7 @@ int enqueue_rhs(lasto_poisson* h, ClusterPlan& P, const lasto_cluster& cl, const
         TRY(launch_multipoles(n, cl.x, cl.y, cl.z, F.b, cl.centre, tabs, plane, P.Q, s));
         TRY(launch_boundary_fill(n, cl.x, cl.y, cl.z, cl.centre[0], cl.centre[1], cl.centre[2], P.Q, F.u, s));
     } else if (h->cfg.boundary == LASTO_BC_EXACT) {
-        TRY(launch_boundary_exact(cl, tabs, F.u, s));   // the multipole scratch holds the moments
+        TRY(launch_boundary_exact(cl, P.mom, F.u, s));
     }   // LASTO_BC_ZERO: the faces stay 0 (Eq. 3.3)
     if (guess) {
         k_copy_interior<<<(unsigned)((n[1] - 2) * (n[2] - 2)), 128, 0, s>>>(guess, F.u, n[0], n[1], n[2]);

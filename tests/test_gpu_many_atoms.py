@@ -73,3 +73,25 @@ def test_raw_deposit_refuses_more():
                       np.ones((12801, 16)))
     with pytest.raises(RuntimeError):
         B.lasto_op_raw_deposit(rc)
+
+
+def test_exact_faces_of_many_atoms_on_a_small_grid():
+    """A solve whose atoms' five moments need more room than the grid's multipole tables."""
+    import torch
+    B = need_gpu()
+    na, n = 600, 17
+    cl = synth.workloads.make_cluster("lattice", 2.0 * _lattice(na, 9) - 8.0, np.random.default_rng(na), n=n, half_width=12.0,
+                                      h_min=1.5, h_max=1.5)
+    cl.R[:] = 0.6
+    dc = B.DeviceCluster(cl, axes=(np.linspace(-12.0, 12.0, n),) * 3)
+    u = torch.zeros((n, n, n), dtype=torch.float64, device="cuda")
+    B.lasto_op_boundary_exact(dc, u)
+    for precision in (B.LASTO_PREC_FP64, B.LASTO_PREC_MIXED):
+        solver = B.Poisson(n_max=n, max_atoms=na, precision=precision, boundary=B.LASTO_BC_EXACT)
+        v, pot = torch.empty((na, 25), dtype=torch.float64, device="cuda"), torch.empty_like(u)
+        st = solver.solve(dc, v, potential=pot)[0]
+        torch.cuda.synchronize()
+        assert st.status == 0 and st.rel_resid <= 1e-10, (st.status, st.rel_resid)
+        face = torch.ones_like(u, dtype=torch.bool)
+        face[1:-1, 1:-1, 1:-1] = False
+        assert torch.equal(pot[face], u[face])
