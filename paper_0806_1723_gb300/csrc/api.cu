@@ -723,7 +723,7 @@ int enqueue_rhs(lasto_poisson* h, ClusterPlan& P, const lasto_cluster& cl, const
         TRY(launch_raw_deposit(ra, P.rec, F.b, nullptr, P.status, s));
     } else {
         TRY(launch_sphere_params(cl, cl.x, cl.y, cl.z, P.rec, nullptr, nullptr, nullptr, nullptr, P.status, s));
-        TRY(launch_deposit(cl, P.rec, h->cfg.precision, F.b, nullptr, nullptr, nullptr, P.status, s));
+        TRY(launch_deposit(cl, P.rec, h->cfg.precision, F.b, nullptr, P.status, s));
     }
     double* tabs = P.mom;
     double* plane = tabs + 5 * ((size_t)n[0] + n[1] + n[2]);
@@ -1936,7 +1936,7 @@ int lasto_op_deposit(const lasto_cluster* cl, int precision, double* b, int* own
     if (!rec.p) return LASTO_ERR_NO_MEMORY;
     cudaError_t e = launch_sphere_params(*cl, cl->x, cl->y, cl->z, rec.as<double>(), nullptr, nullptr, nullptr,
                                          nullptr, status, s);
-    if (e == cudaSuccess) e = launch_deposit(*cl, rec.as<double>(), precision, b, owner, nullptr, nullptr, status, s);
+    if (e == cudaSuccess) e = launch_deposit(*cl, rec.as<double>(), precision, b, owner, status, s);
     return op_status(e);
 }
 

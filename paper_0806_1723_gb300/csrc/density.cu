@@ -364,7 +364,6 @@ struct DepArgs {
     int n[3];
     const double* ax[3];
     const double* rec;
-    const double* clm;
     double* b;
     int* owner;
     int* status;
@@ -400,8 +399,8 @@ constexpr int DF_MAX_ATOMS = 2432;      // most atoms the FP32-pair form takes (
 // bytes of a launch's index lists
 static size_t deposit_smem(bool mixed, int na) { return sizeof(int) * (mixed ? 4 : 2) * (size_t)na; }
 
-cudaError_t launch_deposit(const lasto_cluster& cl, const double* rec, int precision, double* b, int* owner,
-                           const double* /*xm_tab*/, double* /*row_mom*/, int* status, cudaStream_t s)
+cudaError_t launch_deposit(const lasto_cluster& cl, const double* rec, int precision, double* b, int* owner, int* status,
+                           cudaStream_t s)
 {
     cudaError_t e = ensure_monomials();
     if (e != cudaSuccess) return e;
@@ -412,7 +411,6 @@ cudaError_t launch_deposit(const lasto_cluster& cl, const double* rec, int preci
     a.ax[1] = cl.y;
     a.ax[2] = cl.z;
     a.rec = rec;
-    a.clm = cl.c_lm;
     a.b = b;
     a.owner = owner;
     a.status = status;
@@ -1405,11 +1403,7 @@ cudaError_t launch_multipoles(const int n[3], const double* x, const double* y, 
     return cudaGetLastError();
 }
 
-// (the exact faces' five moments per atom use the same array)
-size_t multipole_scratch_doubles(const int n[3])
-{
-    return 5 * ((size_t)n[0] + n[1] + n[2]) + 5 * (size_t)n[1] * n[2] + 15 * (size_t)n[2];
-}
+size_t multipole_scratch_doubles(const int n[3]) { return 5 * ((size_t)n[0] + n[1] + n[2]) + 15 * (size_t)n[2]; }
 
 // ---------------------------------------------------------------- Dirichlet faces
 // slot of x^a y^b z^c (a + b + c = l, 1 <= l <= 4): degree offset + s(s+1)/2 + c, s = b + c

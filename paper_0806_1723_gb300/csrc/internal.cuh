@@ -412,8 +412,8 @@ constexpr int SPHERE_REC_DOUBLES = 116;
 cudaError_t launch_sphere_params(const lasto_cluster& cl, const double* ax0, const double* ax1, const double* ax2,
                                  double* rec, double* q, double* rhoR, double* drhoR, double* coef, int* status,
                                  cudaStream_t s);
-cudaError_t launch_deposit(const lasto_cluster& cl, const double* rec, int precision, double* b, int* owner,
-                           const double* xm_tab, double* row_mom, int* status, cudaStream_t s);
+cudaError_t launch_deposit(const lasto_cluster& cl, const double* rec, int precision, double* b, int* owner, int* status,
+                           cudaStream_t s);
 size_t multipole_scratch_doubles(const int n[3]);
 cudaError_t launch_multipoles(const int n[3], const double* x, const double* y, const double* z, const double* b,
                               const double centre[3], double* tabs, double* plane, double* Q, cudaStream_t s);

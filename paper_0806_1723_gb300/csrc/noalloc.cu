@@ -58,6 +58,6 @@ extern "C" int lasto_op_deposit_noalloc(const lasto_cluster* cl, int precision, 
     // the sphere kernel writes every record the deposit reads, so nothing needs clearing
     cudaError_t e = lasto::launch_sphere_params(*cl, cl->x, cl->y, cl->z, rec, nullptr, nullptr, nullptr, nullptr,
                                                 status, s);
-    if (e == cudaSuccess) e = lasto::launch_deposit(*cl, rec, precision, b, owner, nullptr, nullptr, status, s);
+    if (e == cudaSuccess) e = lasto::launch_deposit(*cl, rec, precision, b, owner, status, s);
     return lasto::op_status(e);
 }
