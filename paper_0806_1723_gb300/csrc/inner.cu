@@ -334,14 +334,18 @@ __device__ __forceinline__ double block_incl_scan(double v, double* wsum)
     return v;
 }
 
-// One block per (atom, IS_LM harmonics).  The radii and their reciprocals once, then per harmonic
+// One block per (atom, `lms` harmonics).  The radii and their reciprocals once, then per harmonic
 // the integrands at the mesh points, the cubic-rule integral over each interval, I1 as a prefix
 // sum and I2 as a suffix sum of the intervals (each thread a contiguous run of intervals, the
-// runs' totals scanned across the block), and V_LM.  Bound: FP64 issue.  The exponential of a
-// radius costs more than its share of a harmonic, so five harmonics share it, and no division is
-// left per point: Pd55, 429 radii 164 us (a block per harmonic) -> 116 us.
+// runs' totals scanned across the block), and V_LM.  Bound: FP64 issue, or for few atoms a block's own
+// chain.  The exponential of a radius costs more than its share of a harmonic, so five harmonics share
+// it where the atoms fill the SMs, and no division is left per point; up to IS_ONE atoms a block takes
+// one harmonic (bitwise the same).  429 radii, a block per harmonic with divisions, then with
+// one and with five harmonics per block: 1 atom 24, 23, 74 us; 13 atoms 53, 47, 74; 40 atoms 119,
+// 105, 115; 55 atoms 166, 137, 115 us.
 constexpr int IS_LM = 5;
-__global__ void __launch_bounds__(IS_NT) k_inner_solve(int na, const double* __restrict__ R,
+constexpr int IS_ONE = 40;
+__global__ void __launch_bounds__(IS_NT) k_inner_solve(int lms, const double* __restrict__ R,
                                                        const double* __restrict__ Z, int n, double r_min,
                                                        const double* __restrict__ rho_lm,
                                                        const double* __restrict__ vR, double* __restrict__ v)
@@ -354,7 +358,7 @@ __global__ void __launch_bounds__(IS_NT) k_inner_solve(int na, const double* __r
     double* g2 = g1 + n;
     double* s1 = g2 + n;
     double* s2 = s1 + n;
-    const int a = blockIdx.x / (NLM / IS_LM), lm0 = (blockIdx.x % (NLM / IS_LM)) * IS_LM;
+    const int a = blockIdx.x / (NLM / lms), lm0 = (blockIdx.x % (NLM / lms)) * lms;
     const double Ra = R[a];
     const double h = log(Ra / r_min) / (n - 1);
     for (int j = threadIdx.x; j < n; j += IS_NT) {
@@ -366,7 +370,7 @@ __global__ void __launch_bounds__(IS_NT) k_inner_solve(int na, const double* __r
     // contiguous runs of intervals per thread: [c0, c1)
     const int m = n - 1, per = (m + IS_NT - 1) / IS_NT;
     const int c0 = min(m, (int)threadIdx.x * per), c1 = min(m, c0 + per);
-    for (int lm = lm0; lm < lm0 + IS_LM; lm++) {
+    for (int lm = lm0; lm < lm0 + lms; lm++) {
         const int L = l_of_lm(lm);
         const double* rho = rho_lm + ((size_t)a * NLM + lm) * n;
         double* out = v + ((size_t)a * NLM + lm) * n;
@@ -467,7 +471,8 @@ cudaError_t launch_inner_solve(int na, const double* R, const double* Z, int n_r
                                          (int)(sizeof(double) * 6 * IS_MAX));
     if (e != cudaSuccess) return e;
     static_assert(NLM % IS_LM == 0, "groups of harmonics");
-    k_inner_solve<<<(unsigned)(na * (NLM / IS_LM)), IS_NT, smem, s>>>(na, R, Z, n_rad, r_min, rho_lm, vR, v);
+    const int lms = na <= IS_ONE ? 1 : IS_LM;
+    k_inner_solve<<<(unsigned)(na * (NLM / lms)), IS_NT, smem, s>>>(lms, R, Z, n_rad, r_min, rho_lm, vR, v);
     return cudaGetLastError();
 }
 
