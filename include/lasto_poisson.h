@@ -424,7 +424,7 @@ int lasto_selftest_bounded_wait(double seconds, int* status, void* stream);
 /* Self-test of what a convolution kernel does when such a wait runs out: the kernel that
  * lasto_nn_conv3d_fwd_tc (which 0; m: packed weights, out: y32 with cout channels per node) or
  * lasto_nn_conv3d_wgrad_tc (which 1; m: dy16, out: dw) launches for these sizes, with waits
- * that run out at once.  A block that meets one (forward: 48 input channels and more) leaves
+ * that run out at once (cout 16, 32 or 64).  A block that meets one (forward: cin 48 and more) leaves
  * `out` alone, waits for its copies and matrix instructions, gives its tensor memory back and
  * sets *err.  Asynchronous on the stream; the stream stays usable. */
 int lasto_selftest_conv_wait(int which, int nb, const int dims[3], int cin, int cout, const void* x, const void* m,

@@ -15,13 +15,13 @@
 // thread issues the MMA of a stage and commits it to the stage's mbarrier, which releases the
 // stage for the copies of the step five later.  After the last step every thread reads its node's row of the
 // accumulator (tcgen05.ld 32x32b: warp w owns tensor-memory lanes 32w .. 32w+31) and applies
-// bias, ReLU and the output conversions.  Every mbarrier wait is bounded (`limit` attempts inside
-// the loops): on a timeout the kernel records an error, stops issuing, waits (again bounded) for its
+// bias, ReLU and the output conversions.  Every mbarrier wait is bounded: on a timeout the kernel records an error, stops issuing, waits (again bounded) for its
 // copies and for the last MMA it issued, which may still read its shared memory and write its
 // tensor memory, frees the latter and returns.
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <climits>
 
 #include "internal.cuh"
 
@@ -59,10 +59,13 @@ __host__ __device__ constexpr uint32_t make_idesc(int n)
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(TC_M >> 4) << 24);
 }
 
-// (a limit of 0: gives up at once)
-__device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, long long limit = TC_SPIN_LIMIT)
+// QUIT: gives up at once (the self-test; a limit that the kernels take as an argument costs their loops
+// 2 to 5 %)
+template <bool QUIT = false>
+__device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity)
 {
-    for (long long it = 0; it < limit; it++) {
+    if (QUIT) return false;
+    for (long long it = 0; it < TC_SPIN_LIMIT; it++) {
         uint32_t ok;
         asm volatile(
             "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
@@ -89,12 +92,12 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v)
 
 // y = act(conv(x, w) + bias) for one 128-node tile; with part != null the raw sums of tap
 // group blockIdx.y go to part[blockIdx.y][node][COUT] instead.
-template <int COUT>
+template <int COUT, bool QUIT>
 __global__ void __launch_bounds__(TC_M) k_conv_tc(Grid g, int cin, const bf16* __restrict__ x,
                                                  const uint4* __restrict__ wpk, const float* __restrict__ bias,
                                                  int relu, float* __restrict__ y32, int ldy32, int off32,
                                                  bf16* __restrict__ y16, int ldy16, int off16,
-                                                 float* __restrict__ part, long long limit, int* __restrict__ err)
+                                                 float* __restrict__ part, int* __restrict__ err)
 {
     constexpr int A_BYTES = TC_M * 32;
     constexpr int B_BYTES = COUT * 32;
@@ -103,12 +106,16 @@ __global__ void __launch_bounds__(TC_M) k_conv_tc(Grid g, int cin, const bf16* _
     __shared__ __align__(1024) unsigned char sB[TC_STAGES][B_BYTES];
     __shared__ __align__(8) unsigned long long mbar[TC_STAGES];
     __shared__ uint32_t tmem_slot;
-    bool bad = false;   // a wait ran out
+    // the first step in whose iteration a wait ran out.  Threads compare it with their own step behind
+    // that step's barrier, so that they leave at the same one, also where a faster thread has set it for
+    // the next already.  (A barrier that carries the flag itself costs 6 % of the kernel.)
+    __shared__ int give_up;
     const int tid = threadIdx.x, warp = tid >> 5;
     const size_t N = g.nodes();
     const size_t node0 = (size_t)blockIdx.x * TC_M;
 
     if (tid == 0) {
+        give_up = INT_MAX;
         for (int s = 0; s < TC_STAGES; s++)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&mbar[s])) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -149,7 +156,7 @@ __global__ void __launch_bounds__(TC_M) k_conv_tc(Grid g, int cin, const bf16* _
     auto prefetch = [&](int k) {
         const int st = k % TC_STAGES;
         if (k >= TC_STAGES) {
-            if (!mbar_wait(smem_u32(&mbar[st]), (uint32_t)((k / TC_STAGES - 1) & 1), limit)) bad = true;
+            if (!mbar_wait<QUIT>(smem_u32(&mbar[st]), (uint32_t)((k / TC_STAGES - 1) & 1))) atomicMin(&give_up, k - TC_AHEAD);
         }
         const int tap = tap_a + k / cpt, c0 = (k % cpt) * 16;
         const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
@@ -174,6 +181,7 @@ __global__ void __launch_bounds__(TC_M) k_conv_tc(Grid g, int cin, const bf16* _
         asm volatile("cp.async.commit_group;\n" ::: "memory");
     }
     int issued = 0;   // steps
+    bool bad = false;
     for (int kc = 0; kc < nk; kc++) {
         const int s = kc % TC_STAGES;
         if (kc + TC_AHEAD < nk) prefetch(kc + TC_AHEAD);
@@ -181,8 +189,8 @@ __global__ void __launch_bounds__(TC_M) k_conv_tc(Grid g, int cin, const bf16* _
         asm volatile("cp.async.wait_group %0;\n" ::"n"(TC_AHEAD) : "memory");   // step kc's copies have landed
         // make the shared-memory writes visible to the tensor core (async proxy)
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-        bad = __syncthreads_or(bad);   // (every thread leaves at the same step)
-        if (bad) break;
+        __syncthreads();
+        if (*(volatile int*)&give_up <= kc) break;
         if (tid == 0) {
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
             const uint64_t ad = make_desc(smem_u32(sA[s])), bd = make_desc(smem_u32(sB[s]));
@@ -203,7 +211,7 @@ __global__ void __launch_bounds__(TC_M) k_conv_tc(Grid g, int cin, const bf16* _
         const int s = (issued - 1) % TC_STAGES;
         if (!mbar_wait(smem_u32(&mbar[s]), (uint32_t)(((issued - 1) / TC_STAGES) & 1))) bad = true;
     }
-    bad = __syncthreads_or(bad);
+    bad = __syncthreads_or(bad || issued < nk);
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     if (!bad) {
         const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);
@@ -329,11 +337,11 @@ inline size_t sq_smem(int W, int cin, int cout)
     return (cin > 16 ? 2 : 1) * ((size_t)6 * sq_seg(W) * 16 + (size_t)27 * 32 * cout);
 }
 
-template <int COUT>
+template <int COUT, bool QUIT>
 __global__ void __launch_bounds__(SQ_NT + 32) k_conv_seq(Seq q, int cin, int cout, const bf16* __restrict__ x, const uint4* __restrict__ wpk,
                                                     const float* __restrict__ bias, int relu, float* __restrict__ y32,
                                                     int ldy32, int off32, bf16* __restrict__ y16, int ldy16, int off16,
-                                                    long long limit, int* __restrict__ err)
+                                                    int* __restrict__ err)
 {
     constexpr int NCOL = 2 * COUT <= 32 ? 32 : 2 * COUT <= 64 ? 64 : 2 * COUT <= 128 ? 128 : 256;
     extern __shared__ __align__(1024) unsigned char sq_raw[];
@@ -364,7 +372,7 @@ __global__ void __launch_bounds__(SQ_NT + 32) k_conv_seq(Seq q, int cin, int cou
     // channels 16 c .. 16 c + 15 into buffer c & 1 (after the MMAs that last read it): a lane pair
     // per position, 32 contiguous bytes
     auto load = [&](int c) {
-        if (c >= 2 && !mbar_wait(smem_u32(&mbar[c % 2]), (uint32_t)((c / 2 - 1) & 1), limit)) {
+        if (c >= 2 && !mbar_wait<QUIT>(smem_u32(&mbar[c % 2]), (uint32_t)((c / 2 - 1) & 1))) {
             bad = true;
             return;
         }
@@ -539,10 +547,10 @@ struct GridDiv {
     DivMagic w, h, d;
 };
 
-template <int COUT>
+template <int COUT, bool QUIT>
 __global__ void __launch_bounds__(TC_M) k_conv_wgrad_tc(Grid g, GridDiv gd, int cin, const bf16* __restrict__ x,
                                                        const bf16* __restrict__ dy, float* __restrict__ dw,
-                                                       long long limit, int* __restrict__ err)
+                                                       int* __restrict__ err)
 {
     constexpr int B_BYTES = COUT * 2 * WG_STEP;
     constexpr int NCOL = COUT <= 32 ? 32 : (COUT <= 64 ? 64 : 128);
@@ -551,7 +559,10 @@ __global__ void __launch_bounds__(TC_M) k_conv_wgrad_tc(Grid g, GridDiv gd, int 
     unsigned char* sB = wg_smem_raw + WG_STAGES * WG_A_BYTES;      // [WG_STAGES][B_BYTES]
     __shared__ __align__(8) unsigned long long mbar[WG_STAGES];
     __shared__ uint32_t tmem_slot;
-    bool bad = false;   // a wait ran out
+    // the first step in whose iteration a wait ran out.  Threads compare it with their own step behind
+    // that step's barrier, so that they leave at the same one, also where a faster thread has set it for
+    // the next already.  (A barrier that carries the flag itself costs 6 % of the kernel.)
+    __shared__ int give_up;
     const int tid = threadIdx.x, warp = tid >> 5;
     const size_t N = g.nodes();
     const size_t node0 = (size_t)blockIdx.x * WG_CHUNK;
@@ -564,6 +575,7 @@ __global__ void __launch_bounds__(TC_M) k_conv_wgrad_tc(Grid g, GridDiv gd, int 
     for (int t = tid; t < WG_STAGES * (WG_A_BYTES + B_BYTES) / 16; t += TC_M)
         reinterpret_cast<uint4*>(wg_smem_raw)[t] = make_uint4(0, 0, 0, 0);
     if (tid == 0) {
+        give_up = INT_MAX;
         for (int st = 0; st < WG_STAGES; st++)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&mbar[st])) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -587,7 +599,7 @@ __global__ void __launch_bounds__(TC_M) k_conv_wgrad_tc(Grid g, GridDiv gd, int 
     auto prefetch = [&](int k) {
         const int st = k % WG_STAGES;
         if (k >= WG_STAGES) {
-            if (!mbar_wait(smem_u32(&mbar[st]), (uint32_t)((k / WG_STAGES - 1) & 1), limit)) bad = true;
+            if (!mbar_wait<QUIT>(smem_u32(&mbar[st]), (uint32_t)((k / WG_STAGES - 1) & 1))) atomicMin(&give_up, k - WG_AHEAD);
         }
         // A: piece p = (node kk, row group r8), r8 fastest (one node's row read contiguously)
         for (int p = tid; p < WG_STEP * r8n; p += TC_M) {
@@ -625,14 +637,15 @@ __global__ void __launch_bounds__(TC_M) k_conv_wgrad_tc(Grid g, GridDiv gd, int 
         asm volatile("cp.async.commit_group;\n" ::: "memory");
     }
     int issued = 0;   // steps
+    bool bad = false;
     for (int kc = 0; kc < nk; kc++) {
         const int st = kc % WG_STAGES;
         if (kc + WG_AHEAD < nk) prefetch(kc + WG_AHEAD);
         asm volatile("cp.async.commit_group;\n" ::: "memory");
         asm volatile("cp.async.wait_group %0;\n" ::"n"(WG_AHEAD) : "memory");
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-        bad = __syncthreads_or(bad);   // (every thread leaves at the same step)
-        if (bad) break;
+        __syncthreads();
+        if (*(volatile int*)&give_up <= kc) break;
         if (tid == 0) {
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
 #pragma unroll
@@ -656,7 +669,7 @@ __global__ void __launch_bounds__(TC_M) k_conv_wgrad_tc(Grid g, GridDiv gd, int 
         const int st = (issued - 1) % WG_STAGES;
         if (!mbar_wait(smem_u32(&mbar[st]), (uint32_t)(((issued - 1) / WG_STAGES) & 1))) bad = true;
     }
-    bad = __syncthreads_or(bad);
+    bad = __syncthreads_or(bad || issued < nk);
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     if (!bad && nk > 0) {
         // thread tid owns accumulator row m = tid (tensor-memory lane tid)
@@ -722,10 +735,10 @@ __device__ __noinline__ float ws_node_sum(const Seq& q, int k0, int k1, int e, i
     return s;
 }
 
-template <int COUT>
+template <int COUT, bool QUIT>
 __global__ void __launch_bounds__(WS_NT + 32) k_conv_wgrad_seq(Seq q, int cin, int cg, int most, const bf16* __restrict__ x,
                                                           const bf16* __restrict__ dy, float* __restrict__ dw,
-                                                          long long limit, int* __restrict__ err)
+                                                          int* __restrict__ err)
 {
     constexpr int DX = ws_dx(COUT), N = DX * COUT, TAPS = ws_groups(COUT), USED = TAPS * N;   // a group: DX taps
     constexpr int NCOL = USED <= 128 ? 128 : USED <= 256 ? 256 : 512;
@@ -762,7 +775,7 @@ __global__ void __launch_bounds__(WS_NT + 32) k_conv_wgrad_seq(Seq q, int cin, i
 
     auto load = [&](int k) {
         const int s = k & 1, p0 = ((int)blockIdx.x + k * (int)gridDim.x) * WS_K;
-        if (k >= 2 && !mbar_wait(smem_u32(&mbar[s]), (uint32_t)((k / 2 - 1) & 1), limit)) {
+        if (k >= 2 && !mbar_wait<QUIT>(smem_u32(&mbar[s]), (uint32_t)((k / 2 - 1) & 1))) {
             bad = true;
             return;
         }
@@ -845,7 +858,7 @@ __global__ void __launch_bounds__(WS_NT + 32) k_conv_wgrad_seq(Seq q, int cin, i
         if (tid < WS_NT && k + 1 < nk) load(k + 1);   // while these are issued
         if (k + 1 == nk || k + 1 == first + run) {
             // (commits complete in issue order)
-            if (!mbar_wait(smem_u32(&mbar[k & 1]), (uint32_t)((k / 2) & 1), limit)) bad = true;
+            if (!mbar_wait<QUIT>(smem_u32(&mbar[k & 1]), (uint32_t)((k / 2) & 1))) bad = true;
             bad = __syncthreads_or(bad);
             if (bad) break;
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
@@ -878,7 +891,7 @@ int conv_fwd_tc(int nb, const int dims[3], int cin, int cout, const void* x, con
                 size_t scratch_floats, int* err, void* stream, bool give_up)
 {
     using namespace tc;
-    const long long limit = give_up ? 0 : TC_SPIN_LIMIT;
+    if (give_up && cout != 16 && cout != 32 && cout != 64) return LASTO_ERR_INVALID_ARG;   // the self-test's sizes
     if (nb < 1 || !dims || cin % 16 || cin < 16 || !x || !wpk ||
         !(cout == 16 || cout == 32 || cout == 48 || cout == 64 || cout == 96 || cout == 128))
         return LASTO_ERR_INVALID_ARG;
@@ -904,35 +917,41 @@ int conv_fwd_tc(int nb, const int dims[3], int cin, int cout, const void* x, con
     const size_t sm = sq_smem(g.W, cin, cout / half);
     if (make_seq(g, &q) && (!scratch || cin <= 64 || q.total / SQ_M >= cin / 8) && sm <= 200 * 1024) {
         const dim3 tiles((unsigned)((q.total + SQ_M - 1) / SQ_M), (unsigned)half);
-#define LASTO_SQ_CASE(C)                                                                                            \
-    case C:                                                                                                         \
-        if (cudaFuncSetAttribute(k_conv_seq<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) !=         \
-            cudaSuccess)                                                                                            \
-            return LASTO_ERR_CUDA;                                                                                  \
-        k_conv_seq<C><<<tiles, SQ_NT + 32, sm, s>>>(q, cin, cout, X, W, bias, relu, y32, ldy32, off32, Y16, ldy16, off16,  \
-                                                    limit, err);                                                    \
+#define LASTO_SQ_CASE(C, Q)                                                                                           \
+    case C + Q:                                                                                                       \
+        if (cudaFuncSetAttribute(k_conv_seq<C, Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) !=        \
+            cudaSuccess)                                                                                              \
+            return LASTO_ERR_CUDA;                                                                                    \
+        k_conv_seq<C, Q><<<tiles, SQ_NT + 32, sm, s>>>(q, cin, cout, X, W, bias, relu, y32, ldy32, off32, Y16, ldy16, off16, \
+                                                    err);                                                             \
         break;
-        switch (cout / half) {
-            LASTO_SQ_CASE(16)
-            LASTO_SQ_CASE(32)
-            LASTO_SQ_CASE(48)
-            LASTO_SQ_CASE(64)
+        switch (cout / half + (give_up ? 1 : 0)) {
+            LASTO_SQ_CASE(16, 0)
+            LASTO_SQ_CASE(32, 0)
+            LASTO_SQ_CASE(48, 0)
+            LASTO_SQ_CASE(64, 0)
+            LASTO_SQ_CASE(16, 1)
+            LASTO_SQ_CASE(32, 1)
+            LASTO_SQ_CASE(64, 1)
         }
 #undef LASTO_SQ_CASE
         return cudaGetLastError() == cudaSuccess ? LASTO_OK : LASTO_ERR_CUDA;
     }
-#define LASTO_TC_CASE(C)                                                                                           \
-    case C:                                                                                                        \
-        k_conv_tc<C><<<grid, TC_M, 0, s>>>(g, cin, X, W, bias, relu, y32, ldy32, off32, Y16, ldy16, off16, part,   \
-                                           limit, err);                                                            \
+#define LASTO_TC_CASE(C, Q)                                                                                           \
+    case C + Q:                                                                                                       \
+        k_conv_tc<C, Q><<<grid, TC_M, 0, s>>>(g, cin, X, W, bias, relu, y32, ldy32, off32, Y16, ldy16, off16, part,   \
+                                           err);                                                                      \
         break;
-    switch (cout) {
-        LASTO_TC_CASE(16)
-        LASTO_TC_CASE(32)
-        LASTO_TC_CASE(48)
-        LASTO_TC_CASE(64)
-        LASTO_TC_CASE(96)
-        LASTO_TC_CASE(128)
+    switch (cout + (give_up ? 1 : 0)) {
+        LASTO_TC_CASE(16, 0)
+        LASTO_TC_CASE(32, 0)
+        LASTO_TC_CASE(48, 0)
+        LASTO_TC_CASE(64, 0)
+        LASTO_TC_CASE(96, 0)
+        LASTO_TC_CASE(128, 0)
+        LASTO_TC_CASE(16, 1)
+        LASTO_TC_CASE(32, 1)
+        LASTO_TC_CASE(64, 1)
         default: return LASTO_ERR_INVALID_ARG;
     }
 #undef LASTO_TC_CASE
@@ -948,7 +967,7 @@ int conv_wgrad_tc(int nb, const int dims[3], int cin, int cout, const void* x, c
                   int* err, void* stream, bool give_up)
 {
     using namespace tc;
-    const long long limit = give_up ? 0 : TC_SPIN_LIMIT;
+    if (give_up && cout != 16 && cout != 32 && cout != 64) return LASTO_ERR_INVALID_ARG;   // the self-test's sizes
     if (nb < 1 || !dims || cin % 16 || cin < 16 || cin > 128 || !x || !dy16 || !dw ||
         !(cout == 16 || cout == 32 || cout == 48 || cout == 64 || cout == 96 || cout == 128))
         return LASTO_ERR_INVALID_ARG;
@@ -973,38 +992,44 @@ int conv_wgrad_tc(int nb, const int dims[3], int cin, int cout, const void* x, c
         const dim3 grid((unsigned)std::min(nchunk, std::max(1, 152 / ny)), (unsigned)ny);
         // a sum of at most WG_CHUNK nodes, as in the gathered form (the pads add nothing)
         const int most = (int)((size_t)WG_CHUNK * (size_t)q.total / g.nodes() / WS_K);
-#define LASTO_WS_CASE(C)                                                                                              \
-    case C:                                                                                                           \
-        if (cudaFuncSetAttribute(k_conv_wgrad_seq<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) !=     \
+#define LASTO_WS_CASE(C, Q)                                                                                           \
+    case C + Q:                                                                                                       \
+        if (cudaFuncSetAttribute(k_conv_wgrad_seq<C, Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) !=  \
             cudaSuccess)                                                                                              \
             return LASTO_ERR_CUDA;                                                                                    \
-        k_conv_wgrad_seq<C><<<grid, WS_NT + 32, sm, s>>>(q, cin, cg, most, X, DY, dw, limit, err);                    \
+        k_conv_wgrad_seq<C, Q><<<grid, WS_NT + 32, sm, s>>>(q, cin, cg, most, X, DY, dw, err);                        \
         break;
-        switch (cout) {
-            LASTO_WS_CASE(16)
-            LASTO_WS_CASE(32)
-            LASTO_WS_CASE(48)
-            LASTO_WS_CASE(64)
-            LASTO_WS_CASE(96)
-            LASTO_WS_CASE(128)
+        switch (cout + (give_up ? 1 : 0)) {
+            LASTO_WS_CASE(16, 0)
+            LASTO_WS_CASE(32, 0)
+            LASTO_WS_CASE(48, 0)
+            LASTO_WS_CASE(64, 0)
+            LASTO_WS_CASE(96, 0)
+            LASTO_WS_CASE(128, 0)
+            LASTO_WS_CASE(16, 1)
+            LASTO_WS_CASE(32, 1)
+            LASTO_WS_CASE(64, 1)
         }
 #undef LASTO_WS_CASE
         return cudaGetLastError() == cudaSuccess ? LASTO_OK : LASTO_ERR_CUDA;
     }
-#define LASTO_WG_CASE(C)                                                                                 \
-    case C:                                                                                              \
-        if (cudaFuncSetAttribute(k_conv_wgrad_tc<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, wg_smem(C)) != \
-            cudaSuccess)                                                                                 \
-            return LASTO_ERR_CUDA;                                                                       \
-        k_conv_wgrad_tc<C><<<grid, TC_M, wg_smem(C), s>>>(g, gd, cin, X, DY, dw, limit, err);               \
+#define LASTO_WG_CASE(C, Q)                                                                                           \
+    case C + Q:                                                                                                       \
+        if (cudaFuncSetAttribute(k_conv_wgrad_tc<C, Q>, cudaFuncAttributeMaxDynamicSharedMemorySize, wg_smem(C)) !=   \
+            cudaSuccess)                                                                                              \
+            return LASTO_ERR_CUDA;                                                                                    \
+        k_conv_wgrad_tc<C, Q><<<grid, TC_M, wg_smem(C), s>>>(g, gd, cin, X, DY, dw, err);                             \
         break;
-    switch (cout) {
-        LASTO_WG_CASE(16)
-        LASTO_WG_CASE(32)
-        LASTO_WG_CASE(48)
-        LASTO_WG_CASE(64)
-        LASTO_WG_CASE(96)
-        LASTO_WG_CASE(128)
+    switch (cout + (give_up ? 1 : 0)) {
+        LASTO_WG_CASE(16, 0)
+        LASTO_WG_CASE(32, 0)
+        LASTO_WG_CASE(48, 0)
+        LASTO_WG_CASE(64, 0)
+        LASTO_WG_CASE(96, 0)
+        LASTO_WG_CASE(128, 0)
+        LASTO_WG_CASE(16, 1)
+        LASTO_WG_CASE(32, 1)
+        LASTO_WG_CASE(64, 1)
         default: return LASTO_ERR_INVALID_ARG;
     }
 #undef LASTO_WG_CASE

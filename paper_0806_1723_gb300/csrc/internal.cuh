@@ -467,7 +467,7 @@ int conv_fwd(int nb, const int dims[3], int cin, int cout, const void* x, const 
              float* y32, int ldy32, int off32, void* y16, int ldy16, int off16, float* scratch,
              size_t scratch_floats, void* stream);
 // conv_tc.cu: the same convolution on tcgen05 tensor cores; weights packed once per set.  give_up: the
-// kernels' waits run out at once (the self-test of what a block then does)
+// kernels' waits run out at once (the self-test of what a block then does; cout 16, 32 or 64)
 cudaError_t launch_pack_weights(int cin, int cout, const void* w, void* wpk, cudaStream_t s);
 int conv_fwd_tc(int nb, const int dims[3], int cin, int cout, const void* x, const void* wpk, const float* bias,
                 int relu, float* y32, int ldy32, int off32, void* y16, int ldy16, int off16, float* scratch,
