@@ -373,35 +373,41 @@ cudaError_t launch_rbgs(const LevelT<T>& L, T* u, const T* b, int colour, cudaSt
 }
 
 // ---------------------------------------------------------------- residual / apply
-// One warp per (j, k) row, a pair of nodes (one of each colour) per lane and step.  Bound in FP64:
+// 2^lg lanes per (j, k) row, a warp where rows are long, a pair of nodes (one of each colour) per lane
+// and step.  Bound in FP64:
 // the pipe (0.6 T operations/s here), 8 per node (six neighbours, the diagonal's sum with the row's
 // y and z part, its product) where the flat form spent 10.  RED: the iterate's last half sweep was
 // black, so the black residuals are zero up to rounding and are written as zeros, half the work.
 // FP64: 129 x 97 x 113 nodes 27.4 -> 22.7 us;
 // red only at 129^3 39.6 -> 19.0 us.
+// Rows beyond RS_ROW pairs are split over blocks, as few long ones leave the chip idle, and rows of fewer
+// than 16 pairs share a warp, as an FP64 operation takes the pipe as long for one lane as for 32 (whole calls:
+// 2049 x 9 x 9 nodes 32 us flat, 50 by rows, 32 so; 9 x 257 x 257 31, 78 and 34).
 constexpr int RS_V = 2;
+constexpr int RS_ROW = 256;
 
 template <typename T, int RED>
 __global__ void __launch_bounds__(NT) k_residual(LevelT<T> L, const T* __restrict__ u, const T* __restrict__ b,
-                                                T* __restrict__ r)
+                                                T* __restrict__ r, int lg)
 {
-    const int nx = L.nx, row = (int)(blockIdx.x * (NT / 32) + (threadIdx.x >> 5));
+    const int nx = L.nx, row = (int)(blockIdx.x * (unsigned)(NT >> lg) + (threadIdx.x >> lg)), lanes = 1 << lg;
     if (row >= L.ny * L.nz) return;
-    const int k = row / L.ny, j = row - k * L.ny, lane = threadIdx.x & 31;
+    const int k = row / L.ny, j = row - k * L.ny, lane = threadIdx.x & (unsigned)(lanes - 1);
     const size_t P0 = (size_t)row * nx, sz = (size_t)nx * L.ny;
+    const int m_end = min((int)(blockIdx.y + 1) * RS_ROW, (nx + 1) / 2);   // pairs
     if (j == 0 || k == 0 || j == L.ny - 1 || k == L.nz - 1) {
-        for (int i = lane; i < nx; i += 32) r[P0 + i] = T(0);
+        for (int i = 2 * (int)blockIdx.y * RS_ROW + lane; i < min(2 * m_end, nx); i += lanes) r[P0 + i] = T(0);
         return;
     }
     const T cmy = L.ax[1].cm[j], cpy = L.ax[1].cp[j], cmz = L.ax[2].cm[k], cpz = L.ax[2].cp[k];
     const T dyz = L.ax[1].dg[j] + L.ax[2].dg[k];
-    for (int m0 = lane; 2 * m0 < nx; m0 += 32 * RS_V) {
+    for (int m0 = (int)blockIdx.y * RS_ROW + lane; m0 < m_end; m0 += lanes * RS_V) {
         T v[RS_V][2];
 #pragma unroll
         for (int q = 0; q < RS_V; q++)
 #pragma unroll
             for (int t = 0; t < 2; t++) {   // t = 0: the red node of the pair
-                const int i = 2 * (m0 + 32 * q) + ((j + k + t) & 1);
+                const int i = 2 * (m0 + lanes * q) + ((j + k + t) & 1);
                 v[q][t] = T(0);
                 if ((RED && t) || i < 1 || i > nx - 2) continue;
                 const T* c = u + P0 + i;
@@ -413,7 +419,7 @@ __global__ void __launch_bounds__(NT) k_residual(LevelT<T> L, const T* __restric
         for (int q = 0; q < RS_V; q++)
 #pragma unroll
             for (int t = 0; t < 2; t++) {
-                const int i = 2 * (m0 + 32 * q) + ((j + k + t) & 1);
+                const int i = 2 * (m0 + lanes * q) + ((j + k + t) & 1);
                 if (i < nx) r[P0 + i] = v[q][t];
             }
     }
@@ -434,11 +440,13 @@ template <typename T>
 cudaError_t launch_residual(const LevelT<T>& L, const T* u, const T* b, T* r, bool red_only, cudaStream_t s)
 {
     if (L.lsh) return cudaErrorInvalidValue;   // natural storage only
-    const unsigned g = (unsigned)(((size_t)L.ny * L.nz + NT / 32 - 1) / (NT / 32));
+    const int lg = L.nx > 31 ? 5 : L.nx > 15 ? 4 : L.nx > 7 ? 3 : 2;
+    const dim3 g((unsigned)(((size_t)L.ny * L.nz + (NT >> lg) - 1) / (NT >> lg)),
+                 (unsigned)((L.nx + 2 * RS_ROW - 1) / (2 * RS_ROW)));
     if (red_only)
-        k_residual<T, 1><<<g, NT, 0, s>>>(L, u, b, r);
+        k_residual<T, 1><<<g, NT, 0, s>>>(L, u, b, r, lg);
     else
-        k_residual<T, 0><<<g, NT, 0, s>>>(L, u, b, r);
+        k_residual<T, 0><<<g, NT, 0, s>>>(L, u, b, r, lg);
     return cudaGetLastError();
 }
 
@@ -453,32 +461,39 @@ cudaError_t launch_apply(const LevelT<T>& L, const T* u, T* Au, cudaStream_t s)
 // ---------------------------------------------------------------- transfers
 // Both as marches along z, a thread per coarse column (or column of cells) and tk coarse planes:
 // the per-axis weights are applied one axis after the other, and a plane's x and y part is shared by
-// the coarse planes on both sides of it.  Blocks: 32 x 4 columns, numbered x first.  tk: 4 where that
-// still gives every SM two blocks, else 1 (the smaller levels wait for their loads: 65^3 to 33^3
-// 9.8 us with marches of 4, 5.3 with 1).
-constexpr int TR_TX = 32, TR_TY = 4;
+// the coarse planes on both sides of it.  Blocks: 32 x 4 columns, numbered x first; 16 x 8 or 8 x 16 where
+// there are no more along x and blocks enough for every SM (whole calls on 9 x 257 x 257 nodes: 47 -> 33 and
+// 44 -> 26 us).  tk: 4 where that still gives every SM two blocks, else 1 (the smaller levels wait for
+// their loads: 65^3 to 33^3 9.8 us with marches of 4, 5.3 with 1).
+constexpr int TR_NT = 128;
+struct MarchShape {
+    int lg, tk;   // 2^lg columns along x per block, tk planes
+};
 
 struct March {
     int I, J, K0, K1;
 };
 
-__device__ __forceinline__ March march_of(int mx, int my, int mz, int tk)
+__device__ __forceinline__ March march_of(int mx, int my, int mz, MarchShape f)
 {
-    const int gx = (mx + TR_TX - 1) / TR_TX, gy = (my + TR_TY - 1) / TR_TY;
+    const int tx = 1 << f.lg, ty = TR_NT >> f.lg, gx = (mx + tx - 1) >> f.lg, gy = (my + ty - 1) / ty;
     const int bz = (int)blockIdx.x / (gx * gy), rem = (int)blockIdx.x - bz * gx * gy, by = rem / gx, bx = rem - by * gx;
     March m;
-    m.I = bx * TR_TX + (int)threadIdx.x % TR_TX;
-    m.J = by * TR_TY + (int)threadIdx.x / TR_TX;
-    m.K0 = bz * tk;
-    m.K1 = min(m.K0 + tk, mz);
+    m.I = bx * tx + ((int)threadIdx.x & (tx - 1));
+    m.J = by * ty + ((int)threadIdx.x >> f.lg);
+    m.K0 = bz * f.tk;
+    m.K1 = min(m.K0 + f.tk, mz);
     return m;
 }
 
-static unsigned march_grid(int mx, int my, int mz, int* tk)
+static unsigned march_grid(int mx, int my, int mz, MarchShape* f)
 {
-    const size_t cols = (size_t)((mx + TR_TX - 1) / TR_TX) * ((my + TR_TY - 1) / TR_TY);
-    *tk = cols * ((mz + 3) / 4) >= 2 * 152 ? 4 : 1;
-    return (unsigned)(cols * ((mz + *tk - 1) / *tk));
+    auto cols = [&](int lg) { return (size_t)((mx + (1 << lg) - 1) >> lg) * (size_t)((my + (TR_NT >> lg) - 1) / (TR_NT >> lg)); };
+    f->lg = 5;
+    if (cols(5) * mz >= 4 * 2 * 152) f->lg = mx > 16 ? 5 : mx > 8 ? 4 : 3;
+    const size_t c = cols(f->lg);
+    f->tk = c * ((mz + 3) / 4) >= 2 * 152 ? 4 : 1;
+    return (unsigned)(c * ((mz + f->tk - 1) / f->tk));
 }
 
 // bc = Vc^-1 P^T Vf r: the 27-point stencil factorises into per-axis weights.  uc (optional): the
@@ -487,10 +502,10 @@ static unsigned march_grid(int mx, int my, int mz, int* tk)
 // sum of the products takes 45.  FP64: 129 x 97 x 113 fine nodes 18.0 -> 15.2 us; RED at
 // 129^3 24.8 -> 14.5 us.
 template <typename T, int RED>
-__global__ void __launch_bounds__(TR_TX * TR_TY) k_restrict(LevelT<T> F, LevelT<T> C, const T* __restrict__ r,
-                                                            T* __restrict__ bc, T* __restrict__ uc, int tk)
+__global__ void __launch_bounds__(TR_NT) k_restrict(LevelT<T> F, LevelT<T> C, const T* __restrict__ r,
+                                                            T* __restrict__ bc, T* __restrict__ uc, MarchShape f)
 {
-    March m = march_of(C.nx - 2, C.ny - 2, C.nz, tk);
+    March m = march_of(C.nx - 2, C.ny - 2, C.nz, f);
     if (m.I >= C.nx - 2 || m.J >= C.ny - 2) return;
     m.I++, m.J++;   // interior columns; the ones next to a face write the face's too
     const size_t csz = (size_t)C.nx * C.ny, fsz = (size_t)F.nx * F.ny;
@@ -549,12 +564,12 @@ template <typename T>
 cudaError_t launch_restrict(const LevelT<T>& F, const LevelT<T>& C, const T* r, T* bc, T* uc, bool red_only, cudaStream_t s)
 {
     if (F.lsh || C.lsh) return cudaErrorInvalidValue;
-    int tk;
-    const unsigned g = march_grid(C.nx - 2, C.ny - 2, C.nz, &tk);
+    MarchShape f;
+    const unsigned g = march_grid(C.nx - 2, C.ny - 2, C.nz, &f);
     if (red_only)
-        k_restrict<T, 1><<<g, TR_TX * TR_TY, 0, s>>>(F, C, r, bc, uc, tk);
+        k_restrict<T, 1><<<g, TR_NT, 0, s>>>(F, C, r, bc, uc, f);
     else
-        k_restrict<T, 0><<<g, TR_TX * TR_TY, 0, s>>>(F, C, r, bc, uc, tk);
+        k_restrict<T, 0><<<g, TR_NT, 0, s>>>(F, C, r, bc, uc, f);
     return cudaGetLastError();
 }
 
@@ -563,10 +578,10 @@ cudaError_t launch_restrict(const LevelT<T>& F, const LevelT<T>& C, const T* r, 
 // cell per step: interpolated along x, then y, then z, 3.25 FP64 operations per fine node with
 // the addition, where a node by itself takes 8 (and 10 in a warp of mixed parities).  129^3 in FP64:
 // 44.7 -> 17.5 us.
-__global__ void __launch_bounds__(TR_TX * TR_TY) k_prolong_cells(LevelT<double> F, LevelT<double> C,
-                                                                 const double* __restrict__ ec, double* __restrict__ u, int tk)
+__global__ void __launch_bounds__(TR_NT) k_prolong_cells(LevelT<double> F, LevelT<double> C,
+                                                                 const double* __restrict__ ec, double* __restrict__ u, MarchShape f)
 {
-    const March m = march_of(C.nx - 1, C.ny - 1, C.nz - 1, tk);
+    const March m = march_of(C.nx - 1, C.ny - 1, C.nz - 1, f);
     if (m.I >= C.nx - 1 || m.J >= C.ny - 1) return;
     const double wx0 = F.ax[0].pl[2 * m.I + 1], wx1 = F.ax[0].pr[2 * m.I + 1];
     const double wy0 = F.ax[1].pl[2 * m.J + 1], wy1 = F.ax[1].pr[2 * m.J + 1];
@@ -729,9 +744,9 @@ cudaError_t launch_prolong_add(const LevelT<T>& F, const LevelT<T>& C, const T* 
             k_prolong_add_rows<0><<<g, 256, 0, s>>>(F, C, ec, u, pf);
     } else {
         if (F.lsh) return cudaErrorInvalidValue;
-        int tk;
-        const unsigned g = march_grid(C.nx - 1, C.ny - 1, C.nz - 1, &tk);
-        k_prolong_cells<<<g, TR_TX * TR_TY, 0, s>>>(F, C, ec, u, tk);
+        MarchShape f;
+        const unsigned g = march_grid(C.nx - 1, C.ny - 1, C.nz - 1, &f);
+        k_prolong_cells<<<g, TR_NT, 0, s>>>(F, C, ec, u, f);
     }
     return cudaGetLastError();
 }
