@@ -66,13 +66,14 @@ __device__ __forceinline__ void direct_eig_axis(const AxisStore& A, T* Q, const 
     __shared__ int r_hi[2], r_lo[2], s_done[2];
     const int tid = threadIdx.x, lane = tid & 31;
     const int m = A.n - 2, ld = m + 1 - (m & 1);
-    const T scale = (T)big;
+    __shared__ T s_scale;
+    if (tid == 0) s_scale = (T)big;
     for (int t = tid; t < m * ld; t += EIG_NT) Q[t] = t / ld == t % ld ? (T)1 : (T)0;   // [m][ld]: row i holds eigenvector i
     if (tid == 0) r_hi[0] = r_hi[1] = r_lo[0] = r_lo[1] = 0;
     __syncthreads();
     for (int i = tid; i < m; i += EIG_NT) {
-        d[i] = (T)(-A.dg[i + 1] / (double)scale);
-        e[i] = i + 1 < m ? (T)(sqrt(A.cp[i + 1] * A.cm[i + 2]) / (double)scale) : (T)0;
+        d[i] = (T)(-A.dg[i + 1] / (double)s_scale);
+        e[i] = i + 1 < m ? (T)(sqrt(A.cp[i + 1] * A.cm[i + 2]) / (double)s_scale) : (T)0;
     }
     __syncthreads();
     const T eps = sizeof(T) == 4 ? (T)6e-8 : (T)1.1e-16;
@@ -163,7 +164,7 @@ __device__ __forceinline__ void direct_eig_axis(const AxisStore& A, T* Q, const 
         out.Ft[dim][i * mp + p] = (O)(v * sv);
     }
     for (int p = tid; p < m; p += EIG_NT) {
-        const O v = (O)(d[p] * scale), most = (O)-low;
+        const O v = (O)(d[p] * s_scale), most = (O)-low;
         out.lam[dim][p] = v > most ? most : v;   // (a NaN stays one)
     }
 }
@@ -175,13 +176,14 @@ __global__ void __launch_bounds__(EIG_NT) k_direct_eig(AxisStore ax0, AxisStore 
     __shared__ double s_big;
     const int dim = blockIdx.x;
     const AxisStore& A = dim == 0 ? ax0 : dim == 1 ? ax1 : ax2;
+    const double length = A.c[A.n - 1] - A.c[0], low = 8.0 / (length * length);
     if (threadIdx.x == 0) {
         double big = 0.0;
         for (int i = 1; i <= A.n - 2; i++) big = fmax(big, A.dg[i]);
         s_big = big;
     }
     __syncthreads();
-    const double big = s_big, length = A.c[A.n - 1] - A.c[0], low = 8.0 / (length * length);
+    const double big = s_big;
     if (sizeof(T) == 4 && 6e-8 * big > EIG_WIDE * low)
         direct_eig_axis(A, reinterpret_cast<double*>(eig_sm), out, dim, mp, big, low);
     else
