@@ -609,7 +609,9 @@ __global__ void __launch_bounds__(TC_M) k_conv_wgrad_tc(Grid g, GridDiv gd, int 
             bool in = node < N;
             size_t nbn = 0;
             if (in) {
-                const unsigned r = (unsigned)node, q1 = div_by(r, gd.w), q2 = div_by(q1, gd.h), b = div_by(q2, gd.d);
+                // (the reciprocals have no form for 1)
+                const unsigned r = (unsigned)node, q1 = g.W > 1 ? div_by(r, gd.w) : r, q2 = g.H > 1 ? div_by(q1, gd.h) : q1,
+                               b = g.D > 1 ? div_by(q2, gd.d) : q2;
                 const int xx = (int)(r - q1 * (unsigned)g.W), yy = (int)(q1 - q2 * (unsigned)g.H);
                 const int z = (int)(q2 - b * (unsigned)g.D);
                 const int tap = tap0 + tl;

@@ -103,3 +103,19 @@ def test_bias_gradient_sums_pairwise():
     exact = sum(v)
     # eight sums of eight rows and their three levels: ten roundings
     assert float((db.double() - exact).abs().max()) <= 10 * 2.0 ** -24 * exact
+
+
+@pytest.mark.parametrize("cin,cout,nb,dims", [(16, 16, 3, (1000, 1, 9)), (32, 48, 2, (1000, 9, 1)), (64, 32, 2, (900, 1, 1)),
+                                              (16, 16, 3, (1, 7, 18)), (64, 96, 1, (7, 1, 18)), (48, 16, 2, (7, 18, 1)),
+                                              (32, 32, 4, (1, 1, 1))])
+def test_axes_of_one_node(cin, cout, nb, dims):
+    """Gathered rows (beyond about 450 nodes) and the padded sequence."""
+    import torch
+    B = need_gpu()
+    g = torch.Generator(device="cuda").manual_seed(dims[0])
+    N = nb * dims[0] * dims[1] * dims[2]
+    x = torch.randn(N, cin, generator=g, device="cuda").bfloat16()
+    dy = torch.randn(N, cout, generator=g, device="cuda").bfloat16()
+    got, ref = wgrad(B, x, dy, nb, dims, cin, cout).double(), wgrad_ref(x, dy, nb, dims)
+    # FP32 sums: the bound of the kernels' own tests
+    assert float((got - ref).abs().max()) <= 2e-5 * float(ref.abs().max())
