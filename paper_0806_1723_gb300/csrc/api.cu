@@ -505,7 +505,8 @@ int tune_level(lasto_poisson* h, LevelStore& S, LevelStore* C, bool finest, cuda
         least = std::min(least, c.us);
     }
     // colour-split storage costs the CG's vector kernels a little (129^3: phases of 72.2 us over split
-    // and 76.3 over natural storage give the same solve)
+    // and 76.3 over natural storage give the same solve; with that factor the choice is the faster
+    // solve's at each of 65, 97, 113, 129, 161, 193, 225 and 257 nodes, the closest 97: 1.83 natural, 1.86 ms split)
     auto cost = [&](const SmoothChoice& c) { return c.fused == 3 ? 1.055f * c.us : c.us; };
     SmoothChoice best;
     best.us = 1e30f;
@@ -535,7 +536,8 @@ int bottom_level(const ClusterPlan& P)
 // and the levels below, or -1.  The first level below the finest that is small enough; level 1
 // only for the FP32 cycle and above 33 nodes: in FP64 the products of a 65^3 level cost what its
 // smoothing does (160 us), and a 65^3 solve keeps its 33^3 level smoothed because its tuning
-// table, which callers read and set, lists that level.  Levels of up to 97 nodes in FP32 against
+// table, which callers read and set, lists that level (Pd13 65^3 1.04 ms; 0.74 with the 33^3 level
+// exact).  Levels of up to 97 nodes in FP32 against
 // up to 49, measured: Pd55 129^3 (65^3 against 33^3) 3677 and 4468 us, Pd561 385^3 (97^3 against
 // 49^3) 41.5 and 43.3 ms, an uneven batch of eight the same within its 2 %.
 template <typename T>

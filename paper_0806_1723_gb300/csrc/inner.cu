@@ -334,7 +334,7 @@ __device__ __forceinline__ double block_incl_scan(double v, double* wsum)
     return v;
 }
 
-// One block per (atom, `lms` harmonics).  The radii and their reciprocals once, then per harmonic
+// One block per (atom, LMS harmonics).  The radii and their reciprocals once, then per harmonic
 // the integrands at the mesh points, the cubic-rule integral over each interval, I1 as a prefix
 // sum and I2 as a suffix sum of the intervals (each thread a contiguous run of intervals, the
 // runs' totals scanned across the block), and V_LM.  Bound: FP64 issue, or for few atoms a block's own
@@ -345,7 +345,8 @@ __device__ __forceinline__ double block_incl_scan(double v, double* wsum)
 // 105, 115; 55 atoms 166, 137, 115 us.
 constexpr int IS_LM = 5;
 constexpr int IS_ONE = 40;
-__global__ void __launch_bounds__(IS_NT) k_inner_solve(int lms, const double* __restrict__ R,
+template <int LMS>
+__global__ void __launch_bounds__(IS_NT) k_inner_solve(const double* __restrict__ R,
                                                        const double* __restrict__ Z, int n, double r_min,
                                                        const double* __restrict__ rho_lm,
                                                        const double* __restrict__ vR, double* __restrict__ v)
@@ -358,7 +359,7 @@ __global__ void __launch_bounds__(IS_NT) k_inner_solve(int lms, const double* __
     double* g2 = g1 + n;
     double* s1 = g2 + n;
     double* s2 = s1 + n;
-    const int a = blockIdx.x / (NLM / lms), lm0 = (blockIdx.x % (NLM / lms)) * lms;
+    const int a = blockIdx.x / (NLM / LMS), lm0 = (blockIdx.x % (NLM / LMS)) * LMS;
     const double Ra = R[a];
     const double h = log(Ra / r_min) / (n - 1);
     for (int j = threadIdx.x; j < n; j += IS_NT) {
@@ -370,7 +371,7 @@ __global__ void __launch_bounds__(IS_NT) k_inner_solve(int lms, const double* __
     // contiguous runs of intervals per thread: [c0, c1)
     const int m = n - 1, per = (m + IS_NT - 1) / IS_NT;
     const int c0 = min(m, (int)threadIdx.x * per), c1 = min(m, c0 + per);
-    for (int lm = lm0; lm < lm0 + lms; lm++) {
+    for (int lm = lm0; lm < lm0 + LMS; lm++) {
         const int L = l_of_lm(lm);
         const double* rho = rho_lm + ((size_t)a * NLM + lm) * n;
         double* out = v + ((size_t)a * NLM + lm) * n;
@@ -467,12 +468,13 @@ cudaError_t launch_inner_solve(int na, const double* R, const double* Z, int n_r
 {
     if (n_rad > IS_MAX) return cudaErrorInvalidValue;
     const size_t smem = sizeof(double) * 6 * (size_t)n_rad;
-    cudaError_t e = cudaFuncSetAttribute(k_inner_solve, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)(sizeof(double) * 6 * IS_MAX));
-    if (e != cudaSuccess) return e;
     static_assert(NLM % IS_LM == 0, "groups of harmonics");
     const int lms = na <= IS_ONE ? 1 : IS_LM;
-    k_inner_solve<<<(unsigned)(na * (NLM / lms)), IS_NT, smem, s>>>(lms, R, Z, n_rad, r_min, rho_lm, vR, v);
+    auto* kernel = lms == 1 ? k_inner_solve<1> : k_inner_solve<IS_LM>;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)(sizeof(double) * 6 * IS_MAX));
+    if (e != cudaSuccess) return e;
+    kernel<<<(unsigned)(na * (NLM / lms)), IS_NT, smem, s>>>(R, Z, n_rad, r_min, rho_lm, vR, v);
     return cudaGetLastError();
 }
 
