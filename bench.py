@@ -1104,12 +1104,12 @@ def deposit_rate(B, synth, stream, flush, dev, probes):
 
 # One Pd561 385^3 deposit launch (k_deposit_df) under ncu (`bench.py --profile deposit`, second
 # launch; one single-pass capture per group of metrics): FP32 FLOP from the sass
-# thread-instruction counts (2 per FFMA: 52.8 G, 1 per FADD: 87.7 G and per FMUL: 58.9 G), the
+# thread-instruction counts (2 per FFMA: 52.8 G, 1 per FADD: 88.2 G and per FMUL: 58.9 G), the
 # warp instructions issued (smsp__inst_executed.sum) and the DRAM bytes (read 1.3 MB + written
-# 638.1 MB).
-DEPOSIT_FP32_FLOP = 252.2e9
-DEPOSIT_WARP_INST = 11.218e9
-DEPOSIT_DRAM_BYTES = 639.4e6
+# 636.8 MB).
+DEPOSIT_FP32_FLOP = 252.7e9
+DEPOSIT_WARP_INST = 11.237e9
+DEPOSIT_DRAM_BYTES = 638.1e6
 MAX_SM_MHZ = 2070.0   # the GB300's maximum SM clock (the clock the timed runs hold)
 
 

@@ -17,8 +17,8 @@
 namespace lasto {
 
 // ---------------------------------------------------------------- eigenvectors
-// One block per axis: the implicit QL algorithm for symmetric tridiagonal matrices (Bowdler,
-// Martin, Reinsch and Wilkinson, 1968) on S scaled by its largest element, in the precision of the
+// One block per axis: the implicit QL algorithm for symmetric tridiagonal matrices (Dubrulle,
+// Martin and Wilkinson, 1968) on S scaled by its largest element, in the precision of the
 // cycle it serves.  Q is a product of plane rotations, so it is orthogonal whatever the axis --
 // also for the near-degenerate pairs of an axis with two refined regions -- and e = Q D Q^T b stays
 // symmetric whatever the rounding.  Definite, which the conjugate gradients also ask of their
@@ -30,7 +30,7 @@ namespace lasto {
 // One lane runs the scalar chain (a rotation is about ten dependent operations)
 // and the other warps apply the rotations of the QL step before to Q, a component per thread.
 // Bound: that chain's latency; it runs beside the deposit.  Parallel cyclic Jacobi in the same
-// place took 697 us at m = 63; this 253 us (m = 95: 510 us; FP64: 279 us at m = 15, 900 us at m = 31).
+// place took 697 us at m = 63; this 253 us (m = 95: 510 us; FP64: 282 us at m = 15, 900 us at m = 31).
 constexpr int EIG_NT = 128;
 // FP64 where FP32's eps times the largest element passes this part of the bound on the smallest
 // eigenvalue: below it that eigenvalue is right to about a seventh.  On 129 nodes over 80 bohr that is at a
