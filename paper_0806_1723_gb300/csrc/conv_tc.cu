@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(TC_M) k_conv_tc(Grid g, int cin, const bf16* _
     // the first step in whose iteration a wait ran out.  Threads compare it with their own step behind
     // that step's barrier, so that they leave at the same one, also where a faster thread has set it for
     // the next already.  (A barrier that carries the flag itself costs 6 % of the kernel.)
-    __shared__ int give_up;
+    __shared__ volatile int give_up;
     const int tid = threadIdx.x, warp = tid >> 5;
     const size_t N = g.nodes();
     const size_t node0 = (size_t)blockIdx.x * TC_M;
@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(TC_M) k_conv_tc(Grid g, int cin, const bf16* _
     auto prefetch = [&](int k) {
         const int st = k % TC_STAGES;
         if (k >= TC_STAGES) {
-            if (!mbar_wait<QUIT>(smem_u32(&mbar[st]), (uint32_t)((k / TC_STAGES - 1) & 1))) atomicMin(&give_up, k - TC_AHEAD);
+            if (!mbar_wait<QUIT>(smem_u32(&mbar[st]), (uint32_t)((k / TC_STAGES - 1) & 1))) give_up = k - TC_AHEAD;
         }
         const int tap = tap_a + k / cpt, c0 = (k % cpt) * 16;
         const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(TC_M) k_conv_tc(Grid g, int cin, const bf16* _
         // make the shared-memory writes visible to the tensor core (async proxy)
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
         __syncthreads();
-        if (*(volatile int*)&give_up <= kc) break;
+        if (give_up <= kc) break;
         if (tid == 0) {
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
             const uint64_t ad = make_desc(smem_u32(sA[s])), bd = make_desc(smem_u32(sB[s]));
@@ -546,6 +546,11 @@ __device__ __forceinline__ uint64_t make_desc_mn(uint32_t saddr, uint32_t lbo, u
 struct GridDiv {
     DivMagic w, h, d;
 };
+// div_by for divisors from 1 on (l = 0: m = 2^31, a shift by 31)
+__device__ __forceinline__ unsigned div_any(unsigned n, DivMagic q)
+{
+    return (unsigned)(((unsigned long long)n * q.m) >> (32 + q.s));
+}
 
 template <int COUT, bool QUIT>
 __global__ void __launch_bounds__(TC_M) k_conv_wgrad_tc(Grid g, GridDiv gd, int cin, const bf16* __restrict__ x,
@@ -562,7 +567,7 @@ __global__ void __launch_bounds__(TC_M) k_conv_wgrad_tc(Grid g, GridDiv gd, int 
     // the first step in whose iteration a wait ran out.  Threads compare it with their own step behind
     // that step's barrier, so that they leave at the same one, also where a faster thread has set it for
     // the next already.  (A barrier that carries the flag itself costs 6 % of the kernel.)
-    __shared__ int give_up;
+    __shared__ volatile int give_up;
     const int tid = threadIdx.x, warp = tid >> 5;
     const size_t N = g.nodes();
     const size_t node0 = (size_t)blockIdx.x * WG_CHUNK;
@@ -599,7 +604,7 @@ __global__ void __launch_bounds__(TC_M) k_conv_wgrad_tc(Grid g, GridDiv gd, int 
     auto prefetch = [&](int k) {
         const int st = k % WG_STAGES;
         if (k >= WG_STAGES) {
-            if (!mbar_wait<QUIT>(smem_u32(&mbar[st]), (uint32_t)((k / WG_STAGES - 1) & 1))) atomicMin(&give_up, k - WG_AHEAD);
+            if (!mbar_wait<QUIT>(smem_u32(&mbar[st]), (uint32_t)((k / WG_STAGES - 1) & 1))) give_up = k - WG_AHEAD;
         }
         // A: piece p = (node kk, row group r8), r8 fastest (one node's row read contiguously)
         for (int p = tid; p < WG_STEP * r8n; p += TC_M) {
@@ -609,9 +614,7 @@ __global__ void __launch_bounds__(TC_M) k_conv_wgrad_tc(Grid g, GridDiv gd, int 
             bool in = node < N;
             size_t nbn = 0;
             if (in) {
-                // (the reciprocals have no form for 1)
-                const unsigned r = (unsigned)node, q1 = g.W > 1 ? div_by(r, gd.w) : r, q2 = g.H > 1 ? div_by(q1, gd.h) : q1,
-                               b = g.D > 1 ? div_by(q2, gd.d) : q2;
+                const unsigned r = (unsigned)node, q1 = div_any(r, gd.w), q2 = div_any(q1, gd.h), b = div_any(q2, gd.d);
                 const int xx = (int)(r - q1 * (unsigned)g.W), yy = (int)(q1 - q2 * (unsigned)g.H);
                 const int z = (int)(q2 - b * (unsigned)g.D);
                 const int tap = tap0 + tl;
@@ -647,7 +650,7 @@ __global__ void __launch_bounds__(TC_M) k_conv_wgrad_tc(Grid g, GridDiv gd, int 
         asm volatile("cp.async.wait_group %0;\n" ::"n"(WG_AHEAD) : "memory");
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
         __syncthreads();
-        if (*(volatile int*)&give_up <= kc) break;
+        if (give_up <= kc) break;
         if (tid == 0) {
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
 #pragma unroll

@@ -154,7 +154,7 @@ struct AxisT {
 // Division of a node index by an invariant divisor as a multiply-high and a shift: with
 // 2^(l-1) < d <= 2^l and m = ceil(2^(31+l) / d) (which fits in 32 bits), floor(n / d) =
 // floor(m n / 2^(31+l)) for every 0 <= n < 2^31 (Granlund and Montgomery, "Division by
-// invariant integers using multiplication", 1994, Theorem 4.2 with N = 31).  d >= 2.  Node indices stay
+// invariant integers using multiplication", 1994, Theorem 4.2 with N = 31).  div_by: d >= 2.  Node indices stay
 // below 2^31 (checked where grids are accepted).
 struct DivMagic {
     unsigned m;
